@@ -41,13 +41,15 @@ __global__ void __launch_bounds__(kMaxThreads, 1) pagd_batch_kernel(BatchParams 
     extern __shared__ __align__(16) char smem[];
     __shared__ double red[32];
     const int ntw = 1 << B.logtw;
-    double2* t64 = (double2*)smem;
-    float2* t32 = (float2*)(smem + (size_t)ntw * sizeof(double2));
+    longlong2* tfx = (longlong2*)smem;
+    float2* t32 = (float2*)(smem + (size_t)ntw * sizeof(longlong2));
     const int stride = kNMax >> B.logtw;
     for (int m = threadIdx.x; m < ntw; m += blockDim.x) {
-        t64[m] = B.tw64[m * stride];
+        tfx[m] = B.twfx[m * stride];
         t32[m] = B.tw32[m * stride];
     }
+    double* sq = (double*)(t32 + ntw);
+    for (int m = threadIdx.x; m < kSq; m += blockDim.x) sq[m] = (double)(m * m);
     Ctl* ctl = (Ctl*)(smem + tw_smem_bytes(B.logtw));
     long long* G = (long long*)(ctl + B.count);  // cost prefix, count + 1 entries
     char* wsm = smem + tw_smem_bytes(B.logtw) + batch_ctl_bytes(B.count);
@@ -107,7 +109,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) pagd_batch_kernel(BatchParams 
             const long long cost = G[i + 1] - G[i];
             if (cost == 0) continue;
             const Params& P = B.PI[i];
-            Tw t{t64, t32, B.logtw, 0, 0, 0, 0};
+            Tw t{tfx, t32, sq, B.logtw, 0, 0, 0, 0};
             batch_split(t, gw, nw, total, G[i], cost, phase_units(P, ctl[i].ph), (int)weighted_unit_cost(P, ctl[i]));
             batch_exec<T>(P, ctl[i], t, wsm, red);
         }

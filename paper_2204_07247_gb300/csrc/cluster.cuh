@@ -47,6 +47,14 @@ __device__ __forceinline__ unsigned long long gtimer_ns() {
 }
 #endif
 
+// twiddles of a line of T: the FP32 table in shared memory, the FP64 one in
+// global memory (the device-wide passes transform FP64 lines in fixed point)
+template <class T> __device__ __forceinline__ const cx<T>* cl_tw(const Params& P, const Tw& tw) {
+    if constexpr (sizeof(T) == 8) return P.tw64;
+    else return tw.t32;
+}
+template <class T> __device__ __forceinline__ int cl_twlog(const Tw& tw) { return sizeof(T) == 8 ? kLogNMax : tw.log; }
+
 constexpr int kClUnits = 8;              // row pairs and column units per CTA
 constexpr int kClRows = 2 * kClUnits;    // rows per CTA
 constexpr int kClSlots = kClUnits + 1;   // column slots (slot 8 of CTA 0: column n / 2)
@@ -232,7 +240,7 @@ __device__ __forceinline__ void cl_col_pass(const Params& P, const Ctl& c, const
                 const C* src = NBX + (size_t)(x0 >> 1) * ps + (size_t)(f * kClSlots) * 2 + (x0 & 1);
                 b0[(size_t)f * PITCH + x0] = pair ? C{src[0].x, src[2 * kClUnits].x} : src[2 * u];
             }
-        const int r = fft_lines_fixed<-1, T, LOGN, kClMaxK>(b0, b1, PITCH, K, tw_of<T>(tw), tw.log, lane);
+        const int r = fft_lines_fixed<-1, T, LOGN, kClMaxK>(b0, b1, PITCH, K, cl_tw<T>(P, tw), cl_twlog<T>(tw), lane);
         C* Xr = r ? b1 : b0;
         C* Xf = r ? b0 : b1;
         if (!pair) {
@@ -292,7 +300,7 @@ __device__ __forceinline__ void cl_col_pass(const Params& P, const Ctl& c, const
                 }
             }
         }
-        const int r2 = fft_lines_fixed<+1, T, LOGN, kClMaxK>(Xr, Xf, PITCH, K, tw_of<T>(tw), tw.log, lane);
+        const int r2 = fft_lines_fixed<+1, T, LOGN, kClMaxK>(Xr, Xf, PITCH, K, cl_tw<T>(P, tw), cl_twlog<T>(tw), lane);
         const C* Yr = r2 ? Xf : Xr;
         // scatter to the row owners: DBX[k1][f][local row], 16 consecutive rows
         // per owner CTA
@@ -367,7 +375,7 @@ __device__ __forceinline__ void cl_row_pass(const Params& P, const Ctl& c, const
                 }
                 b0[(size_t)f * PITCH + xx] = (xx <= HALF) ? C{A.x - B.y, A.y + B.x} : C{A.x + B.y, B.x - A.y};
             }
-        const int r = fft_lines_fixed<+1, T, LOGN, kClMaxK>(b0, b1, PITCH, K, tw_of<T>(tw), tw.log, lane);
+        const int r = fft_lines_fixed<+1, T, LOGN, kClMaxK>(b0, b1, PITCH, K, cl_tw<T>(P, tw), cl_twlog<T>(tw), lane);
         C* Xr = r ? b1 : b0;
         C* Xf = r ? b0 : b1;
         T amax = (T)0;
@@ -410,7 +418,7 @@ __device__ __forceinline__ void cl_row_pass(const Params& P, const Ctl& c, const
                     else qq->x = out[g];
                 }
             }
-        const int r2 = fft_lines_fixed<-1, T, LOGN, kClMaxK>(Xr, Xf, PITCH, K, tw_of<T>(tw), tw.log, lane);
+        const int r2 = fft_lines_fixed<-1, T, LOGN, kClMaxK>(Xr, Xf, PITCH, K, cl_tw<T>(P, tw), cl_twlog<T>(tw), lane);
         const C* Yr = r2 ? Xf : Xr;
         const T hf = (T)0.5;
         // scatter to the column owners: NBX[pair][f][slot][rr], eight slots of

@@ -24,6 +24,7 @@ extern thread_local EmuDim3 threadIdx, blockIdx, blockDim, gridDim;
 struct alignas(8) float2 { float x, y; };
 struct alignas(16) double2 { double x, y; };
 struct alignas(16) float4 { float x, y, z, w; };
+struct alignas(16) longlong2 { long long x, y; };
 
 inline void __syncthreads() {}
 inline void __threadfence() {}
@@ -39,9 +40,17 @@ template <class T> inline T ldcg(const T* p) { return *p; }
 template <class T> inline T ldg(const T* p) { return *p; }
 inline unsigned long long dbl_bits(double d) { unsigned long long u; std::memcpy(&u, &d, 8); return u; }
 inline double bits_dbl(unsigned long long u) { double d; std::memcpy(&d, &u, 8); return d; }
+inline unsigned flt_bits(float f) { unsigned u; std::memcpy(&u, &f, 4); return u; }
+inline float bits_flt(unsigned u) { float f; std::memcpy(&f, &u, 4); return f; }
+inline float warp_xor(float v, int) { return v; }
 #define PAGD_WARP 1
 template <class T> inline T warp_max(T v) { return v; }
 template <class T> inline T warp_sum(T v) { return v; }
+inline unsigned warp_umax(unsigned v) { return v; }
+inline unsigned warp_uadd(unsigned v) { return v; }
+inline int clz32(unsigned v) { return v ? __builtin_clz(v) : 32; }
+inline int clz64(unsigned long long v) { return v ? __builtin_clzll(v) : 64; }
+inline unsigned atomicMax(unsigned* p, unsigned v) { unsigned o = *p; if (v > o) *p = v; return o; }
 // asynchronous 16-byte global -> shared copies (the emulation copies at once)
 inline void cp_async16(void* dst, const void* src) { std::memcpy(dst, src, 16); }
 inline void cp_async_commit() {}
@@ -54,6 +63,9 @@ template <class T> __device__ __forceinline__ T ldcg(const T* p) { return __ldcg
 template <class T> __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
 __device__ __forceinline__ unsigned long long dbl_bits(double d) { return (unsigned long long)__double_as_longlong(d); }
 __device__ __forceinline__ double bits_dbl(unsigned long long u) { return __longlong_as_double((long long)u); }
+__device__ __forceinline__ unsigned flt_bits(float f) { return __float_as_uint(f); }
+__device__ __forceinline__ float bits_flt(unsigned u) { return __uint_as_float(u); }
+__device__ __forceinline__ float warp_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 #define PAGD_WARP 32
 template <class T> __device__ __forceinline__ T warp_max(T v) {
 #pragma unroll
@@ -68,6 +80,10 @@ template <class T> __device__ __forceinline__ T warp_sum(T v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+__device__ __forceinline__ unsigned warp_umax(unsigned v) { return __reduce_max_sync(0xffffffffu, v); }
+__device__ __forceinline__ unsigned warp_uadd(unsigned v) { return __reduce_add_sync(0xffffffffu, v); }
+__device__ __forceinline__ int clz32(unsigned v) { return __clz((int)v); }
+__device__ __forceinline__ int clz64(unsigned long long v) { return __clzll((long long)v); }
 // Asynchronous 16-byte copy global -> shared (cp.async, cached in L2 only):
 // both addresses 16-byte aligned.  Completion per thread in commit groups:
 // cp_async_wait<N>() returns once at most N of this thread's most recent

@@ -142,10 +142,6 @@ __device__ int fft_line_w(cx<T>* b0, cx<T>* b1, int logN, const cx<T>* tw, int l
     return cur;
 }
 
-}  // namespace pagd
-
-namespace pagd {
-
 // ---------------------------------------------------------------------------
 // Compile-time line length: the radix sequence, the per-lane butterfly loops and
 // the line loop unroll, so the loads of all lines a warp owns are in flight
@@ -325,4 +321,24 @@ __device__ __noinline__ int fft_lines_coop(cx<T>* b0, cx<T>* b1, int pitch, int 
     return cur;
 }
 
+template <int S, class T, int NF>
+__device__ __forceinline__ int fft_coop(cx<T>* b0, cx<T>* b1, int logn, int pitch, int nl, const cx<T>* tw, int logTw,
+                                        int tid, int nthr) {
+    if constexpr (NF > 0) {
+        return fft_lines_coop<S, T, ilog2c(NF)>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
+    } else {
+        switch (logn) {
+            case 3: return fft_lines_coop<S, T, 3>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
+            case 4: return fft_lines_coop<S, T, 4>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
+            case 5: return fft_lines_coop<S, T, 5>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
+            case 6: return fft_lines_coop<S, T, 6>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
+            case 7: return fft_lines_coop<S, T, 7>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
+            case 8: return fft_lines_coop<S, T, 8>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
+            default: return fft_lines_coop<S, T, 9>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
+        }
+    }
+}
+
 }  // namespace pagd
+
+#include "fx.cuh"

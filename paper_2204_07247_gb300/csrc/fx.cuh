@@ -1,0 +1,457 @@
+// fx.cuh -- FP64 line transforms in 64-bit block fixed point.
+//
+// GB300 issues an FP64 instruction (FMA, add or conversion alike) at 1/64 of
+// the FP32 rate: measured 64 cycles per warp instruction on one SM
+// sub-partition whatever the active lanes, 19 cycles per SM with all four busy.
+// A 64-bit integer add costs 0.4 cycles per SM and warp, the fixed-point
+// product below 6.5.  A transform is mostly additions, so the lines of every
+// FP64 pass are transformed as 64-bit integers with one exponent per line: a
+// 256-point line takes about 390 SM cycles of arithmetic against 3700 in FP64.
+//
+// The values enter and leave as doubles.  A line is converted at the scale of
+// its largest element (no bit of any value above 2^-8 of it is lost), the sum of the
+// moduli of its points then fixes how far it has to be shifted so that no
+// partial sum of the transform can overflow, and the result is rounded once
+// to double.  The error against a transform in extended precision is no
+// larger than that of the FP64 one it replaces (tests/test_fx_host.py
+// measures both): about a third of it for lines of up to 256 points and for
+// any line whose energy sits in few points, the same for 512 points of noise.
+// Every partial sum of a radix stage is bounded by the sum of the moduli, so
+// the bound holds for any input; a line with a NaN or an infinity comes out NaN.
+//
+// Layout: 16-byte slots, point i of a line at slot i ^ ((i >> 3) & 7), which
+// spreads the strided stores of the first stages over all bank groups.
+#pragma once
+#include "compat.cuh"
+
+namespace pagd {
+
+template <> struct V2<long long> { using type = longlong2; };
+
+// twiddle tables hold cos, sin in units of 2^-61
+constexpr int kFxTw = 61;
+constexpr int kFxNaN = 1 << 28;  // exponent of a line that holds a NaN or an infinity
+
+__host__ __device__ __forceinline__ int fxs(int i) { return i ^ ((i >> 3) & 7); }
+
+// a w 2^-61 rounded, |a| < 2^62, |w| <= sqrt(2) 2^61: both split into a signed
+// high part and a 31-bit low part; the product of the low parts enters with
+// its leading bits
+__device__ __forceinline__ long long fx_mul(long long a, long long w) {
+    const int ah = (int)(a >> 31), al = (int)(a & 0x7fffffff);
+    const int wh = (int)(w >> 31), wl = (int)(w & 0x7fffffff);
+    long long m = (long long)ah * wl + (long long)wh * al;
+    m += (al >> 16) * (wl >> 15);
+    return (((long long)ah * wh) << 1) + ((m + (1ll << 29)) >> 30);
+}
+// complex product in three real ones
+__device__ __forceinline__ longlong2 fx_cmul(longlong2 a, longlong2 w) {
+    const long long k1 = fx_mul(a.x + a.y, w.x);
+    return longlong2{k1 - fx_mul(a.y, w.x + w.y), k1 + fx_mul(a.x, w.y - w.x)};
+}
+
+template <int S> __device__ __forceinline__ void fx_dft8(longlong2* v) {
+    constexpr long long c = 1630477228166597777ll;  // cos(pi / 4) 2^61
+    longlong2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
+    longlong2 o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
+    dft4<S>(e0, e1, e2, e3);
+    dft4<S>(o0, o1, o2, o3);
+    const longlong2 w1{fx_mul(S < 0 ? o1.x + o1.y : o1.x - o1.y, c), fx_mul(S < 0 ? o1.y - o1.x : o1.y + o1.x, c)};
+    const longlong2 w2 = mul_si<S>(o2);
+    const longlong2 w3{fx_mul(S < 0 ? o3.y - o3.x : -o3.x - o3.y, c), fx_mul(S < 0 ? -o3.x - o3.y : o3.x - o3.y, c)};
+    v[0] = cadd(e0, o0);
+    v[4] = csub(e0, o0);
+    v[1] = cadd(e1, w1);
+    v[5] = csub(e1, w1);
+    v[2] = cadd(e2, w2);
+    v[6] = csub(e2, w2);
+    v[3] = cadd(e3, w3);
+    v[7] = csub(e3, w3);
+}
+template <int R, int S> __device__ __forceinline__ void fx_dft(longlong2* v) {
+    if constexpr (R == 2) dft2<S>(v);
+    else if constexpr (R == 4) dft4<S>(v[0], v[1], v[2], v[3]);
+    else fx_dft8<S>(v);
+}
+
+// ------------------------------------------------------------- conversions
+
+__device__ __forceinline__ unsigned fx_hi(double x) { return (unsigned)(dbl_bits(x) >> 32) & 0x7fffffffu; }
+// exponent field of a line from the largest fx_hi of its values
+__device__ __forceinline__ int fx_emax(unsigned hi) { return (int)(hi >> 20); }
+
+// x in units of 2^(emax - 1083): |result| < 2^61
+__device__ __forceinline__ long long fx_from(double x, int emax) {
+    const unsigned long long b = dbl_bits(x);
+    const int e = (int)(b >> 52) & 0x7ff;
+    unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    int r = emax - e;
+    if (r > 63 || e == 0) r = 63;  // below 2^-62 of the largest: zero
+    const long long v = (long long)((m << 8) >> r);
+    return (long long)b < 0 ? -v : v;
+}
+// upper bound of a point's modulus, in units of 2^41
+__device__ __forceinline__ unsigned fx_mag(longlong2 z) {
+    const int x = (int)(z.x >> 41), y = (int)(z.y >> 41);
+    const unsigned ax = (unsigned)(x < 0 ? -x : x) + 1u, ay = (unsigned)(y < 0 ? -y : y) + 1u;
+    const unsigned M = ax > ay ? ax : ay, m = ax > ay ? ay : ax;
+    return M + ((m * 27u) >> 6) + 1u;
+}
+// right shift that brings a line whose moduli sum to less than s 2^41 below 2^61.5
+__device__ __forceinline__ int fx_shift(unsigned s) {
+    const int lz = clz32(s);
+    const int k = 31 - lz + ((s << lz) > 0xb504f333u ? 1 : 0);
+    return k > 20 ? k - 20 : 0;
+}
+__device__ __forceinline__ long long fx_shr(long long a, int sh, long long half) { return (a + half) >> sh; }
+__device__ __forceinline__ long long fx_half(int sh) { return (1ll << sh) >> 1; }
+
+// a 2^-S as a double (round half away, overflow to infinity, below 2^-1022 to zero)
+__device__ __forceinline__ double fx_to(long long a, int S) {
+    const unsigned long long sgn = (unsigned long long)a & 0x8000000000000000ull;
+    const unsigned long long u = a < 0 ? (unsigned long long)-a : (unsigned long long)a;
+    const int lz = clz64(u);
+    const unsigned long long n = u << (lz & 63);
+    const int E = 1086 - lz - S;
+    unsigned long long t = (n >> 11) + ((n >> 10) & 1ull) + ((unsigned long long)(unsigned)(E - 1) << 52);
+    if (E <= 0 || u == 0) t = 0;
+    if (E >= 2047) t = 0x7ff0000000000000ull;
+    if (S > kFxNaN / 2) t = 0x7ff8000000000000ull;
+    return bits_dbl(t | sgn);
+}
+// the exponent S of a converted line: 2^-S is its unit after the shift sh
+__device__ __forceinline__ int fx_scale(int emax, int sh) { return emax == 0x7ff ? kFxNaN : 1083 - emax - sh; }
+
+// FP64 <-> FP32 conversions with integer instructions: the hardware's issue
+// at the FP64 rate (64 cycles per warp and sub-partition), these are about
+// nine integer instructions each.  Rounded to nearest even; FP32 results below 2^-126
+// become zero, as do FP32 inputs below 2^-126.
+__device__ __forceinline__ float to_f32(double x) {
+    const unsigned long long b = dbl_bits(x), m = b & 0x7fffffffffffffffull;
+    const unsigned hi = (unsigned)(m >> 32);
+    const unsigned long long t = m - (896ull << 52);
+    unsigned r = (unsigned)((t + 0x0fffffffull + ((t >> 29) & 1ull)) >> 29);
+    if (hi < 0x38100000u) r = 0u;                                   // below 2^-126
+    if (hi >= 0x47f00000u) r = m > 0x7ff0000000000000ull ? 0x7fc00000u : 0x7f800000u;  // 2^128 and above, inf, NaN
+    return bits_flt(r | ((unsigned)(b >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ double to_f64(float x) {
+    const unsigned b = flt_bits(x), m = b & 0x7fffffffu;
+    unsigned hi = (m >> 3) + (896u << 20), lo = m << 29;
+    if (m < 0x00800000u) { hi = 0u; lo = 0u; }
+    if (m >= 0x7f800000u) hi += 896u << 20;  // inf, NaN
+    hi |= b & 0x80000000u;
+    return bits_dbl(((unsigned long long)hi << 32) | lo);
+}
+template <class T> __device__ __forceinline__ T cvt(double x) {
+    if constexpr (sizeof(T) == 8) return x;
+    else return to_f32(x);
+}
+__device__ __forceinline__ double wide(double x) { return x; }
+__device__ __forceinline__ double wide(float x) { return to_f64(x); }
+
+// Sum of FP32 values without FP64 instructions: the rounding error of every
+// addition is kept (Knuth's two-sum) and summed beside it, 2^-48 of the sum of
+// the magnitudes.
+struct Sum2 {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = h + x, v = s - h;
+        l += (h - (s - v)) + (x - v);
+        h = s;
+    }
+    __device__ __forceinline__ double warp_total() const {
+        Sum2 t = *this;
+#pragma unroll
+        for (int o = kWarp / 2; o > 0; o >>= 1) {
+            const float h2 = warp_xor(t.h, o), l2 = warp_xor(t.l, o);
+            t.add(h2);
+            t.l += l2;
+        }
+        return (double)t.h + (double)t.l;
+    }
+};
+
+// ---------------------------------------------------------- warp-owned line
+
+template <int R, int S, int LOGN, int LOGNS, bool FIRST>
+__device__ __forceinline__ void fx_stage(longlong2* b, int sh, const longlong2* tw, int logTw, int lane) {
+    constexpr int LR = (R == 2) ? 1 : (R == 4) ? 2 : 3;
+    constexpr int NB = 1 << (LOGN - LR), NS = 1 << LOGNS;
+    constexpr int PER = (NB + kWarp - 1) / kWarp;
+    const int twshift = logTw - (LOGNS + LR);
+    longlong2 v[PER * R];
+    const long long half = fx_half(sh);
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        const int j = lane + kWarp * i;
+        if (NB % kWarp == 0 || j < NB) {
+            const int jm = j & (NS - 1);
+            longlong2* u = v + i * R;
+#pragma unroll
+            for (int r = 0; r < R; r++) {
+                u[r] = b[fxs(j + r * NB)];
+                if (FIRST) u[r] = longlong2{fx_shr(u[r].x, sh, half), fx_shr(u[r].y, sh, half)};
+                if (LOGNS > 0 && r > 0) {
+                    longlong2 w = tw[(jm * r) << twshift];
+                    if (S > 0) w.y = -w.y;
+                    u[r] = fx_cmul(u[r], w);
+                }
+            }
+            fx_dft<R, S>(u);
+        }
+    }
+    warp_sync();
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        const int j = lane + kWarp * i;
+        if (NB % kWarp == 0 || j < NB) {
+            const int jm = j & (NS - 1), d = ((j - jm) << LR) + jm;
+#pragma unroll
+            for (int r = 0; r < R; r++) b[fxs(d + r * NS)] = v[i * R + r];
+        }
+    }
+    warp_sync();
+}
+template <int S, int LOGN, int LOGNS>
+__device__ __forceinline__ void fx_stages(longlong2* b, int sh, const longlong2* tw, int logTw, int lane) {
+    if constexpr (LOGNS < LOGN) {
+        constexpr int R = stage_radix(LOGN, LOGNS);
+        fx_stage<R, S, LOGN, LOGNS, LOGNS == 0>(b, sh, tw, logTw, lane);
+        fx_stages<S, LOGN, LOGNS + radix_log(R)>(b, sh, tw, logTw, lane);
+    }
+}
+
+// One line of 1 << LOGN points (slot layout, converted, to be shifted by sh)
+// transformed in place by one warp.  A function of its own: every pass of a
+// kernel shares its code, and its registers do not add to theirs.  Data
+// written before the call and read after it by any lane.
+template <int S, int LOGN>
+static __device__ __noinline__ void fx_line_n(longlong2* b, int sh, const longlong2* tw, int logTw, int lane) {
+    warp_sync();
+    fx_stages<S, LOGN, 0>(b, sh, tw, logTw, lane);
+}
+// NF: the line length, or 0 for the runtime length 1 << logn (8 .. 512)
+template <int S, int NF>
+__device__ __forceinline__ void fx_line(longlong2* b, int logn, int sh, const longlong2* tw, int logTw, int lane) {
+    if constexpr (NF > 0) {
+        fx_line_n<S, ilog2c(NF)>(b, sh, tw, logTw, lane);
+    } else {
+        switch (logn) {
+            case 3: fx_line_n<S, 3>(b, sh, tw, logTw, lane); break;
+            case 4: fx_line_n<S, 4>(b, sh, tw, logTw, lane); break;
+            case 5: fx_line_n<S, 5>(b, sh, tw, logTw, lane); break;
+            case 6: fx_line_n<S, 6>(b, sh, tw, logTw, lane); break;
+            case 7: fx_line_n<S, 7>(b, sh, tw, logTw, lane); break;
+            case 8: fx_line_n<S, 8>(b, sh, tw, logTw, lane); break;
+            default: fx_line_n<S, 9>(b, sh, tw, logTw, lane); break;
+        }
+    }
+}
+
+// the doubles in one slot -> fixed point in place; returns the point's fx_mag
+__device__ __forceinline__ unsigned fx_point(longlong2* slot, int emax) {
+    const double2 z = *(const double2*)slot;
+    const longlong2 f{fx_from(z.x, emax), fx_from(z.y, emax)};
+    *slot = f;
+    return fx_mag(f);
+}
+// Coefficient k < n / 2 of two rows' half spectra, A[k] in slot k and B[k] in
+// slot n - k (k = 0: the real parts of A[0], B[0] in slot 0, of A[n / 2],
+// B[n / 2] in slot n / 2), -> points k and n - k (n / 2) of the packed complex
+// line A + i B in fixed point
+__device__ __forceinline__ unsigned fx_pair_rows(longlong2* b, int k, int n, int emax) {
+    const int k2 = k == 0 ? n >> 1 : n - k;
+    const double2 a = *(const double2*)&b[fxs(k)], c = *(const double2*)&b[fxs(k2)];
+    longlong2 A{fx_from(a.x, emax), fx_from(a.y, emax)}, B{fx_from(c.x, emax), fx_from(c.y, emax)};
+    if (k != 0) {
+        const longlong2 p{A.x - B.y, A.y + B.x};
+        B = longlong2{A.x + B.y, B.x - A.y};
+        A = p;
+    }
+    b[fxs(k)] = A;
+    b[fxs(k2)] = B;
+    return fx_mag(A) + fx_mag(B);
+}
+// A line of n doubles in its slots (each slot written and read by the lane
+// that owns it, lane + kWarp i) -> fixed point in place.  hi: this lane's
+// largest fx_hi.  Returns the line's exponent e and the shift sh that the
+// transform applies (the transformed line's exponent is e - sh).
+struct FxExp {
+    int e, sh;
+};
+static __device__ __noinline__ FxExp fx_convert(longlong2* b, int n, unsigned hi, int lane) {
+    const int emax = fx_emax(warp_umax(hi));
+    unsigned s = 0;
+#pragma unroll 4
+    for (int i = lane; i < n; i += kWarp) s += fx_point(b + fxs(i), emax);
+    return FxExp{fx_scale(emax, 0), fx_shift(warp_uadd(s))};
+}
+static __device__ __noinline__ FxExp fx_convert_rows(longlong2* b, int n, unsigned hi, int lane) {
+    const int emax = fx_emax(warp_umax(hi)), half = n >> 1;
+    unsigned s = 0;
+#pragma unroll 2
+    for (int k = lane; k < half; k += kWarp) s += fx_pair_rows(b, k, n, emax);
+    return FxExp{fx_scale(emax, 0), fx_shift(warp_uadd(s))};
+}
+
+// Global memory -> slots as doubles, by the threads first, first + step, ...
+// (the lanes of a warp or the threads of a CTA); each returns the largest
+// fx_hi of its values.  The loads of kFxLoad points are in flight together.
+// Functions of their own, like the transforms: every pass shares them.
+constexpr int kFxLoad = 4;
+
+// the two rows' half spectra of one field, as fx_pair_rows reads them
+static __device__ __noinline__ unsigned fx_load_rows(longlong2* b, const double2* s0, int n, int rows, int first, int step) {
+    const int half = n >> 1;
+    unsigned hi = 0;
+    for (int k0 = first; k0 < half; k0 += step * kFxLoad) {
+        double2 a[kFxLoad], c[kFxLoad];
+#pragma unroll
+        for (int q = 0; q < kFxLoad; q++) {
+            const int k = k0 + step * q;
+            if (k < half) {
+                a[q] = s0[(size_t)k * rows];
+                c[q] = s0[(size_t)k * rows + 1];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kFxLoad; q++) {
+            const int k = k0 + step * q;
+            if (k < half) {
+                int k2 = n - k;
+                if (k == 0) {  // k = 0 and n / 2: real coefficients
+                    const double2 ah = s0[(size_t)half * rows], ch = s0[(size_t)half * rows + 1];
+                    a[q].y = c[q].x;
+                    c[q] = double2{ah.x, ch.x};
+                    k2 = half;
+                }
+                const unsigned h0 = fx_hi(a[q].x), h1 = fx_hi(a[q].y), h2 = fx_hi(c[q].x), h3 = fx_hi(c[q].y);
+                const unsigned m0 = h0 > h1 ? h0 : h1, m1 = h2 > h3 ? h2 : h3, m = m0 > m1 ? m0 : m1;
+                hi = m > hi ? m : hi;
+                *(double2*)&b[fxs(k)] = a[q];
+                *(double2*)&b[fxs(k2)] = c[q];
+            }
+        }
+    }
+    return hi;
+}
+// n contiguous points
+static __device__ __noinline__ unsigned fx_load(longlong2* b, const double2* s, int n, int first, int step) {
+    unsigned hi = 0;
+    for (int x0 = first; x0 < n; x0 += step * 2 * kFxLoad) {
+        double2 v[2 * kFxLoad];
+#pragma unroll
+        for (int q = 0; q < 2 * kFxLoad; q++)
+            if (x0 + step * q < n) v[q] = s[x0 + step * q];
+#pragma unroll
+        for (int q = 0; q < 2 * kFxLoad; q++) {
+            if (x0 + step * q < n) {
+                const unsigned a = fx_hi(v[q].x), c = fx_hi(v[q].y), m = a > c ? a : c;
+                hi = m > hi ? m : hi;
+                *(double2*)&b[fxs(x0 + step * q)] = v[q];
+            }
+        }
+    }
+    return hi;
+}
+// a transformed packed line of exponent S -> the two rows' half spectra
+static __device__ __noinline__ void fx_store_rows(const longlong2* b, int n, int S, double2* d0, int rows, int first, int step) {
+#pragma unroll 2
+    for (int k = first; k <= (n >> 1); k += step) {
+        const longlong2 zk = b[fxs(k)], zn = b[fxs((n - k) & (n - 1))];
+        double2* d = d0 + (size_t)k * rows;
+        d[0] = double2{fx_to(zk.x + zn.x, S + 1), fx_to(zk.y - zn.y, S + 1)};
+        d[1] = double2{fx_to(zk.y + zn.y, S + 1), fx_to(zn.x - zk.x, S + 1)};
+    }
+}
+static __device__ __noinline__ void fx_store(const longlong2* b, int n, int S, double2* d, int first, int step) {
+#pragma unroll 2
+    for (int x = first; x < n; x += step) {
+        const longlong2 z = b[fxs(x)];
+        d[x] = double2{fx_to(z.x, S), fx_to(z.y, S)};
+    }
+}
+
+// ------------------------------------------------- lines shared by a CTA
+
+template <int R, int S, int LOGN>
+__device__ __forceinline__ void fx_stage_coop(const longlong2* src, longlong2* dst, int nl, int logNs,
+                                              const unsigned* sums, const longlong2* tw, int logTw, int tid,
+                                              int nthr) {
+    constexpr int LR = (R == 2) ? 1 : (R == 4) ? 2 : 3;
+    constexpr int LNB = LOGN - LR, NB = 1 << LNB;
+    const int twshift = logTw - (logNs + LR), nsm = (1 << logNs) - 1, tot = nl << LNB;
+    for (int it = tid; it < tot; it += nthr) {
+        const int l = it >> LNB, j = it & (NB - 1);
+        const longlong2* s = src + (l << LOGN);
+        longlong2* d = dst + (l << LOGN);
+        longlong2 v[R];
+#pragma unroll
+        for (int r = 0; r < R; r++) v[r] = s[fxs(j + r * NB)];
+        const int jm = j & nsm;
+        if (logNs == 0) {
+            const int sh = fx_shift(sums[l]);
+            const long long half = fx_half(sh);
+#pragma unroll
+            for (int r = 0; r < R; r++) v[r] = longlong2{fx_shr(v[r].x, sh, half), fx_shr(v[r].y, sh, half)};
+        } else {
+#pragma unroll
+            for (int r = 1; r < R; r++) {
+                longlong2 w = tw[(jm * r) << twshift];
+                if (S > 0) w.y = -w.y;
+                v[r] = fx_cmul(v[r], w);
+            }
+        }
+        fx_dft<R, S>(v);
+        const int dd = ((j - jm) << LR) + jm;
+#pragma unroll
+        for (int r = 0; r < R; r++) d[fxs(dd + (r << logNs))] = v[r];
+    }
+}
+
+// nl converted lines of 1 << LOGN points in b0 (sums[l]: line l's sum of
+// fx_mag, complete before the call) -> the transforms in b0 (returns 0) or b1
+// (1), visible to every thread on return.  Radix 8 where it gives at least
+// half of the threads a butterfly, else 4: a stage costs a barrier and a round
+// trip through shared memory (about 120 cycles), a radix-4 butterfly's
+// arithmetic about as much, so narrower stages lose more than they spread.
+template <int S, int LOGN>
+__device__ __noinline__ int fx_lines_coop(longlong2* b0, longlong2* b1, int nl, const unsigned* sums,
+                                          const longlong2* tw, int logTw, int tid, int nthr) {
+    longlong2* b[2] = {b0, b1};
+    int cur = 0, logNs = 0;
+    while (logNs < LOGN) {
+        const int rem = LOGN - logNs;
+        const int lr = (rem >= 3 && 2 * (nl << (LOGN - 3)) >= nthr) ? 3 : (rem >= 2 ? 2 : 1);
+        if (logNs > 0) cta_sync();
+        if (lr == 3) fx_stage_coop<8, S, LOGN>(b[cur], b[cur ^ 1], nl, logNs, sums, tw, logTw, tid, nthr);
+        else if (lr == 2) fx_stage_coop<4, S, LOGN>(b[cur], b[cur ^ 1], nl, logNs, sums, tw, logTw, tid, nthr);
+        else fx_stage_coop<2, S, LOGN>(b[cur], b[cur ^ 1], nl, logNs, sums, tw, logTw, tid, nthr);
+        logNs += lr;
+        cur ^= 1;
+    }
+    cta_sync();
+    return cur;
+}
+
+// NF: the line length, or 0 for the runtime length 1 << logn (8 .. 512)
+template <int S, int NF>
+__device__ __forceinline__ int fx_coop(longlong2* b0, longlong2* b1, int logn, int nl, const unsigned* sums,
+                                       const longlong2* tw, int logTw, int tid, int nthr) {
+    if constexpr (NF > 0) {
+        return fx_lines_coop<S, ilog2c(NF)>(b0, b1, nl, sums, tw, logTw, tid, nthr);
+    } else {
+        switch (logn) {
+            case 3: return fx_lines_coop<S, 3>(b0, b1, nl, sums, tw, logTw, tid, nthr);
+            case 4: return fx_lines_coop<S, 4>(b0, b1, nl, sums, tw, logTw, tid, nthr);
+            case 5: return fx_lines_coop<S, 5>(b0, b1, nl, sums, tw, logTw, tid, nthr);
+            case 6: return fx_lines_coop<S, 6>(b0, b1, nl, sums, tw, logTw, tid, nthr);
+            case 7: return fx_lines_coop<S, 7>(b0, b1, nl, sums, tw, logTw, tid, nthr);
+            case 8: return fx_lines_coop<S, 8>(b0, b1, nl, sums, tw, logTw, tid, nthr);
+            default: return fx_lines_coop<S, 9>(b0, b1, nl, sums, tw, logTw, tid, nthr);
+        }
+    }
+}
+
+}  // namespace pagd

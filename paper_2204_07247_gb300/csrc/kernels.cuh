@@ -66,16 +66,18 @@ __global__ void __launch_bounds__(kMaxThreads, 1) pagd_kernel(const __grid_const
     __shared__ double red[32];
     // twiddles exp(-2 pi i m / 2^logtw) staged from the global table
     const int ntw = 1 << P.logtw;
-    double2* t64 = (double2*)smem;
-    float2* t32 = (float2*)(smem + (size_t)ntw * sizeof(double2));
+    longlong2* tfx = (longlong2*)smem;
+    float2* t32 = (float2*)(smem + (size_t)ntw * sizeof(longlong2));
     const int stride = kNMax >> P.logtw;
     for (int m = threadIdx.x; m < ntw; m += blockDim.x) {
-        t64[m] = P.tw64[m * stride];
+        tfx[m] = P.twfx[m * stride];
         t32[m] = P.tw32[m * stride];
     }
+    double* sq = (double*)(t32 + ntw);
+    for (int m = threadIdx.x; m < kSq; m += blockDim.x) sq[m] = (double)(m * m);
     __syncthreads();
     const int wpb = blockDim.x / kWarp;
-    const Tw tw{t64, t32, P.logtw, (int)(threadIdx.x / kWarp) * (int)gridDim.x + (int)blockIdx.x,
+    const Tw tw{tfx, t32, sq, P.logtw, (int)(threadIdx.x / kWarp) * (int)gridDim.x + (int)blockIdx.x,
                 (int)gridDim.x * wpb, 0, -1};
     char* wsm = smem + tw_smem_bytes(P.logtw);
     // The control state is the same in every thread: it lives in shared memory

@@ -65,7 +65,7 @@ struct pagd_solver {
 
 enum {
     O_SC, O_NORMS, O_SUMS, O_STATS, O_TW64, O_TW32, O_U0, O_U1, O_VB, O_G64, O_VBT, O_LBT, O_DD0,
-    O_DD1, O_SS0, O_SS1, O_C0, O_NB, O_DB, O_CL64, O_NB64, O_DB64, O_MASS, O_TRACE, O_VR64, O_NR64, O_WR64, O_LB64, O_YB, O_X, O_X64, O_GH64, O_LCTL, O_END
+    O_DD1, O_SS0, O_SS1, O_C0, O_NB, O_DB, O_CL64, O_NB64, O_DB64, O_MASS, O_TRACE, O_VR64, O_NR64, O_WR64, O_LB64, O_YB, O_X, O_X64, O_GH64, O_LCTL, O_TWFX, O_END
 };
 
 static pagd_status fail(pagd_solver* s, pagd_status st, const char* msg) {
@@ -121,6 +121,7 @@ static void plan_layout(pagd_solver* s) {
     sz[O_X64] = s->dim == 3 ? sizeof(double2) * H * 3 : 0;
     sz[O_GH64] = sizeof(double2) * H;
     sz[O_LCTL] = sizeof(Ctl);
+    sz[O_TWFX] = sizeof(longlong2) * kNMax;
     static_assert(O_END <= (int)(sizeof(((pagd_solver*)nullptr)->off) / sizeof(size_t)), "offset table too small");
     size_t o = 0;
     for (int i = 0; i < O_END; i++) {
@@ -158,6 +159,9 @@ static Params params_for(const pagd_solver* s, char* w) {
     P.k0sq = (twopi / s->L[0]) * (twopi / s->L[0]);
     P.k1sq = (twopi / s->L[last]) * (twopi / s->L[last]);
     P.kmsq = s->dim == 3 ? (twopi / s->L[1]) * (twopi / s->L[1]) : 0.0;
+    P.k0sqf = (float)P.k0sq;
+    P.k1sqf = (float)P.k1sq;
+    P.kmsqf = (float)P.kmsq;
     P.cellvol = 1.0;
     for (int d = 0; d < s->dim; d++) P.cellvol *= s->L[d] / s->n[d];
     P.eps = s->eps;
@@ -165,6 +169,7 @@ static Params params_for(const pagd_solver* s, char* w) {
     P.eta2 = s->eta2;
     P.tau = s->tau;
     P.M = s->M;
+    P.iM = 1.0 / s->M;
     P.s = s->opts.s;
     P.n_eta = s->opts.n_eta;
     P.accel = s->opts.accel;
@@ -182,6 +187,7 @@ static Params params_for(const pagd_solver* s, char* w) {
     P.stats = (StepStat*)(w + s->off[O_STATS]);
     P.tw64 = (const double2*)(w + s->off[O_TW64]);
     P.tw32 = (const float2*)(w + s->off[O_TW32]);
+    P.twfx = (const longlong2*)(w + s->off[O_TWFX]);
     P.U[0] = (double*)(w + s->off[O_U0]);
     P.U[1] = (double*)(w + s->off[O_U1]);
     P.VB = (double*)(w + s->off[O_VB]);
@@ -216,6 +222,24 @@ static Params params_for(const pagd_solver* s, char* w) {
     return P;
 }
 
+// The twiddle tables exp(-2 pi i m / kNMax) from the host libm in long double.
+struct TwTables {
+    std::vector<double2> t64;
+    std::vector<float2> t32;
+    std::vector<longlong2> tfx;
+    TwTables() : t64(kNMax), t32(kNMax), tfx(kNMax) {
+        const long double one = (long double)(1ull << kFxTw);
+        for (int m = 0; m < kNMax; m++) {
+            const long double ang =
+                -2.0L * 3.141592653589793238462643383279502884L * (long double)m / (long double)kNMax;
+            const long double c = cosl(ang), s = sinl(ang);
+            t64[m] = double2{(double)c, (double)s};
+            t32[m] = float2{(float)t64[m].x, (float)t64[m].y};
+            tfx[m] = longlong2{llroundl(c * one), llroundl(s * one)};
+        }
+    }
+};
+
 static Params base_params(const pagd_solver* s) { return params_for(s, s->ws); }
 
 // ------------------------------------------------------- device plumbing
@@ -243,13 +267,15 @@ template <class T> static pagd_status launch(pagd_solver* s, const Params& P) {
     blockDim.x = 1;
     threadIdx.x = 0;
     const int ntw = 1 << P.logtw;
-    double2* t64 = (double2*)base;
-    float2* t32 = (float2*)(base + (size_t)ntw * sizeof(double2));
+    longlong2* tfx = (longlong2*)base;
+    float2* t32 = (float2*)(base + (size_t)ntw * sizeof(longlong2));
     for (int m = 0; m < ntw; m++) {
-        t64[m] = P.tw64[m * (kNMax >> P.logtw)];
+        tfx[m] = P.twfx[m * (kNMax >> P.logtw)];
         t32[m] = P.tw32[m * (kNMax >> P.logtw)];
     }
-    Tw tw{t64, t32, P.logtw, 0, s->grid, 0, -1};
+    double* sq = (double*)(t32 + ntw);
+    for (int m = 0; m < kSq; m++) sq[m] = (double)(m * m);
+    Tw tw{tfx, t32, sq, P.logtw, 0, s->grid, 0, -1};
     char* wsm = base + tw_smem_bytes(P.logtw);
     Ctl c = ctl_init(P);
     const int nf = fixed_len(P.n0, P.n1);
@@ -330,21 +356,24 @@ static pagd_status run_program(pagd_solver* s, Params& P) {
 }
 
 // The FP32 iteration passes stage their inputs through shared memory
-// (row_pass_staged / col_pass_staged) when a warp slice of warp_bytes holds
-// the staging slots (PFC two, FCH one); fixed line lengths only.  PAGD_STAGED=0 keeps the
-// register-staged passes (the same arithmetic, for comparison).
-static bool stage_fits(const pagd_solver* s, size_t warp_bytes) {
-    const int last = s->dim - 1;
-    const int nf = fixed_len(s->n[0], s->n[last]);
-    if (nf == 0 || s->tsize != 4) return false;
+// (row_pass_staged / col_pass_staged; fixed line lengths only): bytes a warp's
+// slice needs for the staging slots (PFC two, FCH one), 0 where they do not
+// stage.  PAGD_STAGED=0 keeps the register-staged passes (the same arithmetic,
+// for comparison).
+static size_t staged_bytes(const pagd_solver* s) {
+    const int nf = fixed_len(s->n[0], s->n[s->dim - 1]);
+    if (nf == 0 || s->tsize != 4) return 0;
     if (const char* e = std::getenv("PAGD_STAGED"))
-        if (e[0] == '0' && e[1] == 0) return false;
-    const int k = k_iter(s->model);
+        if (e[0] == '0' && e[1] == 0) return 0;
+    const int k = k_iter(s->model), sl = staged_slots(s->model);
+    size_t m = std::max(row_staged_smem(nf, k, staged_row_state(s->model), sl), col_staged_smem(nf, k, 3, sl));
     // the middle passes of a cubic grid stage too (mid_pass_staged)
-    if (s->dim == 3 && s->n[1] == nf && mid_staged_smem(nf) > warp_bytes) return false;
-    const int sl = staged_slots(s->model);
-    return row_staged_smem(nf, k, staged_row_state(s->model), sl) <= warp_bytes &&
-           col_staged_smem(nf, k, 3, sl) <= warp_bytes;
+    if (s->dim == 3 && s->n[1] == nf) m = std::max(m, mid_staged_smem(nf));
+    return (m + 15) & ~(size_t)15;
+}
+static bool stage_fits(const pagd_solver* s, size_t warp_bytes) {
+    const size_t need = staged_bytes(s);
+    return need > 0 && need <= warp_bytes;
 }
 
 // One warp per row unit / column / middle unit.  A CTA has as many warps (at
@@ -355,7 +384,8 @@ static void make_plan(pagd_solver* s) {
     const int last = s->dim - 1, nm = s->dim == 3 ? s->n[1] : 1;
     s->logtw = 0;
     for (int d = 0; d < s->dim; d++) s->logtw = std::max(s->logtw, ilog2(s->n[d]));
-    s->warp_bytes = warp_smem_bytes(s->n[0], s->n[last], s->model, s->tsize, fixed_len(s->n[0], s->n[last]), nm);
+    s->warp_bytes = std::max(warp_smem_bytes(s->n[0], s->n[last], s->model, s->tsize, fixed_len(s->n[0], s->n[last]), nm),
+                             staged_bytes(s));
 #ifdef PAGD_EMU
     const int wpb = 1;
 #else
@@ -377,11 +407,11 @@ static void make_plan(pagd_solver* s) {
     s->smem = tw_smem_bytes(s->logtw) + (size_t)wpb * s->warp_bytes;
     // CTA-cooperative units for the passes with FP64 lines when a phase has
     // fewer units than half the warps (most warps would otherwise idle and an
-    // FP64 line would run on one SM sub-partition); fixed line lengths only.
+    // pass's FP64 work would run on one SM sub-partition).
     // PAGD_COOP=0 / 1 overrides the choice.
-    s->coop = (fixed_len(s->n[0], s->n[last]) != 0 && 2 * units <= (long long)s->grid * wpb) ? 1 : 0;
+    s->coop = 2 * units <= (long long)s->grid * wpb ? 1 : 0;
     if (const char* e = std::getenv("PAGD_COOP")) {
-        if ((e[0] == '0' || e[0] == '1') && e[1] == 0) s->coop = fixed_len(s->n[0], s->n[last]) != 0 ? e[0] - '0' : 0;
+        if ((e[0] == '0' || e[0] == '1') && e[1] == 0) s->coop = e[0] - '0';
     }
     // Cluster-resident iterations (cluster.cuh) on square 2D grids of 64, 128
     // or 256 points per axis, when the cluster buffers fit a CTA's shared
@@ -391,6 +421,8 @@ static void make_plan(pagd_solver* s) {
     // device-wide phases run warp-owned.
     s->cl = 0;
     const int nf = fixed_len(s->n[0], s->n[last]);
+    const size_t coop_need = tw_smem_bytes(s->logtw) + coop_smem(std::max(s->n[0], s->n[last]));
+    if (s->coop && s->smem < coop_need) s->smem = coop_need;
     bool want_cl = false;
     if (const char* e = std::getenv("PAGD_CLUSTER")) want_cl = e[0] == '1' && e[1] == 0;
     if (want_cl && s->dim == 2 && cl_size_for(nf) > 0) {
@@ -513,18 +545,10 @@ pagd_status pagd_set_workspace(pagd_solver* s, void* dev_ptr, size_t bytes) {
     if (bytes < s->ws_bytes) return fail(s, PAGD_ENOMEM, "workspace smaller than pagd_workspace_size");
     s->ws = (char*)dev_ptr;
     s->have_state = 0;
-    // twiddles exp(-2 pi i m / kNMax) from the host libm in long double
-    std::vector<double2> t64(kNMax);
-    std::vector<float2> t32(kNMax);
-    for (int m = 0; m < kNMax; m++) {
-        const long double ang = -2.0L * 3.141592653589793238462643383279502884L * (long double)m / (long double)kNMax;
-        t64[m].x = (double)cosl(ang);
-        t64[m].y = (double)sinl(ang);
-        t32[m].x = (float)t64[m].x;
-        t32[m].y = (float)t64[m].y;
-    }
-    pagd_status st = dcopy(s, s->ws + s->off[O_TW64], t64.data(), sizeof(double2) * kNMax);
-    if (st == PAGD_OK) st = dcopy(s, s->ws + s->off[O_TW32], t32.data(), sizeof(float2) * kNMax);
+    const TwTables t;
+    pagd_status st = dcopy(s, s->ws + s->off[O_TW64], t.t64.data(), sizeof(double2) * kNMax);
+    if (st == PAGD_OK) st = dcopy(s, s->ws + s->off[O_TW32], t.t32.data(), sizeof(float2) * kNMax);
+    if (st == PAGD_OK) st = dcopy(s, s->ws + s->off[O_TWFX], t.tfx.data(), sizeof(longlong2) * kNMax);
     if (st == PAGD_OK) st = dsync(s);
     return st;
 }
@@ -561,7 +585,7 @@ static Params run_params(const pagd_solver* s, double* u_out, double dt, int nst
     Params P = base_params(s);
     const bool imex = s->scheme == PAGD_LBDF2 || s->scheme == PAGD_LMP;
     P.prog = imex ? PROG_IMEX : PROG_RUN;
-    P.tol = tol;
+    P.tol = tol + 0.0;  // -0 becomes +0: the device compares norms as integers
     P.dt = dt;
     P.dt_prev0 = (s->step == 0) ? dt : s->dt_prev;
     P.nsteps = nsteps;
@@ -926,11 +950,14 @@ constexpr size_t kStaticWorkspaceBytes = kStaticScratchBytes - kStaticTwBytes;  
 static_assert(kStaticWorkspaceBytes == 8364032, "the limit stated in include/pagd.h");
 #ifndef PAGD_EMU
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
+static __device__ longlong2 g_static_twfx[kNMax];  // the fixed-point twiddle table
 #else
 alignas(256) static unsigned char g_static_scratch[kStaticScratchBytes];
+static longlong2 g_static_twfx[kNMax];
 #endif
 constexpr int kMaxDevices = 64;
 static void* g_static_ptr[kMaxDevices];
+static const longlong2* g_static_twfx_ptr[kMaxDevices];
 static std::mutex g_static_mu;  // guards g_static_ptr and the one-time set-up
 
 // Device address of the static scratch for the current device, with the
@@ -940,23 +967,20 @@ static std::mutex g_static_mu;  // guards g_static_ptr and the one-time set-up
 // with a synchronous cudaMemcpy.  This happens on the first call on each device
 // (make that first call before any stream capture); the lock makes concurrent
 // first calls from several host threads do it once.
-static pagd_status static_scratch(pagd_solver* s, char** out) {
+static pagd_status static_scratch(pagd_solver* s, char** out, const longlong2** twfx) {
 #ifdef PAGD_EMU
     std::lock_guard<std::mutex> lk(g_static_mu);
     if (!g_static_ptr[0]) {
-        std::vector<double2> t64(kNMax);
-        std::vector<float2> t32(kNMax);
-        for (int m = 0; m < kNMax; m++) {
-            const long double ang = -2.0L * 3.141592653589793238462643383279502884L * (long double)m / (long double)kNMax;
-            t64[m] = double2{(double)cosl(ang), (double)sinl(ang)};
-            t32[m] = float2{(float)t64[m].x, (float)t64[m].y};
-        }
-        std::memcpy(g_static_scratch, t64.data(), sizeof(double2) * kNMax);
-        std::memcpy(g_static_scratch + sizeof(double2) * kNMax, t32.data(), sizeof(float2) * kNMax);
+        const TwTables t;
+        std::memcpy(g_static_scratch, t.t64.data(), sizeof(double2) * kNMax);
+        std::memcpy(g_static_scratch + sizeof(double2) * kNMax, t.t32.data(), sizeof(float2) * kNMax);
+        std::memcpy(g_static_twfx, t.tfx.data(), sizeof(longlong2) * kNMax);
+        g_static_twfx_ptr[0] = g_static_twfx;
         g_static_ptr[0] = g_static_scratch;
     }
     (void)s;
     *out = (char*)g_static_ptr[0];
+    *twfx = g_static_twfx_ptr[0];
     return PAGD_OK;
 #else
     int dev = 0;
@@ -968,24 +992,21 @@ static pagd_status static_scratch(pagd_solver* s, char** out) {
         void* ptr = nullptr;
         e = cudaGetSymbolAddress(&ptr, g_static_scratch);
         if (e != cudaSuccess) return cuda_fail(s, e, "cudaGetSymbolAddress of the static scratch");
-        // twiddles exp(-2 pi i m / kNMax) from the host libm in long double
-        std::vector<double2> t64(kNMax);
-        std::vector<float2> t32(kNMax);
-        for (int m = 0; m < kNMax; m++) {
-            const long double ang = -2.0L * 3.141592653589793238462643383279502884L * (long double)m / (long double)kNMax;
-            t64[m].x = (double)cosl(ang);
-            t64[m].y = (double)sinl(ang);
-            t32[m].x = (float)t64[m].x;
-            t32[m].y = (float)t64[m].y;
-        }
-        e = cudaMemcpy(ptr, t64.data(), sizeof(double2) * kNMax, cudaMemcpyHostToDevice);
+        void* fx = nullptr;
+        e = cudaGetSymbolAddress(&fx, g_static_twfx);
+        if (e != cudaSuccess) return cuda_fail(s, e, "cudaGetSymbolAddress of the static twiddle table");
+        const TwTables t;
+        e = cudaMemcpy(ptr, t.t64.data(), sizeof(double2) * kNMax, cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
-            e = cudaMemcpy((char*)ptr + sizeof(double2) * kNMax, t32.data(), sizeof(float2) * kNMax,
+            e = cudaMemcpy((char*)ptr + sizeof(double2) * kNMax, t.t32.data(), sizeof(float2) * kNMax,
                            cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(fx, t.tfx.data(), sizeof(longlong2) * kNMax, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return cuda_fail(s, e, "cudaMemcpy of the static twiddle tables");
+        g_static_twfx_ptr[dev] = (const longlong2*)fx;
         g_static_ptr[dev] = ptr;
     }
     *out = (char*)g_static_ptr[dev];
+    *twfx = g_static_twfx_ptr[dev];
     return PAGD_OK;
 #endif
 }
@@ -1006,7 +1027,8 @@ pagd_status pagd_step_static(pagd_solver* s, const double* un_dev, const double*
         return fail(s, PAGD_EINVAL, buf);
     }
     char* head = nullptr;
-    pagd_status st = static_scratch(s, &head);
+    const longlong2* twfx = nullptr;
+    pagd_status st = static_scratch(s, &head, &twfx);
     if (st != PAGD_OK) return st;
     char* w = head + kStaticTwBytes;
     const size_t b = sizeof(double) * s->npts;
@@ -1017,13 +1039,14 @@ pagd_status pagd_step_static(pagd_solver* s, const double* un_dev, const double*
     Params P = params_for(s, w);
     P.tw64 = (const double2*)head;
     P.tw32 = (const float2*)(head + sizeof(double2) * kNMax);
+    P.twfx = twfx;
     P.trace = nullptr;  // no phase trace: pagd_get_trace reads the solver's own workspace
     const bool imex = s->scheme == PAGD_LBDF2 || s->scheme == PAGD_LMP;
     P.prog = imex ? PROG_IMEX : PROG_RUN;
     P.ref_valid = 0;  // the static scratch holds no reference spectra
     P.cur0 = 0;
     P.step0 = step_index;
-    P.tol = tol;
+    P.tol = tol + 0.0;  // -0 becomes +0: the device compares norms as integers
     P.dt = dt;
     P.dt_prev0 = step_index == 0 ? dt : dt_prev;
     P.nsteps = 1;
@@ -1204,12 +1227,14 @@ template <class T> static pagd_status batch_launch(pagd_batch* b, const BatchPar
     blockDim.x = (unsigned)b->wpb;
     threadIdx.x = 0;
     const int ntw = 1 << B.logtw;
-    double2* t64 = (double2*)base;
-    float2* t32 = (float2*)(base + (size_t)ntw * sizeof(double2));
+    longlong2* tfx = (longlong2*)base;
+    float2* t32 = (float2*)(base + (size_t)ntw * sizeof(longlong2));
     for (int m = 0; m < ntw; m++) {
-        t64[m] = B.tw64[m * (kNMax >> B.logtw)];
+        tfx[m] = B.twfx[m * (kNMax >> B.logtw)];
         t32[m] = B.tw32[m * (kNMax >> B.logtw)];
     }
+    double* sq = (double*)(t32 + ntw);
+    for (int m = 0; m < kSq; m++) sq[m] = (double)(m * m);
     char* wsm = base + tw_smem_bytes(B.logtw) + batch_ctl_bytes(B.count);
     std::vector<Ctl> ctl(B.count);
     std::vector<long long> G(B.count + 1);
@@ -1233,7 +1258,7 @@ template <class T> static pagd_status batch_launch(pagd_batch* b, const BatchPar
                 for (int i = 0; i < B.count; i++) {
                     if (G[i + 1] <= clo || G[i] >= chi || G[i + 1] == G[i]) continue;
                     const Params& P = B.PI[i];
-                    Tw t{t64, t32, B.logtw, 0, 0, 0, 0};
+                    Tw t{tfx, t32, sq, B.logtw, 0, 0, 0, 0};
                     batch_split(t, gw, nw, total, G[i], G[i + 1] - G[i], phase_units(P, ctl[i].ph),
                                 (int)weighted_unit_cost(P, ctl[i]));
                     batch_exec_host<T>(P, ctl[i], t, wsm, red);
@@ -1284,6 +1309,7 @@ pagd_status pagd_batch_create(pagd_batch** out, pagd_solver* const* members, int
         for (int d = 0; d < s->dim; d++) b->logtw = std::max(b->logtw, ilog2(s->n[d]));
         b->warp_bytes = std::max(b->warp_bytes, warp_smem_bytes(s->n[0], s->n[last], s->model, s->tsize,
                                                                 batch_nf(s->n[0], s->n[last]), nm));
+        if (batch_nf(s->n[0], s->n[last])) b->warp_bytes = std::max(b->warp_bytes, staged_bytes(s));
     }
 #ifdef PAGD_EMU
     const int wpb = kEmuBatchWarps;
@@ -1394,7 +1420,7 @@ static pagd_status batch_chunk(pagd_batch* b, double dt, int nsteps, double tol,
     B.count = count;
     B.logtw = b->logtw;
     B.sc = bsc;
-    B.tw64 = PI[0].tw64;
+    B.twfx = PI[0].twfx;
     B.tw32 = PI[0].tw32;
     // tracing on the first member records the launch's global phases there
     B.trace = s0->trace ? (unsigned long long*)(s0->ws + s0->off[O_TRACE]) : nullptr;

@@ -77,7 +77,7 @@ constexpr int kMaxThreads = 256;
 
 // scheme coefficients of one step (see compute_step_coeffs)
 struct StepK {
-    double a, b, c, thv, ts, Ai, rho, gun, thpc, m2;
+    double a, b, c, thv, ts, Ai, rho, gun, thpc, m2, ith, aim;  // ith = 1 / thv, aim = Ai / M
 };
 
 struct Params {
@@ -93,8 +93,9 @@ struct Params {
     long long H;
     long long npts;
     double k0sq, k1sq, kmsq;  // (2 pi / L)^2 of the first, last and middle axes
+    float k0sqf, k1sqf, kmsqf;
     double cellvol;           // product of the spacings
-    double eps, eta1, eta2, tau, M;
+    double eps, eta1, eta2, tau, M, iM;  // iM = 1 / M
     double s;
     int n_eta, accel, max_iter, max_recheck, theta_mode;
     // the PFC FP32 iteration passes stage their inputs by asynchronous copies
@@ -148,8 +149,10 @@ struct Params {
     // the control state the loop hands back to the device-wide machine (a Ctl)
     int cl;
     void* lctl;
+    // twiddle tables of kNMax entries: FP64 (the cluster loop's), FP32, fixed point
     const double2* tw64;
     const float2* tw32;
+    const longlong2* twfx;
     Scal* sc;
     double* mass;  // persistent {K, D, R}: mass excess since set_state, this step's change, and
                    // R, ||d_0||_inf of the last step started from the extrapolation (0: none)
@@ -170,6 +173,10 @@ struct Params {
     double2* out_spec;
 };
 
+struct Beta {
+    double m2, b0, b2, b4;
+};
+
 struct Ctl {
     int ph, step, it, ev, lastev, cur, rech, fail, best_ev;
     int after, mk, m64;  // 3D middle pass: the phase after it, its fields, FP64 buffers
@@ -185,6 +192,7 @@ struct Ctl {
     int rec_pending, rec_ev, rec_bank;
     int acc, acc_cur, acc_it, acc_lastev, acc_ev, reb, ereb, inc, ref_ok, exact_done;
     double resid, base_nrm, best_nrm, acc_resid;
+    Beta bt;             // averaged Newton constants of the current evaluation
 };
 
 // FP32 iterations stop improving once ||d|| reaches about 1e-7 of the FP64
@@ -201,8 +209,9 @@ constexpr int kStagnation = 12;
 // every SM gets a busy warp before any SM gets a second); else the warp owns
 // the contiguous unit range [ulo, uhi) (batched launches).
 struct Tw {
-    const double2* t64;
+    const longlong2* tfx;  // cos, sin in units of 2^-61 (fx.cuh)
     const float2* t32;
+    const double* sq;      // squares 0 .. kSq - 1
     int log;
     int wr, wn, ulo, uhi;
 };
@@ -220,9 +229,6 @@ __device__ __forceinline__ long long thread_rank(const Tw& t) {
     return (long long)t.wr * kWarp + (long long)(threadIdx.x % kWarp);
 }
 __device__ __forceinline__ long long thread_count(const Tw& t) { return (long long)t.wn * kWarp; }
-template <class T> __device__ __forceinline__ const cx<T>* tw_of(const Tw& t);
-template <> __device__ __forceinline__ const cx<double>* tw_of<double>(const Tw& t) { return t.t64; }
-template <> __device__ __forceinline__ const cx<float>* tw_of<float>(const Tw& t) { return t.t32; }
 
 // ---------------------------------------------------------------- helpers
 
@@ -249,6 +255,8 @@ inline StepK compute_step_coeffs(int scheme, int n, double dt, double dtp, doubl
     k.gun = k.a * (1.0 - k.thv) / k.thv;
     k.thpc = (scheme == S_MP && theta_mode == 0) ? 0.5 : 1.0;
     k.m2 = k.a / M;
+    k.ith = 1.0 / k.thv;
+    k.aim = k.Ai / M;
     return k;
 }
 
@@ -264,29 +272,25 @@ __host__ __device__ __forceinline__ const StepK& step_coeffs(const Params& P, in
     return P.kc[n == 0 ? 0 : (step == 0 ? 1 : 2)];
 }
 
-struct Beta {
-    double m2, b0, b2, b4;
-};
-
 // Averaged Newton constants (Sec. 3.4.1) from the grid sums over the argument
 // of the initial guess of this step.
-__device__ __forceinline__ Beta betas(const Params& P, const StepK& k, int bank) {
+__host__ __device__ inline Beta betas_from(const Params& P, const StepK& k, double sum0, double sum2) {
     Beta B;
     const double inv = P.inv_npts;
     B.m2 = k.m2;
-    const double s0 = ldcg(&P.sc->beta_sum[bank][0]) * inv;
+    B.b0 = k.thpc * fabs(sum0 * inv);
     if (P.model == M_PFC) {
-        B.b0 = k.thpc * fabs(s0);
         B.b2 = -2.0 * k.thpc;
         B.b4 = k.thpc;
     } else {
-        const double s2 = ldcg(&P.sc->beta_sum[bank][1]) * inv;
         const double e2 = P.eps * P.eps;
-        B.b0 = k.thpc * fabs(s0);
-        B.b2 = k.thpc * fabs(s2);
+        B.b2 = k.thpc * fabs(sum2 * inv);
         B.b4 = k.thpc * e2 * e2;
     }
     return B;
+}
+__device__ __forceinline__ Beta betas(const Params& P, const StepK& k, int bank) {
+    return betas_from(P, k, ldcg(&P.sc->beta_sum[bank][0]), ldcg(&P.sc->beta_sum[bank][1]));
 }
 
 __device__ __forceinline__ double lam_at(const Params& P, int i) {
@@ -296,21 +300,32 @@ __device__ __forceinline__ double lam_at(const Params& P, int i) {
 // last-axis wavenumber index of column-pass line l (l = k1 nm + km)
 __host__ __device__ __forceinline__ int kl_of(const Params& P, int l) { return l >> P.logm; }
 
-// kappa = |k|^2 at column-pass line l, first-axis index k0
-__device__ __forceinline__ double kappa_at(const Params& P, int l, int k0) {
+// A column-pass line with its part of kappa = |k|^2: the FP64 products of the
+// two fixed axes are formed once per line and kappa costs one FMA per point
+// (FP32 iterations carry no FP64 arithmetic: klf).
+struct Line {
+    int l;
+    double kl;
+    float klf;
+    const double* sq;
+    __device__ __forceinline__ operator int() const { return l; }
+};
+__device__ __forceinline__ Line line_of(const Params& P, const Tw& tw, int l) {
     const int k1 = l >> P.logm, km = l & (P.nm - 1);
-    const int r0 = (k0 <= (P.n0 >> 1)) ? k0 : k0 - P.n0;
-    const int rm = (km <= (P.nm >> 1)) ? km : km - P.nm;
-    return P.k1sq * (double)k1 * (double)k1 + P.kmsq * (double)rm * (double)rm +
-           P.k0sq * (double)r0 * (double)r0;
+    const int rm = (km <= (P.nm >> 1)) ? km : P.nm - km;
+    return Line{l, fma(P.k1sq, tw.sq[k1], P.kmsq * tw.sq[rm]),
+                P.k1sqf * (float)(k1 * k1) + P.kmsqf * (float)(rm * rm), tw.sq};
 }
-
-// kappa in the iteration precision (FP32 iterations carry no FP64 arithmetic)
-template <class T> __device__ __forceinline__ T kappa_t(const Params& P, int l, int k0) {
-    const int k1 = l >> P.logm, km = l & (P.nm - 1);
-    const int r0 = (k0 <= (P.n0 >> 1)) ? k0 : k0 - P.n0;
-    const int rm = (km <= (P.nm >> 1)) ? km : km - P.nm;
-    return (T)P.k1sq * (T)(k1 * k1) + (T)P.kmsq * (T)(rm * rm) + (T)P.k0sq * (T)(r0 * r0);
+__device__ __forceinline__ double kappa_at(const Params& P, const Line& ln, int k0) {
+    return fma(P.k0sq, ln.sq[k0 <= (P.n0 >> 1) ? k0 : P.n0 - k0], ln.kl);
+}
+template <class T> __device__ __forceinline__ T kappa_t(const Params& P, const Line& ln, int k0) {
+    if constexpr (sizeof(T) == 8) {
+        return kappa_at(P, ln, k0);
+    } else {
+        const int r0 = (k0 <= (P.n0 >> 1)) ? k0 : P.n0 - k0;
+        return ln.klf + P.k0sqf * (float)(r0 * r0);
+    }
 }
 
 // index of half-spectrum entry (line l, k0) in the row-major API layout
@@ -340,10 +355,45 @@ __device__ __forceinline__ void publish_sum(double* a, double v) {
     v = warp_sum(v);
     if ((threadIdx.x % kWarp) == 0) atomicAdd(a, v);
 }
-__device__ __forceinline__ void publish_max(unsigned long long* a, double v) {
-    v = warp_max(v);
-    if ((threadIdx.x % kWarp) == 0) atomicMax(a, dbl_bits(v));
+__device__ __forceinline__ void publish_sum(double* a, const Sum2& v) {
+    const double t = v.warp_total();
+    if ((threadIdx.x % kWarp) == 0) atomicAdd(a, t);
 }
+// Running maximum of |x| on the bit patterns: non-negative floating-point
+// numbers compare as integers, a NaN above all of them (an FP64 compare issues
+// at the FP64 rate).
+template <class T> struct MaxAbs;
+template <> struct MaxAbs<float> {
+    unsigned m = 0u;
+    __device__ __forceinline__ void add(float x) {
+        const unsigned b = flt_bits(x) & 0x7fffffffu;
+        m = b > m ? b : m;
+    }
+    __device__ __forceinline__ void publish(unsigned long long* a) const {
+        const unsigned v = warp_umax(m);
+        if ((threadIdx.x % kWarp) == 0) atomicMax(a, dbl_bits(to_f64(bits_flt(v))));
+    }
+};
+template <> struct MaxAbs<double> {
+    unsigned long long m = 0ull;
+    __device__ __forceinline__ void add(double x) {
+        const unsigned long long b = dbl_bits(x) & 0x7fffffffffffffffull;
+        m = b > m ? b : m;
+    }
+    __device__ __forceinline__ void publish(unsigned long long* a) const {
+        const unsigned h = warp_umax((unsigned)(m >> 32));
+        const unsigned l = warp_umax((unsigned)(m >> 32) == h ? (unsigned)m : 0u);
+        if ((threadIdx.x % kWarp) == 0) atomicMax(a, ((unsigned long long)h << 32) | l);
+    }
+};
+// sum of T values: FP64 as they are, FP32 by Sum2
+template <class T> struct SumOf;
+template <> struct SumOf<float> : Sum2 {};
+template <> struct SumOf<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+};
+__device__ __forceinline__ void publish_sum(double* a, const SumOf<double>& v) { publish_sum(a, v.v); }
 
 // ---------------------------------------------------------- pass templates
 
@@ -413,7 +463,7 @@ __device__ void row_pass(const Params& P, const Tw& tw, int kin, int kout, const
                 if (x == 0 || x == half) { A.y = 0; B.y = 0; }
                 Z0[x] = (x <= half) ? CI{A.x - B.y, A.y + B.x} : CI{A.x + B.y, B.x - A.y};
             }
-            const int res = fft_line_w<+1, TI>(Z0, Z1, logn1, tw_of<TI>(tw), tw.log, w.lane);
+            const int res = fft_line_w<+1, TI>(Z0, Z1, logn1, tw.t32, tw.log, w.lane);
             const CI* Zr = res ? Z1 : Z0;
             for (int x = w.lane; x < n1; x += kWarp) {
                 const CI z = Zr[x];
@@ -438,7 +488,7 @@ __device__ void row_pass(const Params& P, const Tw& tw, int kin, int kout, const
             warp_sync();
             for (int x = w.lane; x < n1; x += kWarp)
                 Z0[x] = CO{Rout[(size_t)la * n1 + x], Rout[(size_t)lb * n1 + x]};
-            const int res = fft_line_w<-1, TO>(Z0, Z1, logn1, tw_of<TO>(tw), tw.log, w.lane);
+            const int res = fft_line_w<-1, TO>(Z0, Z1, logn1, tw.t32, tw.log, w.lane);
             const CO* Zr = res ? Z1 : Z0;
             CO* da = dst + (size_t)(la / ru) * H + r0 + (la % ru);
             CO* db = dst + (size_t)(lb / ru) * H + r0 + (lb % ru);
@@ -472,13 +522,14 @@ __device__ void col_pass(const Params& P, const Tw& tw, int kin, int kout, const
     const WarpCtx w = warp_ctx(P, smem);
     const URange ur = units_of(tw, ncols);
     for (int k1 = ur.b; k1 < ur.e; k1 += ur.s) {
+        const Line ln = line_of(P, tw, k1);
         CI* buf[kMaxK + 1];
         CO* obuf[kMaxK + 1];
         for (int i = 0; i < nbi; i++) buf[i] = (CI*)w.mem + (size_t)i * pitch;
         for (int f = 0; f < kin; f++) {
             const CI* s = src + (size_t)f * H + (size_t)k1 * n0;
             for (int k0 = w.lane; k0 < n0; k0 += kWarp) buf[f][k0] = s[k0];
-            const int res = fft_line_w<-1, TI>(buf[f], buf[nbi - 1], logn0, tw_of<TI>(tw), tw.log, w.lane);
+            const int res = fft_line_w<-1, TI>(buf[f], buf[nbi - 1], logn0, tw.t32, tw.log, w.lane);
             if (res) {
                 CI* t = buf[f];
                 buf[f] = buf[nbi - 1];
@@ -493,11 +544,11 @@ __device__ void col_pass(const Params& P, const Tw& tw, int kin, int kout, const
             CI in[kMaxK];
             CO out[kMaxK];
             for (int f = 0; f < kin; f++) in[f] = buf[f][k0];
-            fn(k1, k0, in, out);
+            fn(ln, k0, in, out);
             for (int g = 0; g < kout; g++) obuf[g][k0] = out[g];
         }
         for (int g = 0; g < kout; g++) {
-            const int res = fft_line_w<+1, TO>(obuf[g], obuf[kout], logn0, tw_of<TO>(tw), tw.log, w.lane);
+            const int res = fft_line_w<+1, TO>(obuf[g], obuf[kout], logn0, tw.t32, tw.log, w.lane);
             const CO* r = res ? obuf[kout] : obuf[g];
             CO* d = dst + (size_t)g * H + (size_t)k1 * n0;
             for (int k0 = w.lane; k0 < n0; k0 += kWarp) d[k0] = r[k0];
@@ -603,7 +654,7 @@ __device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
         }
         const CI* Xr = X0;
         if (kin > 0)
-            Xr = fft_lines_fixed<+1, TI, LOGN, kMaxK>(X0, X1, PITCH, kin, tw_of<TI>(tw), tw.log, w.lane) ? X1 : X0;
+            Xr = fft_lines_fixed<+1, TI, LOGN, kMaxK>(X0, X1, PITCH, kin, tw.t32, tw.log, w.lane) ? X1 : X0;
 #pragma unroll 1
         for (int c0 = 0; c0 < NPT; c0 += PCH) {
             if (c0 > 0) {
@@ -640,7 +691,7 @@ __device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
         }
         if (kout > 0) {
             const CO* Yr =
-                fft_lines_fixed<-1, TO, LOGN, kMaxK>(Y0, Y1, PITCH, kout, tw_of<TO>(tw), tw.log, w.lane) ? Y1 : Y0;
+                fft_lines_fixed<-1, TO, LOGN, kMaxK>(Y0, Y1, PITCH, kout, tw.t32, tw.log, w.lane) ? Y1 : Y0;
             const TO hf = (TO)0.5;
             for (int g = 0; g < kout; g++) {
                 CO* d0 = dst + (size_t)g * Hs + r0;
@@ -666,7 +717,7 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
                                cx<TO>* dst, char* smem, Ld&& ld, Ap&& ap) {
     using C = cx<TI>;
     using CO = cx<TO>;
-    using S = decltype(ld(0, 0));
+    using S = decltype(ld(Line{}, 0));
     constexpr int LOGN = ilog2c(NF), PITCH = NF + 2, E = NF / kWarp;
     constexpr int GCH = E < 8 ? E : 8;
     constexpr int PCH = chunk_for((int)sizeof(S), E);
@@ -679,11 +730,12 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
     const URange ur = units_of(tw, ncols);
     constexpr int NCH = E / GCH;  // load chunks per field
     for (int k1 = ur.b; k1 < ur.e; k1 += ur.s) {
+        const Line ln = line_of(P, tw, k1);
         // the per-wavenumber state of the first chunk is loaded first, so that
         // its latency overlaps the lines' and the transform's
         S st[PCH];
 #pragma unroll
-        for (int q = 0; q < PCH; q++) st[q] = ld(k1, w.lane + kWarp * q);
+        for (int q = 0; q < PCH; q++) st[q] = ld(ln, w.lane + kWarp * q);
         // lines of the kin fields, chunk t = (field, GCH points); FP32 lines
         // load chunk t + 1 before storing chunk t to shared memory
         auto load_chunk = [&](int t, C* v) {
@@ -715,7 +767,7 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
         const C* Xr = B0;
         C* Xi = B1;
         if (kin > 0) {
-            const int r = fft_lines_fixed<-1, TI, LOGN, kMaxK>(B0, B1, PITCH, kin, tw_of<TI>(tw), tw.log, w.lane);
+            const int r = fft_lines_fixed<-1, TI, LOGN, kMaxK>(B0, B1, PITCH, kin, tw.t32, tw.log, w.lane);
             Xr = r ? B1 : B0;
             Xi = r ? B0 : B1;
         }
@@ -726,7 +778,7 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
         for (int c0 = 0; c0 < E; c0 += PCH) {
             if (c0 > 0) {
 #pragma unroll
-                for (int q = 0; q < PCH; q++) st[q] = ld(k1, w.lane + kWarp * (c0 + q));
+                for (int q = 0; q < PCH; q++) st[q] = ld(ln, w.lane + kWarp * (c0 + q));
             }
 #pragma unroll
             for (int q = 0; q < PCH; q++) {
@@ -736,7 +788,7 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
 #pragma unroll
                 for (int f = 0; f < kMaxK; f++)
                     if (f < kin) in[f] = Xr[(size_t)f * PITCH + k0];
-                ap(k1, k0, st[q], in, out);
+                ap(ln, k0, st[q], in, out);
 #pragma unroll
                 for (int g = 0; g < kMaxK; g++)
                     if (g < kout) Xo[(size_t)g * PITCH + k0] = out[g];
@@ -745,7 +797,7 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
         if (kout > 0) {
             CO* scratch = (CO*)Xr;
             const int r =
-                fft_lines_fixed<+1, TO, LOGN, kMaxK>(Xo, scratch, PITCH, kout, tw_of<TO>(tw), tw.log, w.lane);
+                fft_lines_fixed<+1, TO, LOGN, kMaxK>(Xo, scratch, PITCH, kout, tw.t32, tw.log, w.lane);
             const CO* Yr = r ? scratch : Xo;
             for (int g = 0; g < kout; g++) {
                 CO* d = dst + (size_t)g * Hs + (size_t)k1 * NF;
@@ -917,6 +969,7 @@ __device__ void col_pass_staged(const Params& P, const Tw& tw, const float2* src
     if (SLOTS == 2) cp_async_commit();
     int s = 0;
     for (int k1 = ur.b; k1 < ur.e; k1 += ur.s, s ^= (SLOTS - 1)) {
+        const Line ln = line_of(P, tw, k1);
         if constexpr (SLOTS == 2) {
             if (k1 + ur.s < ur.e) issue(k1 + ur.s, s ^ 1);
             cp_async_commit();
@@ -941,7 +994,7 @@ __device__ void col_pass_staged(const Params& P, const Tw& tw, const float2* src
             for (int a = 0; a < NS; a++) sv[a] = st[a * NF + k0];
 #pragma unroll
             for (int f = 0; f < K; f++) in[f] = Xr[f * PP + pk];
-            ap(k1, k0, sv, in, out);
+            ap(ln, k0, sv, in, out);
 #pragma unroll
             for (int g = 0; g < K; g++) Xi[g * PP + pk] = out[g];
         }
@@ -961,76 +1014,462 @@ __device__ void col_pass_staged(const Params& P, const Tw& tw, const float2* src
     warp_sync();
 }
 
+// ------------------------------------------------------------- FP64 passes
+//
+// The same passes with lines of doubles, transformed in fixed point (fx.cuh).
+// A line has one buffer of n 16-byte slots: it holds the doubles as loaded,
+// then the fixed-point line, which the transform replaces in place, and after
+// the pointwise step the outputs; kMaxK lines per warp.  NF: line length (0:
+// runtime length).  ld / ap as above.
+
+constexpr int kFxChunk = 2;  // points per lane whose pointwise state is loaded together
+
+// log2 of the number of grid points: the 1 / n_pts of the inverse transform
+// is a shift of the line's exponent
+__device__ __forceinline__ int log_npts(const Params& P) { return P.logn0 + P.logm + P.logn1; }
+
+template <int NF, class Ld, class Ap>
+__device__ void row_pass_fx(const Params& P, const Tw& tw, int kin, int kout, const double2* src, double2* dst,
+                            char* smem, Ld&& ld, Ap&& ap) {
+    using S = decltype(ld(0ll, 0, 0));
+    const int n = NF > 0 ? NF : P.n1, logn = P.logn1, rows = P.rows;
+    const long long Hs = P.H;
+    const WarpCtx w = warp_ctx(P, smem);
+    longlong2* B = (longlong2*)w.mem;
+    const URange ur = units_of(tw, rows / 2);
+    for (int u = ur.b; u < ur.e; u += ur.s) {
+        const int r0 = 2 * u;
+        int sc[kMaxK];
+#pragma unroll 1
+        for (int f = 0; f < kin; f++) {
+            longlong2* b = B + f * n;
+            const FxExp x = fx_convert_rows(b, n, fx_load_rows(b, src + (size_t)f * Hs + r0, n, rows, w.lane, kWarp), w.lane);
+            fx_line<+1, NF>(b, logn, x.sh, tw.tfx, tw.log, w.lane);
+            const int s1 = x.e - x.sh + log_npts(P);
+            if (f == 0) sc[0] = s1;
+            else if (f == 1) sc[1] = s1;
+            else sc[2] = s1;
+        }
+        unsigned hi[kMaxK] = {0u, 0u, 0u};
+        for (int x0 = w.lane; x0 < n; x0 += kWarp * kFxChunk) {
+            S st[2 * kFxChunk];
+#pragma unroll
+            for (int q = 0; q < 2 * kFxChunk; q++) {
+                const int x = x0 + kWarp * (q >> 1), rr = q & 1;
+                if (x < n) st[q] = ld((long long)(r0 + rr) * n + x, r0 + rr, x);
+            }
+#pragma unroll
+            for (int q = 0; q < kFxChunk; q++) {
+                const int x = x0 + kWarp * q;
+                if (x < n) {
+                    longlong2* slot = B + fxs(x);
+                    double in0[kMaxK], in1[kMaxK], out0[kMaxK], out1[kMaxK];
+#pragma unroll
+                    for (int f = 0; f < kMaxK; f++) {
+                        if (f < kin) {
+                            const longlong2 z = slot[f * n];
+                            in0[f] = fx_to(z.x, sc[f]);
+                            in1[f] = fx_to(z.y, sc[f]);
+                        }
+                    }
+                    ap((long long)r0 * n + x, r0, x, st[2 * q], in0, out0);
+                    ap((long long)(r0 + 1) * n + x, r0 + 1, x, st[2 * q + 1], in1, out1);
+#pragma unroll
+                    for (int g = 0; g < kMaxK; g++) {
+                        if (g < kout) {
+                            *(double2*)&slot[g * n] = double2{out0[g], out1[g]};
+                            const unsigned a = fx_hi(out0[g]), b = fx_hi(out1[g]), m = a > b ? a : b;
+                            hi[g] = m > hi[g] ? m : hi[g];
+                        }
+                    }
+                }
+            }
+        }
+#pragma unroll 1
+        for (int g = 0; g < kout; g++) {
+            longlong2* b = B + g * n;
+            const FxExp x = fx_convert(b, n, g == 0 ? hi[0] : (g == 1 ? hi[1] : hi[2]), w.lane);
+            fx_line<-1, NF>(b, logn, x.sh, tw.tfx, tw.log, w.lane);
+            fx_store_rows(b, n, x.e - x.sh, dst + (size_t)g * Hs + r0, rows, w.lane, kWarp);
+        }
+        warp_sync();
+    }
+}
+
+// Column pass; TO = float: the outputs' inverse transforms run in FP32 (kMaxK
+// lines per warp: at most two outputs, the third line's buffer is theirs)
+template <class TO, int NF, class Ld, class Ap>
+__device__ void col_pass_fx(const Params& P, const Tw& tw, int kin, int kout, const double2* src, cx<TO>* dst,
+                            char* smem, Ld&& ld, Ap&& ap) {
+    using CO = cx<TO>;
+    using S = decltype(ld(Line{}, 0));
+    const int n = NF > 0 ? NF : P.n0, logn = P.logn0, ncols = P.ncols;
+    const long long Hs = P.H;
+    const WarpCtx w = warp_ctx(P, smem);
+    longlong2* B = (longlong2*)w.mem;
+    const URange ur = units_of(tw, ncols);
+    for (int k1 = ur.b; k1 < ur.e; k1 += ur.s) {
+        const Line ln = line_of(P, tw, k1);
+        int sc[kMaxK];
+#pragma unroll 1
+        for (int f = 0; f < kin; f++) {
+            longlong2* b = B + f * n;
+            const FxExp x = fx_convert(b, n, fx_load(b, src + (size_t)f * Hs + (size_t)k1 * n, n, w.lane, kWarp), w.lane);
+            const int e = x.e, sh = x.sh;
+            fx_line<-1, NF>(b, logn, sh, tw.tfx, tw.log, w.lane);
+            if (f == 0) sc[0] = e - sh;
+            else if (f == 1) sc[1] = e - sh;
+            else sc[2] = e - sh;
+        }
+        unsigned hi[kMaxK] = {0u, 0u, 0u};
+        for (int x0 = w.lane; x0 < n; x0 += kWarp * kFxChunk) {
+            S st[kFxChunk];
+#pragma unroll
+            for (int q = 0; q < kFxChunk; q++)
+                if (x0 + kWarp * q < n) st[q] = ld(ln, x0 + kWarp * q);
+#pragma unroll
+            for (int q = 0; q < kFxChunk; q++) {
+                const int k0 = x0 + kWarp * q;
+                if (k0 < n) {
+                    longlong2* slot = B + fxs(k0);
+                    double2 in[kMaxK];
+                    CO out[kMaxK];
+#pragma unroll
+                    for (int f = 0; f < kMaxK; f++) {
+                        if (f < kin) {
+                            const longlong2 z = slot[f * n];
+                            in[f] = double2{fx_to(z.x, sc[f]), fx_to(z.y, sc[f])};
+                        }
+                    }
+                    ap(ln, k0, st[q], in, out);
+#pragma unroll
+                    for (int g = 0; g < kMaxK; g++) {
+                        if (g < kout) {
+                            *(CO*)&slot[g * n] = out[g];
+                            if constexpr (sizeof(TO) == 8) {
+                                const unsigned a = fx_hi(out[g].x), c = fx_hi(out[g].y), m = a > c ? a : c;
+                                hi[g] = m > hi[g] ? m : hi[g];
+                            }
+                        }
+                    }
+                }
+            }
+        }
+#pragma unroll 1
+        for (int g = 0; g < kout; g++) {
+            longlong2* b = B + g * n;
+            CO* d = dst + (size_t)g * Hs + (size_t)k1 * n;
+            if constexpr (sizeof(TO) == 8) {
+                const FxExp x = fx_convert(b, n, g == 0 ? hi[0] : (g == 1 ? hi[1] : hi[2]), w.lane);
+                fx_line<+1, NF>(b, logn, x.sh, tw.tfx, tw.log, w.lane);
+                fx_store(b, n, x.e - x.sh, d, w.lane, kWarp);
+            } else {
+                float2* f0 = (float2*)(B + 2 * n);
+                float2* f1 = f0 + n;
+                for (int k0 = w.lane; k0 < n; k0 += kWarp) f0[k0] = *(const float2*)&b[fxs(k0)];
+                int r;
+                if constexpr (NF > 0) r = fft_lines_fixed<+1, float, ilog2c(NF), 1>(f0, f1, n, 1, tw.t32, tw.log, w.lane);
+                else r = fft_line_w<+1, float>(f0, f1, logn, tw.t32, tw.log, w.lane);
+                const float2* y = r ? f1 : f0;
+                for (int k0 = w.lane; k0 < n; k0 += kWarp) d[k0] = y[k0];
+                warp_sync();
+            }
+        }
+        warp_sync();
+    }
+}
+
 // ------------------------------------------------ CTA-cooperative variants
 //
-// The same passes with one unit per CTA: the threads of the CTA load the
-// unit's lines, transform them together (fft_lines_coop), share the pointwise
-// work and store, with CTA barriers in between.  For phases with fewer units
-// than warps (a 256^2 grid has 128 row units and 129 columns): the work of a
-// unit then runs on all four SM sub-partitions, which is what an FP64 line
-// needs on a part whose FP64 rate per sub-partition is low.  Shared memory is
-// the CTA's slice region (one unit needs no more than one warp's slice).
+// One unit per CTA: the threads of the CTA load and convert the unit's lines,
+// transform them together (fx_lines_coop), share the pointwise work and store,
+// with CTA barriers in between.  For phases with fewer units than warps (a
+// 256^2 grid has 128 row units and 129 columns).  The FP64 instructions left
+// in a pass are its pointwise ones: an SM sub-partition issues one in 64
+// cycles, so they have to be spread over all four.  Shared memory: two sets of
+// kMaxK lines and a few words for the lines' exponents.
 
-constexpr int kCoopChunk = 4;  // points per thread whose loads are in flight together
+constexpr int kCoopChunk = 2;  // points per thread whose loads are in flight together
+constexpr size_t coop_smem(int n) { return (size_t)2 * kMaxK * n * 16 + 4 * kMaxK * sizeof(unsigned); }
 
+__device__ __forceinline__ void fx_publish_max(unsigned* a, unsigned v) {
+    v = warp_umax(v);
+    if ((threadIdx.x % kWarp) == 0) atomicMax(a, v);
+}
+__device__ __forceinline__ void fx_publish_sum(unsigned* a, unsigned v) {
+    v = warp_uadd(v);
+    if ((threadIdx.x % kWarp) == 0) atomicAdd(a, v);
+}
+
+template <int NF, class Ld, class Ap>
+__device__ void row_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kout, const double2* src, double2* dst,
+                                 char* smem, Ld&& ld, Ap&& ap) {
+    using S = decltype(ld(0ll, 0, 0));
+    const int n = NF > 0 ? NF : P.n1, logn = NF > 0 ? ilog2c(NF) : P.logn1, half = n >> 1, rows = P.rows;
+    const long long Hs = P.H;
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    longlong2* B0 = (longlong2*)smem;
+    longlong2* B1 = B0 + kMaxK * n;
+    unsigned* red = (unsigned*)(B1 + kMaxK * n);  // [max in, sum in, max out, sum out][field]
+    for (int u = blockIdx.x; u < rows / 2; u += gridDim.x) {
+        const int r0 = 2 * u;
+        for (int i = tid; i < 4 * kMaxK; i += nthr) red[i] = 0u;
+        // the first points' state, in flight during the inverse transforms
+        S st[kCoopChunk];
+#pragma unroll
+        for (int c = 0; c < kCoopChunk; c++) {
+            const int q = tid + nthr * c;
+            if (q < 2 * n) st[c] = ld((long long)(r0 + (q >> logn)) * n + (q & (n - 1)), r0 + (q >> logn), q & (n - 1));
+        }
+        cta_sync();
+        longlong2* X = B0;
+        int sc[kMaxK] = {0, 0, 0};
+        if (kin > 0) {
+            for (int f = 0; f < kin; f++)
+                fx_publish_max(red + f, fx_load_rows(B0 + f * n, src + (size_t)f * Hs + r0, n, rows, tid, nthr));
+            cta_sync();
+            for (int f = 0; f < kin; f++) {
+                const int emax = fx_emax(red[f]);
+                longlong2* b = B0 + f * n;
+                unsigned s = 0;
+                for (int k = tid; k < half; k += nthr) s += fx_pair_rows(b, k, n, emax);
+                fx_publish_sum(red + kMaxK + f, s);
+            }
+            cta_sync();
+            X = fx_coop<+1, NF>(B0, B1, logn, kin, red + kMaxK, tw.tfx, tw.log, tid, nthr) ? B1 : B0;
+#pragma unroll
+            for (int f = 0; f < kMaxK; f++)
+                if (f < kin) sc[f] = fx_scale(fx_emax(red[f]), fx_shift(red[kMaxK + f])) + log_npts(P);
+        }
+        // pointwise: point q = rr n + x of the unit; the outputs replace the
+        // inputs of the same point and row
+        unsigned hi[kMaxK] = {0u, 0u, 0u};
+        for (int q0 = 0; q0 < 2 * n; q0 += nthr * kCoopChunk) {
+            if (q0 > 0) {
+#pragma unroll
+                for (int c = 0; c < kCoopChunk; c++) {
+                    const int q = q0 + tid + nthr * c;
+                    if (q < 2 * n)
+                        st[c] = ld((long long)(r0 + (q >> logn)) * n + (q & (n - 1)), r0 + (q >> logn), q & (n - 1));
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < kCoopChunk; c++) {
+                const int q = q0 + tid + nthr * c;
+                if (q < 2 * n) {
+                    const int rr = q >> logn, x = q & (n - 1);
+                    long long* slot = (long long*)(X + fxs(x)) + rr;
+                    double in[kMaxK], out[kMaxK];
+#pragma unroll
+                    for (int f = 0; f < kMaxK; f++)
+                        if (f < kin) in[f] = fx_to(slot[f * 2 * n], sc[f]);
+                    ap((long long)(r0 + rr) * n + x, r0 + rr, x, st[c], in, out);
+#pragma unroll
+                    for (int g = 0; g < kMaxK; g++) {
+                        if (g < kout) {
+                            *(double*)&slot[g * 2 * n] = out[g];
+                            const unsigned m = fx_hi(out[g]);
+                            hi[g] = m > hi[g] ? m : hi[g];
+                        }
+                    }
+                }
+            }
+        }
+        if (kout > 0) {
+#pragma unroll
+            for (int g = 0; g < kMaxK; g++)
+                if (g < kout) fx_publish_max(red + 2 * kMaxK + g, hi[g]);
+            cta_sync();
+            for (int g = 0; g < kout; g++) {
+                const int emax = fx_emax(red[2 * kMaxK + g]);
+                unsigned s = 0;
+                for (int x = tid; x < n; x += nthr) s += fx_point(X + g * n + fxs(x), emax);
+                fx_publish_sum(red + 3 * kMaxK + g, s);
+            }
+            cta_sync();
+            longlong2* Z = X == B0 ? B1 : B0;
+            const longlong2* Y = fx_coop<-1, NF>(X, Z, logn, kout, red + 3 * kMaxK, tw.tfx, tw.log, tid, nthr) ? Z : X;
+            for (int g = 0; g < kout; g++) {
+                const int e = fx_scale(fx_emax(red[2 * kMaxK + g]), fx_shift(red[3 * kMaxK + g]));
+                fx_store_rows(Y + g * n, n, e, dst + (size_t)g * Hs + r0, rows, tid, nthr);
+            }
+        }
+        cta_sync();  // the next unit reuses the buffers
+    }
+}
+
+template <class TO, int NF, class Ld, class Ap>
+__device__ void col_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kout, const double2* src, cx<TO>* dst,
+                                 char* smem, Ld&& ld, Ap&& ap) {
+    using CO = cx<TO>;
+    using S = decltype(ld(Line{}, 0));
+    const int n = NF > 0 ? NF : P.n0, logn = NF > 0 ? ilog2c(NF) : P.logn0, ncols = P.ncols;
+    const long long Hs = P.H;
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    longlong2* B0 = (longlong2*)smem;
+    longlong2* B1 = B0 + kMaxK * n;
+    unsigned* red = (unsigned*)(B1 + kMaxK * n);
+    for (int k1 = blockIdx.x; k1 < ncols; k1 += gridDim.x) {
+        const Line ln = line_of(P, tw, k1);
+        for (int i = tid; i < 4 * kMaxK; i += nthr) red[i] = 0u;
+        S st[kCoopChunk];
+#pragma unroll
+        for (int c = 0; c < kCoopChunk; c++) {
+            const int k0 = tid + nthr * c;
+            if (k0 < n) st[c] = ld(ln, k0);
+        }
+        cta_sync();
+        longlong2* X = B0;
+        int sc[kMaxK] = {0, 0, 0};
+        if (kin > 0) {
+            for (int f = 0; f < kin; f++)
+                fx_publish_max(red + f, fx_load(B0 + f * n, src + (size_t)f * Hs + (size_t)k1 * n, n, tid, nthr));
+            cta_sync();
+            for (int f = 0; f < kin; f++) {
+                const int emax = fx_emax(red[f]);
+                unsigned s = 0;
+                for (int x = tid; x < n; x += nthr) s += fx_point(B0 + f * n + fxs(x), emax);
+                fx_publish_sum(red + kMaxK + f, s);
+            }
+            cta_sync();
+            X = fx_coop<-1, NF>(B0, B1, logn, kin, red + kMaxK, tw.tfx, tw.log, tid, nthr) ? B1 : B0;
+#pragma unroll
+            for (int f = 0; f < kMaxK; f++)
+                if (f < kin) sc[f] = fx_scale(fx_emax(red[f]), fx_shift(red[kMaxK + f]));
+        }
+        // outputs: doubles in place of the inputs, FP32 lines in the other set
+        longlong2* Z = X == B0 ? B1 : B0;
+        const int pitch = n + 2;
+        unsigned hi[kMaxK] = {0u, 0u, 0u};
+        for (int q0 = 0; q0 < n; q0 += nthr * kCoopChunk) {
+            if (q0 > 0) {
+#pragma unroll
+                for (int c = 0; c < kCoopChunk; c++) {
+                    const int k0 = q0 + tid + nthr * c;
+                    if (k0 < n) st[c] = ld(ln, k0);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < kCoopChunk; c++) {
+                const int k0 = q0 + tid + nthr * c;
+                if (k0 < n) {
+                    longlong2* slot = X + fxs(k0);
+                    double2 in[kMaxK];
+                    CO out[kMaxK];
+#pragma unroll
+                    for (int f = 0; f < kMaxK; f++) {
+                        if (f < kin) {
+                            const longlong2 z = slot[f * n];
+                            in[f] = double2{fx_to(z.x, sc[f]), fx_to(z.y, sc[f])};
+                        }
+                    }
+                    ap(ln, k0, st[c], in, out);
+#pragma unroll
+                    for (int g = 0; g < kMaxK; g++) {
+                        if (g < kout) {
+                            if constexpr (sizeof(TO) == 8) {
+                                *(CO*)&slot[g * n] = out[g];
+                                const unsigned a = fx_hi(out[g].x), c2 = fx_hi(out[g].y), m = a > c2 ? a : c2;
+                                hi[g] = m > hi[g] ? m : hi[g];
+                            } else {
+                                ((CO*)Z)[(size_t)g * pitch + k0] = out[g];
+                            }
+                        }
+                    }
+                }
+            }
+        }
+        if (kout > 0) {
+            if constexpr (sizeof(TO) == 8) {
+#pragma unroll
+                for (int g = 0; g < kMaxK; g++)
+                    if (g < kout) fx_publish_max(red + 2 * kMaxK + g, hi[g]);
+                cta_sync();
+                for (int g = 0; g < kout; g++) {
+                    const int emax = fx_emax(red[2 * kMaxK + g]);
+                    unsigned s = 0;
+                    for (int x = tid; x < n; x += nthr) s += fx_point(X + g * n + fxs(x), emax);
+                    fx_publish_sum(red + 3 * kMaxK + g, s);
+                }
+                cta_sync();
+                const longlong2* Y =
+                    fx_coop<+1, NF>(X, Z, logn, kout, red + 3 * kMaxK, tw.tfx, tw.log, tid, nthr) ? Z : X;
+                for (int g = 0; g < kout; g++)
+                    fx_store(Y + g * n, n, fx_scale(fx_emax(red[2 * kMaxK + g]), fx_shift(red[3 * kMaxK + g])),
+                             dst + (size_t)g * Hs + (size_t)k1 * n, tid, nthr);
+            } else {
+                cta_sync();  // the inputs' buffers become the second set of the FP32 lines
+                float2 *f0 = (float2*)Z, *f1 = (float2*)X;
+                const float2* Y = fft_coop<+1, float, NF>(f0, f1, logn, pitch, kout, tw.t32, tw.log, tid, nthr) ? f1 : f0;
+                for (int it = tid; it < kout * n; it += nthr) {
+                    const int g = it >> logn, x = it & (n - 1);
+                    dst[(size_t)g * Hs + (size_t)k1 * n + x] = Y[(size_t)g * pitch + x];
+                }
+            }
+        }
+        cta_sync();
+    }
+}
+
+// FP32 lines with one unit per CTA (the incremental base evaluations, whose
+// pointwise work is FP64, and the opt-in FP32 iteration passes)
 template <class TI, class TO, int NF, class Ld, class Ap>
 __device__ void row_pass_coop(const Params& P, const Tw& tw, int kin, int kout, const cx<TI>* src, cx<TO>* dst,
                               char* smem, Ld&& ld, Ap&& ap) {
     using CI = cx<TI>;
     using CO = cx<TO>;
     using S = decltype(ld(0ll, 0, 0));
-    constexpr int LOGN = ilog2c(NF), HALF = NF / 2, H1 = HALF + 1, PITCH = NF + 2;
-    const int rows = P.rows;
+    const int n = NF > 0 ? NF : P.n1, logn = NF > 0 ? ilog2c(NF) : P.logn1, half = n >> 1, pitch = n + 2, rows = P.rows;
     const long long Hs = P.H;
     const int tid = threadIdx.x, nthr = blockDim.x;
     CI* X0 = (CI*)smem;
-    CI* X1 = X0 + (size_t)kin * PITCH;
-    CO* Y0 = (CO*)(X1 + (size_t)kin * PITCH);
-    CO* Y1 = Y0 + (size_t)kout * PITCH;
+    CI* X1 = X0 + (size_t)kin * pitch;
+    CO* Y0 = (CO*)(X1 + (size_t)kin * pitch);
+    CO* Y1 = Y0 + (size_t)kout * pitch;
     const TI iscale = (TI)P.inv_npts;
     for (int u = blockIdx.x; u < rows / 2; u += gridDim.x) {
         const int r0 = 2 * u;
         // inverse x-DFT inputs: complex line x of field l packs rows r0, r0 + 1
-        for (int it = tid; it < kin * NF; it += nthr) {
-            const int l = it >> LOGN, x = it & (NF - 1);
-            const int k = (x <= HALF) ? x : NF - x;
+        for (int it = tid; it < kin * n; it += nthr) {
+            const int l = it >> logn, x = it & (n - 1);
+            const int k = (x <= half) ? x : n - x;
             const CI* s0 = src + (size_t)l * Hs + (size_t)k * rows + r0;
             CI A = s0[0], B = s0[1];
-            if (x == 0 || x == HALF) { A.y = 0; B.y = 0; }
-            X0[(size_t)l * PITCH + x] = (x <= HALF) ? CI{A.x - B.y, A.y + B.x} : CI{A.x + B.y, B.x - A.y};
+            if (x == 0 || x == half) { A.y = 0; B.y = 0; }
+            X0[(size_t)l * pitch + x] = (x <= half) ? CI{A.x - B.y, A.y + B.x} : CI{A.x + B.y, B.x - A.y};
         }
         const CI* Xr = X0;
-        if (kin > 0) Xr = fft_lines_coop<+1, TI, LOGN>(X0, X1, PITCH, kin, tw_of<TI>(tw), tw.log, tid, nthr) ? X1 : X0;
-        // pointwise: point q = rr NF + x of the unit (consecutive threads, consecutive x)
-        for (int q0 = 0; q0 < 2 * NF; q0 += nthr * kCoopChunk) {
+        if (kin > 0) Xr = fft_coop<+1, TI, NF>(X0, X1, logn, pitch, kin, tw.t32, tw.log, tid, nthr) ? X1 : X0;
+        // pointwise: point q = rr n + x of the unit (consecutive threads, consecutive x)
+        for (int q0 = 0; q0 < 2 * n; q0 += nthr * kCoopChunk) {
             S st[kCoopChunk];
 #pragma unroll
             for (int c = 0; c < kCoopChunk; c++) {
                 const int q = q0 + tid + nthr * c;
-                if (q < 2 * NF) {
-                    const int rr = q >> LOGN, x = q & (NF - 1);
-                    st[c] = ld((long long)(r0 + rr) * NF + x, r0 + rr, x);
+                if (q < 2 * n) {
+                    const int rr = q >> logn, x = q & (n - 1);
+                    st[c] = ld((long long)(r0 + rr) * n + x, r0 + rr, x);
                 }
             }
 #pragma unroll
             for (int c = 0; c < kCoopChunk; c++) {
                 const int q = q0 + tid + nthr * c;
-                if (q < 2 * NF) {
-                    const int rr = q >> LOGN, x = q & (NF - 1);
+                if (q < 2 * n) {
+                    const int rr = q >> logn, x = q & (n - 1);
                     TI in[kMaxK];
                     TO out[kMaxK];
 #pragma unroll
                     for (int f = 0; f < kMaxK; f++) {
                         if (f < kin) {
-                            const CI z = Xr[(size_t)f * PITCH + x];
+                            const CI z = Xr[(size_t)f * pitch + x];
                             in[f] = (rr ? z.y : z.x) * iscale;
                         }
                     }
-                    ap((long long)(r0 + rr) * NF + x, r0 + rr, x, st[c], in, out);
+                    ap((long long)(r0 + rr) * n + x, r0 + rr, x, st[c], in, out);
 #pragma unroll
                     for (int g = 0; g < kMaxK; g++) {
                         if (g < kout) {
-                            CO* qq = Y0 + (size_t)g * PITCH + x;
+                            CO* qq = Y0 + (size_t)g * pitch + x;
                             if (rr) qq->y = out[g];
                             else qq->x = out[g];
                         }
@@ -1039,14 +1478,14 @@ __device__ void row_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
             }
         }
         if (kout > 0) {
-            const CO* Yr = fft_lines_coop<-1, TO, LOGN>(Y0, Y1, PITCH, kout, tw_of<TO>(tw), tw.log, tid, nthr) ? Y1 : Y0;
+            const CO* Yr = fft_coop<-1, TO, NF>(Y0, Y1, logn, pitch, kout, tw.t32, tw.log, tid, nthr) ? Y1 : Y0;
             const TO hf = (TO)0.5;
-            for (int it = tid; it < kout * H1; it += nthr) {
-                const int g = it / H1, k = it - g * H1;
+            for (int it = tid; it < kout * (half + 1); it += nthr) {
+                const int g = it / (half + 1), k = it - g * (half + 1);
                 CO* d0 = dst + (size_t)g * Hs + r0;
-                const CO* zl = Yr + (size_t)g * PITCH;
+                const CO* zl = Yr + (size_t)g * pitch;
                 const CO zk = zl[k];
-                const CO zn = zl[(NF - k) & (NF - 1)];
+                const CO zn = zl[(n - k) & (n - 1)];
                 d0[(size_t)k * rows] = CO{hf * (zk.x + zn.x), hf * (zk.y - zn.y)};
                 d0[(size_t)k * rows + 1] = CO{hf * (zk.y + zn.y), hf * (zn.x - zk.x)};
             }
@@ -1060,57 +1499,57 @@ __device__ void col_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
                               char* smem, Ld&& ld, Ap&& ap) {
     using C = cx<TI>;
     using CO = cx<TO>;
-    using S = decltype(ld(0, 0));
-    constexpr int LOGN = ilog2c(NF), PITCH = NF + 2;
-    const int ncols = P.ncols;
+    using S = decltype(ld(Line{}, 0));
+    const int n = NF > 0 ? NF : P.n0, logn = NF > 0 ? ilog2c(NF) : P.logn0, pitch = n + 2, ncols = P.ncols;
     const long long Hs = P.H;
     const int kl = kin > kout ? kin : kout;
     const int tid = threadIdx.x, nthr = blockDim.x;
     C* B0 = (C*)smem;
-    C* B1 = B0 + (size_t)kl * PITCH;
+    C* B1 = B0 + (size_t)kl * pitch;
     for (int k1 = blockIdx.x; k1 < ncols; k1 += gridDim.x) {
-        for (int it = tid; it < kin * NF; it += nthr) {
-            const int f = it >> LOGN, x = it & (NF - 1);
-            B0[(size_t)f * PITCH + x] = src[(size_t)f * Hs + (size_t)k1 * NF + x];
+        const Line ln = line_of(P, tw, k1);
+        for (int it = tid; it < kin * n; it += nthr) {
+            const int f = it >> logn, x = it & (n - 1);
+            B0[(size_t)f * pitch + x] = src[(size_t)f * Hs + (size_t)k1 * n + x];
         }
         const C* Xr = B0;
         C* Xi = B1;
         if (kin > 0) {
-            const int r = fft_lines_coop<-1, TI, LOGN>(B0, B1, PITCH, kin, tw_of<TI>(tw), tw.log, tid, nthr);
+            const int r = fft_coop<-1, TI, NF>(B0, B1, logn, pitch, kin, tw.t32, tw.log, tid, nthr);
             Xr = r ? B1 : B0;
             Xi = r ? B0 : B1;
         }
         CO* Xo = (CO*)Xi;
-        for (int q0 = 0; q0 < NF; q0 += nthr * kCoopChunk) {
+        for (int q0 = 0; q0 < n; q0 += nthr * kCoopChunk) {
             S st[kCoopChunk];
 #pragma unroll
             for (int c = 0; c < kCoopChunk; c++) {
                 const int k0 = q0 + tid + nthr * c;
-                if (k0 < NF) st[c] = ld(k1, k0);
+                if (k0 < n) st[c] = ld(ln, k0);
             }
 #pragma unroll
             for (int c = 0; c < kCoopChunk; c++) {
                 const int k0 = q0 + tid + nthr * c;
-                if (k0 < NF) {
+                if (k0 < n) {
                     C in[kMaxK];
                     CO out[kMaxK];
 #pragma unroll
                     for (int f = 0; f < kMaxK; f++)
-                        if (f < kin) in[f] = Xr[(size_t)f * PITCH + k0];
-                    ap(k1, k0, st[c], in, out);
+                        if (f < kin) in[f] = Xr[(size_t)f * pitch + k0];
+                    ap(ln, k0, st[c], in, out);
 #pragma unroll
                     for (int g = 0; g < kMaxK; g++)
-                        if (g < kout) Xo[(size_t)g * PITCH + k0] = out[g];
+                        if (g < kout) Xo[(size_t)g * pitch + k0] = out[g];
                 }
             }
         }
         if (kout > 0) {
             CO* scratch = (CO*)Xr;
-            const int r = fft_lines_coop<+1, TO, LOGN>(Xo, scratch, PITCH, kout, tw_of<TO>(tw), tw.log, tid, nthr);
+            const int r = fft_coop<+1, TO, NF>(Xo, scratch, logn, pitch, kout, tw.t32, tw.log, tid, nthr);
             const CO* Yr = r ? scratch : Xo;
-            for (int it = tid; it < kout * NF; it += nthr) {
-                const int g = it >> LOGN, x = it & (NF - 1);
-                dst[(size_t)g * Hs + (size_t)k1 * NF + x] = Yr[(size_t)g * PITCH + x];
+            for (int it = tid; it < kout * n; it += nthr) {
+                const int g = it >> logn, x = it & (n - 1);
+                dst[(size_t)g * Hs + (size_t)k1 * n + x] = Yr[(size_t)g * pitch + x];
             }
         }
         cta_sync();
@@ -1189,14 +1628,14 @@ __device__ void mid_pass(const Params& P, const Tw& tw, int k, const cx<T>* src,
             if constexpr (L > 0) {
                 if (nm == L) {
                     // cubic grid: both lines in lockstep through the fixed-length stages
-                    r = fft_lines_fixed<S, T, ilog2c(L), kMidG>(B0, B1, pitch, kMidG, tw_of<T>(tw), tw.log, w.lane);
+                    r = fft_lines_fixed<S, T, ilog2c(L), kMidG>(B0, B1, pitch, kMidG, tw.t32, tw.log, w.lane);
                 } else {
                     for (int g = 0; g < kMidG; g++)
-                        r = fft_line_w<S, T>(B0 + g * pitch, B1 + g * pitch, logm, tw_of<T>(tw), tw.log, w.lane);
+                        r = fft_line_w<S, T>(B0 + g * pitch, B1 + g * pitch, logm, tw.t32, tw.log, w.lane);
                 }
             } else {
                 for (int g = 0; g < kMidG; g++)
-                    r = fft_line_w<S, T>(B0 + g * pitch, B1 + g * pitch, logm, tw_of<T>(tw), tw.log, w.lane);
+                    r = fft_line_w<S, T>(B0 + g * pitch, B1 + g * pitch, logm, tw.t32, tw.log, w.lane);
             }
             const C* Br = r ? B1 : B0;
             for (int j = w.lane; j < nv; j += kWarp) {
@@ -1207,6 +1646,74 @@ __device__ void mid_pass(const Params& P, const Tw& tw, int k, const cx<T>* src,
                     const int g = j >> logm, i1 = j & (nm - 1);
                     df[rowbase + j] = Br[g * pitch + i1];
                 }
+            }
+            warp_sync();
+        }
+    }
+}
+
+// The same pass on FP64 lines in fixed point: the unit's kMidG lines one
+// after the other through a warp's line buffers.
+template <int S, int NF>
+__device__ void mid_pass_fx(const Params& P, const Tw& tw, int k, const double2* src, double2* dst, char* smem) {
+    constexpr int L = NF & (kNoCoop - 1);
+    constexpr int CH = 8;
+    const int nm = P.nm, logm = P.logm, n0 = P.n0, rows = P.rows, gpp = P.n0 / kMidG;
+    const long long H = P.H;
+    const int nv = kMidG * nm;
+    const WarpCtx w = warp_ctx(P, smem);
+    longlong2* B = (longlong2*)w.mem;
+    const URange ur = units_of(tw, P.h1 * gpp);
+    for (int u = ur.b; u < ur.e; u += ur.s) {
+        const int k1 = u / gpp, i0 = (u - k1 * gpp) * kMidG;
+        for (int f = 0; f < k; f++) {
+            const double2* sf = src + (size_t)f * H;
+            double2* df = dst + (size_t)f * H;
+            const size_t rowbase = (size_t)k1 * rows + (size_t)i0 * nm;  // [k1][i0][i1]
+            const size_t colbase = (size_t)k1 * nm * n0 + (size_t)i0;    // [k1][km][i0]
+            unsigned hi = 0;  // of the whole unit: one exponent for its lines
+            for (int j0 = w.lane; j0 < nv; j0 += CH * kWarp) {
+                double2 v[CH];
+#pragma unroll
+                for (int q = 0; q < CH; q++) {
+                    const int j = j0 + q * kWarp;
+                    if (j < nv) v[q] = S < 0 ? sf[rowbase + j] : sf[colbase + (size_t)(j / kMidG) * n0 + (j % kMidG)];
+                }
+#pragma unroll
+                for (int q = 0; q < CH; q++) {
+                    const int j = j0 + q * kWarp;
+                    if (j < nv) {
+                        const unsigned a = fx_hi(v[q].x), c = fx_hi(v[q].y), m = a > c ? a : c;
+                        hi = m > hi ? m : hi;
+                        const int g = S < 0 ? j >> logm : j % kMidG, i = S < 0 ? j & (nm - 1) : j / kMidG;
+                        *(double2*)&B[g * nm + fxs(i)] = v[q];
+                    }
+                }
+            }
+            warp_sync();
+            int e[kMidG];
+#pragma unroll
+            for (int g = 0; g < kMidG; g++) {
+                longlong2* b = B + g * nm;
+                const FxExp x = fx_convert(b, nm, hi, w.lane);
+                const int sh = x.sh;
+                e[g] = x.e;
+                if constexpr (L > 0) {
+                    if (nm == L) fx_line<S, L>(b, logm, sh, tw.tfx, tw.log, w.lane);
+                    else fx_line<S, 0>(b, logm, sh, tw.tfx, tw.log, w.lane);
+                } else {
+                    fx_line<S, 0>(b, logm, sh, tw.tfx, tw.log, w.lane);
+                }
+                e[g] -= sh;
+            }
+#pragma unroll 2
+            for (int j = w.lane; j < nv; j += kWarp) {
+                const int g = S < 0 ? j % kMidG : j >> logm, i = S < 0 ? j / kMidG : j & (nm - 1);
+                const longlong2 z = B[g * nm + fxs(i)];
+                const int eg = g == 0 ? e[0] : e[1];
+                const double2 d{fx_to(z.x, eg), fx_to(z.y, eg)};
+                if (S < 0) df[colbase + (size_t)i * n0 + g] = d;
+                else df[rowbase + j] = d;
             }
             warp_sync();
         }
@@ -1305,19 +1812,29 @@ template <class T> __device__ __forceinline__ cx<T>* cdstT(const Params& P) {
     return (cx<T>*)(P.nm > 1 ? P.NB : P.DB);
 }
 
-// dispatch: NF = 0 runs the runtime-length passes (NF may carry kNoCoop)
-// COOP: the pass has the CTA-cooperative variant (by default when it has an
-// FP64 line; phases with FP64 pointwise work on T lines ask for it too)
+// dispatch: NF = 0 runs the runtime-length passes (NF may carry kNoCoop); FP64
+// lines run in fixed point.  COOP: the pass has the CTA-cooperative variant
+// (by default when it has an FP64 line; phases with FP64 pointwise work on T
+// lines ask for it too).  A row pass has lines of one type: TI = double with
+// TO = float has no input lines (kin = 0).
 template <class TI, class TO, int NF, bool COOP = kHasCoop<TI, TO>, class Ld, class Ap>
 __device__ __forceinline__ void rowp(const Params& P, const Tw& tw, int kin, int kout, const cx<TI>* src,
                                      cx<TO>* dst, char* smem, Ld&& ld, Ap&& ap) {
     constexpr int L = NF & (kNoCoop - 1);
-    if constexpr (L == 0) {
-        row_pass<TI, TO>(P, tw, kin, kout, src, dst, smem,
-                         [&](long long p, int row, int x, const TI* in, TO* out) {
-                             const auto s = ld(p, row, x);
-                             ap(p, row, x, s, in, out);
-                         });
+    if constexpr (sizeof(TO) == 8) {
+        static_assert(sizeof(TI) == 8, "lines of one type");
+        if constexpr (COOP && !(NF & kNoCoop)) {
+            if (P.coop) {
+                row_pass_coop_fx<L>(P, tw, kin, kout, src, dst, smem, ld, ap);
+                return;
+            }
+        }
+        row_pass_fx<L>(P, tw, kin, kout, src, dst, smem, ld, ap);
+    } else if constexpr (sizeof(TI) == 8) {
+        rowp<float, TO, NF, COOP>(P, tw, 0, kout, (const float2*)nullptr, dst, smem, ld,
+                                  [&](long long p, int row, int x, const auto& s, const float*, TO* out) {
+                                      ap(p, row, x, s, (const double*)nullptr, out);
+                                  });
     } else {
         if constexpr (COOP && !(NF & kNoCoop)) {
             if (P.coop) {
@@ -1325,7 +1842,14 @@ __device__ __forceinline__ void rowp(const Params& P, const Tw& tw, int kin, int
                 return;
             }
         }
-        row_pass_fixed<TI, TO, L>(P, tw, kin, kout, src, dst, smem, ld, ap);
+        if constexpr (L == 0)
+            row_pass<TI, TO>(P, tw, kin, kout, src, dst, smem,
+                             [&](long long p, int row, int x, const TI* in, TO* out) {
+                                 const auto s = ld(p, row, x);
+                                 ap(p, row, x, s, in, out);
+                             });
+        else
+            row_pass_fixed<TI, TO, L>(P, tw, kin, kout, src, dst, smem, ld, ap);
     }
 }
 
@@ -1333,11 +1857,14 @@ template <class TI, class TO, int NF, bool COOP = kHasCoop<TI, TO>, class Ld, cl
 __device__ __forceinline__ void colp2(const Params& P, const Tw& tw, int kin, int kout, const cx<TI>* src,
                                       cx<TO>* dst, char* smem, Ld&& ld, Ap&& ap) {
     constexpr int L = NF & (kNoCoop - 1);
-    if constexpr (L == 0) {
-        col_pass<TI, TO>(P, tw, kin, kout, src, dst, smem, [&](int k1, int k0, const cx<TI>* in, cx<TO>* out) {
-            const auto s = ld(k1, k0);
-            ap(k1, k0, s, in, out);
-        });
+    if constexpr (sizeof(TI) == 8) {
+        if constexpr (COOP && !(NF & kNoCoop)) {
+            if (P.coop) {
+                col_pass_coop_fx<TO, L>(P, tw, kin, kout, src, dst, smem, ld, ap);
+                return;
+            }
+        }
+        col_pass_fx<TO, L>(P, tw, kin, kout, src, dst, smem, ld, ap);
     } else {
         if constexpr (COOP && !(NF & kNoCoop)) {
             if (P.coop) {
@@ -1345,7 +1872,13 @@ __device__ __forceinline__ void colp2(const Params& P, const Tw& tw, int kin, in
                 return;
             }
         }
-        col_pass_fixed<TI, TO, L>(P, tw, kin, kout, src, dst, smem, ld, ap);
+        if constexpr (L == 0)
+            col_pass<TI, TO>(P, tw, kin, kout, src, dst, smem, [&](const Line& k1, int k0, const cx<TI>* in, cx<TO>* out) {
+                const auto s = ld(k1, k0);
+                ap(k1, k0, s, in, out);
+            });
+        else
+            col_pass_fixed<TI, TO, L>(P, tw, kin, kout, src, dst, smem, ld, ap);
     }
 }
 template <class T, int NF, bool COOP = kHasCoop<T, T>, class Ld, class Ap>
@@ -1402,13 +1935,11 @@ __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, cons
     // the rounding of the removal from accumulating over steps).
     const T* dacc = (const T*)P.DD[c.acc_it & 1];
     const double macc =
-        c.acc ? ldcg(&P.sums[(size_t)(bank ^ 1) * P.nslots + c.acc_lastev]) / (double)P.npts +
-                    ldcg(&P.mass[0]) / (double)P.npts
-              : 0.0;
+        c.acc ? (ldcg(&P.sums[(size_t)(bank ^ 1) * P.nslots + c.acc_lastev]) + ldcg(&P.mass[0])) * P.inv_npts : 0.0;
     double dmass = 0.0;
     // rebase: the candidate of this step
     const T* dreb = (const T*)P.DD[c.it & 1];
-    const double mreb = c.reb ? ldcg(&P.sums[(size_t)bank * P.nslots + c.lastev]) / (double)P.npts : 0.0;
+    const double mreb = c.reb ? ldcg(&P.sums[(size_t)bank * P.nslots + c.lastev]) * P.inv_npts : 0.0;
     // a new step clears its bank's norm and sum slots (a restart of the same
     // step from another initial guess keeps counting in them)
     if (!c.reb && c.gmode != 2 && c.gmode != 3 && c.gmode != 4) {
@@ -1429,16 +1960,19 @@ __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, cons
         P.stats[c.step - 1].used_guess = c.acc_used;
         P.sc->steps_done = c.step;
     }
-    double s0 = 0.0, s2 = 0.0;
-    const float c1e = (float)(1.0 - P.eps), tauf = (float)P.tau, eta1f = (float)P.eta1, eta2f = (float)P.eta2,
-                e2f = (float)(P.eps * P.eps);
+    Sum2 s0, s2;
+    const float c1e = to_f32(1.0 - P.eps), tauf = to_f32(P.tau), eta1f = to_f32(P.eta1), eta2f = to_f32(P.eta2),
+                e2f = to_f32(P.eps * P.eps);
     const int kb = k_base(P.model);
     const bool pfc = P.model == M_PFC;
     const bool reb = c.reb != 0, acc = c.acc != 0;
-    const double ith = 1.0 / k.thv, wth = 1.0 - k.thv;
+    // theta_v = 1 (BDF2): v is the iterate itself; c = 0 (MP, first step): one
+    // history term
+    const double ith = k.ith, wth = 1.0 - k.thv, cg = k.b - k.gun;
+    const bool full = k.thv == 1.0, one = k.c == 0.0;
     double* U0 = P.U[c.cur];
     double* U1 = P.U[c.cur ^ 1];
-    struct St { double vb, g, a, b, d; };
+    struct St { double vb, g, a, b; T d; };
     T* yb = (T*)P.YB;
     cx<TO>* dst = INC ? (cx<TO>*)P.NB : (cx<TO>*)P.NB64;
     const double Ai = k.Ai;
@@ -1453,7 +1987,7 @@ __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, cons
             St s;
             s.vb = P.VB[p];
             s.g = P.G64[p];
-            s.d = reb ? (double)dreb[p] : (acc ? (double)dacc[p] : 0.0);
+            s.d = reb ? dreb[p] : (acc ? dacc[p] : (T)0);
             s.a = reb ? 0.0 : U0[p];   // (before acceptance) u^n of the previous step if acc
             s.b = reb ? 0.0 : U1[p];
             return s;
@@ -1461,48 +1995,56 @@ __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, cons
         [&](long long p, int, int, const St& s, const double*, TO* out) {
             double vb, g;
             if (reb) {
-                vb = s.vb + (s.d - mreb);
+                vb = s.vb + (wide(s.d) - mreb);
                 g = s.g;
             } else {
-                double a = s.a, b = s.b;
+                double a = s.a;
                 if (acc) {
                     // U1 is the previous step's u^n; the accepted u^{n+1} goes to U0
-                    const double va = s.vb + (s.d - macc);
-                    a = (va - wth * s.b) * ith;
+                    const double va = s.vb + (wide(s.d) - macc);
+                    a = full ? va : (va - wth * s.b) * ith;
                     U0[p] = a;
-                    dmass += a - s.b;
                 }
+                const double ut = a - s.b;
+                if (acc) dmass += ut;
                 // initial iterate (Sec. 3.4.2): extrapolation, or the caller's
                 // guess moved to the mass of u^n
-                const double x0 = use_guess ? P.guess[p] + gshift : a + k.rho * (a - b);
-                vb = k.thv * x0 + (1.0 - k.thv) * a;
-                g = k.b * a + k.c * b - k.gun * a;
+                const double x0 = use_guess ? P.guess[p] + gshift : fma(k.rho, ut, a);
+                vb = full ? x0 : fma(k.thv, x0, wth * a);
+                g = one ? cg * a : fma(cg, a, k.c * s.b);
                 P.G64[p] = g;
                 // averaged-Newton sums: preconditioner constants, FP32 is enough
-                const float vf = (float)vb;
+                const float vf = to_f32(vb);
                 if (pfc) {
-                    s0 += (double)(3.0f * vf * vf + c1e);
+                    s0.add(3.0f * vf * vf + c1e);
                 } else {
                     const float f1 = dF1(vf, tauf), f2 = dF2(vf, tauf), f3 = dF3(vf, tauf);
-                    s0 += (double)(f2 * f2 - eta2f * f2 + f3 * f1);
-                    s2 += (double)(e2f * (f2 - eta1f));
+                    s0.add(f2 * f2 - eta2f * f2 + f3 * f1);
+                    s2.add(e2f * (f2 - eta1f));
                 }
             }
             P.VB[p] = vb;
-            vbt[p] = (T)vb;
+            vbt[p] = cvt<T>(vb);
             d0[p] = (T)0;
             d1[p] = (T)0;
             if constexpr (INC) {
                 // a rebase keeps g, so W moves by A_i y (added spectrally); a new
                 // step transforms its W
                 const double y = vb - s.vb, r = s.vb;
-                yb[p] = (T)y;
-                const int o = reb ? 0 : 1;
-                if (!reb) out[0] = (TO)(Ai * vb + g);
-                out[o] = (TO)y;
+                const TO yt = cvt<TO>(y);
+                yb[p] = yt;
+                TO nt = (TO)0;
                 if (pfc) {
-                    const TO yt = (TO)y, rt = (TO)r;
-                    out[o + 1] = yt * ((TO)3 * rt * rt + (TO)3 * rt * yt + yt * yt);
+                    const TO rt = cvt<TO>(r);
+                    nt = yt * ((TO)3 * rt * rt + (TO)3 * rt * yt + yt * yt);
+                }
+                if (reb) {
+                    out[0] = yt;
+                    out[1] = nt;
+                } else {
+                    out[0] = cvt<TO>(fma(Ai, vb, g));
+                    out[1] = yt;
+                    out[2] = nt;
                 }
             } else {
                 out[0] = vb;
@@ -1532,25 +2074,30 @@ __device__ PAGD_COLD void phase_B_inc(const Params& P, const Ctl& c, const Tw& t
 
 // Spectral base gradient C0 = G'_N(VB) (Eqs. misc07 / obj:G'), its
 // preconditioned direction d0 and the first correction delta_1 = theta_v s d0.
+// kappa G = w / M + kappa (rest), with w = A_i v_hat + g_hat and the rest of G
+// in t; the preconditioner is L = den / kappa.  One reciprocal, of kappa den,
+// gives both 1 / kappa and 1 / L (an FP64 division costs as much as six
+// products, and every FP64 instruction 19 SM cycles per warp).
+__device__ __forceinline__ double precond_den(const Beta& B, double kap) {
+    return fma(kap, fma(kap, fma(kap, B.b4, B.b2), B.b0), B.m2);
+}
 template <class T>
-__device__ __forceinline__ void base_direction(const Params& P, const StepK& k, const Beta& B,
-                                               int k1, int k0, double kap, double2 G, double2& d) {
-    const long long idx = (long long)k1 * P.n0 + k0;
-    cx<T>* C0 = (cx<T>*)P.C0;
-    cx<T>* S0 = (cx<T>*)P.SS[0];
-    cx<T>* S1 = (cx<T>*)P.SS[1];
-    if (kap == 0.0) {
-        G = double2{0.0, 0.0};
-        d = double2{0.0, 0.0};
-    } else {
-        const double Lk = B.m2 / kap + B.b0 + B.b2 * kap + B.b4 * kap * kap;
-        if (!(Lk > 0.0)) atomicOr(&P.sc->flags, FLAG_PRECOND);
-        const double il = -1.0 / Lk;
+__device__ __forceinline__ void base_direction(const Params& P, const StepK& k, const Beta& B, double iM, long long idx,
+                                               double kap, double2 w, double2 t, double2& d) {
+    double2 G{0.0, 0.0};
+    d = double2{0.0, 0.0};
+    if (dbl_bits(kap) != 0ull) {
+        const double den = precond_den(B, kap);
+        // not positive, or a NaN
+        if (dbl_bits(den) - 1ull >= 0x7ff0000000000000ull) atomicOr(&P.sc->flags, FLAG_PRECOND);
+        const double r = 1.0 / (kap * den);
+        const double ik = r * den * iM, il = -(r * kap) * kap;
+        G = double2{fma(w.x, ik, t.x), fma(w.y, ik, t.y)};
         d = double2{il * G.x, il * G.y};
     }
-    C0[idx] = cx<T>{(T)G.x, (T)G.y};
-    S0[idx] = cx<T>{(T)0, (T)0};
-    S1[idx] = cx<T>{(T)(k.ts * d.x), (T)(k.ts * d.y)};
+    ((cx<T>*)P.C0)[idx] = cx<T>{cvt<T>(G.x), cvt<T>(G.y)};
+    ((cx<T>*)P.SS[0])[idx] = cx<T>{(T)0, (T)0};
+    ((cx<T>*)P.SS[1])[idx] = cx<T>{cvt<T>(k.ts * d.x), cvt<T>(k.ts * d.y)};
 }
 
 template <class T, int NF>
@@ -1561,51 +2108,42 @@ __device__ PAGD_COLD void phase_C(const Params& P, const Ctl& c, const Tw& tw, c
         P.mass[1] = 0.0;
     }
     const StepK& k = step_coeffs(P, c.step);
-    const Beta B = betas(P, k, c.bsel);
+    const Beta B = c.bt;
     const int kb = k_base(P.model);
-    const double iM = 1.0 / P.M;
-    const double e4 = P.eps * P.eps * P.eps * P.eps;
+    const double iM = P.iM;
     const bool gcached = c.ereb && c.gok;  // g_hat from GH64, not among the inputs
     const int kin = gcached ? kb - 1 : kb;
-    auto ldg_hat = [&](int k1, int k0) {
+    auto ldg_hat = [&](const Line& k1, int k0) {
         return gcached ? P.GH64[(long long)k1 * P.n0 + k0] : double2{0.0, 0.0};
     };
     if (P.model == M_PFC) {
         // the direction is small: its inverse transforms run in T
+        const double c0 = 1.0 - P.eps;
         colp2<double, T, NF>(P, tw, kin, 1, csrc64(P), cdstT<T>(P), smem, ldg_hat,
-                         [&](int k1, int k0, const double2& gh, const double2* in, cx<T>* out) {
-                             const double kap = kappa_at(P, k1, k0);
-                             const double2 v = in[0], g = gcached ? gh : in[1], nl = in[gcached ? 1 : 2];
-                             if (!gcached) P.GH64[(long long)k1 * P.n0 + k0] = g;
-                             P.VR64[(long long)k1 * P.n0 + k0] = v;
-                             P.NR64[(long long)k1 * P.n0 + k0] = nl;
-                             P.WR64[(long long)k1 * P.n0 + k0] = double2{k.Ai * v.x + g.x, k.Ai * v.y + g.y};
-                             double2 G{0.0, 0.0};
-                             if (kap != 0.0) {
-                                 const double Lh = 1.0 - P.eps - 2.0 * kap + kap * kap;
-                                 const double ik = iM / kap;
-                                 G.x = (k.Ai * v.x + g.x) * ik + Lh * v.x + nl.x;
-                                 G.y = (k.Ai * v.y + g.y) * ik + Lh * v.y + nl.y;
-                             }
-                             double2 d;
-                             base_direction<T>(P, k, B, k1, k0, kap, G, d);
-                             out[0] = cx<T>{(T)d.x, (T)d.y};
-                         });
+                             [&](const Line& k1, int k0, const double2& gh, const double2* in, cx<T>* out) {
+                                 const double kap = kappa_at(P, k1, k0);
+                                 const long long idx = (long long)k1.l * P.n0 + k0;
+                                 const double2 v = in[0], g = gcached ? gh : in[1], nl = gcached ? in[1] : in[2];
+                                 const double2 w{fma(k.Ai, v.x, g.x), fma(k.Ai, v.y, g.y)};
+                                 if (!gcached) P.GH64[idx] = g;
+                                 P.VR64[idx] = v;
+                                 P.NR64[idx] = nl;
+                                 P.WR64[idx] = w;
+                                 const double Lh = fma(kap, kap - 2.0, c0);
+                                 double2 d;
+                                 base_direction<T>(P, k, B, iM, idx, kap, w,
+                                                   double2{fma(Lh, v.x, nl.x), fma(Lh, v.y, nl.y)}, d);
+                                 out[0] = cx<T>{cvt<T>(d.x), cvt<T>(d.y)};
+                             });
     } else {
         colp<double, NF>(P, tw, kin, 1, csrc64(P), cdst64(P), smem, ldg_hat,
-                         [&](int k1, int k0, const double2& gh, const double2* in, double2* out) {
+                         [&](const Line& k1, int k0, const double2& gh, const double2* in, double2* out) {
                              const double kap = kappa_at(P, k1, k0);
+                             const long long idx = (long long)k1.l * P.n0 + k0;
                              const double2 v = in[0], g = gcached ? gh : in[1];
-                             if (!gcached) P.GH64[(long long)k1 * P.n0 + k0] = g;
-                             P.VR64[(long long)k1 * P.n0 + k0] = v;
-                             P.WR64[(long long)k1 * P.n0 + k0] = double2{k.Ai * v.x + g.x, k.Ai * v.y + g.y};
-                             double2 G{0.0, 0.0};
-                             if (kap != 0.0) {
-                                 const double ik = iM / kap;
-                                 G.x = (k.Ai * v.x + g.x) * ik + e4 * kap * kap * v.x;
-                                 G.y = (k.Ai * v.y + g.y) * ik + e4 * kap * kap * v.y;
-                             }
-                             P.CL64[(long long)k1 * P.n0 + k0] = G;
+                             if (!gcached) P.GH64[idx] = g;
+                             P.VR64[idx] = v;
+                             P.WR64[idx] = double2{fma(k.Ai, v.x, g.x), fma(k.Ai, v.y, g.y)};
                              out[0] = double2{-kap * v.x, -kap * v.y};
                          });
     }
@@ -1621,7 +2159,7 @@ __device__ PAGD_COLD void phase_D(const Params& P, const Tw& tw, char* smem) {
                              [&](long long p, int, int) { return P.VB[p]; },
                              [&](long long p, int, int, const double& vb, const double* in, double* out) {
                                  const double lb = in[0];
-                                 lbt[p] = (T)lb;
+                                 lbt[p] = cvt<T>(lb);
                                  P.LB64[p] = lb;
                                  const double f1 = dF1(vb, P.tau), f2 = dF2(vb, P.tau);
                                  out[0] = f1;
@@ -1632,28 +2170,30 @@ __device__ PAGD_COLD void phase_D(const Params& P, const Tw& tw, char* smem) {
 template <class T, int NF>
 __device__ PAGD_COLD void phase_E(const Params& P, const Ctl& c, const Tw& tw, char* smem) {
     const StepK& k = step_coeffs(P, c.step);
-    const Beta B = betas(P, k, c.bsel);
-    const double e2 = P.eps * P.eps;
-    const double l1 = lam_at(P, 1);
+    const Beta B = c.bt;
+    const double e2 = P.eps * P.eps, e4 = e2 * e2, iM = P.iM;
+    const double fl = -(1.0 + lam_at(P, 1)) * k.ts;
+    struct St { double2 v, w; };
     // the direction (and Lap of the first correction) are small: inverse in T
     colp2<double, T, NF>(P, tw, 2, 2, csrc64(P), cdstT<T>(P), smem,
-                     [&](int k1, int k0) { return P.CL64[(long long)k1 * P.n0 + k0]; },
-                     [&](int k1, int k0, const double2& lin, const double2* in, cx<T>* out) {
-                         const double kap = kappa_at(P, k1, k0);
-                         const long long idx = (long long)k1 * P.n0 + k0;
-                         P.NR64[idx] = in[0];
-                         P.NR64[idx + P.H] = in[1];
-                         double2 G{0.0, 0.0};
-                         if (kap != 0.0) {
-                             G.x = lin.x + e2 * kap * in[0].x + in[1].x;
-                             G.y = lin.y + e2 * kap * in[0].y + in[1].y;
-                         }
-                         double2 d;
-                         base_direction<T>(P, k, B, k1, k0, kap, G, d);
-                         out[0] = cx<T>{(T)d.x, (T)d.y};
-                         const double f = -kap * (1.0 + l1) * k.ts;
-                         out[1] = cx<T>{(T)(f * d.x), (T)(f * d.y)};
-                     });
+                         [&](const Line& k1, int k0) {
+                             const long long idx = (long long)k1.l * P.n0 + k0;
+                             return St{P.VR64[idx], P.WR64[idx]};
+                         },
+                         [&](const Line& k1, int k0, const St& s, const double2* in, cx<T>* out) {
+                             const double kap = kappa_at(P, k1, k0);
+                             const long long idx = (long long)k1.l * P.n0 + k0;
+                             P.NR64[idx] = in[0];
+                             P.NR64[idx + P.H] = in[1];
+                             const double q = e4 * kap * kap, r = e2 * kap;
+                             double2 d;
+                             base_direction<T>(P, k, B, iM, idx, kap, s.w,
+                                               double2{fma(q, s.v.x, fma(r, in[0].x, in[1].x)),
+                                                       fma(q, s.v.y, fma(r, in[0].y, in[1].y))}, d);
+                             out[0] = cx<T>{cvt<T>(d.x), cvt<T>(d.y)};
+                             const double f = fl * kap;
+                             out[1] = cx<T>{cvt<T>(f * d.x), cvt<T>(f * d.y)};
+                         });
 }
 
 // Incremental base evaluation, column part: the FP64 reference spectra move to
@@ -1667,53 +2207,41 @@ __device__ PAGD_COLD void phase_CN(const Params& P, const Ctl& c, const Tw& tw, 
         P.mass[1] = 0.0;
     }
     const StepK& k = step_coeffs(P, c.step);
-    const Beta B = betas(P, k, c.bsel);
+    const Beta B = c.bt;
     const bool reb = c.ereb != 0;
     const int kb = k_base(P.model);
     const int kin = reb ? kb - 1 : kb;
     const int o = reb ? 0 : 1;  // in[o] = y_hat, in[o + 1] = dN_hat (PFC), in[0] = W_hat (new step)
-    const double iM = 1.0 / P.M, Ai = k.Ai;
-    const double e4 = P.eps * P.eps * P.eps * P.eps;
+    const double iM = P.iM, Ai = k.Ai, c0 = 1.0 - P.eps;
     const bool pfc = P.model == M_PFC;
     struct St { double2 v, n, w; };
     colp<T, NF, true>(
         P, tw, kin, 1, csrcT<T>(P), cdstT<T>(P), smem,
-        [&](int k1, int k0) {
-            const long long idx = (long long)k1 * P.n0 + k0;
+        [&](const Line& k1, int k0) {
+            const long long idx = (long long)k1.l * P.n0 + k0;
             return St{P.VR64[idx], pfc ? P.NR64[idx] : double2{0.0, 0.0}, P.WR64[idx]};
         },
-        [&](int k1, int k0, const St& s, const C* in, C* out) {
-            const long long idx = (long long)k1 * P.n0 + k0;
-            const double kap = kappa_at(P, k1, k0);
-            const double2 yh{(double)in[o].x, (double)in[o].y};
+        [&](const Line& k1, int k0, const St& s, const C* in, C* out) {
+            const long long idx = (long long)k1.l * P.n0 + k0;
+            const C yt = o ? in[1] : in[0];
+            const double2 yh{wide(yt.x), wide(yt.y)};
             const double2 v{s.v.x + yh.x, s.v.y + yh.y};
             P.VR64[idx] = v;
-            const double2 w = reb ? double2{s.w.x + Ai * yh.x, s.w.y + Ai * yh.y}
-                                  : double2{(double)in[0].x, (double)in[0].y};
+            const double2 w = reb ? double2{fma(Ai, yh.x, s.w.x), fma(Ai, yh.y, s.w.y)}
+                                  : double2{wide(in[0].x), wide(in[0].y)};
             P.WR64[idx] = w;
             if (pfc) {
-                const double2 nl{s.n.x + (double)in[o + 1].x, s.n.y + (double)in[o + 1].y};
+                const double kap = kappa_at(P, k1, k0);
+                const C nt = o ? in[2] : in[1];
+                const double2 nl{s.n.x + wide(nt.x), s.n.y + wide(nt.y)};
                 P.NR64[idx] = nl;
-                double2 G{0.0, 0.0};
-                if (kap != 0.0) {
-                    const double Lh = 1.0 - P.eps - 2.0 * kap + kap * kap;
-                    const double ik = iM / kap;
-                    G.x = w.x * ik + Lh * v.x + nl.x;
-                    G.y = w.y * ik + Lh * v.y + nl.y;
-                }
+                const double Lh = fma(kap, kap - 2.0, c0);
                 double2 d;
-                base_direction<T>(P, k, B, k1, k0, kap, G, d);
-                out[0] = C{(T)d.x, (T)d.y};
+                base_direction<T>(P, k, B, iM, idx, kap, w, double2{fma(Lh, v.x, nl.x), fma(Lh, v.y, nl.y)}, d);
+                out[0] = C{cvt<T>(d.x), cvt<T>(d.y)};
             } else {
-                double2 G{0.0, 0.0};
-                if (kap != 0.0) {
-                    const double ik = iM / kap;
-                    G.x = w.x * ik + e4 * kap * kap * v.x;
-                    G.y = w.y * ik + e4 * kap * kap * v.y;
-                }
-                P.CL64[idx] = G;
-                const T f = (T)(-kap);
-                out[0] = C{f * in[o].x, f * in[o].y};
+                const T f = -kappa_t<T>(P, k1, k0);
+                out[0] = C{f * yt.x, f * yt.y};
             }
         });
 }
@@ -1733,12 +2261,12 @@ __device__ PAGD_COLD void phase_DN(const Params& P, const Tw& tw, char* smem) {
         [&](long long p, int, int) { return St{P.VB[p], P.LB64[p], yb[p]}; },
         [&](long long p, int, int, const St& s, const T* in, T* out) {
             const T ly = in[0];
-            const double lbn = s.lb + (double)ly;
+            const double lbn = s.lb + wide(ly);
             P.LB64[p] = lbn;
-            lbt[p] = (T)lbn;
+            lbt[p] = cvt<T>(lbn);
             const T y = s.y;
-            const T b = (T)(s.vb - (double)s.y);
-            const T lb = (T)s.lb;
+            const T b = cvt<T>(s.vb - wide(s.y));
+            const T lb = cvt<T>(s.lb);
             const T f1b = dF1(b, tau), f2b = dF2(b, tau);
             const T df1 = y * ((T)3 * b * b + (T)3 * b * y + y * y + tau * ((T)2 * b + y) - (T)1);
             const T df2 = y * ((T)6 * b + (T)3 * y + (T)2 * tau);
@@ -1752,34 +2280,31 @@ template <class T, int NF>
 __device__ PAGD_COLD void phase_EN(const Params& P, const Ctl& c, const Tw& tw, char* smem) {
     using C = cx<T>;
     const StepK& k = step_coeffs(P, c.step);
-    const Beta B = betas(P, k, c.bsel);
-    const double e2 = P.eps * P.eps;
-    const double l1 = lam_at(P, 1);
+    const Beta B = c.bt;
+    const double e2 = P.eps * P.eps, e4 = e2 * e2, iM = P.iM;
+    const double fl = -(1.0 + lam_at(P, 1)) * k.ts;
     const long long H = P.H;
-    struct St { double2 lin, f1, pp; };
+    struct St { double2 f1, pp, v, w; };
     colp<T, NF, true>(
         P, tw, 2, 2, csrcT<T>(P), cdstT<T>(P), smem,
-        [&](int k1, int k0) {
-            const long long idx = (long long)k1 * P.n0 + k0;
-            return St{P.CL64[idx], P.NR64[idx], P.NR64[idx + H]};
+        [&](const Line& k1, int k0) {
+            const long long idx = (long long)k1.l * P.n0 + k0;
+            return St{P.NR64[idx], P.NR64[idx + H], P.VR64[idx], P.WR64[idx]};
         },
-        [&](int k1, int k0, const St& s, const C* in, C* out) {
-            const long long idx = (long long)k1 * P.n0 + k0;
+        [&](const Line& k1, int k0, const St& s, const C* in, C* out) {
+            const long long idx = (long long)k1.l * P.n0 + k0;
             const double kap = kappa_at(P, k1, k0);
-            const double2 f1{s.f1.x + (double)in[0].x, s.f1.y + (double)in[0].y};
-            const double2 pp{s.pp.x + (double)in[1].x, s.pp.y + (double)in[1].y};
+            const double2 f1{s.f1.x + wide(in[0].x), s.f1.y + wide(in[0].y)};
+            const double2 pp{s.pp.x + wide(in[1].x), s.pp.y + wide(in[1].y)};
             P.NR64[idx] = f1;
             P.NR64[idx + H] = pp;
-            double2 G{0.0, 0.0};
-            if (kap != 0.0) {
-                G.x = s.lin.x + e2 * kap * f1.x + pp.x;
-                G.y = s.lin.y + e2 * kap * f1.y + pp.y;
-            }
+            const double q = e4 * kap * kap, r = e2 * kap;
             double2 d;
-            base_direction<T>(P, k, B, k1, k0, kap, G, d);
-            out[0] = C{(T)d.x, (T)d.y};
-            const double f = -kap * (1.0 + l1) * k.ts;
-            out[1] = C{(T)(f * d.x), (T)(f * d.y)};
+            base_direction<T>(P, k, B, iM, idx, kap, s.w,
+                              double2{fma(q, s.v.x, fma(r, f1.x, pp.x)), fma(q, s.v.y, fma(r, f1.y, pp.y))}, d);
+            out[0] = C{cvt<T>(d.x), cvt<T>(d.y)};
+            const double f = fl * kap;
+            out[1] = C{cvt<T>(f * d.x), cvt<T>(f * d.y)};
         });
 }
 
@@ -1789,8 +2314,8 @@ template <class T> struct RowK {
 };
 template <class T> __device__ __forceinline__ RowK<T> row_consts(const Params& P, const Ctl& c) {
     const StepK& k = step_coeffs(P, c.step);
-    return RowK<T>{(T)lam_at(P, c.it - 1), (T)lam_at(P, c.it), (T)k.ts, (T)P.tau, (T)(P.eps * P.eps),
-                   (T)P.eta1,            (T)P.eta2};
+    return RowK<T>{cvt<T>(lam_at(P, c.it - 1)), cvt<T>(lam_at(P, c.it)), cvt<T>(k.ts), cvt<T>(P.tau),
+                   cvt<T>(P.eps * P.eps), cvt<T>(P.eta1), cvt<T>(P.eta2)};
 }
 
 // One point of the iteration row pass: delta_{i+1} from the direction
@@ -1800,21 +2325,20 @@ template <class T> __device__ __forceinline__ RowK<T> row_consts(const Params& P
 // second variation's nonlinear part).
 template <class T, class TI, bool PFC>
 __device__ __forceinline__ void row_point(const RowK<T>& q, T* dcur, long long p, T dp, T dpp, T b, T lb,
-                                          const TI* in, T* out, TI& amax, double& asum) {
+                                          const TI* in, T* out, MaxAbs<TI>& amax, SumOf<T>& asum) {
     const TI dd = in[0];
     const T de = dp + q.lp * (dp - dpp) + q.ts * (T)dd;
     dcur[p] = de;
-    const TI ad = fabs(dd);
-    amax = (ad > amax || ad != ad) ? ad : amax;
-    asum += (double)de;
+    amax.add(dd);
+    asum.add(de);
     const T y = de + q.l * (de - dp);
     if (PFC) {
-        out[0] = y * ((T)3 * b * b + (T)3 * b * y + y * y);
+        out[0] = y * ((T)3 * b * (b + y) + y * y);
     } else {
         const T tau = q.tau;
         const T ly = (T)in[1];
         const T f1b = dF1(b, tau), f2b = dF2(b, tau);
-        const T df1 = y * ((T)3 * b * b + (T)3 * b * y + y * y + tau * ((T)2 * b + y) - (T)1);
+        const T df1 = y * ((T)3 * b * (b + y) + y * y + tau * ((T)2 * b + y) - (T)1);
         const T df2 = y * ((T)6 * b + (T)3 * y + (T)2 * tau);
         const T f1n = f1b + df1, f2n = f2b + df2;
         out[0] = df1;
@@ -1834,15 +2358,15 @@ __device__ __noinline__ void phase_R_staged(const Params& P, const Ctl& c, const
     const int bank = c.step & 1;
     float* dcur = (float*)P.DD[c.it & 1];
     const float* sp[4] = {(const float*)P.DD[(c.it - 1) & 1], dcur, (const float*)P.VBt, (const float*)P.LBt};
-    float amax = 0.f;
-    double asum = 0.0;
+    MaxAbs<float> amax;
+    SumOf<float> asum;
     row_pass_staged<NF, K, NS, SL>(P, tw, src, (float2*)P.NB, sp, smem,
                                    [&](long long p, int, int, const float* sv, const float* in, float* out) {
                                        row_point<float, float, PFC>(q, dcur, p, sv[0], sv[1], sv[2],
                                                                     NS > 3 ? sv[NS > 3 ? 3 : 0] : 0.f, in, out,
                                                                     amax, asum);
                                    });
-    publish_max(&P.norms[(size_t)bank * P.nslots + c.ev], (double)amax);
+    amax.publish(&P.norms[(size_t)bank * P.nslots + c.ev]);
     publish_sum(&P.sums[(size_t)bank * P.nslots + c.ev], asum);
 }
 
@@ -1859,8 +2383,8 @@ __device__ __noinline__ void phase_R_coop(const Params& P, const Ctl& c, const T
     const float* lbt = (const float*)P.LBt;
     const int K = k_iter(P.model);
     const bool pfc = P.model == M_PFC;
-    float amax = 0.f;
-    double asum = 0.0;
+    MaxAbs<float> amax;
+    SumOf<float> asum;
     struct St { float dp, dpp, b, lb; };
     row_pass_coop<float, float, NF>(
         P, tw, K, K, src, (float2*)P.NB, smem,
@@ -1870,7 +2394,7 @@ __device__ __noinline__ void phase_R_coop(const Params& P, const Ctl& c, const T
             else row_point<float, float, false>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
         });
     // every warp publishes its threads' norm and sum
-    publish_max(&P.norms[(size_t)bank * P.nslots + c.ev], (double)amax);
+    amax.publish(&P.norms[(size_t)bank * P.nslots + c.ev]);
     publish_sum(&P.sums[(size_t)bank * P.nslots + c.ev], asum);
 }
 
@@ -1901,8 +2425,8 @@ __device__ PAGD_HOT void phase_R(const Params& P, const Ctl& c, const Tw& tw, ch
     const T* vbt = (const T*)P.VBt;
     const T* lbt = (const T*)P.LBt;
     const int K = k_iter(P.model);
-    TI amax = (TI)0;
-    double asum = 0.0;
+    MaxAbs<TI> amax;
+    SumOf<T> asum;
     const bool pfc = P.model == M_PFC;
     struct St { T dp, dpp, b, lb; };
     rowp<TI, T, NF>(
@@ -1919,7 +2443,7 @@ __device__ PAGD_HOT void phase_R(const Params& P, const Ctl& c, const Tw& tw, ch
             if (pfc) row_point<T, TI, true>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
             else row_point<T, TI, false>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
         });
-    publish_max(&P.norms[(size_t)bank * P.nslots + c.ev], (double)amax);
+    amax.publish(&P.norms[(size_t)bank * P.nslots + c.ev]);
     publish_sum(&P.sums[(size_t)bank * P.nslots + c.ev], asum);
 }
 
@@ -1931,10 +2455,10 @@ template <class T> struct ColK {
 };
 template <class T> __device__ __forceinline__ ColK<T> col_consts(const Params& P, const Ctl& c) {
     const StepK& k = step_coeffs(P, c.step);
-    const Beta B = betas(P, k, c.bsel);
-    const T e2 = (T)(P.eps * P.eps);
-    return ColK<T>{(T)lam_at(P, c.it), (T)lam_at(P, c.it + 1), (T)k.ts, (T)B.m2, (T)B.b0, (T)B.b2, (T)B.b4,
-                   (T)(k.Ai / P.M),   (T)(1.0 - P.eps),       e2,       e2 * e2};
+    const Beta B = c.bt;
+    const T e2 = cvt<T>(P.eps * P.eps);
+    return ColK<T>{cvt<T>(lam_at(P, c.it)), cvt<T>(lam_at(P, c.it + 1)), cvt<T>(k.ts), cvt<T>(B.m2), cvt<T>(B.b0),
+                   cvt<T>(B.b2), cvt<T>(B.b4), cvt<T>(k.aim), cvt<T>(1.0 - P.eps), e2, e2 * e2};
 }
 
 // One wavenumber of the iteration column pass: ybar_hat, the spectral residual
@@ -1942,18 +2466,20 @@ template <class T> __device__ __forceinline__ ColK<T> col_consts(const Params& P
 // 2), the spectral state update written over the older state, and the outputs
 // to transform (d_hat; FCH also the Laplacian of ybar_{it+1}).
 template <class T, bool PFC>
-__device__ __forceinline__ void col_point(const Params& P, const ColK<T>& q, cx<T>* sprev, int k1, int k0, cx<T> sc,
-                                          cx<T> sp, cx<T> g0, const cx<T>* in, cx<T>* out) {
+__device__ __forceinline__ void col_point(const Params& P, const ColK<T>& q, cx<T>* sprev, const Line& k1, int k0,
+                                          cx<T> sc, cx<T> sp, cx<T> g0, const cx<T>* in, cx<T>* out) {
     using C = cx<T>;
-    const long long idx = (long long)k1 * P.n0 + k0;
+    const long long idx = (long long)k1.l * P.n0 + k0;
     const T kap = kappa_t<T>(P, k1, k0);
     const C yh = C{sc.x + q.l * (sc.x - sp.x), sc.y + q.l * (sc.y - sp.y)};
     C d{(T)0, (T)0};
     if (kap != (T)0) {
-        const T ik = (T)1 / kap;
-        const T il = (T)-1 / (q.m2 * ik + q.b0 + q.b2 * kap + q.b4 * kap * kap);
+        // 1 / kappa and 1 / L = kappa / den from one reciprocal
+        const T den = q.m2 + kap * (q.b0 + kap * (q.b2 + kap * q.b4));
+        const T r = (T)1 / (kap * den);
+        const T ik = r * den, il = -(r * kap) * kap;
         if (PFC) {
-            const T m = q.aim * ik + q.c0 - (T)2 * kap + kap * kap;
+            const T m = q.aim * ik + (q.c0 + kap * (kap - (T)2));
             d.x = il * (g0.x + m * yh.x + in[0].x);
             d.y = il * (g0.y + m * yh.y + in[0].y);
         } else {
@@ -1981,7 +2507,7 @@ __device__ __noinline__ void phase_CI_staged(const Params& P, const Ctl& c, cons
     float2* sprev = (float2*)P.SS[(c.it - 1) & 1];
     const float2* sc3[3] = {(const float2*)P.SS[c.it & 1], sprev, (const float2*)P.C0};
     col_pass_staged<NF, K, 3, SL>(P, tw, csrcT<float>(P), cdstT<float>(P), sc3, smem,
-                                  [&](int k1, int k0, const float2* sv, const float2* in, float2* out) {
+                                  [&](const Line& k1, int k0, const float2* sv, const float2* in, float2* out) {
                                       col_point<float, PFC>(P, q, sprev, k1, k0, sv[0], sv[1], sv[2], in, out);
                                   });
 }
@@ -1998,11 +2524,11 @@ __device__ __noinline__ void phase_CI_coop(const Params& P, const Ctl& c, const 
     struct St { float2 sc, sp, g0; };
     col_pass_coop<float, float, NF>(
         P, tw, K, K, csrcT<float>(P), cdstT<float>(P), smem,
-        [&](int k1, int k0) {
+        [&](const Line& k1, int k0) {
             const long long idx = (long long)k1 * P.n0 + k0;
             return St{scur[idx], sprev[idx], C0[idx]};
         },
-        [&](int k1, int k0, const St& s, const float2* in, float2* out) {
+        [&](const Line& k1, int k0, const St& s, const float2* in, float2* out) {
             if (pfc) col_point<float, true>(P, q, sprev, k1, k0, s.sc, s.sp, s.g0, in, out);
             else col_point<float, false>(P, q, sprev, k1, k0, s.sc, s.sp, s.g0, in, out);
         });
@@ -2037,11 +2563,11 @@ __device__ PAGD_HOT void phase_CI(const Params& P, const Ctl& c, const Tw& tw, c
     struct St { C sc, sp, g0; };
     colp<T, NF>(
         P, tw, K, K, csrcT<T>(P), cdstT<T>(P), smem,
-        [&](int k1, int k0) {
+        [&](const Line& k1, int k0) {
             const long long idx = (long long)k1 * P.n0 + k0;
             return St{scur[idx], sprev[idx], C0[idx]};
         },
-        [&](int k1, int k0, const St& s, const C* in, C* out) {
+        [&](const Line& k1, int k0, const St& s, const C* in, C* out) {
             if (pfc) col_point<T, true>(P, q, sprev, k1, k0, s.sc, s.sp, s.g0, in, out);
             else col_point<T, false>(P, q, sprev, k1, k0, s.sc, s.sp, s.g0, in, out);
         });
@@ -2058,15 +2584,16 @@ __device__ PAGD_COLD void phase_accept(const Params& P, const Ctl& c, const Tw& 
     const T* dc = (const T*)P.DD[c.it & 1];
     const double* un = P.U[c.cur];
     double* unew = P.U[c.cur ^ 1];
-    const double m = (ldcg(&P.sums[(size_t)bank * P.nslots + c.lastev]) + ldcg(&P.mass[0])) / (double)P.npts;
+    const double m = (ldcg(&P.sums[(size_t)bank * P.nslots + c.lastev]) + ldcg(&P.mass[0])) * P.inv_npts;
     const long long gt = thread_rank(tw);
     const long long gs = thread_count(tw);
-    const double ith = 1.0 / k.thv, w = (1.0 - k.thv);
+    const double ith = k.ith, w = (1.0 - k.thv);
+    const bool full = k.thv == 1.0;
     double dmass = 0.0;
     for (long long p = gt; p < P.npts; p += gs) {
-        const double v = P.VB[p] + ((double)dc[p] - m);
+        const double v = P.VB[p] + (wide(dc[p]) - m);
         const double a = un[p];
-        const double x = (v - w * a) * ith;
+        const double x = full ? v : (v - w * a) * ith;
         unew[p] = x;
         dmass += x - a;
         if (P.out_real) P.out_real[p] = x;
@@ -2102,16 +2629,16 @@ __device__ PAGD_COLD void phase_fwd_r(const Params& P, const Tw& tw, char* smem)
 }
 template <int NF>
 __device__ PAGD_COLD void phase_fwd_c(const Params& P, const Tw& tw, char* smem) {
-    colp<double, NF>(P, tw, 1, 0, csrc64(P), (double2*)nullptr, smem, [&](int, int) { return Nil{}; },
-                     [&](int k1, int k0, const Nil&, const double2* in, double2*) {
+    colp<double, NF>(P, tw, 1, 0, csrc64(P), (double2*)nullptr, smem, [&](const Line&, int) { return Nil{}; },
+                     [&](const Line& k1, int k0, const Nil&, const double2* in, double2*) {
                          P.out_spec[api_spec_index(P, k1, k0)] = in[0];
                      });
 }
 template <int NF>
 __device__ PAGD_COLD void phase_inv_c(const Params& P, const Tw& tw, char* smem) {
     colp<double, NF>(P, tw, 0, 1, (const double2*)nullptr, cdst64(P), smem,
-                     [&](int k1, int k0) { return P.in_spec[api_spec_index(P, k1, k0)]; },
-                     [&](int, int, const double2& v, const double2*, double2* out) { out[0] = v; });
+                     [&](const Line& k1, int k0) { return P.in_spec[api_spec_index(P, k1, k0)]; },
+                     [&](const Line&, int, const double2& v, const double2*, double2* out) { out[0] = v; });
 }
 template <int NF>
 __device__ PAGD_COLD void phase_inv_r(const Params& P, const Tw& tw, char* smem) {
@@ -2143,8 +2670,8 @@ __device__ PAGD_COLD void phase_en_c(const Params& P, const Tw& tw, char* smem, 
     double acc = 0.0;
     const bool pfc = P.model == M_PFC;
     const int half = P.n1 >> 1;
-    colp<double, NF>(P, tw, 1, pfc ? 0 : 1, csrc64(P), cdst64(P), smem, [&](int, int) { return Nil{}; },
-                     [&](int k1, int k0, const Nil&, const double2* in, double2* out) {
+    colp<double, NF>(P, tw, 1, pfc ? 0 : 1, csrc64(P), cdst64(P), smem, [&](const Line&, int) { return Nil{}; },
+                     [&](const Line& k1, int k0, const Nil&, const double2* in, double2* out) {
                          const double kap = kappa_at(P, k1, k0);
                          const int kl = kl_of(P, k1);
                          const double w = (kl == 0 || kl == half) ? 1.0 : 2.0;
@@ -2209,8 +2736,8 @@ __device__ PAGD_COLD void phase_rh_r0(const Params& P, const Tw& tw, char* smem)
 template <int NF>
 __device__ PAGD_COLD void phase_rh_c0(const Params& P, const Tw& tw, char* smem) {
     const bool pfc = P.model == M_PFC;
-    colp<double, NF>(P, tw, pfc ? 2 : 1, 1, csrc64(P), cdst64(P), smem, [&](int, int) { return Nil{}; },
-                     [&](int k1, int k0, const Nil&, const double2* in, double2* out) {
+    colp<double, NF>(P, tw, pfc ? 2 : 1, 1, csrc64(P), cdst64(P), smem, [&](const Line&, int) { return Nil{}; },
+                     [&](const Line& k1, int k0, const Nil&, const double2* in, double2* out) {
                          const double kap = kappa_at(P, k1, k0);
                          if (pfc) {
                              const double Lh = 1.0 - P.eps - 2.0 * kap + kap * kap;
@@ -2237,8 +2764,8 @@ template <int NF>
 __device__ PAGD_COLD void phase_rh_c1(const Params& P, const Tw& tw, char* smem) {
     const double e2 = P.eps * P.eps, e4 = e2 * e2;
     colp<double, NF>(P, tw, 2, 1, csrc64(P), cdst64(P), smem,
-                     [&](int k1, int k0) { return P.CL64[(long long)k1 * P.n0 + k0]; },
-                     [&](int k1, int k0, const double2& v, const double2* in, double2* out) {
+                     [&](const Line& k1, int k0) { return P.CL64[(long long)k1 * P.n0 + k0]; },
+                     [&](const Line& k1, int k0, const double2& v, const double2* in, double2* out) {
                          const double kap = kappa_at(P, k1, k0);
                          const double f = -P.M * kap;
                          const double mr = e4 * kap * kap * v.x + e2 * kap * in[0].x + in[1].x;
@@ -2311,21 +2838,21 @@ __device__ __forceinline__ double2 imex_solve(const Params& P, const StepK& k, d
         rx -= M * kap * 0.5 * Lh * un.x;
         ry -= M * kap * 0.5 * Lh * un.y;
     }
-    const double den = k.a + M * kap * half * Lh;
-    return double2{rx / den, ry / den};
+    const double den = 1.0 / (k.a + M * kap * half * Lh);
+    return double2{rx * den, ry * den};
 }
 template <int NF>
 __device__ PAGD_COLD void phase_im_c0(const Params& P, const Ctl& c, const Tw& tw, char* smem) {
     const StepK& k = step_coeffs(P, c.step);
     if (P.model == M_PFC) {
-        colp<double, NF>(P, tw, 3, 1, csrc64(P), cdst64(P), smem, [&](int, int) { return Nil{}; },
-                         [&](int k1, int k0, const Nil&, const double2* in, double2* out) {
+        colp<double, NF>(P, tw, 3, 1, csrc64(P), cdst64(P), smem, [&](const Line&, int) { return Nil{}; },
+                         [&](const Line& k1, int k0, const Nil&, const double2* in, double2* out) {
                              const double kap = kappa_at(P, k1, k0);
                              out[0] = imex_solve(P, k, kap, in[0], in[1], in[2]);
                          });
     } else {
-        colp<double, NF>(P, tw, 3, 1, csrc64(P), cdst64(P), smem, [&](int, int) { return Nil{}; },
-                         [&](int k1, int k0, const Nil&, const double2* in, double2* out) {
+        colp<double, NF>(P, tw, 3, 1, csrc64(P), cdst64(P), smem, [&](const Line&, int) { return Nil{}; },
+                         [&](const Line& k1, int k0, const Nil&, const double2* in, double2* out) {
                              const double kap = kappa_at(P, k1, k0);
                              const long long idx = (long long)k1 * P.n0 + k0;
                              P.CL64[idx] = in[1];
@@ -2353,11 +2880,11 @@ __device__ PAGD_COLD void phase_im_c1(const Params& P, const Ctl& c, const Tw& t
     const double e2 = P.eps * P.eps;
     struct St { double2 un, um; };
     colp<double, NF>(P, tw, 2, 1, csrc64(P), cdst64(P), smem,
-                     [&](int k1, int k0) {
+                     [&](const Line& k1, int k0) {
                          const long long idx = (long long)k1 * P.n0 + k0;
                          return St{P.CL64[idx], P.CL64[idx + P.H]};
                      },
-                     [&](int k1, int k0, const St& s, const double2* in, double2* out) {
+                     [&](const Line& k1, int k0, const St& s, const double2* in, double2* out) {
                          const double kap = kappa_at(P, k1, k0);
                          // -eps^2 Lap F' -> + eps^2 kappa F'_hat
                          const double2 nh{e2 * kap * in[0].x + in[1].x, e2 * kap * in[0].y + in[1].y};
@@ -2411,6 +2938,7 @@ __host__ __device__ inline Ctl ctl_init(const Params& P) {
     c.acc_used = 0;
     c.rec_pending = 0; c.rec_ev = 0; c.rec_bank = 0;
     c.inc = inc_eval(P, c.ref_ok, P.step0, 1);
+    c.bt = betas_from(P, step_coeffs(P, 0), 0.0, 0.0);
     c.resid = 0.0; c.base_nrm = 0.0; c.best_nrm = 0.0; c.acc_resid = 0.0;
     switch (P.prog) {
         case PROG_RUN:
@@ -2497,6 +3025,11 @@ __host__ __device__ inline void mid_insert(const Params& P, int pph, int pinc, i
 // move the base, or iterate on (c.ph = PH_CI).  Shared by the device-wide phase
 // sequence and the cluster-resident iteration loop, so both take the same
 // decisions from the same norms.
+// a <= b for non-negative a, b (false for a NaN a), compared as integers: one
+// thread of every CTA decides between two barriers, and an FP64 compare takes
+// 70 cycles
+__device__ __forceinline__ bool nn_le(double a, double b) { return dbl_bits(a) <= dbl_bits(b); }
+
 template <class T>
 __device__ void ctl_eval(const Params& P, Ctl& c, double nrm) {
     const bool t64 = sizeof(T) == 8;
@@ -2504,8 +3037,8 @@ __device__ void ctl_eval(const Params& P, Ctl& c, double nrm) {
     c.lastev = c.ev;
     c.ev++;
     c.resid = nrm;
-    if (!(nrm <= 1.0e300)) { c.fail = ST_ENAN; c.ph = PH_FAIL; return; }
-    if (c.ph == PH_R1 || nrm < c.best_nrm) { c.best_nrm = nrm; c.best_ev = c.ev; }
+    if (!nn_le(nrm, 1.0e300)) { c.fail = ST_ENAN; c.ph = PH_FAIL; return; }
+    if (c.ph == PH_R1 || !nn_le(c.best_nrm, nrm)) { c.best_nrm = nrm; c.best_ev = c.ev; }
     if (c.ph == PH_R1) c.base_nrm = nrm;
     // the first direction of a step from the extrapolation (Sec. 3.4.2): the
     // record a caller's guess is judged against
@@ -2524,7 +3057,8 @@ __device__ void ctl_eval(const Params& P, Ctl& c, double nrm) {
     // point) errs by about 1e-7 of that shift, so when its norm reaches
     // tol the base moves there and is evaluated exactly.
     const bool inc_norm = c.ph == PH_R1 && c.inc;
-    if (nrm <= P.tol && !fp32_norm && !inc_norm) {
+    const bool conv = nn_le(nrm, P.tol);
+    if (conv && !fp32_norm && !inc_norm) {
         if (c.step + 1 < P.nsteps) {
             // accepted inside the next step's phase B
             c.acc = 1;
@@ -2568,15 +3102,15 @@ __device__ void ctl_eval(const Params& P, Ctl& c, double nrm) {
         c.bsel = 3;
         c.inc = t64 ? 0 : inc_eval(P, c.ref_ok, P.step0 + c.step, 1);
         c.ph = PH_B;
-    } else if ((fp32_norm && (nrm <= P.tol || nrm <= kRebaseRatio * c.base_nrm ||
+    } else if ((fp32_norm && (conv || nn_le(nrm, kRebaseRatio * c.base_nrm) ||
                               c.ev - c.best_ev >= kStagnation)) ||
-               (inc_norm && nrm <= P.tol)) {
+               (inc_norm && conv)) {
         if (c.rech >= P.max_recheck) { c.fail = ST_ENOCONV; c.ph = PH_FAIL; return; }
         c.rech++;
         c.reb = 1;
         // a rebase that may accept is evaluated exactly; one that only
         // moves the base past the FP32 floor may be incremental
-        c.inc = (nrm <= P.tol || !c.exact_done) ? 0 : inc_eval(P, c.ref_ok, P.step0 + c.step, 0);
+        c.inc = (conv || !c.exact_done) ? 0 : inc_eval(P, c.ref_ok, P.step0 + c.step, 0);
         c.ph = PH_B;
     } else {
         c.ph = PH_CI;
@@ -2615,6 +3149,7 @@ __device__ void ctl_step(const Params& P, Ctl& c) {
             // evaluations of the guess probe (they count in the step's cost)
             if (!c.reb && c.gmode != 2 && c.gmode != 3 && c.gmode != 4) { c.ev = 0; c.rech = 0; }
             c.rec_pending = 0;  // phase B stored it
+            c.bt = betas(P, step_coeffs(P, c.step), c.bsel);
             c.ereb = c.reb;  // the evaluation started by B is a rebase (kept through C..E)
             c.acc = 0;
             c.reb = 0;
@@ -2717,19 +3252,22 @@ __device__ PAGD_DISPATCH void exec_cold(const Params& P, const Ctl& c, const Tw&
     }
 }
 
-// the FP32 middle passes of a cubic grid run staged (mid_pass_staged) when
-// the launch stages its iteration passes; returns whether it ran them (only
-// fixed line lengths instantiate the staged pass)
+// The middle pass on the iteration buffers: fixed point for T = double, else
+// staged (mid_pass_staged) on a cubic grid when the launch stages its
+// iteration passes (only fixed line lengths instantiate the staged pass)
 template <class T, int NF, int S>
-__device__ __forceinline__ bool mid_pass_staged_if(const Params& P, const Tw& tw, int k, const void* src, void* dst,
-                                                   char* smem) {
-    if constexpr (sizeof(T) == 4 && (NF & (kNoCoop - 1)) != 0) {
-        if (P.stage && P.nm == (NF & (kNoCoop - 1))) {
-            mid_pass_staged<NF & (kNoCoop - 1), S>(P, tw, k, (const float2*)src, (float2*)dst, smem);
-            return true;
+__device__ __forceinline__ void mid_iter(const Params& P, const Tw& tw, int k, const void* src, void* dst, char* smem) {
+    if constexpr (sizeof(T) == 8) {
+        mid_pass_fx<S, NF>(P, tw, k, (const double2*)src, (double2*)dst, smem);
+    } else {
+        if constexpr ((NF & (kNoCoop - 1)) != 0) {
+            if (P.stage && P.nm == (NF & (kNoCoop - 1))) {
+                mid_pass_staged<NF & (kNoCoop - 1), S>(P, tw, k, (const float2*)src, (float2*)dst, smem);
+                return;
+            }
         }
+        mid_pass<float, S, NF>(P, tw, k, (const float2*)src, (float2*)dst, smem);
     }
-    return false;
 }
 
 template <class T, int NF>
@@ -2739,56 +3277,54 @@ __device__ __forceinline__ void exec_phase(const Params& P, const Ctl& c, const 
         case PH_RI: phase_R<T, T, NF>(P, c, tw, smem, red, (const cx<T>*)P.DB); break;
         case PH_CI: phase_CI<T, NF>(P, c, tw, smem); break;
         case PH_MF:
-            if (c.m64) mid_pass<double, -1, NF>(P, tw, c.mk, P.NB64, P.X64, smem);
-            else if (!mid_pass_staged_if<T, NF, -1>(P, tw, c.mk, P.NB, P.X, smem))
-                mid_pass<T, -1, NF>(P, tw, c.mk, (const cx<T>*)P.NB, (cx<T>*)P.X, smem);
+            if (c.m64) mid_pass_fx<-1, NF>(P, tw, c.mk, P.NB64, P.X64, smem);
+            else mid_iter<T, NF, -1>(P, tw, c.mk, P.NB, P.X, smem);
             break;
         case PH_MI:
-            if (c.m64) mid_pass<double, +1, NF>(P, tw, c.mk, P.NB64, P.DB64, smem);
-            else if (!mid_pass_staged_if<T, NF, +1>(P, tw, c.mk, P.NB, P.DB, smem))
-                mid_pass<T, +1, NF>(P, tw, c.mk, (const cx<T>*)P.NB, (cx<T>*)P.DB, smem);
+            if (c.m64) mid_pass_fx<+1, NF>(P, tw, c.mk, P.NB64, P.DB64, smem);
+            else mid_iter<T, NF, +1>(P, tw, c.mk, P.NB, P.DB, smem);
             break;
         default: exec_cold<T, NF>(P, c, tw, smem, red); break;
     }
 }
 
-// shared memory per warp needed by any phase (bytes, 16-byte multiple);
+// shared memory per warp needed by any phase (bytes, 16-byte multiple): kMaxK
+// line buffers of the FP64 passes (the middle pass uses kMidG of them), the
+// FP32 passes' lines (FP32-mixed only: the iteration fields and the three
+// fields of an incremental base evaluation);
 // nf = 0: runtime-length passes, else the fixed-length ones; nm: middle axis
 inline size_t warp_smem_bytes(int n0, int n1, int model, int tsize, int nf, int nm = 1) {
     size_t m = 0;
     auto upd = [&](size_t v) { if (v > m) m = v; };
-    if (nm > 1) upd(mid_warp_smem(nm, 8));  // middle passes (3D), FP64 worst case
-    const int ki = k_iter(model);
-    if (nf == 0) {
-        upd(row_warp_smem(n1, 0, 8, 3, 8));            // B (PFC: 3 fields) / IMEX R0
-        upd(row_warp_smem(n1, 1, 8, 2, 8));            // D / IMEX R1 / energy / DFT
-        upd(row_warp_smem(n1, 0, 8, 1, 8));
-        upd(row_warp_smem(n1, ki, 8, ki, tsize));      // R1
-        upd(row_warp_smem(n1, ki, tsize, ki, tsize));  // RI
-        upd(col_warp_smem(n0, 3, 8));                  // C / IMEX C0
-        upd(col_warp_smem(n0, 2, 8));                  // E
-        upd(col_warp_smem(n0, ki, tsize));             // CI
-        upd(col_warp_smem_mixed(n0, 3, 8, 1, tsize));  // exact C (PFC): FP64 in, direction out
-        upd(col_warp_smem_mixed(n0, 2, 8, 2, tsize));  // exact E (FCH)
-    } else {
-        const size_t p = (size_t)(nf + 2);
-        auto rowf = [&](int kin, int szin, int kout, int szout) {
-            return 2 * p * ((size_t)kin * 2 * szin + (size_t)kout * 2 * szout);
-        };
-        auto colf = [&](int k, int sz) { return 2 * p * (size_t)k * 2 * sz; };
-        upd(rowf(0, 8, 3, 8));
-        upd(rowf(1, 8, 2, 8));
-        upd(rowf(ki, 8, ki, tsize));
-        upd(rowf(ki, tsize, ki, tsize));
-        upd(colf(3, 8));
-        upd(colf(2, 8));
-        upd(colf(ki, tsize));
+    const int nmax = n0 > n1 ? n0 : n1;
+    upd((size_t)kMaxK * 16 * nmax);
+    upd((size_t)kMidG * 16 * nm);
+    const int ki = k_iter(model), kb = k_base(model);
+    if (tsize == 4) {
+        if (nm > 1) upd(mid_warp_smem(nm, 4));
+        if (nf == 0) {
+            upd(row_warp_smem(n1, 0, 4, kb, 4));
+            upd(row_warp_smem(n1, 1, 4, 2, 4));
+            upd(row_warp_smem(n1, ki, 4, ki, 4));
+            upd(col_warp_smem(n0, kb, 4));
+        } else {
+            const size_t p = (size_t)(nf + 2);
+            auto rowf = [&](int kin, int kout) { return 2 * p * (size_t)(kin + kout) * 8; };
+            upd(rowf(0, kb));
+            upd(rowf(1, 2));
+            upd(rowf(ki, ki));
+            upd(2 * p * (size_t)kb * 8);
+        }
     }
     return (m + 15) & ~(size_t)15;
 }
 
-// twiddle tables in shared memory: 1 << logtw entries, FP64 then FP32
-__host__ __device__ inline size_t tw_smem_bytes(int logtw) { return ((size_t)1 << logtw) * (16 + 8); }
+// tables in shared memory: 1 << logtw twiddles, fixed point then FP32, and the
+// squares of the wavenumber indices
+constexpr int kSq = 258;  // indices to 256 (512 points per axis), a multiple of 16 bytes
+__host__ __device__ inline size_t tw_smem_bytes(int logtw) {
+    return ((size_t)1 << logtw) * (16 + 8) + kSq * sizeof(double);
+}
 
 // the fixed line length used for an n0 x n1 grid (0: runtime-length passes)
 inline int fixed_len(int n0, int n1) {
@@ -2812,8 +3348,8 @@ struct BatchParams {
     unsigned long long* trace;
     int trace_cap;
     int* ntrace;
-    const double2* tw64;
     const float2* tw32;
+    const longlong2* twfx;
 };
 
 // work units of a phase and the points one unit touches: column lines, middle
