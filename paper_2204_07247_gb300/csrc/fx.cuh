@@ -44,10 +44,11 @@ __device__ __forceinline__ long long fx_mul(long long a, long long w) {
     m += (al >> 16) * (wl >> 15);
     return (((long long)ah * wh) << 1) + ((m + (1ll << 29)) >> 30);
 }
-// complex product in three real ones
-__device__ __forceinline__ longlong2 fx_cmul(longlong2 a, longlong2 w) {
-    const long long k1 = fx_mul(a.x + a.y, w.x);
-    return longlong2{k1 - fx_mul(a.y, w.x + w.y), k1 + fx_mul(a.x, w.y - w.x)};
+// a w (S < 0) or a conj(w) (S > 0) in three real products
+template <int S> __device__ __forceinline__ longlong2 fx_cmul(longlong2 a, longlong2 w) {
+    const long long k1 = fx_mul(a.x + a.y, w.x), p = w.x + w.y, q = w.y - w.x;
+    if (S < 0) return longlong2{k1 - fx_mul(a.y, p), k1 + fx_mul(a.x, q)};
+    return longlong2{k1 + fx_mul(a.y, q), k1 - fx_mul(a.x, p)};
 }
 
 template <int S> __device__ __forceinline__ void fx_dft8(longlong2* v) {
@@ -106,19 +107,26 @@ __device__ __forceinline__ int fx_shift(unsigned s) {
 __device__ __forceinline__ long long fx_shr(long long a, int sh, long long half) { return (a + half) >> sh; }
 __device__ __forceinline__ long long fx_half(int sh) { return (1ll << sh) >> 1; }
 
-// a 2^-S as a double (round half away, overflow to infinity, below 2^-1022 to zero)
-__device__ __forceinline__ double fx_to(long long a, int S) {
+// a 2^-S as a double (round half away), |a| < 2^63.  FAST: S in [kFxLo, kFxUp], where
+// no value overflows or falls below 2^-1022 (else to infinity and zero; NaN
+// for a line marked kFxNaN).
+constexpr int kFxLo = -900, kFxUp = 1000;
+template <bool FAST> __device__ __forceinline__ double fx_to_t(long long a, int S) {
     const unsigned long long sgn = (unsigned long long)a & 0x8000000000000000ull;
     const unsigned long long u = a < 0 ? (unsigned long long)-a : (unsigned long long)a;
-    const int lz = clz64(u);
-    const unsigned long long n = u << (lz & 63);
-    const int E = 1086 - lz - S;
-    unsigned long long t = (n >> 11) + ((n >> 10) & 1ull) + ((unsigned long long)(unsigned)(E - 1) << 52);
-    if (E <= 0 || u == 0) t = 0;
-    if (E >= 2047) t = 0x7ff0000000000000ull;
-    if (S > kFxNaN / 2) t = 0x7ff8000000000000ull;
+    const int lz = clz64(u);  // at least 1
+    const unsigned long long n = u << ((lz - 1) & 63);
+    const int E = 1085 - lz - S;
+    unsigned long long t = ((n + 0x200ull) >> 10) + ((unsigned long long)(unsigned)E << 52);
+    if (u == 0 || (!FAST && E < 0)) t = 0;
+    if (!FAST) {
+        if (E >= 2046) t = 0x7ff0000000000000ull;
+        if (S > kFxNaN / 2) t = 0x7ff8000000000000ull;
+    }
     return bits_dbl(t | sgn);
 }
+__device__ __forceinline__ bool fx_fast(int S) { return S >= kFxLo && S <= kFxUp; }
+__device__ __forceinline__ double fx_to(long long a, int S) { return fx_to_t<false>(a, S); }
 // the exponent S of a converted line: 2^-S is its unit after the shift sh
 __device__ __forceinline__ int fx_scale(int emax, int sh) { return emax == 0x7ff ? kFxNaN : 1083 - emax - sh; }
 
@@ -143,6 +151,21 @@ __device__ __forceinline__ double to_f64(float x) {
     hi |= b & 0x80000000u;
     return bits_dbl(((unsigned long long)hi << 32) | lo);
 }
+// 1 / x for a positive normal x in three FP64 instructions (the compiled
+// division takes 364 cycles, six times one): an FP32 reciprocal of the
+// significand, then one step of Newton's iteration for 1 / x with its next
+// term, x0 (1 + e + e^2) with e = 1 - m x0 (|e| <= 2^-21, so e^3 is below the
+// rounding), and the exponent by integer arithmetic.  Other x: the division.
+__device__ __forceinline__ double rcp64(double x) {
+    const unsigned long long b = dbl_bits(x);
+    const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+    if (hi - 0x00100000u >= 0x7fa00000u) return 1.0 / x;
+    const float m = bits_flt(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
+    const double x0 = to_f64(1.0f / m), md = bits_dbl((b & 0xfffffffffffffull) | 0x3ff0000000000000ull);
+    const double e = fma(-md, x0, 1.0), y = fma(x0, fma(e, e, e), x0);
+    return bits_dbl(dbl_bits(y) + ((unsigned long long)(1023u - (hi >> 20)) << 52));
+}
+__device__ __forceinline__ float rcp64(float x) { return 1.0f / x; }
 template <class T> __device__ __forceinline__ T cvt(double x) {
     if constexpr (sizeof(T) == 8) return x;
     else return to_f32(x);
@@ -174,6 +197,12 @@ struct Sum2 {
 
 // ---------------------------------------------------------- warp-owned line
 
+// radix of the stage that starts at LOGNS: as stage_radix, but 4, 8, 4 for 128
+// points, whose first and last butterflies then cover all lanes
+__host__ __device__ constexpr int fx_radix(int logn, int logns) {
+    return logn == 7 ? (logns == 2 ? 8 : 4) : stage_radix(logn, logns);
+}
+
 template <int R, int S, int LOGN, int LOGNS, bool FIRST>
 __device__ __forceinline__ void fx_stage(longlong2* b, int sh, const longlong2* tw, int logTw, int lane) {
     constexpr int LR = (R == 2) ? 1 : (R == 4) ? 2 : 3;
@@ -192,11 +221,7 @@ __device__ __forceinline__ void fx_stage(longlong2* b, int sh, const longlong2* 
             for (int r = 0; r < R; r++) {
                 u[r] = b[fxs(j + r * NB)];
                 if (FIRST) u[r] = longlong2{fx_shr(u[r].x, sh, half), fx_shr(u[r].y, sh, half)};
-                if (LOGNS > 0 && r > 0) {
-                    longlong2 w = tw[(jm * r) << twshift];
-                    if (S > 0) w.y = -w.y;
-                    u[r] = fx_cmul(u[r], w);
-                }
+                if (LOGNS > 0 && r > 0) u[r] = fx_cmul<S>(u[r], tw[(jm * r) << twshift]);
             }
             fx_dft<R, S>(u);
         }
@@ -216,7 +241,7 @@ __device__ __forceinline__ void fx_stage(longlong2* b, int sh, const longlong2* 
 template <int S, int LOGN, int LOGNS>
 __device__ __forceinline__ void fx_stages(longlong2* b, int sh, const longlong2* tw, int logTw, int lane) {
     if constexpr (LOGNS < LOGN) {
-        constexpr int R = stage_radix(LOGN, LOGNS);
+        constexpr int R = fx_radix(LOGN, LOGNS);
         fx_stage<R, S, LOGN, LOGNS, LOGNS == 0>(b, sh, tw, logTw, lane);
         fx_stages<S, LOGN, LOGNS + radix_log(R)>(b, sh, tw, logTw, lane);
     }
@@ -356,20 +381,204 @@ static __device__ __noinline__ unsigned fx_load(longlong2* b, const double2* s, 
     return hi;
 }
 // a transformed packed line of exponent S -> the two rows' half spectra
-static __device__ __noinline__ void fx_store_rows(const longlong2* b, int n, int S, double2* d0, int rows, int first, int step) {
+template <bool FAST>
+__device__ __forceinline__ void fx_store_rows_t(const longlong2* b, int n, int S, double2* d0, int rows, int first, int step) {
 #pragma unroll 2
     for (int k = first; k <= (n >> 1); k += step) {
         const longlong2 zk = b[fxs(k)], zn = b[fxs((n - k) & (n - 1))];
         double2* d = d0 + (size_t)k * rows;
-        d[0] = double2{fx_to(zk.x + zn.x, S + 1), fx_to(zk.y - zn.y, S + 1)};
-        d[1] = double2{fx_to(zk.y + zn.y, S + 1), fx_to(zn.x - zk.x, S + 1)};
+        d[0] = double2{fx_to_t<FAST>(zk.x + zn.x, S), fx_to_t<FAST>(zk.y - zn.y, S)};
+        d[1] = double2{fx_to_t<FAST>(zk.y + zn.y, S), fx_to_t<FAST>(zn.x - zk.x, S)};
     }
 }
-static __device__ __noinline__ void fx_store(const longlong2* b, int n, int S, double2* d, int first, int step) {
+static __device__ __noinline__ void fx_store_rows(const longlong2* b, int n, int S, double2* d0, int rows, int first, int step) {
+    if (fx_fast(S + 1)) fx_store_rows_t<true>(b, n, S + 1, d0, rows, first, step);
+    else fx_store_rows_t<false>(b, n, S + 1, d0, rows, first, step);
+}
+template <bool FAST>
+__device__ __forceinline__ void fx_store_t(const longlong2* b, int n, int S, double2* d, int first, int step) {
 #pragma unroll 2
     for (int x = first; x < n; x += step) {
         const longlong2 z = b[fxs(x)];
-        d[x] = double2{fx_to(z.x, S), fx_to(z.y, S)};
+        d[x] = double2{fx_to_t<FAST>(z.x, S), fx_to_t<FAST>(z.y, S)};
+    }
+}
+static __device__ __noinline__ void fx_store(const longlong2* b, int n, int S, double2* d, int first, int step) {
+    if (fx_fast(S)) fx_store_t<true>(b, n, S, d, first, step);
+    else fx_store_t<false>(b, n, S, d, first, step);
+}
+
+// --------------------------------------- lines between memory and registers
+//
+// Lines of 128, 256 and 512 points: a lane holds points lane + kWarp i in
+// registers, which are whole butterflies of the first and of the last stage,
+// so a line is converted and its first stage done before it goes to shared
+// memory, and a line on its way out is converted to doubles from the registers
+// of its last stage: two round trips through shared memory instead of five.
+
+// v (converted, to be shifted by sh) -> first stage -> b
+template <int S, int LOGN> __device__ __forceinline__ void fx_first(const longlong2* v, longlong2* b, int sh, int lane) {
+    constexpr int R = fx_radix(LOGN, 0), NB = (1 << LOGN) / R, PER = NB / kWarp;
+    const long long half = fx_half(sh);
+    warp_sync();
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        longlong2 u[R];
+#pragma unroll
+        for (int r = 0; r < R; r++)
+            u[r] = longlong2{fx_shr(v[i + r * PER].x, sh, half), fx_shr(v[i + r * PER].y, sh, half)};
+        fx_dft<R, S>(u);
+#pragma unroll
+        for (int r = 0; r < R; r++) b[fxs((lane + kWarp * i) * R + r)] = u[r];
+    }
+    warp_sync();
+}
+// b (all stages but the last done) -> v
+template <int S, int LOGN>
+__device__ __forceinline__ void fx_last(longlong2* v, const longlong2* b, const longlong2* tw, int logTw, int lane) {
+    constexpr int R = LOGN == 9 ? 8 : 4, LR = radix_log(R), NB = (1 << LOGN) / R, PER = NB / kWarp;
+    const int twshift = logTw - LOGN;
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        const int j = lane + kWarp * i;
+        longlong2 u[R];
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+            u[r] = b[fxs(j + r * NB)];
+            if (r > 0) u[r] = fx_cmul<S>(u[r], tw[(j * r) << twshift]);
+        }
+        fx_dft<R, S>(u);
+#pragma unroll
+        for (int r = 0; r < R; r++) v[i + r * PER] = u[r];
+    }
+    warp_sync();
+    (void)LR;
+}
+template <int S, int LOGN, int LOGNS, int END>
+__device__ __forceinline__ void fx_middle(longlong2* b, const longlong2* tw, int logTw, int lane) {
+    if constexpr (LOGNS < END) {
+        constexpr int R = fx_radix(LOGN, LOGNS);
+        fx_stage<R, S, LOGN, LOGNS, false>(b, 0, tw, logTw, lane);
+        fx_middle<S, LOGN, LOGNS + radix_log(R), END>(b, tw, logTw, lane);
+    }
+}
+// doubles in registers -> fixed point in registers
+template <int E> __device__ __forceinline__ FxExp fx_regs(const double2* z, longlong2* v) {
+    unsigned hi = 0, s = 0;
+#pragma unroll
+    for (int i = 0; i < E; i++) {
+        const unsigned a = fx_hi(z[i].x), c = fx_hi(z[i].y), m = a > c ? a : c;
+        hi = m > hi ? m : hi;
+    }
+    const int emax = fx_emax(warp_umax(hi));
+#pragma unroll
+    for (int i = 0; i < E; i++) {
+        v[i] = longlong2{fx_from(z[i].x, emax), fx_from(z[i].y, emax)};
+        s += fx_mag(v[i]);
+    }
+    return FxExp{fx_scale(emax, 0), fx_shift(warp_uadd(s))};
+}
+template <int E> __device__ __forceinline__ void fx_put(const longlong2* v, int S, double2* d, int stride, int lane) {
+    if (fx_fast(S)) {
+#pragma unroll
+        for (int i = 0; i < E; i++)
+            d[(size_t)(lane + kWarp * i) * stride] = double2{fx_to_t<true>(v[i].x, S), fx_to_t<true>(v[i].y, S)};
+    } else {
+#pragma unroll 1
+        for (int i = 0; i < E; i++) {
+            longlong2 t = v[0];
+#pragma unroll
+            for (int q = 1; q < E; q++)
+                if (q == i) t = v[q];
+            d[(size_t)(lane + kWarp * i) * stride] = double2{fx_to(t.x, S), fx_to(t.y, S)};
+        }
+    }
+}
+// points s[i stride] of a line -> its transform in the slots of b; returns the exponent
+template <int S, int LOGN>
+__device__ __noinline__ int fx_line_in(longlong2* b, const double2* s, int stride, const longlong2* tw, int logTw, int lane) {
+    constexpr int E = (1 << LOGN) / kWarp;
+    double2 z[E];
+    longlong2 v[E];
+#pragma unroll
+    for (int i = 0; i < E; i++) z[i] = s[(size_t)(lane + kWarp * i) * stride];
+    const FxExp x = fx_regs<E>(z, v);
+    fx_first<S, LOGN>(v, b, x.sh, lane);
+    fx_middle<S, LOGN, radix_log(fx_radix(LOGN, 0)), LOGN>(b, tw, logTw, lane);
+    return x.e - x.sh;
+}
+// doubles in the lane's slots of b -> the transform at d[i stride]
+template <int S, int LOGN>
+__device__ __noinline__ void fx_line_out(longlong2* b, double2* d, int stride, const longlong2* tw, int logTw, int lane) {
+    constexpr int E = (1 << LOGN) / kWarp, END = LOGN - (LOGN == 9 ? 3 : 2);
+    longlong2 v[E];
+    double2 z[E];
+#pragma unroll
+    for (int i = 0; i < E; i++) z[i] = *(const double2*)&b[fxs(lane + kWarp * i)];
+    const FxExp x = fx_regs<E>(z, v);
+    fx_first<S, LOGN>(v, b, x.sh, lane);
+    fx_middle<S, LOGN, radix_log(fx_radix(LOGN, 0)), END>(b, tw, logTw, lane);
+    fx_last<S, LOGN>(v, b, tw, logTw, lane);
+    fx_put<E>(v, x.e - x.sh, d, stride, lane);
+}
+// doubles in the lane's slots of b -> the transform in the slots; returns the exponent
+template <int S, int LOGN>
+__device__ __noinline__ int fx_line_mid(longlong2* b, const longlong2* tw, int logTw, int lane) {
+    constexpr int E = (1 << LOGN) / kWarp;
+    longlong2 v[E];
+    double2 z[E];
+#pragma unroll
+    for (int i = 0; i < E; i++) z[i] = *(const double2*)&b[fxs(lane + kWarp * i)];
+    const FxExp x = fx_regs<E>(z, v);
+    fx_first<S, LOGN>(v, b, x.sh, lane);
+    fx_middle<S, LOGN, radix_log(fx_radix(LOGN, 0)), LOGN>(b, tw, logTw, lane);
+    return x.e - x.sh;
+}
+// s[i ss] -> the transform at d[i ds]
+template <int S, int LOGN>
+__device__ __noinline__ void fx_line_move(longlong2* b, const double2* s, int ss, double2* d, int ds, const longlong2* tw,
+                                          int logTw, int lane) {
+    constexpr int E = (1 << LOGN) / kWarp, END = LOGN - (LOGN == 9 ? 3 : 2);
+    double2 z[E];
+    longlong2 v[E];
+#pragma unroll
+    for (int i = 0; i < E; i++) z[i] = s[(size_t)(lane + kWarp * i) * ss];
+    const FxExp x = fx_regs<E>(z, v);
+    fx_first<S, LOGN>(v, b, x.sh, lane);
+    fx_middle<S, LOGN, radix_log(fx_radix(LOGN, 0)), END>(b, tw, logTw, lane);
+    fx_last<S, LOGN>(v, b, tw, logTw, lane);
+    fx_put<E>(v, x.e - x.sh, d, ds, lane);
+}
+// line lengths with those forms
+__host__ __device__ constexpr bool fx_regs_ok(int nf) { return nf == 128 || nf == 256 || nf == 512; }
+
+// The passes' entries for a line of n = 1 << logn points (NF: n, or 0 for the
+// runtime length): memory -> transform in the slots (in), slots' doubles ->
+// transform in the slots (mid), slots' doubles -> transform in memory (out).
+// hi: this lane's largest fx_hi of its slots.  in and mid return the exponent.
+template <int S, int NF>
+__device__ __forceinline__ int fx_in(longlong2* b, const double2* s, int n, int logn, const longlong2* tw, int logTw, int lane) {
+    if constexpr (fx_regs_ok(NF)) return fx_line_in<S, ilog2c(NF)>(b, s, 1, tw, logTw, lane);
+    const FxExp x = fx_convert(b, n, fx_load(b, s, n, lane, kWarp), lane);
+    fx_line<S, NF>(b, logn, x.sh, tw, logTw, lane);
+    return x.e - x.sh;
+}
+template <int S, int NF>
+__device__ __forceinline__ int fx_mid(longlong2* b, unsigned hi, int n, int logn, const longlong2* tw, int logTw, int lane) {
+    if constexpr (fx_regs_ok(NF)) return fx_line_mid<S, ilog2c(NF)>(b, tw, logTw, lane);
+    const FxExp x = fx_convert(b, n, hi, lane);
+    fx_line<S, NF>(b, logn, x.sh, tw, logTw, lane);
+    return x.e - x.sh;
+}
+template <int S, int NF>
+__device__ __forceinline__ void fx_out(longlong2* b, unsigned hi, double2* d, int n, int logn, const longlong2* tw, int logTw,
+                                       int lane) {
+    if constexpr (fx_regs_ok(NF)) {
+        fx_line_out<S, ilog2c(NF)>(b, d, 1, tw, logTw, lane);
+    } else {
+        const FxExp x = fx_convert(b, n, hi, lane);
+        fx_line<S, NF>(b, logn, x.sh, tw, logTw, lane);
+        fx_store(b, n, x.e - x.sh, d, lane, kWarp);
     }
 }
 
@@ -397,11 +606,7 @@ __device__ __forceinline__ void fx_stage_coop(const longlong2* src, longlong2* d
             for (int r = 0; r < R; r++) v[r] = longlong2{fx_shr(v[r].x, sh, half), fx_shr(v[r].y, sh, half)};
         } else {
 #pragma unroll
-            for (int r = 1; r < R; r++) {
-                longlong2 w = tw[(jm * r) << twshift];
-                if (S > 0) w.y = -w.y;
-                v[r] = fx_cmul(v[r], w);
-            }
+            for (int r = 1; r < R; r++) v[r] = fx_cmul<S>(v[r], tw[(jm * r) << twshift]);
         }
         fx_dft<R, S>(v);
         const int dd = ((j - jm) << LR) + jm;

@@ -61,7 +61,7 @@ static __device__ bool grid_barrier(Scal* sc, unsigned& gen) {
 }
 
 template <class T, int NF>
-__global__ void __launch_bounds__(kMaxThreads, 1) pagd_kernel(const __grid_constant__ Params P) {
+__global__ void __launch_bounds__(kMaxThreads, kMaxCtas) pagd_kernel(const __grid_constant__ Params P) {
     extern __shared__ __align__(16) char smem[];
     __shared__ double red[32];
     // twiddles exp(-2 pi i m / 2^logtw) staged from the global table

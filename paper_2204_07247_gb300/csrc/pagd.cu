@@ -36,6 +36,7 @@ thread_local EmuDim3 threadIdx{0, 0, 0}, blockIdx{0, 0, 0}, blockDim{1, 1, 1}, g
 
 constexpr int kMaxChunk = 4096;
 constexpr size_t kMaxSmem = 227 * 1024;  // dynamic shared memory per CTA on sm_103a
+constexpr size_t kMaxSmem2 = 113 * 1024 - 2048;  // per CTA with two on an SM (1 KB reserved and up to 1 KB static each)
 constexpr int kMaxBatch = 4096;
 constexpr int kTraceCap = 8192;  // phase records kept per launch when tracing
 // FP32-mixed: steps between exact FP64 recomputations of the reference spectra
@@ -389,15 +390,21 @@ static void make_plan(pagd_solver* s) {
 #ifdef PAGD_EMU
     const int wpb = 1;
 #else
-    const size_t room = kMaxSmem - tw_smem_bytes(s->logtw);
-    int wpb = (int)std::min<size_t>((size_t)(kMaxThreads / 32), room / s->warp_bytes);
+    // the warps of one CTA per SM, and of each of two
+    const size_t tws = tw_smem_bytes(s->logtw), room2 = kMaxSmem2 - tws;
+    int wpb = (int)std::min<size_t>((size_t)(kMaxThreads / 32), (kMaxSmem - tws) / s->warp_bytes);
+    const int wpb2 = (int)std::min<size_t>((size_t)(kMaxThreads / 32), room2 / s->warp_bytes);
     if (wpb < 1) wpb = 1;
 #endif
-    s->threads = wpb * 32;
     const long long rows = rows_of(s);
     long long units = rows / 2;
     if ((long long)s->h1 * nm > units) units = (long long)s->h1 * nm;
     const int sms = num_sms();
+#ifndef PAGD_EMU
+    // units for more warps than one CTA per SM has: two CTAs where they hold more
+    if (units > (long long)sms * wpb && 2 * wpb2 > wpb) wpb = wpb2;
+#endif
+    s->threads = wpb * 32;
     s->grid = units < sms ? (int)units : sms;
     if ((long long)s->grid < (units + wpb - 1) / wpb) {
         const long long g = (units + wpb - 1) / wpb;

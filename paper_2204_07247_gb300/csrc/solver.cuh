@@ -74,6 +74,12 @@ constexpr int kMaxK = 3;        // fields per pass
 // the register file); the launch picks as many as the warps' shared memory
 // slices allow
 constexpr int kMaxThreads = 256;
+// CTAs of the single-instance kernel per SM (128 registers a thread): a warp's
+// line transform is a chain of shared-memory round trips and integer products
+// that keeps an SM sub-partition a quarter busy (a 256-point line takes one
+// warp 9200 cycles from load to store, eight warps 11500), so grids with units
+// enough run 16 warps per SM
+constexpr int kMaxCtas = 2;
 
 // scheme coefficients of one step (see compute_step_coeffs)
 struct StepK {
@@ -838,7 +844,7 @@ __host__ __device__ constexpr size_t col_staged_smem(int n, int k, int ns, int s
 // staging slots per model: PFC (one field) prefetches the next unit into a
 // second slot; FCH (two fields, four state arrays) has room for one slot,
 // which still puts all of a unit's reads in flight at once
-__host__ __device__ constexpr int staged_slots(int model) { return model == 0 ? 2 : 1; }
+__host__ __device__ constexpr int staged_slots(int) { return 1; }
 __host__ __device__ constexpr int staged_row_state(int model) { return model == 0 ? 3 : 4; }
 
 template <int NF, int K, int NS, int SLOTS, class Ap>
@@ -1088,9 +1094,8 @@ __device__ void row_pass_fx(const Params& P, const Tw& tw, int kin, int kout, co
 #pragma unroll 1
         for (int g = 0; g < kout; g++) {
             longlong2* b = B + g * n;
-            const FxExp x = fx_convert(b, n, g == 0 ? hi[0] : (g == 1 ? hi[1] : hi[2]), w.lane);
-            fx_line<-1, NF>(b, logn, x.sh, tw.tfx, tw.log, w.lane);
-            fx_store_rows(b, n, x.e - x.sh, dst + (size_t)g * Hs + r0, rows, w.lane, kWarp);
+            const int e = fx_mid<-1, NF>(b, g == 0 ? hi[0] : (g == 1 ? hi[1] : hi[2]), n, logn, tw.tfx, tw.log, w.lane);
+            fx_store_rows(b, n, e, dst + (size_t)g * Hs + r0, rows, w.lane, kWarp);
         }
         warp_sync();
     }
@@ -1114,12 +1119,10 @@ __device__ void col_pass_fx(const Params& P, const Tw& tw, int kin, int kout, co
 #pragma unroll 1
         for (int f = 0; f < kin; f++) {
             longlong2* b = B + f * n;
-            const FxExp x = fx_convert(b, n, fx_load(b, src + (size_t)f * Hs + (size_t)k1 * n, n, w.lane, kWarp), w.lane);
-            const int e = x.e, sh = x.sh;
-            fx_line<-1, NF>(b, logn, sh, tw.tfx, tw.log, w.lane);
-            if (f == 0) sc[0] = e - sh;
-            else if (f == 1) sc[1] = e - sh;
-            else sc[2] = e - sh;
+            const int e = fx_in<-1, NF>(b, src + (size_t)f * Hs + (size_t)k1 * n, n, logn, tw.tfx, tw.log, w.lane);
+            if (f == 0) sc[0] = e;
+            else if (f == 1) sc[1] = e;
+            else sc[2] = e;
         }
         unsigned hi[kMaxK] = {0u, 0u, 0u};
         for (int x0 = w.lane; x0 < n; x0 += kWarp * kFxChunk) {
@@ -1160,9 +1163,7 @@ __device__ void col_pass_fx(const Params& P, const Tw& tw, int kin, int kout, co
             longlong2* b = B + g * n;
             CO* d = dst + (size_t)g * Hs + (size_t)k1 * n;
             if constexpr (sizeof(TO) == 8) {
-                const FxExp x = fx_convert(b, n, g == 0 ? hi[0] : (g == 1 ? hi[1] : hi[2]), w.lane);
-                fx_line<+1, NF>(b, logn, x.sh, tw.tfx, tw.log, w.lane);
-                fx_store(b, n, x.e - x.sh, d, w.lane, kWarp);
+                fx_out<+1, NF>(b, g == 0 ? hi[0] : (g == 1 ? hi[1] : hi[2]), d, n, logn, tw.tfx, tw.log, w.lane);
             } else {
                 float2* f0 = (float2*)(B + 2 * n);
                 float2* f1 = f0 + n;
@@ -1671,6 +1672,17 @@ __device__ void mid_pass_fx(const Params& P, const Tw& tw, int k, const double2*
             double2* df = dst + (size_t)f * H;
             const size_t rowbase = (size_t)k1 * rows + (size_t)i0 * nm;  // [k1][i0][i1]
             const size_t colbase = (size_t)k1 * nm * n0 + (size_t)i0;    // [k1][km][i0]
+            if constexpr (fx_regs_ok(L)) {
+                if (nm == L) {  // cubic grid
+#pragma unroll 1
+                    for (int g = 0; g < kMidG; g++) {
+                        const size_t rb = rowbase + (size_t)g * nm, cb = colbase + g;
+                        if (S < 0) fx_line_move<S, ilog2c(L)>(B, sf + rb, 1, df + cb, n0, tw.tfx, tw.log, w.lane);
+                        else fx_line_move<S, ilog2c(L)>(B, sf + cb, n0, df + rb, 1, tw.tfx, tw.log, w.lane);
+                    }
+                    continue;
+                }
+            }
             unsigned hi = 0;  // of the whole unit: one exponent for its lines
             for (int j0 = w.lane; j0 < nv; j0 += CH * kWarp) {
                 double2 v[CH];
@@ -2090,7 +2102,7 @@ __device__ __forceinline__ void base_direction(const Params& P, const StepK& k, 
         const double den = precond_den(B, kap);
         // not positive, or a NaN
         if (dbl_bits(den) - 1ull >= 0x7ff0000000000000ull) atomicOr(&P.sc->flags, FLAG_PRECOND);
-        const double r = 1.0 / (kap * den);
+        const double r = rcp64(kap * den);
         const double ik = r * den * iM, il = -(r * kap) * kap;
         G = double2{fma(w.x, ik, t.x), fma(w.y, ik, t.y)};
         d = double2{il * G.x, il * G.y};
@@ -2476,7 +2488,7 @@ __device__ __forceinline__ void col_point(const Params& P, const ColK<T>& q, cx<
     if (kap != (T)0) {
         // 1 / kappa and 1 / L = kappa / den from one reciprocal
         const T den = q.m2 + kap * (q.b0 + kap * (q.b2 + kap * q.b4));
-        const T r = (T)1 / (kap * den);
+        const T r = rcp64(kap * den);
         const T ik = r * den, il = -(r * kap) * kap;
         if (PFC) {
             const T m = q.aim * ik + (q.c0 + kap * (kap - (T)2));
@@ -2838,7 +2850,7 @@ __device__ __forceinline__ double2 imex_solve(const Params& P, const StepK& k, d
         rx -= M * kap * 0.5 * Lh * un.x;
         ry -= M * kap * 0.5 * Lh * un.y;
     }
-    const double den = 1.0 / (k.a + M * kap * half * Lh);
+    const double den = rcp64(k.a + M * kap * half * Lh);
     return double2{rx * den, ry * den};
 }
 template <int NF>
