@@ -21,13 +21,15 @@
 //
 // Parameters are one flat FP32 array in this order: P [C][2], b_P [C]; for
 // each layer W [C][C] (W[o][c]), b [C], R [C][C][M0 M1][2] (R[o][c][m], re, im);
-// Q [C], b_Q.  The DFTs over the kept modes are computed directly (two
-// separable stages per direction), not with a full FFT.
+// Q [C], b_Q.  Only the kept modes of the DFTs are computed, one axis after the
+// other; a layer is one pass over its activations (k_tile).
 #include "../../include/pagd_sno.h"
+#include "fft.cuh"
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -37,128 +39,419 @@
 namespace {
 
 constexpr int kThr = 256;
+constexpr int kTile = 512;       // points of a tile (k_tile)
+constexpr int kPitch = kTile + 4;  // of a channel's points in shared memory: rows 16 bytes apart in the banks
 
+// A tile is kTile points: R = 16 / QC rows of the last axis (or 1 / JB of one), whose
+// points x1 = j + J q (q < QC, J = n1 / QC) go one j to a lane, so that a lane
+// holds a QC-point subsequence and the 32 lanes of a warp a whole row (J <= 32)
+// or 32 of its residues.
 struct SnoDims {
     int n0, n1, np, C, L, M0, M1, M;
+    int QC, J, JB, R, NT;  // NT: tiles of a sample
 };
 
-__device__ __forceinline__ float gelu_f(float x) {
-    // GELU with the tanh form (Hendrycks and Gimpel, 2016)
+// tanh form of GELU (Hendrycks and Gimpel, 2016) and its derivative
+__device__ __forceinline__ float gelu_t(float x) {
     const float k = 0.7978845608028654f;  // sqrt(2 / pi)
-    const float u = k * (x + 0.044715f * x * x * x);
-    return 0.5f * x * (1.f + tanhf(u));
+    return tanhf(k * (x + 0.044715f * x * x * x));
 }
-__device__ __forceinline__ float gelu_grad(float x) {
+__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.f + gelu_t(x)); }
+__device__ __forceinline__ float gelu_grad(float x, float t) {
     const float k = 0.7978845608028654f;
-    const float u = k * (x + 0.044715f * x * x * x);
-    const float t = tanhf(u);
     return 0.5f * (1.f + t) + 0.5f * x * (1.f - t * t) * k * (1.f + 3.f * 0.044715f * x * x);
 }
 
 __device__ __forceinline__ int k0_of(int m0, int M0, int n0) { return m0 < M0 / 2 ? m0 : n0 - M0 + m0; }
 
-// exp(sign 2 pi i j / n) from sincospif
-__device__ __forceinline__ float2 cis(int j, int n, float sign) {
+// exp(-2 pi i j / n), j < n, from sincospif: the tables of both axes, written
+// once when the workspace is handed in
+__global__ void k_tables(float2* t, int n) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
     float s, c;
     sincospif(2.f * (float)j / (float)n, &s, &c);
-    return make_float2(c, sign * s);
-}
-// the block's table t[j] = exp(-2 pi i j / n), j < n (conjugate for the inverse)
-__device__ __forceinline__ void fill_tw(float2* t, int n) {
-    for (int j = threadIdx.x; j < n; j += blockDim.x) t[j] = cis(j, n, -1.f);
-    __syncthreads();
+    t[j] = make_float2(c, -s);
 }
 
-// ---------------------------------------------------------------- lift
-// a = [u^n, s_in (u^n - u^{n-1})], v0 = P a + b_P
-__global__ void k_lift(SnoDims d, const float* prm, const double* un, const double* unm1, float s_in, float* a,
-                       float* v0, int B) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
-    if (p >= d.np) return;
-    const size_t o = (size_t)b * d.np + p;
-    const float a0 = (float)un[o], a1 = (float)(s_in * (un[o] - unm1[o]));
-    a[((size_t)b * 2 + 0) * d.np + p] = a0;
-    a[((size_t)b * 2 + 1) * d.np + p] = a1;
-    for (int c = 0; c < d.C; c++)
-        v0[((size_t)b * d.C + c) * d.np + p] = prm[2 * c] * a0 + prm[2 * c + 1] * a1 + prm[2 * d.C + c];
+// cos(2 pi k / 16)
+__host__ __device__ constexpr float cos16(int k) {
+    const float c[16] = {1.f, 0.92387953251128674f, 0.70710678118654752f, 0.38268343236508977f,
+                         0.f, -0.38268343236508977f, -0.70710678118654752f, -0.92387953251128674f,
+                         -1.f, -0.92387953251128674f, -0.70710678118654752f, -0.38268343236508977f,
+                         0.f, 0.38268343236508977f, 0.70710678118654752f, 0.92387953251128674f};
+    return c[k & 15];
+}
+__host__ __device__ constexpr float sin16(int k) { return cos16(k - 4 + 16); }
+
+// Y[c] = sum_q x[q] exp(-2 pi i c q / QC), c = 0 .. QC / 2, of real x, from the
+// even and odd parts of x
+template <int QC> __device__ __forceinline__ void rdft(const float* x, float2* Y) {
+    constexpr int h = QC / 2, st = 16 / QC;
+    if constexpr (QC == 1) {
+        Y[0] = make_float2(x[0], 0.f);
+    } else {
+        float S[h > 1 ? h : 1], D[h > 1 ? h : 1];
+#pragma unroll
+        for (int q = 1; q < h; q++) {
+            S[q] = x[q] + x[QC - q];
+            D[q] = x[q] - x[QC - q];
+        }
+#pragma unroll
+        for (int c = 0; c <= h; c++) {
+            float re = (c & 1) ? x[0] - x[h] : x[0] + x[h], im = 0.f;
+#pragma unroll
+            for (int q = 1; q < h; q++) {
+                re = fmaf(S[q], cos16(c * q * st), re);
+                if (c > 0 && c < h) im = fmaf(D[q], -sin16(c * q * st), im);
+            }
+            Y[c] = make_float2(re, im);
+        }
+    }
+}
+// y[q] = Re sum_c Z[c] exp(+2 pi i c q / QC), c < QC
+template <int QC> __device__ __forceinline__ void irdft(const float2* Z, float* y) {
+    constexpr int h = QC / 2, st = 16 / QC;
+    if constexpr (QC == 1) {
+        y[0] = Z[0].x;
+    } else {
+        float A[h > 1 ? h : 1], B[h > 1 ? h : 1];
+#pragma unroll
+        for (int c = 1; c < h; c++) {
+            A[c] = Z[c].x + Z[QC - c].x;
+            B[c] = Z[c].y - Z[QC - c].y;
+        }
+#pragma unroll
+        for (int q = 0; q <= h; q++) {
+            float e = (q & 1) ? Z[0].x - Z[h].x : Z[0].x + Z[h].x, o = 0.f;
+#pragma unroll
+            for (int c = 1; c < h; c++) {
+                e = fmaf(A[c], cos16(c * q * st), e);
+                if (q > 0 && q < h) o = fmaf(B[c], sin16(c * q * st), o);
+            }
+            y[q] = e - o;
+            if (q > 0 && q < h) y[QC - q] = e + o;
+        }
+    }
 }
 
-// ------------------------------------------------- truncated DFT, forward
-// stage 1 (last axis): T[r][m1] = sum_x1 X[r][x1] e^{-2 pi i m1 x1 / n1}, one block per row r
-__global__ void k_dft_rows(SnoDims d, const float* X, float2* T) {
-    __shared__ float2 part[kThr / 32][32];
-    extern __shared__ float2 tw[];  // n1 entries
-    fill_tw(tw, d.n1);
-    const int r = blockIdx.x;
-    const float* x = X + (size_t)r * d.n1;
-    float2 acc[32];
-    for (int m = 0; m < d.M1; m++) acc[m] = make_float2(0.f, 0.f);
-    for (int x1 = threadIdx.x; x1 < d.n1; x1 += blockDim.x) {
-        const float v = x[x1];
-        for (int m = 0; m < d.M1; m++) {
-            const float2 e = tw[(m * x1) & (d.n1 - 1)];
-            acc[m].x += v * e.x;
-            acc[m].y += v * e.y;
+// Sums of V = 2 MM values over the lanes of a warp, dealt to the lanes: each
+// exchange halves the values a lane still holds.  On return lane l holds values
+// l V / 32 .. (V = 32 or 64).
+template <int V> __device__ __forceinline__ void reduce_deal(float* v, int lane) {
+    int cnt = V;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const bool up = (lane & s) != 0;
+        const int hf = cnt / 2;
+#pragma unroll
+        for (int i = 0; i < V / 2; i++) {
+            if (i < hf) {
+                const float give = up ? v[i] : v[i + hf], keep = up ? v[i + hf] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, give, s);
+            }
         }
+        cnt = hf;
     }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int m = 0; m < d.M1; m++) {
-        float re = acc[m].x, im = acc[m].y;
-        for (int s = 16; s > 0; s >>= 1) {
-            re += __shfl_xor_sync(0xffffffffu, re, s);
-            im += __shfl_xor_sync(0xffffffffu, im, s);
+}
+
+// What a tile kernel does at its points (k_tile)
+enum { T_LIFT, T_LAYER, T_GUESS, T_LOSS, T_BACK, T_BACK0 };
+
+struct TileArgs {
+    const float* prm;     // P, b_P (T_LIFT)
+    const double *un, *unm1, *target;
+    float s_in;
+    double rho, s_out, inv_s_out, dscale;  // dscale = 2 / (np B)
+    const float* W;       // the layer's W [C][C] and bias
+    const float* bias;
+    const float* Q;       // Q [C], b_Q
+    const float2* G;      // modes [B][C][M] of the spectral part
+    const float* vin;     // [B][C][np]: v_l, or dz_l
+    const float* zprev;   // z_{l-1} (T_BACK)
+    float* vout;          // v_{l+1}, or dz_{l-1}; nullable
+    float* z;             // nullable
+    float2* T;            // row transforms [B][C][n0 JB][M1] of the tile's output
+    const float2 *tw0, *tw1;
+    double* guess;
+    double* loss;
+    float* part;          // per-block sums: T_LOSS [C + 1], T_BACK0 [C][3]
+};
+
+// One tile of every channel, in one block:
+//   the spectral part at the tile's points from its modes (first axis by a
+//   direct sum over the M0 kept modes, last axis by twiddles and a QC-point
+//   real transform per lane), the channel mixing W v, the pointwise function,
+//   and the tile's part of the last-axis transform of the result, whose first-
+//   axis sums k_cols takes.
+// The activations are read and written once per layer; per point and channel
+// the transforms cost 2 x 15 multiply-adds and the mixing C.  FP32 throughout.
+// CT: channels rounded up to 16 or 32; MM: kept modes of the last axis to 16
+// or 32.  Dynamic shared memory: tile_smem().
+template <int MODE, int QC, int CT, int MM>
+__global__ void __launch_bounds__(kThr, CT <= 16 ? 2 : 1) k_tile(SnoDims d, TileArgs a) {
+    constexpr int R = 16 / QC;
+    extern __shared__ __align__(16) float sm[];
+    float* y = sm;                                  // [C][kPitch]
+    float* sw = y + d.C * kPitch;                   // [CT][CT] row = output channel, [CT] bias
+    float2* tj = (float2*)(sw + CT * CT + CT);      // [M1][32] exp(-2 pi i m1 j / n1)
+    float2* U = tj + d.M1 * 32;                     // [R][C][M1]
+    float2* e0 = U + R * d.C * d.M1;                // [R][M0] exp(-2 pi i k0 x0 / n0)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.y;
+    const int rg = blockIdx.x / d.JB, jb = blockIdx.x - rg * d.JB, x00 = rg * R, j = jb * 32 + lane;
+    const size_t bc = (size_t)b * d.C;
+    for (int i = tid; i < d.M1 * 32; i += kThr) tj[i] = a.tw1[((i >> 5) * (jb * 32 + (i & 31))) & (d.n1 - 1)];
+    if constexpr (MODE != T_LIFT) {
+        for (int i = tid; i < CT * CT; i += kThr) {
+            const int o = i / CT, c = i % CT;
+            const bool in = o < d.C && c < d.C;
+            sw[i] = !in ? 0.f : (MODE == T_BACK || MODE == T_BACK0) ? a.W[c * d.C + o] : a.W[o * d.C + c];
         }
-        if (lane == 0) part[w][m] = make_float2(re, im);
+        for (int i = tid; i < CT; i += kThr)
+            sw[CT * CT + i] = (i < d.C && MODE != T_BACK && MODE != T_BACK0) ? a.bias[i] : 0.f;
+        for (int i = tid; i < R * d.M0; i += kThr) {
+            const int rr = i / d.M0, m0 = i - rr * d.M0;
+            e0[i] = a.tw0[(k0_of(m0, d.M0, d.n0) * (x00 + rr)) & (d.n0 - 1)];
+        }
+        __syncthreads();
+        // first axis: U[rr][o][m1] = w sum_m0 G[o][m0][m1] exp(+2 pi i k0 x0 / n0)
+        const bool back = MODE == T_BACK || MODE == T_BACK0;
+        const float inv = 1.f / (float)d.np;
+        for (int i = tid; i < d.C * d.M1; i += kThr) {
+            const int o = i / d.M1, m1 = i - o * d.M1;
+            const float2* g = a.G + (bc + o) * d.M + m1;
+            float2 s[R];
+#pragma unroll
+            for (int rr = 0; rr < R; rr++) s[rr] = make_float2(0.f, 0.f);
+#pragma unroll 4
+            for (int m0 = 0; m0 < d.M0; m0++) {
+                const float2 v = g[m0 * d.M1];
+#pragma unroll
+                for (int rr = 0; rr < R; rr++) {
+                    const float2 e = e0[rr * d.M0 + m0];  // conjugated
+                    s[rr].x += v.x * e.x + v.y * e.y;
+                    s[rr].y += v.y * e.x - v.x * e.y;
+                }
+            }
+            const float w = back ? 1.f : (m1 == 0 ? inv : 2.f * inv);
+#pragma unroll
+            for (int rr = 0; rr < R; rr++) U[(rr * d.C + o) * d.M1 + m1] = make_float2(w * s[rr].x, w * s[rr].y);
+        }
+        __syncthreads();
+        // last axis: a lane's QC points of row rr, channel o
+        for (int p = warp; p < R * d.C; p += kThr / 32) {
+            const int rr = p / d.C, o = p - rr * d.C;
+            float2 Z[QC];
+#pragma unroll
+            for (int c = 0; c < QC; c++) Z[c] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int m = 0; m < MM; m++) {
+                if (m < d.M1) {
+                    const float2 u = U[p * d.M1 + m], e = tj[m * 32 + lane];  // conjugated
+                    Z[m % QC].x += u.x * e.x + u.y * e.y;
+                    Z[m % QC].y += u.y * e.x - u.x * e.y;
+                }
+            }
+            float v[QC];
+            irdft<QC>(Z, v);
+#pragma unroll
+            for (int q = 0; q < QC; q++) y[o * kPitch + (rr * QC + q) * 32 + lane] = v[q];
+        }
     }
     __syncthreads();
-    if (threadIdx.x < d.M1) {
+    // pointwise
+    double lacc = 0.0;
+    float qacc[CT + 1];   // T_LOSS: sums of dout v_L, dout
+    float pacc[3][MODE == T_BACK0 ? CT : 1];
+    if constexpr (MODE == T_LOSS)
+        for (int c = 0; c <= CT; c++) qacc[c] = 0.f;
+    if constexpr (MODE == T_BACK0)
+        for (int c = 0; c < CT; c++) pacc[0][c] = pacc[1][c] = pacc[2][c] = 0.f;
+#pragma unroll 1
+    for (int s = tid; s < kTile; s += kThr) {
+        const int x0 = x00 + s / (QC * 32), q = (s >> 5) % QC, x1 = j + d.J * q;
+        const bool in = x0 < d.n0 && j < d.J;
+        const size_t p = in ? (size_t)x0 * d.n1 + x1 : 0, ip = (size_t)b * d.np + p;
+        if constexpr (MODE == T_LIFT) {
+            const double u = in ? a.un[ip] : 0.0, um = in ? a.unm1[ip] : 0.0;
+            const float a0 = pagd::to_f32(u), a1 = pagd::to_f32(a.s_in * (u - um));
+            for (int c = 0; c < d.C; c++) {
+                const float v = in ? a.prm[2 * c] * a0 + a.prm[2 * c + 1] * a1 + a.prm[2 * d.C + c] : 0.f;
+                if (in) a.vout[(bc + c) * d.np + p] = v;
+                y[c * kPitch + s] = v;
+            }
+        } else {
+            float vin[CT];
+#pragma unroll
+            for (int c = 0; c < CT; c++) vin[c] = (c < d.C && in) ? a.vin[(bc + c) * d.np + p] : 0.f;
+            float out = 0.f;
+            float tn[MODE == T_LOSS ? CT : 1], zz[MODE == T_LOSS ? CT : 1];
+#pragma unroll
+            for (int o = 0; o < CT; o++) {
+                if (o < d.C) {
+                    float f = sw[CT * CT + o] + y[o * kPitch + s];
+#pragma unroll
+                    for (int c = 0; c < CT; c += 4) {
+                        const float4 w = *(const float4*)&sw[o * CT + c];
+                        f = fmaf(w.x, vin[c], fmaf(w.y, vin[c + 1], fmaf(w.z, vin[c + 2], fmaf(w.w, vin[c + 3], f))));
+                    }
+                    const size_t i = (bc + o) * d.np + p;
+                    if constexpr (MODE == T_LAYER) {
+                        const float v = gelu_f(f);
+                        if (in) {
+                            if (a.z) a.z[i] = f;
+                            a.vout[i] = v;
+                        }
+                        y[o * kPitch + s] = in ? v : 0.f;
+                    } else if constexpr (MODE == T_GUESS) {
+                        out = fmaf(a.Q[o], gelu_f(f), out);
+                    } else if constexpr (MODE == T_LOSS) {
+                        tn[o] = gelu_t(f);
+                        zz[o] = f;
+                        out = fmaf(a.Q[o], 0.5f * f * (1.f + tn[o]), out);
+                    } else if constexpr (MODE == T_BACK) {
+                        const float z = in ? a.zprev[i] : 0.f;
+                        const float g = f * gelu_grad(z, gelu_t(z));
+                        if (in) a.vout[i] = g;
+                        y[o * kPitch + s] = in ? g : 0.f;
+                    } else {
+                        y[o * kPitch + s] = in ? f : 0.f;  // dv_0
+                    }
+                }
+            }
+            if constexpr (MODE == T_GUESS || MODE == T_LOSS) {
+                const float o = out + a.Q[d.C];
+                const double u = in ? a.un[ip] : 0.0, um = in ? a.unm1[ip] : 0.0, ext = fma(a.rho, u - um, u);
+                if constexpr (MODE == T_GUESS) {
+                    if (in) a.guess[ip] = fma(a.s_out, pagd::to_f64(o), ext);
+                } else {
+                    const double e = in ? pagd::to_f64(o) - (a.target[ip] - ext) * a.inv_s_out : 0.0;
+                    lacc = fma(e, e, lacc);
+                    const float g = pagd::to_f32(a.dscale * e);
+#pragma unroll
+                    for (int c = 0; c < CT; c++) {
+                        if (c < d.C) {
+                            qacc[c] = fmaf(g, 0.5f * zz[c] * (1.f + tn[c]), qacc[c]);
+                            const float dz = a.Q[c] * g * gelu_grad(zz[c], tn[c]);
+                            if (in) a.vout[(bc + c) * d.np + p] = dz;
+                            y[c * kPitch + s] = in ? dz : 0.f;
+                        }
+                    }
+                    qacc[CT] += g;
+                }
+            }
+            if constexpr (MODE == T_BACK0) {
+                const double u = in ? a.un[ip] : 0.0, um = in ? a.unm1[ip] : 0.0;
+                const float a0 = pagd::to_f32(u), a1 = pagd::to_f32(a.s_in * (u - um));
+#pragma unroll
+                for (int c = 0; c < CT; c++) {
+                    if (c < d.C) {
+                        const float g = y[c * kPitch + s];
+                        pacc[0][c] = fmaf(g, a0, pacc[0][c]);
+                        pacc[1][c] = fmaf(g, a1, pacc[1][c]);
+                        pacc[2][c] += g;
+                    }
+                }
+            }
+        }
+    }
+    if constexpr (MODE == T_LOSS || MODE == T_BACK0) {
+        // block sums of the per-thread accumulators -> one row of part
+        constexpr int NV = MODE == T_LOSS ? CT + 1 : 3 * CT;
+        float* red = (float*)U;  // [kThr / 32][NV]: the spectral part's buffers are free
+        const int nv = MODE == T_LOSS ? d.C + 1 : 3 * d.C;
+#pragma unroll
+        for (int c = 0; c < NV; c++) {
+            float v;
+            if constexpr (MODE == T_LOSS) v = qacc[c];
+            else v = pacc[c % 3][c / 3];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) red[warp * NV + c] = v;
+        }
+        if constexpr (MODE == T_LOSS) {
+            for (int o = 16; o > 0; o >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, o);
+            if (lane == 0) atomicAdd(a.loss, lacc * (0.5 * a.dscale));
+        }
+        __syncthreads();
+        for (int i = tid; i < nv; i += kThr) {
+            const int c = (MODE == T_LOSS && i == d.C) ? CT : i;
+            float v = 0.f;
+            for (int w = 0; w < kThr / 32; w++) v += red[w * NV + c];
+            a.part[((size_t)b * gridDim.x + blockIdx.x) * nv + i] = v;
+        }
+    }
+    if constexpr (MODE == T_LIFT || MODE == T_LAYER || MODE == T_LOSS || MODE == T_BACK) {
+        __syncthreads();
+        // last-axis transform of the tile's rows
+        for (int pq = warp; pq < R * d.C; pq += kThr / 32) {
+            const int rr = pq / d.C, o = pq - rr * d.C, x0 = x00 + rr;
+            float v[QC];
+            float2 Y[QC / 2 + 1];
+#pragma unroll
+            for (int q = 0; q < QC; q++) v[q] = y[o * kPitch + (rr * QC + q) * 32 + lane];
+            rdft<QC>(v, Y);
+            float acc[2 * MM];
+#pragma unroll
+            for (int m = 0; m < MM; m++) {
+                constexpr int h = QC / 2;
+                const int c = m % QC;
+                float2 w = c <= h ? Y[c] : make_float2(Y[QC - c].x, -Y[QC - c].y);
+                const float2 e = m < d.M1 ? tj[m * 32 + lane] : make_float2(0.f, 0.f);
+                acc[2 * m] = w.x * e.x - w.y * e.y;
+                acc[2 * m + 1] = w.x * e.y + w.y * e.x;
+            }
+            reduce_deal<2 * MM>(acc, lane);
+            if (x0 < d.n0) {
+                float* t = (float*)(a.T + ((bc + o) * (size_t)(d.n0 * d.JB) + (size_t)x0 * d.JB + jb) * d.M1);
+                if constexpr (MM == 32) {
+                    if (lane < d.M1) *(float2*)&t[2 * lane] = make_float2(acc[0], acc[1]);
+                } else {
+                    if (lane < 2 * d.M1) t[lane] = acc[0];
+                }
+            }
+        }
+    }
+}
+
+static size_t tile_smem(const SnoDims& d, int CT) {
+    const size_t red = (size_t)(kThr / 32) * 3 * CT * sizeof(float);
+    size_t spec = sizeof(float2) * ((size_t)d.R * d.C * d.M1 + (size_t)d.R * d.M0);
+    if (spec < red) spec = red;
+    return sizeof(float) * ((size_t)d.C * kPitch + CT * CT + CT) + sizeof(float2) * (size_t)d.M1 * 32 + spec;
+}
+
+// First axis: F[g][m0][m1] = sum over the rows r of T[g][r][m1] exp(-2 pi i k0 x0(r) / n0), one
+// block per channel g, a thread per mode and share of the rows
+constexpr int kColThr = 1024;
+__global__ void __launch_bounds__(kColThr) k_cols(SnoDims d, const float2* T, const float2* tw0, float2* F) {
+    extern __shared__ __align__(16) float2 cs[];  // n0 twiddles, then the shares' sums
+    float2* part = cs + d.n0;
+    for (int i = threadIdx.x; i < d.n0; i += kColThr) cs[i] = tw0[i];
+    __syncthreads();
+    int mp = 32;
+    while (mp < d.M) mp <<= 1;
+    const int g = blockIdx.x, m = threadIdx.x & (mp - 1), q = threadIdx.x / mp, nq = kColThr / mp, nr = d.n0 * d.JB;
+    if (m < d.M) {
+        const int m0 = m / d.M1, m1 = m - m0 * d.M1, k0 = k0_of(m0, d.M0, d.n0);
+        const float2* t = T + (size_t)g * nr * d.M1 + m1;
         float2 s = make_float2(0.f, 0.f);
-        for (int i = 0; i < (int)(blockDim.x >> 5); i++) {
-            s.x += part[i][threadIdx.x].x;
-            s.y += part[i][threadIdx.x].y;
+#pragma unroll 4
+        for (int r = q; r < nr; r += nq) {
+            const float2 v = t[(size_t)r * d.M1], e = cs[(k0 * (r / d.JB)) & (d.n0 - 1)];
+            s.x += v.x * e.x - v.y * e.y;
+            s.y += v.x * e.y + v.y * e.x;
         }
-        T[(size_t)r * d.M1 + threadIdx.x] = s;
+        part[q * mp + m] = s;
     }
-}
-
-// stage 2 (first axis): F[g][m0][m1] = sum_x0 T[g][x0][m1] e^{-2 pi i k0 x0 / n0}, one block per
-// channel g, one thread per mode
-__global__ void k_dft_cols(SnoDims d, const float2* T, float2* F) {
-    extern __shared__ float2 tw[];  // n0 entries
-    fill_tw(tw, d.n0);
-    const int g = blockIdx.x, m = threadIdx.x;
-    if (m >= d.M) return;
-    const int m0 = m / d.M1, m1 = m % d.M1, k0 = k0_of(m0, d.M0, d.n0);
-    const float2* t = T + (size_t)g * d.n0 * d.M1 + m1;
-    float2 s = make_float2(0.f, 0.f);
-    for (int x0 = 0; x0 < d.n0; x0++) {
-        const float2 v = t[(size_t)x0 * d.M1];
-        const float2 e = tw[(k0 * x0) & (d.n0 - 1)];
-        s.x += v.x * e.x - v.y * e.y;
-        s.y += v.x * e.y + v.y * e.x;
+    __syncthreads();
+    for (int i = threadIdx.x; i < d.M; i += kColThr) {
+        float2 s = part[i];
+        for (int k = 1; k < nq; k++) {
+            s.x += part[k * mp + i].x;
+            s.y += part[k * mp + i].y;
+        }
+        F[(size_t)g * d.M + i] = s;
     }
-    F[(size_t)g * d.M + m] = s;
-}
-
-// ------------------------------------------------ truncated DFT, inverse
-// stage 1 (first axis): U[g][x0][m1] = sum_m0 X[g][m0][m1] e^{+2 pi i k0 x0 / n0}
-__global__ void k_idft_cols(SnoDims d, const float2* X, float2* U) {
-    extern __shared__ float2 tw[];  // n0 entries
-    fill_tw(tw, d.n0);
-    const int g = blockIdx.y;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;  // x0 * M1 + m1
-    if (i >= d.n0 * d.M1) return;
-    const int x0 = i / d.M1, m1 = i % d.M1;
-    float2 s = make_float2(0.f, 0.f);
-    for (int m0 = 0; m0 < d.M0; m0++) {
-        const float2 v = X[(size_t)g * d.M + m0 * d.M1 + m1];
-        const int k0 = k0_of(m0, d.M0, d.n0);
-        float2 e = tw[(k0 * x0) & (d.n0 - 1)];
-        e.y = -e.y;
-        s.x += v.x * e.x - v.y * e.y;
-        s.y += v.x * e.y + v.y * e.x;
-    }
-    U[(size_t)g * d.n0 * d.M1 + i] = s;
 }
 
 // ---------------------------------------------------------------- mixing
@@ -169,258 +462,158 @@ __global__ void k_mix(SnoDims d, const float* R, const float2* F, float2* G) {
     if (i >= d.C * d.M) return;
     const int o = i / d.M, m = i % d.M;
     float2 s = make_float2(0.f, 0.f);
+#pragma unroll 4
     for (int c = 0; c < d.C; c++) {
-        const float* r = R + (((size_t)o * d.C + c) * d.M + m) * 2;
+        const float* rp = R + (((size_t)o * d.C + c) * d.M + m) * 2;  // may start at an odd float
+        const float2 r = make_float2(rp[0], rp[1]);
         const float2 f = F[((size_t)b * d.C + c) * d.M + m];
-        s.x += r[0] * f.x - r[1] * f.y;
-        s.y += r[0] * f.y + r[1] * f.x;
+        s.x += r.x * f.x - r.y * f.y;
+        s.y += r.x * f.y + r.y * f.x;
     }
     G[((size_t)b * d.C + o) * d.M + m] = s;
 }
 
-// ----------------------------------------------- layer: W v + b + K v, GELU
-// One block per (row x0, sample b); U holds the first-axis inverse of G.
-__global__ void k_layer(SnoDims d, const float* W, const float* bias, const float2* U, const float* v, float* z,
-                        float* vn, int last_act) {
-    extern __shared__ float2 su[];  // [C][M1], then the table of n1 twiddles
-    __shared__ float sw[32 * 32 + 32];
-    float2* tw = su + d.C * d.M1;
-    fill_tw(tw, d.n1);
-    const int x0 = blockIdx.x, b = blockIdx.y;
-    for (int i = threadIdx.x; i < d.C * d.M1; i += blockDim.x) {
-        const int o = i / d.M1, m1 = i % d.M1;
-        su[i] = U[(((size_t)b * d.C + o) * d.n0 + x0) * d.M1 + m1];
-    }
-    for (int i = threadIdx.x; i < d.C * d.C; i += blockDim.x) sw[i] = W[i];
-    for (int i = threadIdx.x; i < d.C; i += blockDim.x) sw[d.C * d.C + i] = bias[i];
-    __syncthreads();
-    const float inv = 1.f / (float)d.np;
-    for (int x1 = threadIdx.x; x1 < d.n1; x1 += blockDim.x) {
-        const size_t p = (size_t)x0 * d.n1 + x1;
-        float vin[32];
-        for (int c = 0; c < d.C; c++) vin[c] = v[((size_t)b * d.C + c) * d.np + p];
-        for (int o = 0; o < d.C; o++) {
-            float y = 0.f;
-            for (int m1 = 0; m1 < d.M1; m1++) {
-                const float2 e = tw[(m1 * x1) & (d.n1 - 1)];  // conjugated below: exp(+i ...)
-                const float2 u = su[o * d.M1 + m1];
-                y += (m1 == 0 ? 1.f : 2.f) * (u.x * e.x + u.y * e.y);
-            }
-            float s = sw[d.C * d.C + o] + y * inv;
-            for (int c = 0; c < d.C; c++) s += sw[o * d.C + c] * vin[c];
-            z[((size_t)b * d.C + o) * d.np + p] = s;
-            vn[((size_t)b * d.C + o) * d.np + p] = last_act ? gelu_f(s) : s;
+// spectral part of the backward pass: dG[b][o][m] = (w_m / np) DFT(dz)[b][o][m];
+// dR[o][c][m] = sum_b dG conj(F), dF[b][c][m] = sum_o conj(R) dG.  One block per
+// channel c and 32 modes, the o split over its warps.
+__global__ void __launch_bounds__(kThr) k_mix_back(SnoDims d, const float* R, const float2* F, const float2* dZ, float* dR,
+                                                   float2* dF, int B) {
+    __shared__ float2 red[kThr / 32][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.y, m = blockIdx.x * 32 + lane;
+    const bool in = m < d.M;
+    const int mm = in ? m : 0;
+    const float wm = (mm % d.M1 == 0 ? 1.f : 2.f) / (float)d.np;
+    float2 acc[4], r[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int o = w + 8 * k;
+        acc[k] = r[k] = make_float2(0.f, 0.f);
+        if (o < d.C) {
+            const float* rp = R + (((size_t)o * d.C + c) * d.M + mm) * 2;  // may start at an odd float
+            r[k] = make_float2(rp[0], rp[1]);
         }
     }
-}
-
-// ---------------------------------------------------------- projection
-// out = Q v + b_Q.  Inference: guess = un + rho (un - unm1) + s_out out.
-// Training: loss and dout = 2 (out - t) / (np B), t = (target - extrapolation) / s_out.
-__global__ void k_proj(SnoDims d, const float* Q, const float* v, const double* un, const double* unm1, double rho,
-                       double s_out, double* guess, const double* target, float* dout, double* loss, int B) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
-    double l = 0.0;
-    if (p < d.np) {
-        float o = Q[d.C];
-        for (int c = 0; c < d.C; c++) o += Q[c] * v[((size_t)b * d.C + c) * d.np + p];
-        const size_t i = (size_t)b * d.np + p;
-        const double ext = un[i] + rho * (un[i] - unm1[i]);
-        if (guess) guess[i] = ext + s_out * (double)o;
-        if (target) {
-            const double t = (target[i] - ext) / s_out;
-            const double e = (double)o - t;
-            l = e * e;
-            dout[i] = (float)(2.0 * e / ((double)d.np * B));
-        }
-    }
-    if (loss) {
-        for (int s = 16; s > 0; s >>= 1) l += __shfl_xor_sync(0xffffffffu, l, s);
-        if ((threadIdx.x & 31) == 0) atomicAdd(loss, l / ((double)d.np * B));
-    }
-}
-
-// --------------------------------------------------------------- backward
-// Sums over points of per-point products go to per-block partial rows, summed
-// by k_sum_rows into the gradient (no float atomics on hot addresses).
-
-// projection: dQ[c] = sum dout v_L[c], db_Q = sum dout; dv_L[c] = Q[c] dout
-__global__ void k_proj_back(SnoDims d, const float* Q, const float* v, const float* dout, float* dv, float* part, int B) {
-    __shared__ float red[kThr / 32][33];
-    const int p = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
-    float acc[33];
-    for (int c = 0; c <= d.C; c++) acc[c] = 0.f;
-    if (p < d.np) {
-        const float g = dout[(size_t)b * d.np + p];
-        for (int c = 0; c < d.C; c++) {
-            const size_t i = ((size_t)b * d.C + c) * d.np + p;
-            acc[c] = g * v[i];
-            dv[i] = Q[c] * g;
-        }
-        acc[d.C] = g;
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int c = 0; c <= d.C; c++) {
-        float x = acc[c];
-        for (int s = 16; s > 0; s >>= 1) x += __shfl_xor_sync(0xffffffffu, x, s);
-        if (lane == 0) red[w][c] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x <= d.C) {
-        float s = 0.f;
-        for (int i = 0; i < (int)(blockDim.x >> 5); i++) s += red[i][threadIdx.x];
-        part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (d.C + 1) + threadIdx.x] = s;
-    }
-}
-
-// layer, pointwise part: dz = dvn GELU'(z) (kept for the weight gradients and
-// the spectral part) and dv = W^T dz
-__global__ void k_layer_back(SnoDims d, const float* W, const float* z, const float* dvn, float* dz, float* dv,
-                             int B) {
-    __shared__ float sw[32 * 32];
-    for (int i = threadIdx.x; i < d.C * d.C; i += blockDim.x) sw[i] = W[i];
-    __syncthreads();
-    const int p = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
-    if (p >= d.np) return;
-    float g[32];
-    for (int o = 0; o < d.C; o++) {
-        const size_t i = ((size_t)b * d.C + o) * d.np + p;
-        g[o] = dvn[i] * gelu_grad(z[i]);
-        dz[i] = g[o];
-    }
-    for (int c = 0; c < d.C; c++) {
-        float s = 0.f;
-        for (int o = 0; o < d.C; o++) s += sw[o * d.C + c] * g[o];
-        dv[((size_t)b * d.C + c) * d.np + p] = s;
-    }
-}
-
-// per row (x0, b) partial sums dW[o][c] = sum dz[o] v[c] and db[o] = sum dz[o]:
-// the row is staged in shared memory in chunks, one thread per (o, c)
-constexpr int kWChunk = 128;
-__global__ void k_wgrad(SnoDims d, const float* dz, const float* v, float* part) {
-    __shared__ float sdz[32][kWChunk];
-    __shared__ float sv[32][kWChunk];
-    const int x0 = blockIdx.x, b = blockIdx.y;
-    const int nrow = d.C * d.C + d.C;
-    float acc[8];
-    for (int q = 0; q < 8; q++) acc[q] = 0.f;
-    for (int c0 = 0; c0 < d.n1; c0 += kWChunk) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < d.C * kWChunk; i += blockDim.x) {
-            const int ch = i / kWChunk, x = i % kWChunk;
-            const size_t p = ((size_t)b * d.C + ch) * d.np + (size_t)x0 * d.n1 + c0 + x;
-            const bool in = c0 + x < d.n1;
-            sdz[ch][x] = in ? dz[p] : 0.f;
-            sv[ch][x] = in ? v[p] : 0.f;
-        }
-        __syncthreads();
-        for (int q = 0, i = threadIdx.x; i < nrow && q < 8; i += blockDim.x, q++) {
-            float s = 0.f;
-            if (i < d.C * d.C) {
-                const int o = i / d.C, c = i % d.C;
-                for (int x = 0; x < kWChunk; x++) s += sdz[o][x] * sv[c][x];
-            } else {
-                const int o = i - d.C * d.C;
-                for (int x = 0; x < kWChunk; x++) s += sdz[o][x];
-            }
-            acc[q] += s;
-        }
-    }
-    for (int q = 0, i = threadIdx.x; i < nrow && q < 8; i += blockDim.x, q++)
-        part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * nrow + i] = acc[q];
-}
-
-// spectral part: dG[b][o][m] = (w_m / np) DFT(dz)[b][o][m] (already in G form);
-// dR[o][c][m] += sum_b dG conj(F), dF[b][c][m] = sum_o conj(R) dG
-__global__ void k_mix_back(SnoDims d, const float* R, const float2* F, const float2* dZ, float* dR, float2* dF, int B) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;  // c * M + m
-    if (i >= d.C * d.M) return;
-    const int c = i / d.M, m = i % d.M, m1 = m % d.M1;
-    const float wm = (m1 == 0 ? 1.f : 2.f) / (float)d.np;
     for (int b = 0; b < B; b++) {
-        const float2 f = F[((size_t)b * d.C + c) * d.M + m];
+        const float2 f = F[((size_t)b * d.C + c) * d.M + mm];
         float2 s = make_float2(0.f, 0.f);
-        for (int o = 0; o < d.C; o++) {
-            float2 g = dZ[((size_t)b * d.C + o) * d.M + m];
-            g.x *= wm;
-            g.y *= wm;
-            const float* r = R + (((size_t)o * d.C + c) * d.M + m) * 2;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int o = w + 8 * k;
+            if (o < d.C) {
+                float2 g = dZ[((size_t)b * d.C + o) * d.M + mm];
+                g.x *= wm;
+                g.y *= wm;
+                acc[k].x += g.x * f.x + g.y * f.y;  // dG conj(F)
+                acc[k].y += g.y * f.x - g.x * f.y;
+                s.x += r[k].x * g.x + r[k].y * g.y;  // conj(R) dG
+                s.y += r[k].x * g.y - r[k].y * g.x;
+            }
+        }
+        __syncthreads();
+        red[w][lane] = s;
+        __syncthreads();
+        if (w == 0 && in) {
+            for (int q = 1; q < kThr / 32; q++) {
+                s.x += red[q][lane].x;
+                s.y += red[q][lane].y;
+            }
+            dF[((size_t)b * d.C + c) * d.M + m] = s;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int o = w + 8 * k;
+        if (o < d.C && in) {
             float* dr = dR + (((size_t)o * d.C + c) * d.M + m) * 2;
-            dr[0] += g.x * f.x + g.y * f.y;  // dG conj(F)
-            dr[1] += g.y * f.x - g.x * f.y;
-            s.x += r[0] * g.x + r[1] * g.y;  // conj(R) dG
-            s.y += r[0] * g.y - r[1] * g.x;
+            dr[0] = acc[k].x;
+            dr[1] = acc[k].y;
         }
-        dF[((size_t)b * d.C + c) * d.M + m] = s;
     }
 }
 
-// dv[g](x) += sum over kept modes of Re(U[g][x0][m1] e^{+2 pi i m1 x1 / n1}) (the adjoint of the
-// forward truncated DFT; U is the first-axis inverse of dF, no weights, no 1/np)
-__global__ void k_idft_rows_add(SnoDims d, const float2* U, float* dv, int G) {
-    extern __shared__ float2 tw[];  // n1 entries
-    fill_tw(tw, d.n1);
-    const int x0 = blockIdx.x, g = blockIdx.y;
-    for (int x1 = threadIdx.x; x1 < d.n1; x1 += blockDim.x) {
-        float s = 0.f;
-        for (int m1 = 0; m1 < d.M1; m1++) {
-            const float2 e = tw[(m1 * x1) & (d.n1 - 1)];  // exp(+i ...) = conj
-            const float2 u = U[((size_t)g * d.n0 + x0) * d.M1 + m1];
-            s += u.x * e.x + u.y * e.y;
+// Partial sums over kTile consecutive points dW[o][c] = sum dz[o] v[c] and
+// db[o] = sum dz[o] -> row of part.  Both channels sets are staged in shared
+// memory; a warp takes kTile / 8 of the points, a lane a (CT / 4) x (CT / 8)
+// block of the products, four points per shared load.
+template <int CT>
+__global__ void __launch_bounds__(kThr) k_wgrad(SnoDims d, const float* dz, const float* v, float* part) {
+    extern __shared__ __align__(16) float sm[];
+    float *sd = sm, *sv = sm + CT * kPitch;
+    constexpr int NO = CT / 4, NC = CT / 8;  // lanes: 4 x 8
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, b = blockIdx.y, p0 = blockIdx.x * kTile;
+    for (int i = tid; i < CT * (kTile / 4); i += kThr) {
+        const int ch = i / (kTile / 4), x = 4 * (i % (kTile / 4));
+        float4 g = make_float4(0.f, 0.f, 0.f, 0.f), u = g;
+        if (ch < d.C && p0 + x < d.np) {  // np is a multiple of 4
+            g = *(const float4*)&dz[((size_t)b * d.C + ch) * d.np + p0 + x];
+            u = *(const float4*)&v[((size_t)b * d.C + ch) * d.np + p0 + x];
         }
-        dv[(size_t)g * d.np + (size_t)x0 * d.n1 + x1] += s;
+        *(float4*)&sd[ch * kPitch + x] = g;
+        *(float4*)&sv[ch * kPitch + x] = u;
     }
-}
-
-// lift: dP[c][j] = sum dv0[c] a[j], db_P[c] = sum dv0[c]; per-block partials [C][3]
-__global__ void k_lift_back(SnoDims d, const float* a, const float* dv0, float* part, int B) {
-    __shared__ float red[kThr / 32][96];
-    const int p = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
-    float a0 = 0.f, a1 = 0.f;
-    if (p < d.np) {
-        a0 = a[((size_t)b * 2) * d.np + p];
-        a1 = a[((size_t)b * 2 + 1) * d.np + p];
+    __syncthreads();
+    const int o0 = lane >> 3, c0 = lane & 7;
+    float acc[NO][NC], bs[NO];
+#pragma unroll
+    for (int i = 0; i < NO; i++) {
+        bs[i] = 0.f;
+#pragma unroll
+        for (int k = 0; k < NC; k++) acc[i][k] = 0.f;
     }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int c = 0; c < d.C; c++) {
-        const float g = p < d.np ? dv0[((size_t)b * d.C + c) * d.np + p] : 0.f;
-        float x0 = g * a0, x1 = g * a1, x2 = g;
-        for (int s = 16; s > 0; s >>= 1) {
-            x0 += __shfl_xor_sync(0xffffffffu, x0, s);
-            x1 += __shfl_xor_sync(0xffffffffu, x1, s);
-            x2 += __shfl_xor_sync(0xffffffffu, x2, s);
-        }
-        if (lane == 0) {
-            red[w][3 * c] = x0;
-            red[w][3 * c + 1] = x1;
-            red[w][3 * c + 2] = x2;
+#pragma unroll 2
+    for (int x = w * (kTile / 8); x < (w + 1) * (kTile / 8); x += 4) {
+        float4 g[NO], u[NC];
+#pragma unroll
+        for (int i = 0; i < NO; i++) g[i] = *(const float4*)&sd[(o0 + 4 * i) * kPitch + x];
+#pragma unroll
+        for (int k = 0; k < NC; k++) u[k] = *(const float4*)&sv[(c0 + 8 * k) * kPitch + x];
+#pragma unroll
+        for (int i = 0; i < NO; i++) {
+            bs[i] += (g[i].x + g[i].y) + (g[i].z + g[i].w);
+#pragma unroll
+            for (int k = 0; k < NC; k++)
+                acc[i][k] = fmaf(g[i].x, u[k].x, fmaf(g[i].y, u[k].y, fmaf(g[i].z, u[k].z, fmaf(g[i].w, u[k].w, acc[i][k]))));
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < 3 * d.C; i += blockDim.x) {
+    float* red = sm;  // [8 warps][CT][CT + 1]
+#pragma unroll
+    for (int i = 0; i < NO; i++) {
+        const int o = o0 + 4 * i;
+#pragma unroll
+        for (int k = 0; k < NC; k++) red[(w * CT + o) * (CT + 1) + c0 + 8 * k] = acc[i][k];
+        if (c0 == 0) red[(w * CT + o) * (CT + 1) + CT] = bs[i];
+    }
+    __syncthreads();
+    const int nrow = d.C * d.C + d.C;
+    for (int i = tid; i < nrow; i += kThr) {
+        const int o = i < d.C * d.C ? i / d.C : i - d.C * d.C, c = i < d.C * d.C ? i % d.C : CT;
         float s = 0.f;
-        for (int q = 0; q < (int)(blockDim.x >> 5); q++) s += red[q][i];
-        part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (3 * d.C) + i] = s;
+        for (int q = 0; q < 8; q++) s += red[(q * CT + o) * (CT + 1) + c];
+        part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * nrow + i] = s;
     }
 }
 
-// out[j] += sum over rows of part[row][j]
-__global__ void k_sum_rows(const float* part, int rows, int cols, float* out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= cols) return;
-    double s = 0.0;
-    for (int r = 0; r < rows; r++) s += part[(size_t)r * cols + j];
-    out[j] += (float)s;
-}
-
-// lift partials are [C][3] = (dP0, dP1, db); the gradient layout is P[C][2] then b_P[C]
-__global__ void k_lift_scatter(const float* sums, float* grad, int C) {
-    const int c = threadIdx.x;
-    if (c >= C) return;
-    grad[2 * c] += sums[3 * c];
-    grad[2 * c + 1] += sums[3 * c + 1];
-    grad[2 * C + c] += sums[3 * c + 2];
+// out[col(j)] = sum over rows of part[row][j], the rounding errors kept (Sum2); lift: the
+// partials [C][3] = (dP0, dP1, db) go to the layout P [C][2], b_P [C]
+constexpr int kSumThr = 1024;
+__global__ void __launch_bounds__(kSumThr) k_sum_rows(const float* part, int rows, int cols, float* out, int lift) {
+    __shared__ float rh[kSumThr / 32][33], rl[kSumThr / 32][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
+    pagd::Sum2 s;
+    if (j < cols)
+        for (int r = w; r < rows; r += kSumThr / 32) s.add(part[(size_t)r * cols + j]);
+    rh[w][lane] = s.h;
+    rl[w][lane] = s.l;
+    __syncthreads();
+    if (w == 0 && j < cols) {
+        for (int q = 1; q < kSumThr / 32; q++) {
+            s.add(rh[q][lane]);
+            s.l += rl[q][lane];
+        }
+        const int o = !lift ? j : (j % 3 < 2 ? 2 * (j / 3) + j % 3 : 2 * lift + j / 3);
+        out[o] = s.h + s.l;
+    }
 }
 
 // Adam (Kingma and Ba, 2015) with bias correction
@@ -452,9 +645,7 @@ struct sno_net {
     void* stream;
     char* ws;
     size_t ws_bytes;
-    size_t off_a, off_v, off_z, off_F, off_G, off_T, off_U, off_dv, off_dv2, off_dz, off_dout, off_part, off_dF,
-        off_loss, off_sums;
-    size_t part_rows;
+    size_t off_v, off_z, off_F, off_G, off_T, off_dz, off_dz2, off_part, off_dF, off_loss, off_tw0, off_tw1;
     std::string err;
 };
 
@@ -480,23 +671,19 @@ static void plan(sno_net* s) {
         o += (bytes + 255) & ~(size_t)255;
         return at;
     };
-    s->off_a = take(sizeof(float) * B * 2 * np);
-    s->off_v = take(sizeof(float) * B * d.C * np * (d.L + 1));
-    s->off_z = take(sizeof(float) * B * d.C * np * d.L);
+    s->off_v = take(sizeof(float) * B * d.C * np * d.L);
+    s->off_z = take(sizeof(float) * B * d.C * np * (d.L > 1 ? d.L - 1 : 0));
     s->off_F = take(sizeof(float2) * B * d.C * d.M * d.L);
     s->off_G = take(sizeof(float2) * B * d.C * d.M);
-    s->off_T = take(sizeof(float2) * B * d.C * d.n0 * d.M1);
-    s->off_U = take(sizeof(float2) * B * d.C * d.n0 * d.M1);
-    s->off_dv = take(sizeof(float) * B * d.C * np);
-    s->off_dv2 = take(sizeof(float) * B * d.C * np);
+    s->off_T = take(sizeof(float2) * B * d.C * d.n0 * d.JB * d.M1);
     s->off_dz = take(sizeof(float) * B * d.C * np);
-    s->off_dout = take(sizeof(float) * B * np);
-    const size_t rows_pt = B * (size_t)((np + kThr - 1) / kThr), rows_row = B * (size_t)d.n0;
-    s->part_rows = rows_pt > rows_row ? rows_pt : rows_row;
-    s->off_part = take(sizeof(float) * s->part_rows * (size_t)(d.C * d.C + d.C + 3 * d.C + 1));
+    s->off_dz2 = take(sizeof(float) * B * d.C * np);
+    const size_t rows = B * std::max<size_t>((size_t)d.NT, (np + kTile - 1) / kTile);
+    s->off_part = take(sizeof(float) * rows * std::max<size_t>((size_t)d.C * d.C + d.C, (size_t)3 * d.C));
     s->off_dF = take(sizeof(float2) * B * d.C * d.M);
     s->off_loss = take(sizeof(double));
-    s->off_sums = take(sizeof(float) * (size_t)(d.C * d.C + d.C + 3 * d.C + 1));
+    s->off_tw0 = take(sizeof(float2) * d.n0);
+    s->off_tw1 = take(sizeof(float2) * d.n1);
     s->ws_bytes = o;
 }
 
@@ -506,33 +693,84 @@ static void plan(sno_net* s) {
         if (e_ != cudaSuccess) return sno_fail(s, PAGD_ECUDA, cudaGetErrorString(e_)); \
     } while (0)
 
-// the whole forward pass for B samples; activations stay in the workspace
-static pagd_status forward(sno_net* s, const float* prm, const double* un, const double* unm1, float s_in, int B) {
+template <int MODE, int QC, int CT, int MM>
+static cudaError_t launch_tile(const SnoDims& d, const TileArgs& a, int B, cudaStream_t st) {
+    const size_t smem = tile_smem(d, CT);
+    if (smem > 48 * 1024) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k_tile<MODE, QC, CT, MM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    k_tile<MODE, QC, CT, MM><<<dim3(d.NT, B), kThr, smem, st>>>(d, a);
+    return cudaGetLastError();
+}
+template <int MODE, int QC> static cudaError_t tile_qc(const SnoDims& d, const TileArgs& a, int B, cudaStream_t st) {
+    if (d.C <= 16) return d.M1 <= 16 ? launch_tile<MODE, QC, 16, 16>(d, a, B, st) : launch_tile<MODE, QC, 16, 32>(d, a, B, st);
+    return d.M1 <= 16 ? launch_tile<MODE, QC, 32, 16>(d, a, B, st) : launch_tile<MODE, QC, 32, 32>(d, a, B, st);
+}
+template <int MODE> static cudaError_t tile(const SnoDims& d, const TileArgs& a, int B, cudaStream_t st) {
+    if (d.QC == 16) return tile_qc<MODE, 16>(d, a, B, st);
+    if (d.QC == 4) return tile_qc<MODE, 4>(d, a, B, st);
+    return tile_qc<MODE, 1>(d, a, B, st);
+}
+template <int CT> static cudaError_t launch_wgrad(const SnoDims& d, const float* dz, const float* v, float* part, int B,
+                                                  cudaStream_t st) {
+    const size_t smem = std::max<size_t>((size_t)2 * CT * kPitch, (size_t)8 * CT * (CT + 1)) * sizeof(float);
+    const cudaError_t e = cudaFuncSetAttribute(k_wgrad<CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_wgrad<CT><<<dim3((d.np + kTile - 1) / kTile, B), kThr, smem, st>>>(d, dz, v, part);
+    return cudaGetLastError();
+}
+
+static TileArgs tile_args(const sno_net* s, const float* prm, const double* un, const double* unm1, float s_in) {
+    TileArgs a = {};
+    a.prm = prm;
+    a.un = un;
+    a.unm1 = unm1;
+    a.s_in = s_in;
+    a.Q = prm + off_Q(s->d);
+    a.G = (const float2*)(s->ws + s->off_G);
+    a.T = (float2*)(s->ws + s->off_T);
+    a.tw0 = (const float2*)(s->ws + s->off_tw0);
+    a.tw1 = (const float2*)(s->ws + s->off_tw1);
+    return a;
+}
+static void set_layer(TileArgs& a, const SnoDims& d, int l) {
+    a.W = a.prm + off_layer(d, l);
+    a.bias = a.W + d.C * d.C;
+}
+
+// T -> the modes F
+static void launch_cols(const sno_net* s, int G, const float2* T, float2* F) {
+    const SnoDims& d = s->d;
+    k_cols<<<G, kColThr, sizeof(float2) * (d.n0 + kColThr), (cudaStream_t)s->stream>>>(
+        d, T, (const float2*)(s->ws + s->off_tw0), F);
+}
+
+// The forward pass for B samples up to the modes of the last layer; v_l (and,
+// with train, z_l) stay in the workspace.  The last layer's pass is the caller's.
+static pagd_status forward(sno_net* s, TileArgs& a, int B, bool train) {
     const SnoDims& d = s->d;
     cudaStream_t st = (cudaStream_t)s->stream;
     char* w = s->ws;
-    float* a = (float*)(w + s->off_a);
     float* v = (float*)(w + s->off_v);
     float* z = (float*)(w + s->off_z);
     float2* F = (float2*)(w + s->off_F);
     float2* G = (float2*)(w + s->off_G);
-    float2* T = (float2*)(w + s->off_T);
-    float2* U = (float2*)(w + s->off_U);
     const size_t vs = (size_t)B * d.C * d.np;  // one layer of activations
-    const dim3 gp((d.np + kThr - 1) / kThr, B);
-    k_lift<<<gp, kThr, 0, st>>>(d, prm, un, unm1, s_in, a, v, B);
+    a.vout = v;
+    CK(tile<T_LIFT>(d, a, B, st));
     for (int l = 0; l < d.L; l++) {
-        const float* L = prm + off_layer(d, l);
-        const float* W = L;
-        const float* bias = L + d.C * d.C;
-        const float* R = L + d.C * d.C + d.C;
         float2* Fl = F + (size_t)l * B * d.C * d.M;
-        k_dft_rows<<<B * d.C * d.n0, kThr, sizeof(float2) * d.n1, st>>>(d, v + l * vs, T);
-        k_dft_cols<<<B * d.C, d.M, sizeof(float2) * d.n0, st>>>(d, T, Fl);
-        k_mix<<<dim3((d.C * d.M + kThr - 1) / kThr, B), kThr, 0, st>>>(d, R, Fl, G);
-        k_idft_cols<<<dim3((d.n0 * d.M1 + kThr - 1) / kThr, B * d.C), kThr, sizeof(float2) * d.n0, st>>>(d, G, U);
-        k_layer<<<dim3(d.n0, B), kThr, sizeof(float2) * (d.C * d.M1 + d.n1), st>>>(d, W, bias, U, v + l * vs,
-                                                                                   z + l * vs, v + (l + 1) * vs, 1);
+        set_layer(a, d, l);
+        launch_cols(s, B * d.C, a.T, Fl);
+        k_mix<<<dim3((d.C * d.M + kThr - 1) / kThr, B), kThr, 0, st>>>(d, a.bias + d.C, Fl, G);
+        a.vin = v + l * vs;
+        if (l + 1 < d.L) {
+            a.vout = v + (l + 1) * vs;
+            a.z = train ? z + l * vs : nullptr;
+            CK(tile<T_LAYER>(d, a, B, st));
+        }
     }
     CK(cudaGetLastError());
     return PAGD_OK;
@@ -551,7 +789,13 @@ pagd_status sno_create(sno_net** out, int n0, int n1, int channels, int layers, 
         return PAGD_EINVAL;
     sno_net* s = new (std::nothrow) sno_net();
     if (!s) return PAGD_ENOMEM;
-    s->d = SnoDims{n0, n1, n0 * n1, channels, layers, modes0, modes1, modes0 * modes1};
+    SnoDims& d = s->d;
+    d = SnoDims{n0, n1, n0 * n1, channels, layers, modes0, modes1, modes0 * modes1, 0, 0, 0, 0, 0};
+    d.QC = n1 >= 512 ? 16 : n1 >= 64 ? 4 : 1;
+    d.J = n1 / d.QC;
+    d.JB = d.J > 32 ? d.J / 32 : 1;
+    d.R = 16 / d.QC;
+    d.NT = (n0 + d.R - 1) / d.R * d.JB;
     s->batch = batch;
     s->stream = stream;
     s->ws = nullptr;
@@ -577,6 +821,12 @@ pagd_status sno_set_workspace(sno_net* s, void* dev, size_t bytes) {
     if (((uintptr_t)dev & 255) != 0) return sno_fail(s, PAGD_EINVAL, "workspace not 256-byte aligned");
     if (bytes < s->ws_bytes) return sno_fail(s, PAGD_ENOMEM, "workspace too small");
     s->ws = (char*)dev;
+    // the twiddle tables, once per workspace, on the network's stream
+    cudaStream_t st = (cudaStream_t)s->stream;
+    const SnoDims& d = s->d;
+    k_tables<<<(d.n0 + kThr - 1) / kThr, kThr, 0, st>>>((float2*)(s->ws + s->off_tw0), d.n0);
+    k_tables<<<(d.n1 + kThr - 1) / kThr, kThr, 0, st>>>((float2*)(s->ws + s->off_tw1), d.n1);
+    CK(cudaGetLastError());
     return PAGD_OK;
 }
 
@@ -585,13 +835,13 @@ pagd_status sno_predict(sno_net* s, const float* params, const double* un, const
     if (!s || !params || !un || !unm1 || !guess) return PAGD_EINVAL;
     if (!s->ws) return sno_fail(s, PAGD_ESTATE, "no workspace");
     if (nsamples < 1 || nsamples > s->batch) return sno_fail(s, PAGD_EINVAL, "bad sample count");
-    pagd_status r = forward(s, params, un, unm1, (float)s_in, nsamples);
+    TileArgs a = tile_args(s, params, un, unm1, (float)s_in);
+    a.rho = rho;
+    a.s_out = s_out;
+    a.guess = guess;
+    const pagd_status r = forward(s, a, nsamples, false);
     if (r != PAGD_OK) return r;
-    const SnoDims& d = s->d;
-    const float* vL = (const float*)(s->ws + s->off_v) + (size_t)d.L * nsamples * d.C * d.np;
-    k_proj<<<dim3((d.np + kThr - 1) / kThr, nsamples), kThr, 0, (cudaStream_t)s->stream>>>(
-        d, params + off_Q(d), vL, un, unm1, rho, s_out, guess, nullptr, nullptr, nullptr, nsamples);
-    CK(cudaGetLastError());
+    CK(tile<T_GUESS>(s->d, a, nsamples, (cudaStream_t)s->stream));
     CK(cudaStreamSynchronize((cudaStream_t)s->stream));
     return PAGD_OK;
 }
@@ -605,58 +855,56 @@ pagd_status sno_loss_grad(sno_net* s, const float* params, const double* un, con
     const SnoDims& d = s->d;
     const int B = nsamples;
     cudaStream_t st = (cudaStream_t)s->stream;
-    pagd_status r = forward(s, params, un, unm1, (float)s_in, B);
-    if (r != PAGD_OK) return r;
     char* w = s->ws;
-    float* a = (float*)(w + s->off_a);
     float* v = (float*)(w + s->off_v);
     float* z = (float*)(w + s->off_z);
     float2* F = (float2*)(w + s->off_F);
-    float2* T = (float2*)(w + s->off_T);
-    float2* U = (float2*)(w + s->off_U);
     float2* dZ = (float2*)(w + s->off_G);
     float2* dF = (float2*)(w + s->off_dF);
-    float* dv = (float*)(w + s->off_dv);
-    float* dv2 = (float*)(w + s->off_dv2);
     float* dz = (float*)(w + s->off_dz);
-    float* dout = (float*)(w + s->off_dout);
+    float* dz2 = (float*)(w + s->off_dz2);
     float* part = (float*)(w + s->off_part);
-    float* sums = (float*)(w + s->off_sums);
     double* dloss = (double*)(w + s->off_loss);
     const size_t vs = (size_t)B * d.C * d.np;
-    const dim3 gp((d.np + kThr - 1) / kThr, B);
-    CK(cudaMemsetAsync(grad, 0, sizeof(float) * param_count(d), st));
+    const int nrow = d.C * d.C + d.C, tiles = d.NT * B, wrows = (d.np + kTile - 1) / kTile * B;
     CK(cudaMemsetAsync(dloss, 0, sizeof(double), st));
-    const float* Q = params + off_Q(d);
-    float* gQ = grad + off_Q(d);
-    k_proj<<<gp, kThr, 0, st>>>(d, Q, v + (size_t)d.L * vs, un, unm1, rho, s_out, nullptr, target, dout, dloss, B);
-    k_proj_back<<<gp, kThr, 0, st>>>(d, Q, v + (size_t)d.L * vs, dout, dv, part, B);
-    k_sum_rows<<<1, 64, 0, st>>>(part, (int)(gp.x * gp.y), d.C + 1, gQ);
+    TileArgs a = tile_args(s, params, un, unm1, (float)s_in);
+    a.target = target;
+    a.rho = rho;
+    a.inv_s_out = 1.0 / s_out;
+    a.dscale = 2.0 / ((double)d.np * B);
+    a.loss = dloss;
+    a.part = part;
+    const pagd_status r = forward(s, a, B, true);
+    if (r != PAGD_OK) return r;
+    // last layer, projection, loss, and the way back to dz of the last layer
+    a.vout = dz;
+    CK(tile<T_LOSS>(d, a, B, st));
+    auto sum_rows = [&](int rows, int cols, float* out, int lift) {
+        k_sum_rows<<<(cols + 31) / 32, kSumThr, 0, st>>>(part, rows, cols, out, lift);
+    };
+    sum_rows(tiles, d.C + 1, grad + off_Q(d), 0);
+    a.G = dF;
     for (int l = d.L - 1; l >= 0; l--) {
-        const float* L = params + off_layer(d, l);
-        const float* W = L;
-        const float* R = L + d.C * d.C + d.C;
         float* gL = grad + off_layer(d, l);
-        float* gR = gL + d.C * d.C + d.C;
-        const int nrow = d.C * d.C + d.C;
-        // pointwise part: dz, dv2 = W^T dz, then dW, db
-        k_layer_back<<<gp, kThr, 0, st>>>(d, W, z + (size_t)l * vs, dv, dz, dv2, B);
-        k_wgrad<<<dim3(d.n0, B), kThr, 0, st>>>(d, dz, v + (size_t)l * vs, part);
-        k_sum_rows<<<(nrow + 63) / 64, 64, 0, st>>>(part, d.n0 * B, nrow, gL);
-        // spectral part: DFT(dz) -> dG (weights applied in k_mix_back), dR, dF, dv2 += IDFT(dF)
-        k_dft_rows<<<B * d.C * d.n0, kThr, sizeof(float2) * d.n1, st>>>(d, dz, T);
-        k_dft_cols<<<B * d.C, d.M, sizeof(float2) * d.n0, st>>>(d, T, dZ);
-        k_mix_back<<<(d.C * d.M + kThr - 1) / kThr, kThr, 0, st>>>(d, R, F + (size_t)l * B * d.C * d.M, dZ, gR, dF, B);
-        k_idft_cols<<<dim3((d.n0 * d.M1 + kThr - 1) / kThr, B * d.C), kThr, sizeof(float2) * d.n0, st>>>(d, dF, U);
-        k_idft_rows_add<<<dim3(d.n0, B * d.C), kThr, sizeof(float2) * d.n1, st>>>(d, U, dv2, B * d.C);
-        float* t = dv;
-        dv = dv2;
-        dv2 = t;
+        set_layer(a, d, l);
+        launch_cols(s, B * d.C, a.T, dZ);
+        k_mix_back<<<dim3((d.M + 31) / 32, d.C), kThr, 0, st>>>(d, a.bias + d.C, F + (size_t)l * B * d.C * d.M, dZ,
+                                                              gL + nrow, dF, B);
+        if (d.C <= 16) CK(launch_wgrad<16>(d, dz, v + (size_t)l * vs, part, B, st));
+        else CK(launch_wgrad<32>(d, dz, v + (size_t)l * vs, part, B, st));
+        sum_rows(wrows, nrow, gL, 0);
+        a.vin = dz;
+        a.vout = dz2;
+        if (l > 0) {
+            a.zprev = z + (size_t)(l - 1) * vs;
+            CK(tile<T_BACK>(d, a, B, st));
+        } else {
+            CK(tile<T_BACK0>(d, a, B, st));
+        }
+        std::swap(dz, dz2);
     }
-    k_lift_back<<<gp, kThr, 0, st>>>(d, a, dv, part, B);
-    CK(cudaMemsetAsync(sums, 0, sizeof(float) * 3 * d.C, st));
-    k_sum_rows<<<(3 * d.C + 63) / 64, 64, 0, st>>>(part, (int)(gp.x * gp.y), 3 * d.C, sums);
-    k_lift_scatter<<<1, 32, 0, st>>>(sums, grad, d.C);
+    sum_rows(tiles, 3 * d.C, grad, d.C);
     CK(cudaGetLastError());
     if (loss) CK(cudaMemcpyAsync(loss, dloss, sizeof(double), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
