@@ -41,8 +41,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) pagd_batch_kernel(BatchParams 
     extern __shared__ __align__(16) char smem[];
     __shared__ double red[32];
     const int ntw = 1 << B.logtw;
-    longlong2* tfx = (longlong2*)smem;
-    float2* t32 = (float2*)(smem + (size_t)ntw * sizeof(longlong2));
+    FxTw* tfx = (FxTw*)smem;
+    float2* t32 = (float2*)(smem + (size_t)ntw * sizeof(FxTw));
     const int stride = kNMax >> B.logtw;
     for (int m = threadIdx.x; m < ntw; m += blockDim.x) {
         tfx[m] = B.twfx[m * stride];

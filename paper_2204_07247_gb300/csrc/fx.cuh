@@ -28,31 +28,42 @@ namespace pagd {
 
 template <> struct V2<long long> { using type = longlong2; };
 
-// twiddle tables hold cos, sin in units of 2^-61
+// twiddle tables hold cos and sin in units of 2^-61 (FxTw)
 constexpr int kFxTw = 61;
 constexpr int kFxNaN = 1 << 28;  // exponent of a line that holds a NaN or an infinity
 
 __host__ __device__ __forceinline__ int fxs(int i) { return i ^ ((i >> 3) & 7); }
 
-// a w 2^-61 rounded, |a| < 2^62, |w| <= sqrt(2) 2^61: both split into a signed
-// high part and a 31-bit low part; the product of the low parts enters with
-// its leading bits
-__device__ __forceinline__ long long fx_mul(long long a, long long w) {
-    const int ah = (int)(a >> 31), al = (int)(a & 0x7fffffff);
-    const int wh = (int)(w >> 31), wl = (int)(w & 0x7fffffff);
-    long long m = (long long)ah * wl + (long long)wh * al;
-    m += (al >> 16) * (wl >> 15);
-    return (((long long)ah * wh) << 1) + ((m + (1ll << 29)) >> 30);
+// A factor w, |w| <= sqrt(2) in units of 2^-61, as h 2^31 + l with 0 <= l < 2^31
+struct FxW {
+    int h, l;
+};
+__host__ __device__ constexpr FxW fx_split(long long w) { return FxW{(int)(w >> 31), (int)(w & 0x7fffffff)}; }
+// A twiddle c + i s: the factors c, c + s, s - c of fx_cmul, split when the
+// table is made (six integer instructions less per complex product)
+struct alignas(8) FxTw {
+    FxW c, p, q;
+};
+__host__ __device__ constexpr FxTw fx_tw(long long c, long long s) { return FxTw{fx_split(c), fx_split(c + s), fx_split(s - c)}; }
+
+// a w 2^-61 rounded, |a| < 2^62: a split like w; the product of the low parts
+// enters with its leading bits
+__device__ __forceinline__ long long fx_mul(long long a, FxW w) {
+    const int ah = (int)(a >> 31), al = (int)a & 0x7fffffff;
+    long long m = (long long)ah * w.l + (1ll << 29);
+    m += (long long)w.h * al;
+    m += (al >> 16) * (w.l >> 15);
+    return (((long long)ah * w.h) << 1) + (m >> 30);
 }
 // a w (S < 0) or a conj(w) (S > 0) in three real products
-template <int S> __device__ __forceinline__ longlong2 fx_cmul(longlong2 a, longlong2 w) {
-    const long long k1 = fx_mul(a.x + a.y, w.x), p = w.x + w.y, q = w.y - w.x;
-    if (S < 0) return longlong2{k1 - fx_mul(a.y, p), k1 + fx_mul(a.x, q)};
-    return longlong2{k1 + fx_mul(a.y, q), k1 - fx_mul(a.x, p)};
+template <int S> __device__ __forceinline__ longlong2 fx_cmul(longlong2 a, const FxTw& w) {
+    const long long k1 = fx_mul(a.x + a.y, w.c);
+    if (S < 0) return longlong2{k1 - fx_mul(a.y, w.p), k1 + fx_mul(a.x, w.q)};
+    return longlong2{k1 + fx_mul(a.y, w.q), k1 - fx_mul(a.x, w.p)};
 }
 
 template <int S> __device__ __forceinline__ void fx_dft8(longlong2* v) {
-    constexpr long long c = 1630477228166597777ll;  // cos(pi / 4) 2^61
+    constexpr FxW c = fx_split(1630477228166597777ll);  // cos(pi / 4) 2^61
     longlong2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
     longlong2 o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
     dft4<S>(e0, e1, e2, e3);
@@ -204,7 +215,7 @@ __host__ __device__ constexpr int fx_radix(int logn, int logns) {
 }
 
 template <int R, int S, int LOGN, int LOGNS, bool FIRST>
-__device__ __forceinline__ void fx_stage(longlong2* b, int sh, const longlong2* tw, int logTw, int lane) {
+__device__ __forceinline__ void fx_stage(longlong2* b, int sh, const FxTw* tw, int logTw, int lane) {
     constexpr int LR = (R == 2) ? 1 : (R == 4) ? 2 : 3;
     constexpr int NB = 1 << (LOGN - LR), NS = 1 << LOGNS;
     constexpr int PER = (NB + kWarp - 1) / kWarp;
@@ -239,7 +250,7 @@ __device__ __forceinline__ void fx_stage(longlong2* b, int sh, const longlong2* 
     warp_sync();
 }
 template <int S, int LOGN, int LOGNS>
-__device__ __forceinline__ void fx_stages(longlong2* b, int sh, const longlong2* tw, int logTw, int lane) {
+__device__ __forceinline__ void fx_stages(longlong2* b, int sh, const FxTw* tw, int logTw, int lane) {
     if constexpr (LOGNS < LOGN) {
         constexpr int R = fx_radix(LOGN, LOGNS);
         fx_stage<R, S, LOGN, LOGNS, LOGNS == 0>(b, sh, tw, logTw, lane);
@@ -252,13 +263,13 @@ __device__ __forceinline__ void fx_stages(longlong2* b, int sh, const longlong2*
 // kernel shares its code, and its registers do not add to theirs.  Data
 // written before the call and read after it by any lane.
 template <int S, int LOGN>
-static __device__ __noinline__ void fx_line_n(longlong2* b, int sh, const longlong2* tw, int logTw, int lane) {
+static __device__ __noinline__ void fx_line_n(longlong2* b, int sh, const FxTw* tw, int logTw, int lane) {
     warp_sync();
     fx_stages<S, LOGN, 0>(b, sh, tw, logTw, lane);
 }
 // NF: the line length, or 0 for the runtime length 1 << logn (8 .. 512)
 template <int S, int NF>
-__device__ __forceinline__ void fx_line(longlong2* b, int logn, int sh, const longlong2* tw, int logTw, int lane) {
+__device__ __forceinline__ void fx_line(longlong2* b, int logn, int sh, const FxTw* tw, int logTw, int lane) {
     if constexpr (NF > 0) {
         fx_line_n<S, ilog2c(NF)>(b, sh, tw, logTw, lane);
     } else {
@@ -435,7 +446,7 @@ template <int S, int LOGN> __device__ __forceinline__ void fx_first(const longlo
 }
 // b (all stages but the last done) -> v
 template <int S, int LOGN>
-__device__ __forceinline__ void fx_last(longlong2* v, const longlong2* b, const longlong2* tw, int logTw, int lane) {
+__device__ __forceinline__ void fx_last(longlong2* v, const longlong2* b, const FxTw* tw, int logTw, int lane) {
     constexpr int R = LOGN == 9 ? 8 : 4, LR = radix_log(R), NB = (1 << LOGN) / R, PER = NB / kWarp;
     const int twshift = logTw - LOGN;
 #pragma unroll
@@ -455,7 +466,7 @@ __device__ __forceinline__ void fx_last(longlong2* v, const longlong2* b, const 
     (void)LR;
 }
 template <int S, int LOGN, int LOGNS, int END>
-__device__ __forceinline__ void fx_middle(longlong2* b, const longlong2* tw, int logTw, int lane) {
+__device__ __forceinline__ void fx_middle(longlong2* b, const FxTw* tw, int logTw, int lane) {
     if constexpr (LOGNS < END) {
         constexpr int R = fx_radix(LOGN, LOGNS);
         fx_stage<R, S, LOGN, LOGNS, false>(b, 0, tw, logTw, lane);
@@ -496,7 +507,7 @@ template <int E> __device__ __forceinline__ void fx_put(const longlong2* v, int 
 }
 // points s[i stride] of a line -> its transform in the slots of b; returns the exponent
 template <int S, int LOGN>
-__device__ __noinline__ int fx_line_in(longlong2* b, const double2* s, int stride, const longlong2* tw, int logTw, int lane) {
+__device__ __noinline__ int fx_line_in(longlong2* b, const double2* s, int stride, const FxTw* tw, int logTw, int lane) {
     constexpr int E = (1 << LOGN) / kWarp;
     double2 z[E];
     longlong2 v[E];
@@ -509,7 +520,7 @@ __device__ __noinline__ int fx_line_in(longlong2* b, const double2* s, int strid
 }
 // doubles in the lane's slots of b -> the transform at d[i stride]
 template <int S, int LOGN>
-__device__ __noinline__ void fx_line_out(longlong2* b, double2* d, int stride, const longlong2* tw, int logTw, int lane) {
+__device__ __noinline__ void fx_line_out(longlong2* b, double2* d, int stride, const FxTw* tw, int logTw, int lane) {
     constexpr int E = (1 << LOGN) / kWarp, END = LOGN - (LOGN == 9 ? 3 : 2);
     longlong2 v[E];
     double2 z[E];
@@ -523,7 +534,7 @@ __device__ __noinline__ void fx_line_out(longlong2* b, double2* d, int stride, c
 }
 // doubles in the lane's slots of b -> the transform in the slots; returns the exponent
 template <int S, int LOGN>
-__device__ __noinline__ int fx_line_mid(longlong2* b, const longlong2* tw, int logTw, int lane) {
+__device__ __noinline__ int fx_line_mid(longlong2* b, const FxTw* tw, int logTw, int lane) {
     constexpr int E = (1 << LOGN) / kWarp;
     longlong2 v[E];
     double2 z[E];
@@ -536,7 +547,7 @@ __device__ __noinline__ int fx_line_mid(longlong2* b, const longlong2* tw, int l
 }
 // s[i ss] -> the transform at d[i ds]
 template <int S, int LOGN>
-__device__ __noinline__ void fx_line_move(longlong2* b, const double2* s, int ss, double2* d, int ds, const longlong2* tw,
+__device__ __noinline__ void fx_line_move(longlong2* b, const double2* s, int ss, double2* d, int ds, const FxTw* tw,
                                           int logTw, int lane) {
     constexpr int E = (1 << LOGN) / kWarp, END = LOGN - (LOGN == 9 ? 3 : 2);
     double2 z[E];
@@ -557,21 +568,21 @@ __host__ __device__ constexpr bool fx_regs_ok(int nf) { return nf == 128 || nf =
 // transform in the slots (mid), slots' doubles -> transform in memory (out).
 // hi: this lane's largest fx_hi of its slots.  in and mid return the exponent.
 template <int S, int NF>
-__device__ __forceinline__ int fx_in(longlong2* b, const double2* s, int n, int logn, const longlong2* tw, int logTw, int lane) {
+__device__ __forceinline__ int fx_in(longlong2* b, const double2* s, int n, int logn, const FxTw* tw, int logTw, int lane) {
     if constexpr (fx_regs_ok(NF)) return fx_line_in<S, ilog2c(NF)>(b, s, 1, tw, logTw, lane);
     const FxExp x = fx_convert(b, n, fx_load(b, s, n, lane, kWarp), lane);
     fx_line<S, NF>(b, logn, x.sh, tw, logTw, lane);
     return x.e - x.sh;
 }
 template <int S, int NF>
-__device__ __forceinline__ int fx_mid(longlong2* b, unsigned hi, int n, int logn, const longlong2* tw, int logTw, int lane) {
+__device__ __forceinline__ int fx_mid(longlong2* b, unsigned hi, int n, int logn, const FxTw* tw, int logTw, int lane) {
     if constexpr (fx_regs_ok(NF)) return fx_line_mid<S, ilog2c(NF)>(b, tw, logTw, lane);
     const FxExp x = fx_convert(b, n, hi, lane);
     fx_line<S, NF>(b, logn, x.sh, tw, logTw, lane);
     return x.e - x.sh;
 }
 template <int S, int NF>
-__device__ __forceinline__ void fx_out(longlong2* b, unsigned hi, double2* d, int n, int logn, const longlong2* tw, int logTw,
+__device__ __forceinline__ void fx_out(longlong2* b, unsigned hi, double2* d, int n, int logn, const FxTw* tw, int logTw,
                                        int lane) {
     if constexpr (fx_regs_ok(NF)) {
         fx_line_out<S, ilog2c(NF)>(b, d, 1, tw, logTw, lane);
@@ -583,23 +594,165 @@ __device__ __forceinline__ void fx_out(longlong2* b, unsigned hi, double2* d, in
 }
 
 // ------------------------------------------------- lines shared by a CTA
+//
+// nl lines of n = 1 << logn points, line l in slots l n .., dealt to the
+// threads of a CTA over (line, point) so that all lines' loads are in flight
+// together.  red: [largest fx_hi][line], [sum of fx_mag][line] (zero before).
 
-template <int R, int S, int LOGN>
-__device__ __forceinline__ void fx_stage_coop(const longlong2* src, longlong2* dst, int nl, int logNs,
-                                              const unsigned* sums, const longlong2* tw, int logTw, int tid,
-                                              int nthr) {
+__device__ __forceinline__ void fxc_put_max(unsigned* red, int l, bool in, unsigned v, int n) {
+    if (n >= kWarp) {  // a warp's points are of one line
+        v = warp_umax(in ? v : 0u);
+        if ((threadIdx.x % kWarp) == 0) atomicMax(red + l, v);
+    } else if (in) {
+        atomicMax(red + l, v);
+    }
+}
+__device__ __forceinline__ void fxc_put_sum(unsigned* red, int l, bool in, unsigned v, int n) {
+    if (n >= kWarp) {
+        v = warp_uadd(in ? v : 0u);
+        if ((threadIdx.x % kWarp) == 0) atomicAdd(red + l, v);
+    } else if (in) {
+        atomicAdd(red + l, v);
+    }
+}
+// columns: line l's points at s + l H
+static __device__ __noinline__ void fxc_load(longlong2* b, const double2* s, long long H, int nl, int logn, unsigned* red,
+                                             int tid, int nthr) {
+    const int n = 1 << logn, tot = nl << logn, lane = tid % kWarp;
+    for (int i0 = tid - lane; i0 < tot; i0 += nthr * kFxLoad) {
+        double2 v[kFxLoad];
+#pragma unroll
+        for (int q = 0; q < kFxLoad; q++) {
+            const int i = i0 + lane + nthr * q;
+            if (i < tot) v[q] = s[(size_t)(i >> logn) * H + (i & (n - 1))];
+        }
+#pragma unroll
+        for (int q = 0; q < kFxLoad; q++) {
+            const int iw = i0 + nthr * q, i = iw + lane;
+            if (iw < tot) {
+                const bool in = i < tot;
+                unsigned m = 0;
+                if (in) {
+                    const unsigned a = fx_hi(v[q].x), c = fx_hi(v[q].y);
+                    m = a > c ? a : c;
+                    *(double2*)&b[(i >> logn << logn) + fxs(i & (n - 1))] = v[q];
+                }
+                fxc_put_max(red, in ? i >> logn : 0, in, m, n);
+            }
+        }
+    }
+}
+// row pairs: line l's coefficients at s + l H + k rows, as fx_pair_rows reads them
+static __device__ __noinline__ void fxc_load_rows(longlong2* b, const double2* s, long long H, int rows, int nl, int logn,
+                                                  unsigned* red, int tid, int nthr) {
+    const int n = 1 << logn, half = n >> 1, tot = nl * half, lane = tid % kWarp;
+    for (int i0 = tid - lane; i0 < tot; i0 += nthr * 2) {
+        double2 a[2], c[2];
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            const int i = i0 + lane + nthr * q;
+            if (i < tot) {
+                const double2* p = s + (size_t)(i >> (logn - 1)) * H + (size_t)(i & (half - 1)) * rows;
+                a[q] = p[0];
+                c[q] = p[1];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            const int iw = i0 + nthr * q, i = iw + lane;
+            if (iw < tot) {
+                const bool in = i < tot;
+                const int l = in ? i >> (logn - 1) : 0, k = i & (half - 1);
+                unsigned m = 0;
+                if (in) {
+                    int k2 = n - k;
+                    if (k == 0) {  // k = 0 and n / 2: real coefficients
+                        const double2* p = s + (size_t)l * H + (size_t)half * rows;
+                        a[q].y = c[q].x;
+                        c[q] = double2{p[0].x, p[1].x};
+                        k2 = half;
+                    }
+                    const unsigned h0 = fx_hi(a[q].x), h1 = fx_hi(a[q].y), h2 = fx_hi(c[q].x), h3 = fx_hi(c[q].y);
+                    const unsigned m0 = h0 > h1 ? h0 : h1, m1 = h2 > h3 ? h2 : h3;
+                    m = m0 > m1 ? m0 : m1;
+                    *(double2*)&b[l * n + fxs(k)] = a[q];
+                    *(double2*)&b[l * n + fxs(k2)] = c[q];
+                }
+                fxc_put_max(red, l, in, m, half);
+            }
+        }
+    }
+}
+// the doubles in the slots -> fixed point in place (rows: of fxc_load_rows)
+static __device__ __noinline__ void fxc_convert(longlong2* b, int nl, int logn, unsigned* red, unsigned* sums, int tid,
+                                                int nthr) {
+    const int n = 1 << logn, tot = nl << logn, lane = tid % kWarp;
+    for (int iw = tid - lane; iw < tot; iw += nthr) {
+        const int i = iw + lane, l = i < tot ? i >> logn : 0;
+        unsigned s = 0;
+        if (i < tot) s = fx_point(b + (l << logn) + fxs(i & (n - 1)), fx_emax(red[l]));
+        fxc_put_sum(sums, l, i < tot, s, n);
+    }
+}
+static __device__ __noinline__ void fxc_convert_rows(longlong2* b, int nl, int logn, unsigned* red, unsigned* sums, int tid,
+                                                     int nthr) {
+    const int n = 1 << logn, half = n >> 1, tot = nl * half, lane = tid % kWarp;
+    for (int iw = tid - lane; iw < tot; iw += nthr) {
+        const int i = iw + lane, l = i < tot ? i >> (logn - 1) : 0;
+        unsigned s = 0;
+        if (i < tot) s = fx_pair_rows(b + l * n, i & (half - 1), n, fx_emax(red[l]));
+        fxc_put_sum(sums, l, i < tot, s, half);
+    }
+}
+__device__ __forceinline__ int fxc_scale(const unsigned* red, const unsigned* sums, int l) {
+    return fx_scale(fx_emax(red[l]), fx_shift(sums[l]));
+}
+// transformed lines -> memory
+static __device__ __noinline__ void fxc_store(const longlong2* b, double2* d, long long H, int nl, int logn,
+                                              const unsigned* red, const unsigned* sums, int tid, int nthr) {
+    const int n = 1 << logn, tot = nl << logn;
+#pragma unroll 2
+    for (int i = tid; i < tot; i += nthr) {
+        const int l = i >> logn, x = i & (n - 1), S = fxc_scale(red, sums, l);
+        const longlong2 z = b[(l << logn) + fxs(x)];
+        d[(size_t)l * H + x] = fx_fast(S) ? double2{fx_to_t<true>(z.x, S), fx_to_t<true>(z.y, S)}
+                                          : double2{fx_to(z.x, S), fx_to(z.y, S)};
+    }
+}
+static __device__ __noinline__ void fxc_store_rows(const longlong2* b, double2* d0, long long H, int rows, int nl, int logn,
+                                                   const unsigned* red, const unsigned* sums, int tid, int nthr) {
+    const int n = 1 << logn, half = n >> 1, tot = nl * half;
+    // coefficients k < n / 2, then n / 2 of every line
+    for (int i = tid; i < tot + nl; i += nthr) {
+        const int l = i < tot ? i >> (logn - 1) : i - tot, k = i < tot ? i & (half - 1) : half, S = fxc_scale(red, sums, l) + 1;
+        const longlong2 zk = b[l * n + fxs(k)], zn = b[l * n + fxs((n - k) & (n - 1))];
+        const longlong2 A{zk.x + zn.x, zk.y - zn.y}, B{zk.y + zn.y, zn.x - zk.x};
+        double2* d = d0 + (size_t)l * H + (size_t)k * rows;
+        if (fx_fast(S)) {
+            d[0] = double2{fx_to_t<true>(A.x, S), fx_to_t<true>(A.y, S)};
+            d[1] = double2{fx_to_t<true>(B.x, S), fx_to_t<true>(B.y, S)};
+        } else {
+            d[0] = double2{fx_to(A.x, S), fx_to(A.y, S)};
+            d[1] = double2{fx_to(B.x, S), fx_to(B.y, S)};
+        }
+    }
+}
+
+template <int R, int S, int LOGN, int LOGNS>
+__device__ __forceinline__ void fx_stage_coop(const longlong2* src, longlong2* dst, int nl, const unsigned* sums,
+                                              const FxTw* tw, int logTw, int tid, int nthr) {
     constexpr int LR = (R == 2) ? 1 : (R == 4) ? 2 : 3;
-    constexpr int LNB = LOGN - LR, NB = 1 << LNB;
-    const int twshift = logTw - (logNs + LR), nsm = (1 << logNs) - 1, tot = nl << LNB;
+    constexpr int LNB = LOGN - LR, NB = 1 << LNB, NS = 1 << LOGNS;
+    const int twshift = logTw - (LOGNS + LR), tot = nl << LNB;
+#pragma unroll 1
     for (int it = tid; it < tot; it += nthr) {
-        const int l = it >> LNB, j = it & (NB - 1);
+        const int l = it >> LNB, j = it & (NB - 1), jm = j & (NS - 1);
         const longlong2* s = src + (l << LOGN);
         longlong2* d = dst + (l << LOGN);
         longlong2 v[R];
 #pragma unroll
         for (int r = 0; r < R; r++) v[r] = s[fxs(j + r * NB)];
-        const int jm = j & nsm;
-        if (logNs == 0) {
+        if (LOGNS == 0) {
             const int sh = fx_shift(sums[l]);
             const long long half = fx_half(sh);
 #pragma unroll
@@ -611,39 +764,39 @@ __device__ __forceinline__ void fx_stage_coop(const longlong2* src, longlong2* d
         fx_dft<R, S>(v);
         const int dd = ((j - jm) << LR) + jm;
 #pragma unroll
-        for (int r = 0; r < R; r++) d[fxs(dd + (r << logNs))] = v[r];
+        for (int r = 0; r < R; r++) d[fxs(dd + (r << LOGNS))] = v[r];
+    }
+}
+// radix of a shared line's stage: 4, and 8 for the first stage of an odd number of levels
+__host__ __device__ constexpr int fxc_radix(int logn, int logns) { return logns == 0 && (logn & 1) ? 8 : 4; }
+template <int S, int LOGN, int LOGNS>
+__device__ __forceinline__ int fx_stages_coop(longlong2* b0, longlong2* b1, int nl, const unsigned* sums, const FxTw* tw,
+                                              int logTw, int tid, int nthr) {
+    if constexpr (LOGNS < LOGN) {
+        constexpr int R = fxc_radix(LOGN, LOGNS);
+        fx_stage_coop<R, S, LOGN, LOGNS>(b0, b1, nl, sums, tw, logTw, tid, nthr);
+        cta_sync();
+        return 1 ^ fx_stages_coop<S, LOGN, LOGNS + radix_log(R)>(b1, b0, nl, sums, tw, logTw, tid, nthr);
+    } else {
+        return 0;
     }
 }
 
-// nl converted lines of 1 << LOGN points in b0 (sums[l]: line l's sum of
-// fx_mag, complete before the call) -> the transforms in b0 (returns 0) or b1
-// (1), visible to every thread on return.  Radix 8 where it gives at least
-// half of the threads a butterfly, else 4: a stage costs a barrier and a round
-// trip through shared memory (about 120 cycles), a radix-4 butterfly's
-// arithmetic about as much, so narrower stages lose more than they spread.
+// nl converted lines of 1 << LOGN points in b0 (sums complete before the call)
+// -> the transforms in b0 (returns 0) or b1 (1), visible to every thread on
+// return.  Radix 4: a stage costs a barrier and a round trip through shared
+// memory; a lone warp on a sub-partition issues a product in about 30 cycles,
+// and wider radices leave more of them idle.
 template <int S, int LOGN>
-__device__ __noinline__ int fx_lines_coop(longlong2* b0, longlong2* b1, int nl, const unsigned* sums,
-                                          const longlong2* tw, int logTw, int tid, int nthr) {
-    longlong2* b[2] = {b0, b1};
-    int cur = 0, logNs = 0;
-    while (logNs < LOGN) {
-        const int rem = LOGN - logNs;
-        const int lr = (rem >= 3 && 2 * (nl << (LOGN - 3)) >= nthr) ? 3 : (rem >= 2 ? 2 : 1);
-        if (logNs > 0) cta_sync();
-        if (lr == 3) fx_stage_coop<8, S, LOGN>(b[cur], b[cur ^ 1], nl, logNs, sums, tw, logTw, tid, nthr);
-        else if (lr == 2) fx_stage_coop<4, S, LOGN>(b[cur], b[cur ^ 1], nl, logNs, sums, tw, logTw, tid, nthr);
-        else fx_stage_coop<2, S, LOGN>(b[cur], b[cur ^ 1], nl, logNs, sums, tw, logTw, tid, nthr);
-        logNs += lr;
-        cur ^= 1;
-    }
-    cta_sync();
-    return cur;
+__device__ __noinline__ int fx_lines_coop(longlong2* b0, longlong2* b1, int nl, const unsigned* sums, const FxTw* tw,
+                                          int logTw, int tid, int nthr) {
+    return fx_stages_coop<S, LOGN, 0>(b0, b1, nl, sums, tw, logTw, tid, nthr);
 }
 
 // NF: the line length, or 0 for the runtime length 1 << logn (8 .. 512)
 template <int S, int NF>
-__device__ __forceinline__ int fx_coop(longlong2* b0, longlong2* b1, int logn, int nl, const unsigned* sums,
-                                       const longlong2* tw, int logTw, int tid, int nthr) {
+__device__ __forceinline__ int fx_coop(longlong2* b0, longlong2* b1, int logn, int nl, const unsigned* sums, const FxTw* tw,
+                                       int logTw, int tid, int nthr) {
     if constexpr (NF > 0) {
         return fx_lines_coop<S, ilog2c(NF)>(b0, b1, nl, sums, tw, logTw, tid, nthr);
     } else {

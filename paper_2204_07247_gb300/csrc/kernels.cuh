@@ -66,8 +66,8 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxCtas) pagd_kernel(const __gri
     __shared__ double red[32];
     // twiddles exp(-2 pi i m / 2^logtw) staged from the global table
     const int ntw = 1 << P.logtw;
-    longlong2* tfx = (longlong2*)smem;
-    float2* t32 = (float2*)(smem + (size_t)ntw * sizeof(longlong2));
+    FxTw* tfx = (FxTw*)smem;
+    float2* t32 = (float2*)(smem + (size_t)ntw * sizeof(FxTw));
     const int stride = kNMax >> P.logtw;
     for (int m = threadIdx.x; m < ntw; m += blockDim.x) {
         tfx[m] = P.twfx[m * stride];

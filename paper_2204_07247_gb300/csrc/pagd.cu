@@ -122,7 +122,7 @@ static void plan_layout(pagd_solver* s) {
     sz[O_X64] = s->dim == 3 ? sizeof(double2) * H * 3 : 0;
     sz[O_GH64] = sizeof(double2) * H;
     sz[O_LCTL] = sizeof(Ctl);
-    sz[O_TWFX] = sizeof(longlong2) * kNMax;
+    sz[O_TWFX] = sizeof(FxTw) * kNMax;
     static_assert(O_END <= (int)(sizeof(((pagd_solver*)nullptr)->off) / sizeof(size_t)), "offset table too small");
     size_t o = 0;
     for (int i = 0; i < O_END; i++) {
@@ -188,7 +188,7 @@ static Params params_for(const pagd_solver* s, char* w) {
     P.stats = (StepStat*)(w + s->off[O_STATS]);
     P.tw64 = (const double2*)(w + s->off[O_TW64]);
     P.tw32 = (const float2*)(w + s->off[O_TW32]);
-    P.twfx = (const longlong2*)(w + s->off[O_TWFX]);
+    P.twfx = (const FxTw*)(w + s->off[O_TWFX]);
     P.U[0] = (double*)(w + s->off[O_U0]);
     P.U[1] = (double*)(w + s->off[O_U1]);
     P.VB = (double*)(w + s->off[O_VB]);
@@ -227,7 +227,7 @@ static Params params_for(const pagd_solver* s, char* w) {
 struct TwTables {
     std::vector<double2> t64;
     std::vector<float2> t32;
-    std::vector<longlong2> tfx;
+    std::vector<FxTw> tfx;
     TwTables() : t64(kNMax), t32(kNMax), tfx(kNMax) {
         const long double one = (long double)(1ull << kFxTw);
         for (int m = 0; m < kNMax; m++) {
@@ -236,7 +236,7 @@ struct TwTables {
             const long double c = cosl(ang), s = sinl(ang);
             t64[m] = double2{(double)c, (double)s};
             t32[m] = float2{(float)t64[m].x, (float)t64[m].y};
-            tfx[m] = longlong2{llroundl(c * one), llroundl(s * one)};
+            tfx[m] = fx_tw(llroundl(c * one), llroundl(s * one));
         }
     }
 };
@@ -268,8 +268,8 @@ template <class T> static pagd_status launch(pagd_solver* s, const Params& P) {
     blockDim.x = 1;
     threadIdx.x = 0;
     const int ntw = 1 << P.logtw;
-    longlong2* tfx = (longlong2*)base;
-    float2* t32 = (float2*)(base + (size_t)ntw * sizeof(longlong2));
+    FxTw* tfx = (FxTw*)base;
+    float2* t32 = (float2*)(base + (size_t)ntw * sizeof(FxTw));
     for (int m = 0; m < ntw; m++) {
         tfx[m] = P.twfx[m * (kNMax >> P.logtw)];
         t32[m] = P.tw32[m * (kNMax >> P.logtw)];
@@ -357,19 +357,19 @@ static pagd_status run_program(pagd_solver* s, Params& P) {
 }
 
 // The FP32 iteration passes stage their inputs through shared memory
-// (row_pass_staged / col_pass_staged; fixed line lengths only): bytes a warp's
+// (row_pass_staged / col_pass_staged; line lengths 64 to 512): bytes a warp's
 // slice needs for the staging slots (PFC two, FCH one), 0 where they do not
 // stage.  PAGD_STAGED=0 keeps the register-staged passes (the same arithmetic,
 // for comparison).
 static size_t staged_bytes(const pagd_solver* s) {
-    const int nf = fixed_len(s->n[0], s->n[s->dim - 1]);
-    if (nf == 0 || s->tsize != 4) return 0;
+    const int n0 = s->n[0], n1 = s->n[s->dim - 1];
+    if (!stage_len(n0) || !stage_len(n1) || s->tsize != 4) return 0;
     if (const char* e = std::getenv("PAGD_STAGED"))
         if (e[0] == '0' && e[1] == 0) return 0;
     const int k = k_iter(s->model), sl = staged_slots(s->model);
-    size_t m = std::max(row_staged_smem(nf, k, staged_row_state(s->model), sl), col_staged_smem(nf, k, 3, sl));
+    size_t m = std::max(row_staged_smem(n1, k, staged_row_state(s->model), sl), col_staged_smem(n0, k, 3, sl));
     // the middle passes of a cubic grid stage too (mid_pass_staged)
-    if (s->dim == 3 && s->n[1] == nf) m = std::max(m, mid_staged_smem(nf));
+    if (s->dim == 3 && n0 == n1 && s->n[1] == n0) m = std::max(m, mid_staged_smem(n0));
     return (m + 15) & ~(size_t)15;
 }
 static bool stage_fits(const pagd_solver* s, size_t warp_bytes) {
@@ -555,7 +555,7 @@ pagd_status pagd_set_workspace(pagd_solver* s, void* dev_ptr, size_t bytes) {
     const TwTables t;
     pagd_status st = dcopy(s, s->ws + s->off[O_TW64], t.t64.data(), sizeof(double2) * kNMax);
     if (st == PAGD_OK) st = dcopy(s, s->ws + s->off[O_TW32], t.t32.data(), sizeof(float2) * kNMax);
-    if (st == PAGD_OK) st = dcopy(s, s->ws + s->off[O_TWFX], t.tfx.data(), sizeof(longlong2) * kNMax);
+    if (st == PAGD_OK) st = dcopy(s, s->ws + s->off[O_TWFX], t.tfx.data(), sizeof(FxTw) * kNMax);
     if (st == PAGD_OK) st = dsync(s);
     return st;
 }
@@ -957,14 +957,14 @@ constexpr size_t kStaticWorkspaceBytes = kStaticScratchBytes - kStaticTwBytes;  
 static_assert(kStaticWorkspaceBytes == 8364032, "the limit stated in include/pagd.h");
 #ifndef PAGD_EMU
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
-static __device__ longlong2 g_static_twfx[kNMax];  // the fixed-point twiddle table
+static __device__ FxTw g_static_twfx[kNMax];  // the fixed-point twiddle table
 #else
 alignas(256) static unsigned char g_static_scratch[kStaticScratchBytes];
-static longlong2 g_static_twfx[kNMax];
+static FxTw g_static_twfx[kNMax];
 #endif
 constexpr int kMaxDevices = 64;
 static void* g_static_ptr[kMaxDevices];
-static const longlong2* g_static_twfx_ptr[kMaxDevices];
+static const FxTw* g_static_twfx_ptr[kMaxDevices];
 static std::mutex g_static_mu;  // guards g_static_ptr and the one-time set-up
 
 // Device address of the static scratch for the current device, with the
@@ -974,14 +974,14 @@ static std::mutex g_static_mu;  // guards g_static_ptr and the one-time set-up
 // with a synchronous cudaMemcpy.  This happens on the first call on each device
 // (make that first call before any stream capture); the lock makes concurrent
 // first calls from several host threads do it once.
-static pagd_status static_scratch(pagd_solver* s, char** out, const longlong2** twfx) {
+static pagd_status static_scratch(pagd_solver* s, char** out, const FxTw** twfx) {
 #ifdef PAGD_EMU
     std::lock_guard<std::mutex> lk(g_static_mu);
     if (!g_static_ptr[0]) {
         const TwTables t;
         std::memcpy(g_static_scratch, t.t64.data(), sizeof(double2) * kNMax);
         std::memcpy(g_static_scratch + sizeof(double2) * kNMax, t.t32.data(), sizeof(float2) * kNMax);
-        std::memcpy(g_static_twfx, t.tfx.data(), sizeof(longlong2) * kNMax);
+        std::memcpy(g_static_twfx, t.tfx.data(), sizeof(FxTw) * kNMax);
         g_static_twfx_ptr[0] = g_static_twfx;
         g_static_ptr[0] = g_static_scratch;
     }
@@ -1007,9 +1007,9 @@ static pagd_status static_scratch(pagd_solver* s, char** out, const longlong2** 
         if (e == cudaSuccess)
             e = cudaMemcpy((char*)ptr + sizeof(double2) * kNMax, t.t32.data(), sizeof(float2) * kNMax,
                            cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(fx, t.tfx.data(), sizeof(longlong2) * kNMax, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(fx, t.tfx.data(), sizeof(FxTw) * kNMax, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return cuda_fail(s, e, "cudaMemcpy of the static twiddle tables");
-        g_static_twfx_ptr[dev] = (const longlong2*)fx;
+        g_static_twfx_ptr[dev] = (const FxTw*)fx;
         g_static_ptr[dev] = ptr;
     }
     *out = (char*)g_static_ptr[dev];
@@ -1034,7 +1034,7 @@ pagd_status pagd_step_static(pagd_solver* s, const double* un_dev, const double*
         return fail(s, PAGD_EINVAL, buf);
     }
     char* head = nullptr;
-    const longlong2* twfx = nullptr;
+    const FxTw* twfx = nullptr;
     pagd_status st = static_scratch(s, &head, &twfx);
     if (st != PAGD_OK) return st;
     char* w = head + kStaticTwBytes;
@@ -1234,8 +1234,8 @@ template <class T> static pagd_status batch_launch(pagd_batch* b, const BatchPar
     blockDim.x = (unsigned)b->wpb;
     threadIdx.x = 0;
     const int ntw = 1 << B.logtw;
-    longlong2* tfx = (longlong2*)base;
-    float2* t32 = (float2*)(base + (size_t)ntw * sizeof(longlong2));
+    FxTw* tfx = (FxTw*)base;
+    float2* t32 = (float2*)(base + (size_t)ntw * sizeof(FxTw));
     for (int m = 0; m < ntw; m++) {
         tfx[m] = B.twfx[m * (kNMax >> B.logtw)];
         t32[m] = B.tw32[m * (kNMax >> B.logtw)];
@@ -1316,7 +1316,7 @@ pagd_status pagd_batch_create(pagd_batch** out, pagd_solver* const* members, int
         for (int d = 0; d < s->dim; d++) b->logtw = std::max(b->logtw, ilog2(s->n[d]));
         b->warp_bytes = std::max(b->warp_bytes, warp_smem_bytes(s->n[0], s->n[last], s->model, s->tsize,
                                                                 batch_nf(s->n[0], s->n[last]), nm));
-        if (batch_nf(s->n[0], s->n[last])) b->warp_bytes = std::max(b->warp_bytes, staged_bytes(s));
+        b->warp_bytes = std::max(b->warp_bytes, staged_bytes(s));
     }
 #ifdef PAGD_EMU
     const int wpb = kEmuBatchWarps;

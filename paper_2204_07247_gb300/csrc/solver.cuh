@@ -158,7 +158,7 @@ struct Params {
     // twiddle tables of kNMax entries: FP64 (the cluster loop's), FP32, fixed point
     const double2* tw64;
     const float2* tw32;
-    const longlong2* twfx;
+    const FxTw* twfx;
     Scal* sc;
     double* mass;  // persistent {K, D, R}: mass excess since set_state, this step's change, and
                    // R, ||d_0||_inf of the last step started from the extrapolation (0: none)
@@ -215,7 +215,7 @@ constexpr int kStagnation = 12;
 // every SM gets a busy warp before any SM gets a second); else the warp owns
 // the contiguous unit range [ulo, uhi) (batched launches).
 struct Tw {
-    const longlong2* tfx;  // cos, sin in units of 2^-61 (fx.cuh)
+    const FxTw* tfx;       // fixed-point twiddles (fx.cuh)
     const float2* t32;
     const double* sq;      // squares 0 .. kSq - 1
     int log;
@@ -1197,16 +1197,11 @@ __device__ __forceinline__ void fx_publish_max(unsigned* a, unsigned v) {
     v = warp_umax(v);
     if ((threadIdx.x % kWarp) == 0) atomicMax(a, v);
 }
-__device__ __forceinline__ void fx_publish_sum(unsigned* a, unsigned v) {
-    v = warp_uadd(v);
-    if ((threadIdx.x % kWarp) == 0) atomicAdd(a, v);
-}
-
 template <int NF, class Ld, class Ap>
 __device__ void row_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kout, const double2* src, double2* dst,
                                  char* smem, Ld&& ld, Ap&& ap) {
     using S = decltype(ld(0ll, 0, 0));
-    const int n = NF > 0 ? NF : P.n1, logn = NF > 0 ? ilog2c(NF) : P.logn1, half = n >> 1, rows = P.rows;
+    const int n = NF > 0 ? NF : P.n1, logn = NF > 0 ? ilog2c(NF) : P.logn1, rows = P.rows;
     const long long Hs = P.H;
     const int tid = threadIdx.x, nthr = blockDim.x;
     longlong2* B0 = (longlong2*)smem;
@@ -1226,21 +1221,14 @@ __device__ void row_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
         longlong2* X = B0;
         int sc[kMaxK] = {0, 0, 0};
         if (kin > 0) {
-            for (int f = 0; f < kin; f++)
-                fx_publish_max(red + f, fx_load_rows(B0 + f * n, src + (size_t)f * Hs + r0, n, rows, tid, nthr));
+            fxc_load_rows(B0, src + r0, Hs, rows, kin, logn, red, tid, nthr);
             cta_sync();
-            for (int f = 0; f < kin; f++) {
-                const int emax = fx_emax(red[f]);
-                longlong2* b = B0 + f * n;
-                unsigned s = 0;
-                for (int k = tid; k < half; k += nthr) s += fx_pair_rows(b, k, n, emax);
-                fx_publish_sum(red + kMaxK + f, s);
-            }
+            fxc_convert_rows(B0, kin, logn, red, red + kMaxK, tid, nthr);
             cta_sync();
             X = fx_coop<+1, NF>(B0, B1, logn, kin, red + kMaxK, tw.tfx, tw.log, tid, nthr) ? B1 : B0;
 #pragma unroll
             for (int f = 0; f < kMaxK; f++)
-                if (f < kin) sc[f] = fx_scale(fx_emax(red[f]), fx_shift(red[kMaxK + f])) + log_npts(P);
+                if (f < kin) sc[f] = fxc_scale(red, red + kMaxK, f) + log_npts(P);
         }
         // pointwise: point q = rr n + x of the unit; the outputs replace the
         // inputs of the same point and row
@@ -1281,19 +1269,11 @@ __device__ void row_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
             for (int g = 0; g < kMaxK; g++)
                 if (g < kout) fx_publish_max(red + 2 * kMaxK + g, hi[g]);
             cta_sync();
-            for (int g = 0; g < kout; g++) {
-                const int emax = fx_emax(red[2 * kMaxK + g]);
-                unsigned s = 0;
-                for (int x = tid; x < n; x += nthr) s += fx_point(X + g * n + fxs(x), emax);
-                fx_publish_sum(red + 3 * kMaxK + g, s);
-            }
+            fxc_convert(X, kout, logn, red + 2 * kMaxK, red + 3 * kMaxK, tid, nthr);
             cta_sync();
             longlong2* Z = X == B0 ? B1 : B0;
             const longlong2* Y = fx_coop<-1, NF>(X, Z, logn, kout, red + 3 * kMaxK, tw.tfx, tw.log, tid, nthr) ? Z : X;
-            for (int g = 0; g < kout; g++) {
-                const int e = fx_scale(fx_emax(red[2 * kMaxK + g]), fx_shift(red[3 * kMaxK + g]));
-                fx_store_rows(Y + g * n, n, e, dst + (size_t)g * Hs + r0, rows, tid, nthr);
-            }
+            fxc_store_rows(Y, dst + r0, Hs, rows, kout, logn, red + 2 * kMaxK, red + 3 * kMaxK, tid, nthr);
         }
         cta_sync();  // the next unit reuses the buffers
     }
@@ -1323,20 +1303,14 @@ __device__ void col_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
         longlong2* X = B0;
         int sc[kMaxK] = {0, 0, 0};
         if (kin > 0) {
-            for (int f = 0; f < kin; f++)
-                fx_publish_max(red + f, fx_load(B0 + f * n, src + (size_t)f * Hs + (size_t)k1 * n, n, tid, nthr));
+            fxc_load(B0, src + (size_t)k1 * n, Hs, kin, logn, red, tid, nthr);
             cta_sync();
-            for (int f = 0; f < kin; f++) {
-                const int emax = fx_emax(red[f]);
-                unsigned s = 0;
-                for (int x = tid; x < n; x += nthr) s += fx_point(B0 + f * n + fxs(x), emax);
-                fx_publish_sum(red + kMaxK + f, s);
-            }
+            fxc_convert(B0, kin, logn, red, red + kMaxK, tid, nthr);
             cta_sync();
             X = fx_coop<-1, NF>(B0, B1, logn, kin, red + kMaxK, tw.tfx, tw.log, tid, nthr) ? B1 : B0;
 #pragma unroll
             for (int f = 0; f < kMaxK; f++)
-                if (f < kin) sc[f] = fx_scale(fx_emax(red[f]), fx_shift(red[kMaxK + f]));
+                if (f < kin) sc[f] = fxc_scale(red, red + kMaxK, f);
         }
         // outputs: doubles in place of the inputs, FP32 lines in the other set
         longlong2* Z = X == B0 ? B1 : B0;
@@ -1386,18 +1360,11 @@ __device__ void col_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
                 for (int g = 0; g < kMaxK; g++)
                     if (g < kout) fx_publish_max(red + 2 * kMaxK + g, hi[g]);
                 cta_sync();
-                for (int g = 0; g < kout; g++) {
-                    const int emax = fx_emax(red[2 * kMaxK + g]);
-                    unsigned s = 0;
-                    for (int x = tid; x < n; x += nthr) s += fx_point(X + g * n + fxs(x), emax);
-                    fx_publish_sum(red + 3 * kMaxK + g, s);
-                }
+                fxc_convert(X, kout, logn, red + 2 * kMaxK, red + 3 * kMaxK, tid, nthr);
                 cta_sync();
                 const longlong2* Y =
                     fx_coop<+1, NF>(X, Z, logn, kout, red + 3 * kMaxK, tw.tfx, tw.log, tid, nthr) ? Z : X;
-                for (int g = 0; g < kout; g++)
-                    fx_store(Y + g * n, n, fx_scale(fx_emax(red[2 * kMaxK + g]), fx_shift(red[3 * kMaxK + g])),
-                             dst + (size_t)g * Hs + (size_t)k1 * n, tid, nthr);
+                fxc_store(Y, dst + (size_t)k1 * n, Hs, kout, logn, red + 2 * kMaxK, red + 3 * kMaxK, tid, nthr);
             } else {
                 cta_sync();  // the inputs' buffers become the second set of the FP32 lines
                 float2 *f0 = (float2*)Z, *f1 = (float2*)X;
@@ -2382,6 +2349,13 @@ __device__ __noinline__ void phase_R_staged(const Params& P, const Ctl& c, const
     publish_sum(&P.sums[(size_t)bank * P.nslots + c.ev], asum);
 }
 
+template <int L>
+__device__ __forceinline__ void phase_R_staged_of(const Params& P, const Ctl& c, const Tw& tw, char* smem,
+                                                  const float2* src) {
+    if (P.model == M_PFC) phase_R_staged<L, true>(P, c, tw, smem, src);
+    else phase_R_staged<L, false>(P, c, tw, smem, src);
+}
+
 // The FP32 iteration row pass with CTA-cooperative units (row_pass_coop), an
 // opt-in alternative (Params::coop32) for grids with fewer row units than
 // SMs, where one warp per unit leaves most of an SM idle.
@@ -2416,13 +2390,22 @@ __device__ __noinline__ void phase_R_coop(const Params& P, const Ctl& c, const T
 template <class TI, class T, int NF>
 __device__ PAGD_HOT void phase_R(const Params& P, const Ctl& c, const Tw& tw, char* smem, double* red,
                         const cx<TI>* src) {
-    if constexpr (sizeof(TI) == 4 && sizeof(T) == 4 && (NF & (kNoCoop - 1)) != 0) {
+    if constexpr (sizeof(TI) == 4 && sizeof(T) == 4) {
         if (P.stage) {
-            if (P.model == M_PFC) phase_R_staged<NF & (kNoCoop - 1), true>(P, c, tw, smem, (const float2*)src);
-            else phase_R_staged<NF & (kNoCoop - 1), false>(P, c, tw, smem, (const float2*)src);
+            constexpr int L = NF & (kNoCoop - 1);
+            if constexpr (L != 0) {
+                phase_R_staged_of<L>(P, c, tw, smem, (const float2*)src);
+            } else {  // a rectangular grid: the row passes' line length
+                switch (P.n1) {
+                    case 64: phase_R_staged_of<64>(P, c, tw, smem, (const float2*)src); break;
+                    case 128: phase_R_staged_of<128>(P, c, tw, smem, (const float2*)src); break;
+                    case 256: phase_R_staged_of<256>(P, c, tw, smem, (const float2*)src); break;
+                    default: phase_R_staged_of<512>(P, c, tw, smem, (const float2*)src); break;
+                }
+            }
             return;
         }
-        if constexpr (!(NF & kNoCoop)) {
+        if constexpr (!(NF & kNoCoop) && NF != 0) {
             if (P.coop32) {
                 phase_R_coop<NF>(P, c, tw, smem, (const float2*)src);
                 return;
@@ -2524,6 +2507,11 @@ __device__ __noinline__ void phase_CI_staged(const Params& P, const Ctl& c, cons
                                   });
 }
 
+template <int L> __device__ __forceinline__ void phase_CI_staged_of(const Params& P, const Ctl& c, const Tw& tw, char* smem) {
+    if (P.model == M_PFC) phase_CI_staged<L, true>(P, c, tw, smem);
+    else phase_CI_staged<L, false>(P, c, tw, smem);
+}
+
 // The FP32 iteration column pass with CTA-cooperative units (col_pass_coop).
 template <int NF>
 __device__ __noinline__ void phase_CI_coop(const Params& P, const Ctl& c, const Tw& tw, char* smem) {
@@ -2552,13 +2540,22 @@ __device__ __noinline__ void phase_CI_coop(const Params& P, const Ctl& c, const 
 template <class T, int NF>
 __device__ PAGD_HOT void phase_CI(const Params& P, const Ctl& c, const Tw& tw, char* smem) {
     using C = cx<T>;
-    if constexpr (sizeof(T) == 4 && (NF & (kNoCoop - 1)) != 0) {
+    if constexpr (sizeof(T) == 4) {
         if (P.stage) {
-            if (P.model == M_PFC) phase_CI_staged<NF & (kNoCoop - 1), true>(P, c, tw, smem);
-            else phase_CI_staged<NF & (kNoCoop - 1), false>(P, c, tw, smem);
+            constexpr int L = NF & (kNoCoop - 1);
+            if constexpr (L != 0) {
+                phase_CI_staged_of<L>(P, c, tw, smem);
+            } else {
+                switch (P.n0) {
+                    case 64: phase_CI_staged_of<64>(P, c, tw, smem); break;
+                    case 128: phase_CI_staged_of<128>(P, c, tw, smem); break;
+                    case 256: phase_CI_staged_of<256>(P, c, tw, smem); break;
+                    default: phase_CI_staged_of<512>(P, c, tw, smem); break;
+                }
+            }
             return;
         }
-        if constexpr (!(NF & kNoCoop)) {
+        if constexpr (!(NF & kNoCoop) && NF != 0) {
             if (P.coop32) {
                 phase_CI_coop<NF>(P, c, tw, smem);
                 return;
@@ -3335,8 +3332,13 @@ inline size_t warp_smem_bytes(int n0, int n1, int model, int tsize, int nf, int 
 // squares of the wavenumber indices
 constexpr int kSq = 258;  // indices to 256 (512 points per axis), a multiple of 16 bytes
 __host__ __device__ inline size_t tw_smem_bytes(int logtw) {
-    return ((size_t)1 << logtw) * (16 + 8) + kSq * sizeof(double);
+    return ((size_t)1 << logtw) * (sizeof(FxTw) + sizeof(float2)) + kSq * sizeof(double);
 }
+
+// line lengths of the staged FP32 passes; a rectangular grid of two of them
+// stages too, each pass with its own line's length (PFC 256 x 512: row pass
+// 19.7 us through the runtime-length pass, column pass 13.1)
+__host__ __device__ inline bool stage_len(int n) { return n == 64 || n == 128 || n == 256 || n == 512; }
 
 // the fixed line length used for an n0 x n1 grid (0: runtime-length passes)
 inline int fixed_len(int n0, int n1) {
@@ -3361,7 +3363,7 @@ struct BatchParams {
     int trace_cap;
     int* ntrace;
     const float2* tw32;
-    const longlong2* twfx;
+    const FxTw* twfx;
 };
 
 // work units of a phase and the points one unit touches: column lines, middle
