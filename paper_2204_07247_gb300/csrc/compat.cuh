@@ -27,6 +27,7 @@ struct alignas(16) float4 { float x, y, z, w; };
 struct alignas(16) longlong2 { long long x, y; };
 
 inline void __syncthreads() {}
+inline void pair_sync(int) {}
 inline void __threadfence() {}
 inline double atomicAdd(double* p, double v) { double o = *p; *p = o + v; return o; }
 inline unsigned atomicAdd(unsigned* p, unsigned v) { unsigned o = *p; *p = o + v; return o; }
@@ -66,6 +67,8 @@ __device__ __forceinline__ double bits_dbl(unsigned long long u) { return __long
 __device__ __forceinline__ unsigned flt_bits(float f) { return __float_as_uint(f); }
 __device__ __forceinline__ float bits_flt(unsigned u) { return __uint_as_float(u); }
 __device__ __forceinline__ float warp_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+// barrier of the two warps of pair p
+__device__ __forceinline__ void pair_sync(int p) { asm volatile("bar.sync %0, 64;" ::"r"(p + 1) : "memory"); }
 #define PAGD_WARP 32
 template <class T> __device__ __forceinline__ T warp_max(T v) {
 #pragma unroll

@@ -264,25 +264,22 @@ __device__ __forceinline__ void cta_sync() {
 #endif
 }
 
-template <int R, int S, class T, int LOGN>
-__device__ __forceinline__ void stage_coop(const cx<T>* src, cx<T>* dst, int pitch, int nl, int logNs,
-                                           const cx<T>* tw, int logTw, int tid, int nthr) {
+template <int R, int S, class T, int LOGN, int LOGNS>
+__device__ __forceinline__ void stage_coop(const cx<T>* src, cx<T>* dst, int pitch, int nl, const cx<T>* tw, int logTw,
+                                           int tid, int nthr) {
     using C = cx<T>;
     constexpr int LR = (R == 2) ? 1 : (R == 4) ? 2 : 3;
-    constexpr int LNB = LOGN - LR;
-    constexpr int NB = 1 << LNB;
-    const int twshift = logTw - (logNs + LR);
-    const int nsm = (1 << logNs) - 1;
-    const int tot = nl << LNB;
+    constexpr int LNB = LOGN - LR, NB = 1 << LNB, NS = 1 << LOGNS;
+    const int twshift = logTw - (LOGNS + LR), tot = nl << LNB;
+#pragma unroll 1
     for (int it = tid; it < tot; it += nthr) {
-        const int l = it >> LNB, j = it & (NB - 1);
+        const int l = it >> LNB, j = it & (NB - 1), jm = j & (NS - 1);
         const C* s = src + l * pitch;
         C* d = dst + l * pitch;
         C v[R];
 #pragma unroll
         for (int r = 0; r < R; r++) v[r] = s[j + r * NB];
-        const int jm = j & nsm;
-        if (jm) {
+        if (LOGNS > 0) {
 #pragma unroll
             for (int r = 1; r < R; r++) {
                 C w = tw[(jm * r) << twshift];
@@ -293,32 +290,33 @@ __device__ __forceinline__ void stage_coop(const cx<T>* src, cx<T>* dst, int pit
         dftR<R, S>(v);
         const int idxD = ((j - jm) << LR) + jm;
 #pragma unroll
-        for (int r = 0; r < R; r++) d[idxD + (r << logNs)] = v[r];
+        for (int r = 0; r < R; r++) d[idxD + r * NS] = v[r];
+    }
+}
+// radix of a shared line's stage: 4, and 8 for the first stage of an odd
+// number of levels (radix 2, which gives every thread a butterfly, needs twice
+// the barriers and shared-memory round trips and was slower)
+__host__ __device__ constexpr int coop_radix(int logn, int logns) { return logns == 0 && (logn & 1) ? 8 : 4; }
+template <int S, class T, int LOGN, int LOGNS>
+__device__ __forceinline__ int stages_coop(cx<T>* b0, cx<T>* b1, int pitch, int nl, const cx<T>* tw, int logTw, int tid,
+                                           int nthr) {
+    if constexpr (LOGNS < LOGN) {
+        constexpr int R = coop_radix(LOGN, LOGNS);
+        stage_coop<R, S, T, LOGN, LOGNS>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
+        cta_sync();
+        return 1 ^ stages_coop<S, T, LOGN, LOGNS + radix_log(R)>(b1, b0, pitch, nl, tw, logTw, tid, nthr);
+    } else {
+        return 0;
     }
 }
 
 // nl lines of length 1 << LOGN in b0 (written by any thread before the call)
-// -> result in b0 (returns 0) or b1 (1), visible to every thread on return.
-// Each stage takes the largest radix (8, 4, 2) whose butterflies still cover
-// the nthr threads.
+// -> result in b0 (returns 0) or b1 (1), visible to every thread on return
 template <int S, class T, int LOGN>
 __device__ __noinline__ int fft_lines_coop(cx<T>* b0, cx<T>* b1, int pitch, int nl, const cx<T>* tw, int logTw, int tid,
-                              int nthr) {
-    cx<T>* b[2] = {b0, b1};
-    int cur = 0, logNs = 0;
-    while (logNs < LOGN) {
-        const int rem = LOGN - logNs;
-        int lr = rem >= 3 ? 3 : rem;
-        while (lr > 1 && (nl << (LOGN - lr)) < nthr) lr--;
-        cta_sync();
-        if (lr == 3) stage_coop<8, S, T, LOGN>(b[cur], b[cur ^ 1], pitch, nl, logNs, tw, logTw, tid, nthr);
-        else if (lr == 2) stage_coop<4, S, T, LOGN>(b[cur], b[cur ^ 1], pitch, nl, logNs, tw, logTw, tid, nthr);
-        else stage_coop<2, S, T, LOGN>(b[cur], b[cur ^ 1], pitch, nl, logNs, tw, logTw, tid, nthr);
-        logNs += lr;
-        cur ^= 1;
-    }
+                                           int nthr) {
     cta_sync();
-    return cur;
+    return stages_coop<S, T, LOGN, 0>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
 }
 
 template <int S, class T, int NF>

@@ -767,13 +767,11 @@ __device__ __forceinline__ void fx_stage_coop(const longlong2* src, longlong2* d
         for (int r = 0; r < R; r++) d[fxs(dd + (r << LOGNS))] = v[r];
     }
 }
-// radix of a shared line's stage: 4, and 8 for the first stage of an odd number of levels
-__host__ __device__ constexpr int fxc_radix(int logn, int logns) { return logns == 0 && (logn & 1) ? 8 : 4; }
 template <int S, int LOGN, int LOGNS>
 __device__ __forceinline__ int fx_stages_coop(longlong2* b0, longlong2* b1, int nl, const unsigned* sums, const FxTw* tw,
                                               int logTw, int tid, int nthr) {
     if constexpr (LOGNS < LOGN) {
-        constexpr int R = fxc_radix(LOGN, LOGNS);
+        constexpr int R = coop_radix(LOGN, LOGNS);
         fx_stage_coop<R, S, LOGN, LOGNS>(b0, b1, nl, sums, tw, logTw, tid, nthr);
         cta_sync();
         return 1 ^ fx_stages_coop<S, LOGN, LOGNS + radix_log(R)>(b1, b0, nl, sums, tw, logTw, tid, nthr);

@@ -421,36 +421,44 @@ static size_t tile_smem(const SnoDims& d, int CT) {
 }
 
 // First axis: F[g][m0][m1] = sum over the rows r of T[g][r][m1] exp(-2 pi i k0 x0(r) / n0), one
-// block per channel g, a thread per mode and share of the rows
-constexpr int kColThr = 1024;
+// block per channel g, a thread per mode and share of the rows; the rows go
+// through shared memory, kColRows at a time, loaded together
+constexpr int kColThr = 1024, kColRows = 512;
 __global__ void __launch_bounds__(kColThr) k_cols(SnoDims d, const float2* T, const float2* tw0, float2* F) {
-    extern __shared__ __align__(16) float2 cs[];  // n0 twiddles, then the shares' sums
-    float2* part = cs + d.n0;
+    extern __shared__ __align__(16) float2 cs[];  // n0 twiddles, the rows, the shares' sums
+    float2* rw = cs + d.n0;
+    float2* part = rw + kColRows * d.M1;
     for (int i = threadIdx.x; i < d.n0; i += kColThr) cs[i] = tw0[i];
-    __syncthreads();
     int mp = 32;
     while (mp < d.M) mp <<= 1;
     const int g = blockIdx.x, m = threadIdx.x & (mp - 1), q = threadIdx.x / mp, nq = kColThr / mp, nr = d.n0 * d.JB;
-    if (m < d.M) {
-        const int m0 = m / d.M1, m1 = m - m0 * d.M1, k0 = k0_of(m0, d.M0, d.n0);
-        const float2* t = T + (size_t)g * nr * d.M1 + m1;
-        float2 s = make_float2(0.f, 0.f);
+    const int m0 = m / d.M1, m1 = m - m0 * d.M1, k0 = k0_of(m0, d.M0, d.n0);
+    float2 s = make_float2(0.f, 0.f);
+    for (int c0 = 0; c0 < nr; c0 += kColRows) {
+        const int cr = nr - c0 < kColRows ? nr - c0 : kColRows;
+        const float2* t = T + ((size_t)g * nr + c0) * d.M1;
+        __syncthreads();
 #pragma unroll 4
-        for (int r = q; r < nr; r += nq) {
-            const float2 v = t[(size_t)r * d.M1], e = cs[(k0 * (r / d.JB)) & (d.n0 - 1)];
-            s.x += v.x * e.x - v.y * e.y;
-            s.y += v.x * e.y + v.y * e.x;
+        for (int i = threadIdx.x; i < cr * d.M1; i += kColThr) rw[i] = t[i];
+        __syncthreads();
+        if (m < d.M) {
+#pragma unroll 4
+            for (int r = q; r < cr; r += nq) {
+                const float2 v = rw[r * d.M1 + m1], e = cs[(k0 * ((c0 + r) / d.JB)) & (d.n0 - 1)];
+                s.x += v.x * e.x - v.y * e.y;
+                s.y += v.x * e.y + v.y * e.x;
+            }
         }
-        part[q * mp + m] = s;
     }
+    if (m < d.M) part[q * mp + m] = s;
     __syncthreads();
     for (int i = threadIdx.x; i < d.M; i += kColThr) {
-        float2 s = part[i];
+        float2 f = part[i];
         for (int k = 1; k < nq; k++) {
-            s.x += part[k * mp + i].x;
-            s.y += part[k * mp + i].y;
+            f.x += part[k * mp + i].x;
+            f.y += part[k * mp + i].y;
         }
-        F[(size_t)g * d.M + i] = s;
+        F[(size_t)g * d.M + i] = f;
     }
 }
 
@@ -741,10 +749,13 @@ static void set_layer(TileArgs& a, const SnoDims& d, int l) {
 }
 
 // T -> the modes F
-static void launch_cols(const sno_net* s, int G, const float2* T, float2* F) {
+static cudaError_t launch_cols(const sno_net* s, int G, const float2* T, float2* F) {
     const SnoDims& d = s->d;
-    k_cols<<<G, kColThr, sizeof(float2) * (d.n0 + kColThr), (cudaStream_t)s->stream>>>(
-        d, T, (const float2*)(s->ws + s->off_tw0), F);
+    const size_t smem = sizeof(float2) * (d.n0 + (size_t)kColRows * d.M1 + kColThr);
+    const cudaError_t e = cudaFuncSetAttribute(k_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_cols<<<G, kColThr, smem, (cudaStream_t)s->stream>>>(d, T, (const float2*)(s->ws + s->off_tw0), F);
+    return cudaGetLastError();
 }
 
 // The forward pass for B samples up to the modes of the last layer; v_l (and,
@@ -763,7 +774,7 @@ static pagd_status forward(sno_net* s, TileArgs& a, int B, bool train) {
     for (int l = 0; l < d.L; l++) {
         float2* Fl = F + (size_t)l * B * d.C * d.M;
         set_layer(a, d, l);
-        launch_cols(s, B * d.C, a.T, Fl);
+        CK(launch_cols(s, B * d.C, a.T, Fl));
         k_mix<<<dim3((d.C * d.M + kThr - 1) / kThr, B), kThr, 0, st>>>(d, a.bias + d.C, Fl, G);
         a.vin = v + l * vs;
         if (l + 1 < d.L) {
@@ -888,7 +899,7 @@ pagd_status sno_loss_grad(sno_net* s, const float* params, const double* un, con
     for (int l = d.L - 1; l >= 0; l--) {
         float* gL = grad + off_layer(d, l);
         set_layer(a, d, l);
-        launch_cols(s, B * d.C, a.T, dZ);
+        CK(launch_cols(s, B * d.C, a.T, dZ));
         k_mix_back<<<dim3((d.M + 31) / 32, d.C), kThr, 0, st>>>(d, a.bias + d.C, F + (size_t)l * B * d.C * d.M, dZ,
                                                               gL + nrow, dF, B);
         if (d.C <= 16) CK(launch_wgrad<16>(d, dz, v + (size_t)l * vs, part, B, st));

@@ -1020,6 +1020,173 @@ __device__ void col_pass_staged(const Params& P, const Tw& tw, const float2* src
     warp_sync();
 }
 
+// ------------------------------------------- staged passes by pairs of warps
+//
+// The staged passes of two fields (FCH) with a unit shared by two warps, for
+// grids with no more units than pairs: one warp on an otherwise idle SM takes
+// about 6 us for a unit, most of it issuing its two lines' butterflies and
+// pointwise work one after the other.  Warp f of a pair stages and transforms
+// field f; the pointwise step is split by row (row pass) or by halves of the
+// line (column pass).  The pair's unit lives in the slice of its first warp.
+// The same arithmetic as row_pass_staged / col_pass_staged.  (The emulation
+// runs both warps' parts of each step between two pair barriers in turn.)
+struct Pair {
+    int id, f0, f1, b, e, s;  // pair of the CTA, this warp's parts [f0, f1), its units
+};
+__device__ __forceinline__ Pair pair_of(const Tw& tw, int units) {
+#ifdef PAGD_EMU
+    return Pair{0, 0, 2, tw.wr, units, tw.wn};
+#else
+    const int w = threadIdx.x / kWarp, np = blockDim.x / (2 * kWarp);
+    return Pair{w >> 1, w & 1, (w & 1) + 1, (w >> 1) * (int)gridDim.x + (int)blockIdx.x, (w >> 1) < np ? units : 0,
+                np * (int)gridDim.x};
+#endif
+}
+// whether the launch's pairs hold every unit at once
+__device__ __forceinline__ bool pairs_hold(const Tw& tw, int units) {
+#ifdef PAGD_EMU
+    return units > 0;
+#else
+    return units <= (int)(blockDim.x / (2 * kWarp)) * (int)gridDim.x;
+#endif
+}
+
+template <int NF, int NS, class Ap>
+__device__ void row_pass_pair(const Params& P, const Tw& tw, const float2* src, float2* dst, const float* const* sp,
+                              char* smem, Ap&& ap) {
+    constexpr int LOGN = ilog2c(NF), HALF = NF / 2, H1 = HALF + 1, PP = padded_len(NF), E = NF / kWarp, K = 2;
+    const int rows = P.rows, lane = threadIdx.x % kWarp;
+    const long long Hs = P.H;
+    const Pair pr = pair_of(tw, rows / 2);
+    char* mem = smem + (size_t)(2 * pr.id) * P.warp_bytes;
+    float2* X0 = (float2*)mem;
+    float2* X1 = X0 + K * PP;
+    float4* sq = (float4*)(X1 + K * PP);
+    float* st = (float*)(sq + K * H1);
+    const float iscale = (float)P.inv_npts;
+    for (int u = pr.b; u < pr.e; u += pr.s) {
+        const int r0 = 2 * u;
+        float2 *Xr = X0, *Xo = X1;
+        for (int f = pr.f0; f < pr.f1; f++) {
+            // field f's pieces and row f's state
+            for (int k = lane; k < H1; k += kWarp)
+                cp_async16(sq + f * H1 + k, src + (size_t)f * Hs + (size_t)k * rows + r0);
+            cp_async_commit();
+#pragma unroll
+            for (int a = 0; a < NS; a++)
+                for (int j = lane; j < NF / 4; j += kWarp)
+                    cp_async16(st + (a * 2 + f) * NF + 4 * j, sp[a] + (size_t)(r0 + f) * NF + 4 * j);
+            cp_async_commit();
+            cp_async_wait<1>();
+            warp_sync();
+#pragma unroll
+            for (int i = 0; i < E; i++) {
+                const int x = lane + kWarp * i;
+                const int k = (x <= HALF) ? x : NF - x;
+                const float4 v = sq[f * H1 + k];
+                float2 A{v.x, v.y}, B{v.z, v.w};
+                if (x == 0 || x == HALF) { A.y = 0.f; B.y = 0.f; }
+                X0[f * PP + pix<true>(x)] =
+                    (x <= HALF) ? float2{A.x - B.y, A.y + B.x} : float2{A.x + B.y, B.x - A.y};
+            }
+            const int r = fft_lines_fixed<+1, float, LOGN, 1, true>(X0 + f * PP, X1 + f * PP, PP, 1, tw.t32, tw.log, lane);
+            Xr = r ? X1 : X0;
+            Xo = r ? X0 : X1;
+            cp_async_wait<0>();
+        }
+        pair_sync(pr.id);
+        for (int rr = pr.f0; rr < pr.f1; rr++) {
+#pragma unroll
+            for (int i = 0; i < E; i++) {
+                const int x = lane + kWarp * i, px = pix<true>(x);
+                float sv[NS], in[K], out[K];
+#pragma unroll
+                for (int a = 0; a < NS; a++) sv[a] = st[(a * 2 + rr) * NF + x];
+#pragma unroll
+                for (int f = 0; f < K; f++) in[f] = ((const float*)&Xr[f * PP + px])[rr] * iscale;
+                ap((long long)(r0 + rr) * NF + x, r0 + rr, x, sv, in, out);
+#pragma unroll
+                for (int g = 0; g < K; g++) ((float*)&Xr[g * PP + px])[rr] = out[g];
+            }
+        }
+        pair_sync(pr.id);
+        for (int g = pr.f0; g < pr.f1; g++) {
+            const int r2 = fft_lines_fixed<-1, float, LOGN, 1, true>(Xr + g * PP, Xo + g * PP, PP, 1, tw.t32, tw.log, lane);
+            const float2* zl = (r2 ? Xo : Xr) + g * PP;
+            float4* d0 = (float4*)(dst + (size_t)g * Hs + r0);
+            for (int k = lane; k <= HALF; k += kWarp) {
+                const float2 zk = zl[pix<true>(k)], zn = zl[pix<true>((NF - k) & (NF - 1))];
+                d0[(size_t)k * (rows / 2)] =
+                    float4{0.5f * (zk.x + zn.x), 0.5f * (zk.y - zn.y), 0.5f * (zk.y + zn.y), 0.5f * (zn.x - zk.x)};
+            }
+        }
+        pair_sync(pr.id);
+    }
+}
+
+template <int NF, int NS, class Ap>
+__device__ void col_pass_pair(const Params& P, const Tw& tw, const float2* src, float2* dst, const float2* const* sc,
+                              char* smem, Ap&& ap) {
+    constexpr int LOGN = ilog2c(NF), PP = padded_len(NF), E = NF / kWarp, K = 2;
+    const int lane = threadIdx.x % kWarp;
+    const long long Hs = P.H;
+    const Pair pr = pair_of(tw, P.ncols);
+    char* mem = smem + (size_t)(2 * pr.id) * P.warp_bytes;
+    float2* B0 = (float2*)mem;
+    float2* B1 = B0 + K * PP;
+    float2* sl = B1 + K * PP;      // the input lines
+    float2* st = sl + K * NF;      // the state lines
+    for (int k1 = pr.b; k1 < pr.e; k1 += pr.s) {
+        const Line ln = line_of(P, tw, k1);
+        float2 *Xr = B0, *Xi = B1;
+        for (int f = pr.f0; f < pr.f1; f++) {
+            for (int j = lane; j < NF / 2; j += kWarp)
+                cp_async16(sl + f * NF + 2 * j, src + (size_t)f * Hs + (size_t)k1 * NF + 2 * j);
+            cp_async_commit();
+            // this warp's half of the line's state
+#pragma unroll
+            for (int a = 0; a < NS; a++)
+                for (int j = lane; j < NF / 4; j += kWarp)
+                    cp_async16(st + a * NF + f * (NF / 2) + 2 * j, sc[a] + (size_t)k1 * NF + f * (NF / 2) + 2 * j);
+            cp_async_commit();
+            cp_async_wait<1>();
+            warp_sync();
+            const int r = fft_lines_fixed_into_padded<-1, float, LOGN, 1>(sl + f * NF, NF, B0 + f * PP, B1 + f * PP, PP, 1,
+                                                                          tw.t32, tw.log, lane);
+            Xr = r ? B1 : B0;
+            Xi = r ? B0 : B1;
+            cp_async_wait<0>();
+        }
+        pair_sync(pr.id);
+        for (int h = pr.f0; h < pr.f1; h++) {
+#pragma unroll
+            for (int i = 0; i < E / 2; i++) {
+                const int k0 = h * (NF / 2) + lane + kWarp * i, pk = pix<true>(k0);
+                float2 sv[NS], in[K], out[K];
+#pragma unroll
+                for (int a = 0; a < NS; a++) sv[a] = st[a * NF + k0];
+#pragma unroll
+                for (int f = 0; f < K; f++) in[f] = Xr[f * PP + pk];
+                ap(ln, k0, sv, in, out);
+#pragma unroll
+                for (int g = 0; g < K; g++) Xi[g * PP + pk] = out[g];
+            }
+        }
+        pair_sync(pr.id);
+        for (int g = pr.f0; g < pr.f1; g++) {
+            const float2* y =
+                (fft_lines_fixed<+1, float, LOGN, 1, true>(Xi + g * PP, Xr + g * PP, PP, 1, tw.t32, tw.log, lane) ? Xr : Xi) +
+                g * PP;
+            float4* d = (float4*)(dst + (size_t)g * Hs + (size_t)k1 * NF);
+            for (int j = lane; j < NF / 2; j += kWarp) {
+                const int q = pix<true>(2 * j);  // 2j and 2j + 1 share a 16-point group
+                d[j] = float4{y[q].x, y[q].y, y[q + 1].x, y[q + 1].y};
+            }
+        }
+        pair_sync(pr.id);
+    }
+}
+
 // ------------------------------------------------------------- FP64 passes
 //
 // The same passes with lines of doubles, transformed in fixed point (fx.cuh).
@@ -2339,12 +2506,19 @@ __device__ __noinline__ void phase_R_staged(const Params& P, const Ctl& c, const
     const float* sp[4] = {(const float*)P.DD[(c.it - 1) & 1], dcur, (const float*)P.VBt, (const float*)P.LBt};
     MaxAbs<float> amax;
     SumOf<float> asum;
-    row_pass_staged<NF, K, NS, SL>(P, tw, src, (float2*)P.NB, sp, smem,
-                                   [&](long long p, int, int, const float* sv, const float* in, float* out) {
-                                       row_point<float, float, PFC>(q, dcur, p, sv[0], sv[1], sv[2],
-                                                                    NS > 3 ? sv[NS > 3 ? 3 : 0] : 0.f, in, out,
-                                                                    amax, asum);
-                                   });
+    auto pt = [&](long long p, int, int, const float* sv, const float* in, float* out) {
+        row_point<float, float, PFC>(q, dcur, p, sv[0], sv[1], sv[2], NS > 3 ? sv[NS > 3 ? 3 : 0] : 0.f, in, out, amax,
+                                     asum);
+    };
+    if constexpr (!PFC && NF % (2 * kWarp) == 0) {
+        if (P.coop && pairs_hold(tw, P.rows / 2)) {
+            row_pass_pair<NF, NS>(P, tw, src, (float2*)P.NB, sp, smem, pt);
+            amax.publish(&P.norms[(size_t)bank * P.nslots + c.ev]);
+            publish_sum(&P.sums[(size_t)bank * P.nslots + c.ev], asum);
+            return;
+        }
+    }
+    row_pass_staged<NF, K, NS, SL>(P, tw, src, (float2*)P.NB, sp, smem, pt);
     amax.publish(&P.norms[(size_t)bank * P.nslots + c.ev]);
     publish_sum(&P.sums[(size_t)bank * P.nslots + c.ev], asum);
 }
@@ -2501,10 +2675,16 @@ __device__ __noinline__ void phase_CI_staged(const Params& P, const Ctl& c, cons
     const ColK<float> q = col_consts<float>(P, c);
     float2* sprev = (float2*)P.SS[(c.it - 1) & 1];
     const float2* sc3[3] = {(const float2*)P.SS[c.it & 1], sprev, (const float2*)P.C0};
-    col_pass_staged<NF, K, 3, SL>(P, tw, csrcT<float>(P), cdstT<float>(P), sc3, smem,
-                                  [&](const Line& k1, int k0, const float2* sv, const float2* in, float2* out) {
-                                      col_point<float, PFC>(P, q, sprev, k1, k0, sv[0], sv[1], sv[2], in, out);
-                                  });
+    auto pt = [&](const Line& k1, int k0, const float2* sv, const float2* in, float2* out) {
+        col_point<float, PFC>(P, q, sprev, k1, k0, sv[0], sv[1], sv[2], in, out);
+    };
+    if constexpr (!PFC && NF % (2 * kWarp) == 0) {
+        if (P.coop && pairs_hold(tw, P.ncols)) {
+            col_pass_pair<NF, 3>(P, tw, csrcT<float>(P), cdstT<float>(P), sc3, smem, pt);
+            return;
+        }
+    }
+    col_pass_staged<NF, K, 3, SL>(P, tw, csrcT<float>(P), cdstT<float>(P), sc3, smem, pt);
 }
 
 template <int L> __device__ __forceinline__ void phase_CI_staged_of(const Params& P, const Ctl& c, const Tw& tw, char* smem) {
