@@ -51,15 +51,17 @@ struct SnoDims {
     int QC, J, JB, R, NT;  // NT: tiles of a sample
 };
 
-// tanh form of GELU (Hendrycks and Gimpel, 2016) and its derivative
-__device__ __forceinline__ float gelu_t(float x) {
-    const float k = 0.7978845608028654f;  // sqrt(2 / pi)
-    return tanhf(k * (x + 0.044715f * x * x * x));
+// tanh form of GELU (Hendrycks and Gimpel, 2016), x (1 + tanh u) / 2 = x sigma(2 u)
+// with the logistic function sigma: no branch, no cancellation for u < 0
+__device__ __forceinline__ float gelu_s(float x) {
+    const float k = 1.5957691216057308f;  // 2 sqrt(2 / pi)
+    return 1.f / (1.f + expf(-k * (x + 0.044715f * x * x * x)));
 }
-__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.f + gelu_t(x)); }
-__device__ __forceinline__ float gelu_grad(float x, float t) {
-    const float k = 0.7978845608028654f;
-    return 0.5f * (1.f + t) + 0.5f * x * (1.f - t * t) * k * (1.f + 3.f * 0.044715f * x * x);
+__device__ __forceinline__ float gelu_f(float x) { return x * gelu_s(x); }
+// its derivative at x, s = gelu_s(x)
+__device__ __forceinline__ float gelu_grad(float x, float s) {
+    const float k = 1.5957691216057308f;
+    return s + x * s * (1.f - s) * k * (1.f + 3.f * 0.044715f * x * x);
 }
 
 __device__ __forceinline__ int k0_of(int m0, int M0, int n0) { return m0 < M0 / 2 ? m0 : n0 - M0 + m0; }
@@ -189,7 +191,7 @@ struct TileArgs {
 // CT: channels rounded up to 16 or 32; MM: kept modes of the last axis to 16
 // or 32.  Dynamic shared memory: tile_smem().
 template <int MODE, int QC, int CT, int MM>
-__global__ void __launch_bounds__(kThr, CT <= 16 ? 2 : 1) k_tile(SnoDims d, TileArgs a) {
+__global__ void __launch_bounds__(kThr, CT <= 16 ? 3 : 1) k_tile(SnoDims d, TileArgs a) {
     constexpr int R = 16 / QC;
     extern __shared__ __align__(16) float sm[];
     float* y = sm;                                  // [C][kPitch]
@@ -267,89 +269,128 @@ __global__ void __launch_bounds__(kThr, CT <= 16 ? 2 : 1) k_tile(SnoDims d, Tile
         for (int c = 0; c <= CT; c++) qacc[c] = 0.f;
     if constexpr (MODE == T_BACK0)
         for (int c = 0; c < CT; c++) pacc[0][c] = pacc[1][c] = pacc[2][c] = 0.f;
+    // PT points of a thread go together where few registers are live (in the
+    // other modes two were slower: layer 150 -> 190 us for 8 states of 512^2)
+    constexpr int PT = MODE == T_LIFT || MODE == T_BACK0 ? 2 : 1;
 #pragma unroll 1
-    for (int s = tid; s < kTile; s += kThr) {
-        const int x0 = x00 + s / (QC * 32), q = (s >> 5) % QC, x1 = j + d.J * q;
-        const bool in = x0 < d.n0 && j < d.J;
-        const size_t p = in ? (size_t)x0 * d.n1 + x1 : 0, ip = (size_t)b * d.np + p;
+    for (int s0 = tid; s0 < kTile; s0 += kThr * PT) {
+        bool in[PT];
+        size_t pp[PT];
+#pragma unroll
+        for (int t = 0; t < PT; t++) {
+            const int s = s0 + kThr * t, x0 = x00 + s / (QC * 32), q = (s >> 5) % QC, x1 = j + d.J * q;
+            in[t] = x0 < d.n0 && j < d.J;
+            pp[t] = in[t] ? (size_t)x0 * d.n1 + x1 : 0;
+        }
         if constexpr (MODE == T_LIFT) {
-            const double u = in ? a.un[ip] : 0.0, um = in ? a.unm1[ip] : 0.0;
-            const float a0 = pagd::to_f32(u), a1 = pagd::to_f32(a.s_in * (u - um));
+            float a0[PT], a1[PT];
+#pragma unroll
+            for (int t = 0; t < PT; t++) {
+                const size_t ip = (size_t)b * d.np + pp[t];
+                const double u = in[t] ? a.un[ip] : 0.0, um = in[t] ? a.unm1[ip] : 0.0;
+                a0[t] = pagd::to_f32(u);
+                a1[t] = pagd::to_f32(a.s_in * (u - um));
+            }
             for (int c = 0; c < d.C; c++) {
-                const float v = in ? a.prm[2 * c] * a0 + a.prm[2 * c + 1] * a1 + a.prm[2 * d.C + c] : 0.f;
-                if (in) a.vout[(bc + c) * d.np + p] = v;
-                y[c * kPitch + s] = v;
+                const float p0 = a.prm[2 * c], p1 = a.prm[2 * c + 1], p2 = a.prm[2 * d.C + c];
+#pragma unroll
+                for (int t = 0; t < PT; t++) {
+                    const float v = in[t] ? p0 * a0[t] + p1 * a1[t] + p2 : 0.f;
+                    if (in[t]) a.vout[(bc + c) * d.np + pp[t]] = v;
+                    y[c * kPitch + s0 + kThr * t] = v;
+                }
             }
         } else {
-            float vin[CT];
+            float vin[PT][CT];
 #pragma unroll
-            for (int c = 0; c < CT; c++) vin[c] = (c < d.C && in) ? a.vin[(bc + c) * d.np + p] : 0.f;
-            float out = 0.f;
-            float tn[MODE == T_LOSS ? CT : 1], zz[MODE == T_LOSS ? CT : 1];
+            for (int t = 0; t < PT; t++)
+#pragma unroll
+                for (int c = 0; c < CT; c++) vin[t][c] = (c < d.C && in[t]) ? a.vin[(bc + c) * d.np + pp[t]] : 0.f;
+            float out[PT];
+            float sg[MODE == T_LOSS ? CT : 1], zz[MODE == T_LOSS ? CT : 1];
+#pragma unroll
+            for (int t = 0; t < PT; t++) out[t] = 0.f;
 #pragma unroll
             for (int o = 0; o < CT; o++) {
                 if (o < d.C) {
-                    float f = sw[CT * CT + o] + y[o * kPitch + s];
+                    float f[PT];
+#pragma unroll
+                    for (int t = 0; t < PT; t++) f[t] = sw[CT * CT + o] + y[o * kPitch + s0 + kThr * t];
 #pragma unroll
                     for (int c = 0; c < CT; c += 4) {
                         const float4 w = *(const float4*)&sw[o * CT + c];
-                        f = fmaf(w.x, vin[c], fmaf(w.y, vin[c + 1], fmaf(w.z, vin[c + 2], fmaf(w.w, vin[c + 3], f))));
+#pragma unroll
+                        for (int t = 0; t < PT; t++)
+                            f[t] = fmaf(w.x, vin[t][c],
+                                        fmaf(w.y, vin[t][c + 1], fmaf(w.z, vin[t][c + 2], fmaf(w.w, vin[t][c + 3], f[t]))));
                     }
-                    const size_t i = (bc + o) * d.np + p;
-                    if constexpr (MODE == T_LAYER) {
-                        const float v = gelu_f(f);
-                        if (in) {
-                            if (a.z) a.z[i] = f;
-                            a.vout[i] = v;
+#pragma unroll
+                    for (int t = 0; t < PT; t++) {
+                        const size_t i = (bc + o) * d.np + pp[t];
+                        float* ys = &y[o * kPitch + s0 + kThr * t];
+                        if constexpr (MODE == T_LAYER) {
+                            const float v = gelu_f(f[t]);
+                            if (in[t]) {
+                                if (a.z) a.z[i] = f[t];
+                                a.vout[i] = v;
+                            }
+                            *ys = in[t] ? v : 0.f;
+                        } else if constexpr (MODE == T_GUESS) {
+                            out[t] = fmaf(a.Q[o], gelu_f(f[t]), out[t]);
+                        } else if constexpr (MODE == T_LOSS) {
+                            sg[o] = gelu_s(f[t]);
+                            zz[o] = f[t];
+                            out[t] = fmaf(a.Q[o], f[t] * sg[o], out[t]);
+                        } else if constexpr (MODE == T_BACK) {
+                            const float z = in[t] ? a.zprev[i] : 0.f;
+                            const float g = f[t] * gelu_grad(z, gelu_s(z));
+                            if (in[t]) a.vout[i] = g;
+                            *ys = in[t] ? g : 0.f;
+                        } else {
+                            *ys = in[t] ? f[t] : 0.f;  // dv_0
                         }
-                        y[o * kPitch + s] = in ? v : 0.f;
-                    } else if constexpr (MODE == T_GUESS) {
-                        out = fmaf(a.Q[o], gelu_f(f), out);
-                    } else if constexpr (MODE == T_LOSS) {
-                        tn[o] = gelu_t(f);
-                        zz[o] = f;
-                        out = fmaf(a.Q[o], 0.5f * f * (1.f + tn[o]), out);
-                    } else if constexpr (MODE == T_BACK) {
-                        const float z = in ? a.zprev[i] : 0.f;
-                        const float g = f * gelu_grad(z, gelu_t(z));
-                        if (in) a.vout[i] = g;
-                        y[o * kPitch + s] = in ? g : 0.f;
-                    } else {
-                        y[o * kPitch + s] = in ? f : 0.f;  // dv_0
                     }
                 }
             }
             if constexpr (MODE == T_GUESS || MODE == T_LOSS) {
-                const float o = out + a.Q[d.C];
-                const double u = in ? a.un[ip] : 0.0, um = in ? a.unm1[ip] : 0.0, ext = fma(a.rho, u - um, u);
-                if constexpr (MODE == T_GUESS) {
-                    if (in) a.guess[ip] = fma(a.s_out, pagd::to_f64(o), ext);
-                } else {
-                    const double e = in ? pagd::to_f64(o) - (a.target[ip] - ext) * a.inv_s_out : 0.0;
-                    lacc = fma(e, e, lacc);
-                    const float g = pagd::to_f32(a.dscale * e);
 #pragma unroll
-                    for (int c = 0; c < CT; c++) {
-                        if (c < d.C) {
-                            qacc[c] = fmaf(g, 0.5f * zz[c] * (1.f + tn[c]), qacc[c]);
-                            const float dz = a.Q[c] * g * gelu_grad(zz[c], tn[c]);
-                            if (in) a.vout[(bc + c) * d.np + p] = dz;
-                            y[c * kPitch + s] = in ? dz : 0.f;
+                for (int t = 0; t < PT; t++) {
+                    const float o = out[t] + a.Q[d.C];
+                    const size_t ip = (size_t)b * d.np + pp[t];
+                    const double u = in[t] ? a.un[ip] : 0.0, um = in[t] ? a.unm1[ip] : 0.0, ext = fma(a.rho, u - um, u);
+                    if constexpr (MODE == T_GUESS) {
+                        if (in[t]) a.guess[ip] = fma(a.s_out, pagd::to_f64(o), ext);
+                    } else {
+                        const double e = in[t] ? pagd::to_f64(o) - (a.target[ip] - ext) * a.inv_s_out : 0.0;
+                        lacc = fma(e, e, lacc);
+                        const float g = pagd::to_f32(a.dscale * e);
+#pragma unroll
+                        for (int c = 0; c < CT; c++) {
+                            if (c < d.C) {
+                                qacc[c] = fmaf(g, zz[c] * sg[c], qacc[c]);
+                                const float dz = a.Q[c] * g * gelu_grad(zz[c], sg[c]);
+                                if (in[t]) a.vout[(bc + c) * d.np + pp[t]] = dz;
+                                y[c * kPitch + s0 + kThr * t] = in[t] ? dz : 0.f;
+                            }
                         }
+                        qacc[CT] += g;
                     }
-                    qacc[CT] += g;
                 }
             }
             if constexpr (MODE == T_BACK0) {
-                const double u = in ? a.un[ip] : 0.0, um = in ? a.unm1[ip] : 0.0;
-                const float a0 = pagd::to_f32(u), a1 = pagd::to_f32(a.s_in * (u - um));
 #pragma unroll
-                for (int c = 0; c < CT; c++) {
-                    if (c < d.C) {
-                        const float g = y[c * kPitch + s];
-                        pacc[0][c] = fmaf(g, a0, pacc[0][c]);
-                        pacc[1][c] = fmaf(g, a1, pacc[1][c]);
-                        pacc[2][c] += g;
+                for (int t = 0; t < PT; t++) {
+                    const size_t ip = (size_t)b * d.np + pp[t];
+                    const double u = in[t] ? a.un[ip] : 0.0, um = in[t] ? a.unm1[ip] : 0.0;
+                    const float a0 = pagd::to_f32(u), a1 = pagd::to_f32(a.s_in * (u - um));
+#pragma unroll
+                    for (int c = 0; c < CT; c++) {
+                        if (c < d.C) {
+                            const float g = y[c * kPitch + s0 + kThr * t];
+                            pacc[0][c] = fmaf(g, a0, pacc[0][c]);
+                            pacc[1][c] = fmaf(g, a1, pacc[1][c]);
+                            pacc[2][c] += g;
+                        }
                     }
                 }
             }
