@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) pagd_batch_kernel(BatchParams 
             const long long cost = G[i + 1] - G[i];
             if (cost == 0) continue;
             const Params& P = B.PI[i];
-            Tw t{tfx, t32, sq, B.logtw, 0, 0, 0, 0};
+            Tw t{tfx, t32, sq, B.logtw, 0, 0, 0, 0, 0, 0, nullptr};
             batch_split(t, gw, nw, total, G[i], cost, phase_units(P, ctl[i].ph), (int)weighted_unit_cost(P, ctl[i]));
             batch_exec<T>(P, ctl[i], t, wsm, red);
         }

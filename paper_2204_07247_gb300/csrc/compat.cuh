@@ -28,6 +28,10 @@ struct alignas(16) longlong2 { long long x, y; };
 
 inline void __syncthreads() {}
 inline void pair_sync(int) {}
+inline double warp_xor(double v, int) { return v; }
+inline unsigned long long warp_xor(unsigned long long v, int) { return v; }
+inline unsigned warp_bcast(unsigned v) { return v; }
+inline void __threadfence_block() {}
 inline void __threadfence() {}
 inline double atomicAdd(double* p, double v) { double o = *p; *p = o + v; return o; }
 inline unsigned atomicAdd(unsigned* p, unsigned v) { unsigned o = *p; *p = o + v; return o; }
@@ -66,7 +70,9 @@ __device__ __forceinline__ unsigned long long dbl_bits(double d) { return (unsig
 __device__ __forceinline__ double bits_dbl(unsigned long long u) { return __longlong_as_double((long long)u); }
 __device__ __forceinline__ unsigned flt_bits(float f) { return __float_as_uint(f); }
 __device__ __forceinline__ float bits_flt(unsigned u) { return __uint_as_float(u); }
-__device__ __forceinline__ float warp_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+template <class T> __device__ __forceinline__ T warp_xor(T v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+// lane 0's value
+__device__ __forceinline__ unsigned warp_bcast(unsigned v) { return __shfl_sync(0xffffffffu, v, 0); }
 // barrier of the two warps of pair p
 __device__ __forceinline__ void pair_sync(int p) { asm volatile("bar.sync %0, 64;" ::"r"(p + 1) : "memory"); }
 #define PAGD_WARP 32

@@ -264,22 +264,21 @@ __device__ __forceinline__ void cta_sync() {
 #endif
 }
 
-template <int R, int S, class T, int LOGN, int LOGNS>
-__device__ __forceinline__ void stage_coop(const cx<T>* src, cx<T>* dst, int pitch, int nl, const cx<T>* tw, int logTw,
-                                           int tid, int nthr) {
+template <int R, int S, class T, bool FIRST>
+__device__ __forceinline__ void stage_coop(const cx<T>* src, cx<T>* dst, int logn, int logNs, int pitch, int nl,
+                                           const cx<T>* tw, int logTw, int tid, int nthr) {
     using C = cx<T>;
     constexpr int LR = (R == 2) ? 1 : (R == 4) ? 2 : 3;
-    constexpr int LNB = LOGN - LR, NB = 1 << LNB, NS = 1 << LOGNS;
-    const int twshift = logTw - (LOGNS + LR), tot = nl << LNB;
+    const int lnb = logn - LR, nsm = (1 << logNs) - 1, twshift = logTw - (logNs + LR), tot = nl << lnb;
 #pragma unroll 1
     for (int it = tid; it < tot; it += nthr) {
-        const int l = it >> LNB, j = it & (NB - 1), jm = j & (NS - 1);
+        const int l = it >> lnb, j = it & ((1 << lnb) - 1), jm = j & nsm;
         const C* s = src + l * pitch;
         C* d = dst + l * pitch;
         C v[R];
 #pragma unroll
-        for (int r = 0; r < R; r++) v[r] = s[j + r * NB];
-        if (LOGNS > 0) {
+        for (int r = 0; r < R; r++) v[r] = s[j + (r << lnb)];
+        if (!FIRST) {
 #pragma unroll
             for (int r = 1; r < R; r++) {
                 C w = tw[(jm * r) << twshift];
@@ -290,51 +289,37 @@ __device__ __forceinline__ void stage_coop(const cx<T>* src, cx<T>* dst, int pit
         dftR<R, S>(v);
         const int idxD = ((j - jm) << LR) + jm;
 #pragma unroll
-        for (int r = 0; r < R; r++) d[idxD + r * NS] = v[r];
-    }
-}
-// radix of a shared line's stage: 4, and 8 for the first stage of an odd
-// number of levels (radix 2, which gives every thread a butterfly, needs twice
-// the barriers and shared-memory round trips and was slower)
-__host__ __device__ constexpr int coop_radix(int logn, int logns) { return logns == 0 && (logn & 1) ? 8 : 4; }
-template <int S, class T, int LOGN, int LOGNS>
-__device__ __forceinline__ int stages_coop(cx<T>* b0, cx<T>* b1, int pitch, int nl, const cx<T>* tw, int logTw, int tid,
-                                           int nthr) {
-    if constexpr (LOGNS < LOGN) {
-        constexpr int R = coop_radix(LOGN, LOGNS);
-        stage_coop<R, S, T, LOGN, LOGNS>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
-        cta_sync();
-        return 1 ^ stages_coop<S, T, LOGN, LOGNS + radix_log(R)>(b1, b0, pitch, nl, tw, logTw, tid, nthr);
-    } else {
-        return 0;
+        for (int r = 0; r < R; r++) d[idxD + (r << logNs)] = v[r];
     }
 }
 
-// nl lines of length 1 << LOGN in b0 (written by any thread before the call)
-// -> result in b0 (returns 0) or b1 (1), visible to every thread on return
-template <int S, class T, int LOGN>
-__device__ __noinline__ int fft_lines_coop(cx<T>* b0, cx<T>* b1, int pitch, int nl, const cx<T>* tw, int logTw, int tid,
-                                           int nthr) {
+// nl lines of length 1 << logn in b0 (written by any thread before the call)
+// -> result in b0 (returns 0) or b1 (1), visible to every thread on return.
+// Radix 4, and 8 for the first stage of an odd number of levels (radix 2, which
+// gives every thread a butterfly, needs twice the barriers and shared-memory
+// round trips and was slower); the stages share their code.
+template <int S, class T>
+__device__ __noinline__ int fft_coop(cx<T>* b0, cx<T>* b1, int logn, int pitch, int nl, const cx<T>* tw, int logTw,
+                                     int tid, int nthr) {
+    cx<T>*s = b0, *d = b1;
+    int logNs = 2, r = 1;
     cta_sync();
-    return stages_coop<S, T, LOGN, 0>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
-}
-
-template <int S, class T, int NF>
-__device__ __forceinline__ int fft_coop(cx<T>* b0, cx<T>* b1, int logn, int pitch, int nl, const cx<T>* tw, int logTw,
-                                        int tid, int nthr) {
-    if constexpr (NF > 0) {
-        return fft_lines_coop<S, T, ilog2c(NF)>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
+    if (logn & 1) {
+        stage_coop<8, S, T, true>(s, d, logn, 0, pitch, nl, tw, logTw, tid, nthr);
+        logNs = 3;
     } else {
-        switch (logn) {
-            case 3: return fft_lines_coop<S, T, 3>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
-            case 4: return fft_lines_coop<S, T, 4>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
-            case 5: return fft_lines_coop<S, T, 5>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
-            case 6: return fft_lines_coop<S, T, 6>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
-            case 7: return fft_lines_coop<S, T, 7>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
-            case 8: return fft_lines_coop<S, T, 8>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
-            default: return fft_lines_coop<S, T, 9>(b0, b1, pitch, nl, tw, logTw, tid, nthr);
-        }
+        stage_coop<4, S, T, true>(s, d, logn, 0, pitch, nl, tw, logTw, tid, nthr);
     }
+    cta_sync();
+#pragma unroll 1
+    for (; logNs < logn; logNs += 2, r ^= 1) {
+        cx<T>* t = s;
+        s = d;
+        d = t;
+        stage_coop<4, S, T, false>(s, d, logn, logNs, pitch, nl, tw, logTw, tid, nthr);
+        cta_sync();
+    }
+    return r;
 }
 
 }  // namespace pagd

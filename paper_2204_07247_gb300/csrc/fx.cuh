@@ -647,7 +647,7 @@ static __device__ __noinline__ void fxc_load_rows(longlong2* b, const double2* s
                                                   unsigned* red, int tid, int nthr) {
     const int n = 1 << logn, half = n >> 1, tot = nl * half, lane = tid % kWarp;
     for (int i0 = tid - lane; i0 < tot; i0 += nthr * 2) {
-        double2 a[2], c[2];
+        double2 a[2], c[2], e[2];
 #pragma unroll
         for (int q = 0; q < 2; q++) {
             const int i = i0 + lane + nthr * q;
@@ -655,6 +655,10 @@ static __device__ __noinline__ void fxc_load_rows(longlong2* b, const double2* s
                 const double2* p = s + (size_t)(i >> (logn - 1)) * H + (size_t)(i & (half - 1)) * rows;
                 a[q] = p[0];
                 c[q] = p[1];
+                if ((i & (half - 1)) == 0) {  // n / 2, with k = 0
+                    p += (size_t)half * rows;
+                    e[q] = double2{p[0].x, p[1].x};
+                }
             }
         }
 #pragma unroll
@@ -667,9 +671,8 @@ static __device__ __noinline__ void fxc_load_rows(longlong2* b, const double2* s
                 if (in) {
                     int k2 = n - k;
                     if (k == 0) {  // k = 0 and n / 2: real coefficients
-                        const double2* p = s + (size_t)l * H + (size_t)half * rows;
                         a[q].y = c[q].x;
-                        c[q] = double2{p[0].x, p[1].x};
+                        c[q] = e[q];
                         k2 = half;
                     }
                     const unsigned h0 = fx_hi(a[q].x), h1 = fx_hi(a[q].y), h2 = fx_hi(c[q].x), h3 = fx_hi(c[q].y);
@@ -707,52 +710,65 @@ static __device__ __noinline__ void fxc_convert_rows(longlong2* b, int nl, int l
 __device__ __forceinline__ int fxc_scale(const unsigned* red, const unsigned* sums, int l) {
     return fx_scale(fx_emax(red[l]), fx_shift(sums[l]));
 }
-// transformed lines -> memory
-static __device__ __noinline__ void fxc_store(const longlong2* b, double2* d, long long H, int nl, int logn,
-                                              const unsigned* red, const unsigned* sums, int tid, int nthr) {
+// transformed lines -> memory (FAST as fx_to_t)
+__device__ __forceinline__ bool fxc_fast(const unsigned* red, const unsigned* sums, int nl) {
+    bool fast = true;
+    for (int l = 0; l < nl; l++) fast = fast && fx_fast(fxc_scale(red, sums, l)) && fx_fast(fxc_scale(red, sums, l) + 1);
+    return fast;
+}
+template <bool FAST>
+__device__ __noinline__ void fxc_store_t(const longlong2* b, double2* d, long long H, int nl, int logn, const unsigned* red,
+                                         const unsigned* sums, int tid, int nthr) {
     const int n = 1 << logn, tot = nl << logn;
-#pragma unroll 2
+#pragma unroll 1
     for (int i = tid; i < tot; i += nthr) {
         const int l = i >> logn, x = i & (n - 1), S = fxc_scale(red, sums, l);
         const longlong2 z = b[(l << logn) + fxs(x)];
-        d[(size_t)l * H + x] = fx_fast(S) ? double2{fx_to_t<true>(z.x, S), fx_to_t<true>(z.y, S)}
-                                          : double2{fx_to(z.x, S), fx_to(z.y, S)};
+        d[(size_t)l * H + x] = double2{fx_to_t<FAST>(z.x, S), fx_to_t<FAST>(z.y, S)};
     }
 }
-static __device__ __noinline__ void fxc_store_rows(const longlong2* b, double2* d0, long long H, int rows, int nl, int logn,
-                                                   const unsigned* red, const unsigned* sums, int tid, int nthr) {
+__device__ __forceinline__ void fxc_store(const longlong2* b, double2* d, long long H, int nl, int logn,
+                                          const unsigned* red, const unsigned* sums, int tid, int nthr) {
+    if (fxc_fast(red, sums, nl)) fxc_store_t<true>(b, d, H, nl, logn, red, sums, tid, nthr);
+    else fxc_store_t<false>(b, d, H, nl, logn, red, sums, tid, nthr);
+}
+template <bool FAST>
+__device__ __noinline__ void fxc_store_rows_t(const longlong2* b, double2* d0, long long H, int rows, int nl, int logn,
+                                              const unsigned* red, const unsigned* sums, int tid, int nthr) {
     const int n = 1 << logn, half = n >> 1, tot = nl * half;
     // coefficients k < n / 2, then n / 2 of every line
+#pragma unroll 1
     for (int i = tid; i < tot + nl; i += nthr) {
         const int l = i < tot ? i >> (logn - 1) : i - tot, k = i < tot ? i & (half - 1) : half, S = fxc_scale(red, sums, l) + 1;
         const longlong2 zk = b[l * n + fxs(k)], zn = b[l * n + fxs((n - k) & (n - 1))];
-        const longlong2 A{zk.x + zn.x, zk.y - zn.y}, B{zk.y + zn.y, zn.x - zk.x};
         double2* d = d0 + (size_t)l * H + (size_t)k * rows;
-        if (fx_fast(S)) {
-            d[0] = double2{fx_to_t<true>(A.x, S), fx_to_t<true>(A.y, S)};
-            d[1] = double2{fx_to_t<true>(B.x, S), fx_to_t<true>(B.y, S)};
-        } else {
-            d[0] = double2{fx_to(A.x, S), fx_to(A.y, S)};
-            d[1] = double2{fx_to(B.x, S), fx_to(B.y, S)};
-        }
+        d[0] = double2{fx_to_t<FAST>(zk.x + zn.x, S), fx_to_t<FAST>(zk.y - zn.y, S)};
+        d[1] = double2{fx_to_t<FAST>(zk.y + zn.y, S), fx_to_t<FAST>(zn.x - zk.x, S)};
     }
 }
+__device__ __forceinline__ void fxc_store_rows(const longlong2* b, double2* d0, long long H, int rows, int nl, int logn,
+                                               const unsigned* red, const unsigned* sums, int tid, int nthr) {
+    if (fxc_fast(red, sums, nl)) fxc_store_rows_t<true>(b, d0, H, rows, nl, logn, red, sums, tid, nthr);
+    else fxc_store_rows_t<false>(b, d0, H, rows, nl, logn, red, sums, tid, nthr);
+}
 
-template <int R, int S, int LOGN, int LOGNS>
-__device__ __forceinline__ void fx_stage_coop(const longlong2* src, longlong2* dst, int nl, const unsigned* sums,
-                                              const FxTw* tw, int logTw, int tid, int nthr) {
+// One radix-R stage at runtime lengths: the stages of a line share their code.
+// (A unit runs each instruction of a pass a few times only: an SM missed 390
+// times per phase in its instruction cache with a copy per stage and length.)
+template <int R, int S, bool FIRST>
+__device__ __forceinline__ void fx_stage_coop(const longlong2* src, longlong2* dst, int logn, int logNs, int nl,
+                                              const unsigned* sums, const FxTw* tw, int logTw, int tid, int nthr) {
     constexpr int LR = (R == 2) ? 1 : (R == 4) ? 2 : 3;
-    constexpr int LNB = LOGN - LR, NB = 1 << LNB, NS = 1 << LOGNS;
-    const int twshift = logTw - (LOGNS + LR), tot = nl << LNB;
+    const int lnb = logn - LR, nsm = (1 << logNs) - 1, twshift = logTw - (logNs + LR), tot = nl << lnb;
 #pragma unroll 1
     for (int it = tid; it < tot; it += nthr) {
-        const int l = it >> LNB, j = it & (NB - 1), jm = j & (NS - 1);
-        const longlong2* s = src + (l << LOGN);
-        longlong2* d = dst + (l << LOGN);
+        const int l = it >> lnb, j = it & ((1 << lnb) - 1), jm = j & nsm;
+        const longlong2* s = src + (l << logn);
+        longlong2* d = dst + (l << logn);
         longlong2 v[R];
 #pragma unroll
-        for (int r = 0; r < R; r++) v[r] = s[fxs(j + r * NB)];
-        if (LOGNS == 0) {
+        for (int r = 0; r < R; r++) v[r] = s[fxs(j + (r << lnb))];
+        if (FIRST) {
             const int sh = fx_shift(sums[l]);
             const long long half = fx_half(sh);
 #pragma unroll
@@ -764,50 +780,68 @@ __device__ __forceinline__ void fx_stage_coop(const longlong2* src, longlong2* d
         fx_dft<R, S>(v);
         const int dd = ((j - jm) << LR) + jm;
 #pragma unroll
-        for (int r = 0; r < R; r++) d[fxs(dd + (r << LOGNS))] = v[r];
+        for (int r = 0; r < R; r++) d[fxs(dd + (r << logNs))] = v[r];
     }
 }
-template <int S, int LOGN, int LOGNS>
-__device__ __forceinline__ int fx_stages_coop(longlong2* b0, longlong2* b1, int nl, const unsigned* sums, const FxTw* tw,
-                                              int logTw, int tid, int nthr) {
-    if constexpr (LOGNS < LOGN) {
-        constexpr int R = coop_radix(LOGN, LOGNS);
-        fx_stage_coop<R, S, LOGN, LOGNS>(b0, b1, nl, sums, tw, logTw, tid, nthr);
-        cta_sync();
-        return 1 ^ fx_stages_coop<S, LOGN, LOGNS + radix_log(R)>(b1, b0, nl, sums, tw, logTw, tid, nthr);
-    } else {
-        return 0;
+#ifndef PAGD_EMU
+__device__ __forceinline__ longlong2 fx_xor(longlong2 v, int o) {
+    return longlong2{__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)};
+}
+// A radix-4 stage with twiddles, a point per thread: four lanes share a
+// butterfly, each one input's complex product, and combine by shuffles.  For
+// lines of up to 64 points, which otherwise keep half a warp busy: 64 points
+// 2050 -> 1600 cycles, 128 the same, 256 slower (2800 -> 3000).
+template <int S>
+__device__ __forceinline__ void fx_stage_quad(const longlong2* src, longlong2* dst, int logn, int logNs, int nl,
+                                              const FxTw* tw, int logTw, int tid, int nthr) {
+    const int lnb = logn - 2, twshift = logTw - (logNs + 2), tot = nl << logn;
+#pragma unroll 1
+    for (int i0 = tid & ~31; i0 < tot; i0 += nthr) {  // whole warps: nl << logn may end inside one
+        const int it = i0 + (tid & 31), on = it < tot ? it : 0;
+        const int l = on >> logn, j = (on & ((1 << logn) - 1)) >> 2, r = on & 3, jm = j & ((1 << logNs) - 1);
+        longlong2 v = fx_cmul<S>(src[(l << logn) + fxs(j + (r << lnb))], tw[(jm * r) << twshift]);
+        longlong2 o = fx_xor(v, 2);
+        v = r < 2 ? cadd(v, o) : csub(o, v);       // p0 + p2, p1 + p3, p0 - p2, p1 - p3
+        if (r == 3) v = mul_si<S>(v);
+        o = fx_xor(v, 1);
+        v = (r & 1) ? csub(o, v) : cadd(v, o);     // outputs 0, 2, 1, 3
+        const int k = (r >> 1) | ((r & 1) << 1);
+        if (it < tot) dst[(l << logn) + fxs(((j - jm) << 2) + jm + (k << logNs))] = v;
     }
 }
+#endif
 
-// nl converted lines of 1 << LOGN points in b0 (sums complete before the call)
+// nl converted lines of 1 << logn points in b0 (sums complete before the call)
 // -> the transforms in b0 (returns 0) or b1 (1), visible to every thread on
-// return.  Radix 4: a stage costs a barrier and a round trip through shared
-// memory; a lone warp on a sub-partition issues a product in about 30 cycles,
-// and wider radices leave more of them idle.
-template <int S, int LOGN>
-__device__ __noinline__ int fx_lines_coop(longlong2* b0, longlong2* b1, int nl, const unsigned* sums, const FxTw* tw,
-                                          int logTw, int tid, int nthr) {
-    return fx_stages_coop<S, LOGN, 0>(b0, b1, nl, sums, tw, logTw, tid, nthr);
-}
-
-// NF: the line length, or 0 for the runtime length 1 << logn (8 .. 512)
-template <int S, int NF>
-__device__ __forceinline__ int fx_coop(longlong2* b0, longlong2* b1, int logn, int nl, const unsigned* sums, const FxTw* tw,
-                                       int logTw, int tid, int nthr) {
-    if constexpr (NF > 0) {
-        return fx_lines_coop<S, ilog2c(NF)>(b0, b1, nl, sums, tw, logTw, tid, nthr);
+// return.  Radix 4, and 8 for the first stage of an odd number of levels: a
+// stage costs a barrier and a round trip through shared memory; a lone warp on
+// a sub-partition issues a product in about 30 cycles, and wider radices leave
+// more of them idle.
+template <int S>
+__device__ __noinline__ int fx_coop(longlong2* b0, longlong2* b1, int logn, int nl, const unsigned* sums, const FxTw* tw,
+                                    int logTw, int tid, int nthr) {
+    longlong2 *s = b0, *d = b1;
+    int logNs = 2, r = 1;
+    if (logn & 1) {
+        fx_stage_coop<8, S, true>(s, d, logn, 0, nl, sums, tw, logTw, tid, nthr);
+        logNs = 3;
     } else {
-        switch (logn) {
-            case 3: return fx_lines_coop<S, 3>(b0, b1, nl, sums, tw, logTw, tid, nthr);
-            case 4: return fx_lines_coop<S, 4>(b0, b1, nl, sums, tw, logTw, tid, nthr);
-            case 5: return fx_lines_coop<S, 5>(b0, b1, nl, sums, tw, logTw, tid, nthr);
-            case 6: return fx_lines_coop<S, 6>(b0, b1, nl, sums, tw, logTw, tid, nthr);
-            case 7: return fx_lines_coop<S, 7>(b0, b1, nl, sums, tw, logTw, tid, nthr);
-            case 8: return fx_lines_coop<S, 8>(b0, b1, nl, sums, tw, logTw, tid, nthr);
-            default: return fx_lines_coop<S, 9>(b0, b1, nl, sums, tw, logTw, tid, nthr);
-        }
+        fx_stage_coop<4, S, true>(s, d, logn, 0, nl, sums, tw, logTw, tid, nthr);
     }
+    cta_sync();
+#pragma unroll 1
+    for (; logNs < logn; logNs += 2, r ^= 1) {
+        longlong2* t = s;
+        s = d;
+        d = t;
+#ifndef PAGD_EMU
+        if (logn <= 6 && (nl << logn) <= nthr) fx_stage_quad<S>(s, d, logn, logNs, nl, tw, logTw, tid, nthr);
+        else
+#endif
+            fx_stage_coop<4, S, false>(s, d, logn, logNs, nl, sums, tw, logTw, tid, nthr);
+        cta_sync();
+    }
+    return r;
 }
 
 }  // namespace pagd

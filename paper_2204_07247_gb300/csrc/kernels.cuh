@@ -64,6 +64,7 @@ template <class T, int NF>
 __global__ void __launch_bounds__(kMaxThreads, kMaxCtas) pagd_kernel(const __grid_constant__ Params P) {
     extern __shared__ __align__(16) char smem[];
     __shared__ double red[32];
+    __shared__ CtaRed cr;
     // twiddles exp(-2 pi i m / 2^logtw) staged from the global table
     const int ntw = 1 << P.logtw;
     FxTw* tfx = (FxTw*)smem;
@@ -77,8 +78,9 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxCtas) pagd_kernel(const __gri
     for (int m = threadIdx.x; m < kSq; m += blockDim.x) sq[m] = (double)(m * m);
     __syncthreads();
     const int wpb = blockDim.x / kWarp;
-    const Tw tw{tfx, t32, sq, P.logtw, (int)(threadIdx.x / kWarp) * (int)gridDim.x + (int)blockIdx.x,
-                (int)gridDim.x * wpb, 0, -1};
+    const int wr = (int)(threadIdx.x / kWarp) * (int)gridDim.x + (int)blockIdx.x, wn = (int)gridDim.x * wpb;
+    const Tw tw{tfx, t32, sq, P.logtw, wr, wn, 0, -1, P.one && threadIdx.x >= kWarp ? kIdleRank : wr,
+                P.one ? (int)gridDim.x : wn, &cr};
     char* wsm = smem + tw_smem_bytes(P.logtw);
     // The control state is the same in every thread: it lives in shared memory
     // and thread 0 advances it between two CTA barriers, which keeps its ~40
@@ -87,6 +89,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxCtas) pagd_kernel(const __gri
     unsigned gen = 0;
     int ntr = 0;
     if (threadIdx.x == 0) {
+        cr.count = 0u;
         c = ctl_init(P);
         if (P.trace && blockIdx.x == 0) {
             P.trace[0] = (unsigned long long)PH_DONE;  // start marker
@@ -117,7 +120,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxCtas) pagd_kernel(const __gri
                 unsigned* dst = (unsigned*)&c;
                 for (int i = 0; i < (int)(sizeof(Ctl) / sizeof(unsigned)); i++) dst[i] = __ldcg(src + i);
             }
-            ctl_advance<T>(P, c);
+            if (cl_phase || !ctl_fast<T>(P, c)) ctl_advance<T>(P, c);
         }
         __syncthreads();
     }

@@ -36,7 +36,7 @@ thread_local EmuDim3 threadIdx{0, 0, 0}, blockIdx{0, 0, 0}, blockDim{1, 1, 1}, g
 
 constexpr int kMaxChunk = 4096;
 constexpr size_t kMaxSmem = 227 * 1024;  // dynamic shared memory per CTA on sm_103a
-constexpr size_t kMaxSmem2 = 113 * 1024 - 2048;  // per CTA with two on an SM (1 KB reserved and up to 1 KB static each)
+constexpr size_t kMaxSmem2 = 113 * 1024 - 1024;  // per CTA with two on an SM (1 KB reserved, up to 1 KB static each)
 constexpr int kMaxBatch = 4096;
 constexpr int kTraceCap = 8192;  // phase records kept per launch when tracing
 // FP32-mixed: steps between exact FP64 recomputations of the reference spectra
@@ -56,7 +56,7 @@ struct pagd_solver {
     size_t ws_bytes;
     char* ws;
     // launch plan (grid_used: the grid of the last launch)
-    int grid, logtw, threads, coop, cl, stage, coop32, grid_used;
+    int grid, logtw, threads, coop, one, cl, stage, coop32, grid_used;
     size_t smem, warp_bytes;
     // state
     int have_state, step, cur, trace, ref_valid;
@@ -154,6 +154,7 @@ static Params params_for(const pagd_solver* s, char* w) {
     P.inv_npts = 1.0 / (double)s->npts;
     P.warp_bytes = (long long)s->warp_bytes;
     P.coop = s->coop;
+    P.one = s->one;
     P.stage = s->stage;
     P.coop32 = s->coop32;
     const double twopi = 6.283185307179586476925286766559;
@@ -276,7 +277,7 @@ template <class T> static pagd_status launch(pagd_solver* s, const Params& P) {
     }
     double* sq = (double*)(t32 + ntw);
     for (int m = 0; m < kSq; m++) sq[m] = (double)(m * m);
-    Tw tw{tfx, t32, sq, P.logtw, 0, s->grid, 0, -1};
+    Tw tw{tfx, t32, sq, P.logtw, 0, s->grid, 0, -1, 0, s->grid, nullptr};
     char* wsm = base + tw_smem_bytes(P.logtw);
     Ctl c = ctl_init(P);
     const int nf = fixed_len(P.n0, P.n1);
@@ -294,7 +295,7 @@ template <class T> static pagd_status launch(pagd_solver* s, const Params& P) {
         }
         for (int b = 0; b < s->grid; b++) {
             blockIdx.x = (unsigned)b;
-            tw.wr = b;
+            tw.wr = tw.ur = b;
             switch (nf) {
                 case 64: exec_phase<T, 64>(P, c, tw, wsm, red); break;
                 case 128: exec_phase<T, 128>(P, c, tw, wsm, red); break;
@@ -445,6 +446,19 @@ static void make_plan(pagd_solver* s) {
             if (nf == 256) s->coop = 0;
         }
     }
+    // A 2D grid with more units than SMs but at most twice as many (512^2: 256
+    // row units, 257 columns): a CTA per unit, two on an SM, instead of two
+    // rounds of one; a CTA then needs shared memory for one unit only.
+    s->one = 0;
+#ifndef PAGD_EMU
+    const size_t one_need = std::max(coop_need, tws + s->warp_bytes);
+    if (s->coop && !s->cl && s->dim == 2 && units > sms && units <= (long long)kMaxCtas * sms && one_need <= kMaxSmem2) {
+        s->one = 1;
+        s->grid = (int)units;
+        s->threads = kMaxThreads;
+        s->smem = one_need;
+    }
+#endif
     s->stage = (!s->cl && stage_fits(s, s->warp_bytes)) ? 1 : 0;
     // FP32 iteration passes with CTA-cooperative units (unstaged FP32 passes
     // of fixed line length): opt-in with PAGD_COOP32=1.  Measured slower on
@@ -1265,7 +1279,7 @@ template <class T> static pagd_status batch_launch(pagd_batch* b, const BatchPar
                 for (int i = 0; i < B.count; i++) {
                     if (G[i + 1] <= clo || G[i] >= chi || G[i + 1] == G[i]) continue;
                     const Params& P = B.PI[i];
-                    Tw t{tfx, t32, sq, B.logtw, 0, 0, 0, 0};
+                    Tw t{tfx, t32, sq, B.logtw, 0, 0, 0, 0, 0, 0, nullptr};
                     batch_split(t, gw, nw, total, G[i], G[i + 1] - G[i], phase_units(P, ctl[i].ph),
                                 (int)weighted_unit_cost(P, ctl[i]));
                     batch_exec_host<T>(P, ctl[i], t, wsm, red);

@@ -109,6 +109,9 @@ struct Params {
     int stage;
     // PROG_PASS: the iteration pass it repeats (PH_RI, PH_CI, PH_MF, PH_MI)
     int pass;
+    // one warp (FCH: pair) per CTA owns units, and only it has a slice of shared
+    // memory (grids whose CTAs have one unit each, two CTAs per SM)
+    int one;
     // the FP32 iteration passes run CTA-cooperative units (phase_R_coop /
     // phase_CI_coop; opt-in, single-instance launches, unstaged passes)
     int coop32;
@@ -199,6 +202,7 @@ struct Ctl {
     int acc, acc_cur, acc_it, acc_lastev, acc_ev, reb, ereb, inc, ref_ok, exact_done;
     double resid, base_nrm, best_nrm, acc_resid;
     Beta bt;             // averaged Newton constants of the current evaluation
+    double reb_nrm;      // kRebaseRatio base_nrm
 };
 
 // FP32 iterations stop improving once ||d|| reaches about 1e-7 of the FP64
@@ -206,6 +210,13 @@ struct Ctl {
 // before that floor is reached.
 constexpr double kRebaseRatio = 1.0e-6;
 constexpr int kStagnation = 12;
+
+// one slot per warp of a CTA (publish_group)
+struct CtaRed {
+    double v[3][8];
+    unsigned long long m[8];
+    unsigned count;
+};
 
 // Per-thread pass context: the twiddle tables exp(-2 pi i m / (1 << log))
 // staged in shared memory, and how the work of the current phase of one
@@ -220,13 +231,15 @@ struct Tw {
     const double* sq;      // squares 0 .. kSq - 1
     int log;
     int wr, wn, ulo, uhi;
+    int ur, un;  // rank and number of the warps that own units (round robin)
+    CtaRed* cr;  // the CTA's reduction slots (null: every warp publishes by itself)
 };
 
 struct URange {
     int b, e, s;
 };
 __device__ __forceinline__ URange units_of(const Tw& t, int units) {
-    if (t.uhi < 0) return URange{t.wr, units, t.wn};
+    if (t.uhi < 0) return URange{t.ur, units, t.un};
     return URange{t.ulo, t.uhi < units ? t.uhi : units, 1};
 }
 // the one thread of the instance's warps that writes per-instance scalars
@@ -357,13 +370,63 @@ __device__ __forceinline__ double nanmax(double a, double b) { return (b > a || 
 // Grid-wide reductions: every warp reduces its lanes with shuffles and lane 0
 // publishes the partial with an atomic, so no CTA-wide barrier is needed
 // inside a phase (warps of a CTA never wait for each other's units).
+// (Adding nothing is left out: atomics of all warps on one address follow each
+// other at the L2, about 2 ns each.)
+__device__ __forceinline__ void add_nonzero(double* a, double v) {
+    if (dbl_bits(v) << 1) atomicAdd(a, v);
+}
 __device__ __forceinline__ void publish_sum(double* a, double v) {
     v = warp_sum(v);
-    if ((threadIdx.x % kWarp) == 0) atomicAdd(a, v);
+    if ((threadIdx.x % kWarp) == 0) add_nonzero(a, v);
 }
-__device__ __forceinline__ void publish_sum(double* a, const Sum2& v) {
-    const double t = v.warp_total();
-    if ((threadIdx.x % kWarp) == 0) atomicAdd(a, t);
+// A phase's maximum and sums of this warp (the same in every lane) into global
+// memory.  Where the launch has slots for it, the warps of a CTA leave theirs
+// in shared memory and the last one to come publishes for all (no barrier): of
+// 1032 atomics on one address in a phase of a 256^2 grid, 129 are left.
+// all: every warp of the CTA publishes in this phase and may have a share.
+constexpr unsigned kFewCtas = 64;  // so few CTAs' atomics cost less than the meeting (PFC 64^2, 33 CTAs: 0.3 us)
+template <int N>
+__device__ __forceinline__ void publish_group(const Tw& tw, bool all, unsigned long long* ma, unsigned long long m,
+                                              double* const (&a)[N], const double (&v)[N]) {
+    const int lane = threadIdx.x % kWarp;
+    if (!all || !tw.cr || gridDim.x <= kFewCtas) {
+        if (lane == 0) {
+            if (m) atomicMax(ma, m);
+#pragma unroll
+            for (int i = 0; i < N; i++) add_nonzero(a[i], v[i]);
+        }
+        return;
+    }
+    CtaRed* cr = tw.cr;
+    const unsigned w = threadIdx.x / kWarp, nw = blockDim.x / kWarp;
+    unsigned last = 0;
+    if (lane == 0) {
+        cr->m[w] = m;
+#pragma unroll
+        for (int i = 0; i < N; i++) cr->v[i][w] = v[i];
+        __threadfence_block();
+        last = atomicAdd(&cr->count, 1u) == nw - 1 ? 1u : 0u;
+        __threadfence_block();
+    }
+    if (!warp_bcast(last)) return;
+    const bool in = (unsigned)lane < nw;
+    unsigned long long mt = in ? cr->m[lane] : 0ull;
+    double t[N];
+#pragma unroll
+    for (int i = 0; i < N; i++) t[i] = in ? cr->v[i][lane] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        const unsigned long long u = warp_xor(mt, o);
+        mt = u > mt ? u : mt;
+#pragma unroll
+        for (int i = 0; i < N; i++) t[i] += warp_xor(t[i], o);
+    }
+    if (lane == 0) {
+        cr->count = 0u;
+        if (mt) atomicMax(ma, mt);
+#pragma unroll
+        for (int i = 0; i < N; i++) add_nonzero(a[i], t[i]);
+    }
 }
 // Running maximum of |x| on the bit patterns: non-negative floating-point
 // numbers compare as integers, a NaN above all of them (an FP64 compare issues
@@ -375,10 +438,8 @@ template <> struct MaxAbs<float> {
         const unsigned b = flt_bits(x) & 0x7fffffffu;
         m = b > m ? b : m;
     }
-    __device__ __forceinline__ void publish(unsigned long long* a) const {
-        const unsigned v = warp_umax(m);
-        if ((threadIdx.x % kWarp) == 0) atomicMax(a, dbl_bits(to_f64(bits_flt(v))));
-    }
+    // the FP64 bits of the warp's maximum
+    __device__ __forceinline__ unsigned long long warp_bits() const { return dbl_bits(to_f64(bits_flt(warp_umax(m)))); }
 };
 template <> struct MaxAbs<double> {
     unsigned long long m = 0ull;
@@ -386,10 +447,10 @@ template <> struct MaxAbs<double> {
         const unsigned long long b = dbl_bits(x) & 0x7fffffffffffffffull;
         m = b > m ? b : m;
     }
-    __device__ __forceinline__ void publish(unsigned long long* a) const {
+    __device__ __forceinline__ unsigned long long warp_bits() const {
         const unsigned h = warp_umax((unsigned)(m >> 32));
         const unsigned l = warp_umax((unsigned)(m >> 32) == h ? (unsigned)m : 0u);
-        if ((threadIdx.x % kWarp) == 0) atomicMax(a, ((unsigned long long)h << 32) | l);
+        return ((unsigned long long)h << 32) | l;
     }
 };
 // sum of T values: FP64 as they are, FP32 by Sum2
@@ -398,8 +459,16 @@ template <> struct SumOf<float> : Sum2 {};
 template <> struct SumOf<double> {
     double v = 0.0;
     __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ double warp_total() const { return warp_sum(v); }
 };
-__device__ __forceinline__ void publish_sum(double* a, const SumOf<double>& v) { publish_sum(a, v.v); }
+// the norm and the sum of a row pass's evaluation
+template <class TI, class T>
+__device__ __forceinline__ void publish_eval(const Params& P, const Tw& tw, bool all, int bank, int ev,
+                                             const MaxAbs<TI>& amax, const SumOf<T>& asum) {
+    double* const a[1] = {&P.sums[(size_t)bank * P.nslots + ev]};
+    const double v[1] = {asum.warp_total()};
+    publish_group<1>(tw, all, &P.norms[(size_t)bank * P.nslots + ev], amax.warp_bits(), a, v);
+}
 
 // ---------------------------------------------------------- pass templates
 
@@ -1033,21 +1102,21 @@ __device__ void col_pass_staged(const Params& P, const Tw& tw, const float2* src
 struct Pair {
     int id, f0, f1, b, e, s;  // pair of the CTA, this warp's parts [f0, f1), its units
 };
-__device__ __forceinline__ Pair pair_of(const Tw& tw, int units) {
+__device__ __forceinline__ Pair pair_of(const Params& P, const Tw& tw, int units) {
 #ifdef PAGD_EMU
     return Pair{0, 0, 2, tw.wr, units, tw.wn};
 #else
-    const int w = threadIdx.x / kWarp, np = blockDim.x / (2 * kWarp);
+    const int w = threadIdx.x / kWarp, np = P.one ? 1 : blockDim.x / (2 * kWarp);
     return Pair{w >> 1, w & 1, (w & 1) + 1, (w >> 1) * (int)gridDim.x + (int)blockIdx.x, (w >> 1) < np ? units : 0,
                 np * (int)gridDim.x};
 #endif
 }
 // whether the launch's pairs hold every unit at once
-__device__ __forceinline__ bool pairs_hold(const Tw& tw, int units) {
+__device__ __forceinline__ bool pairs_hold(const Params& P, int units) {
 #ifdef PAGD_EMU
     return units > 0;
 #else
-    return units <= (int)(blockDim.x / (2 * kWarp)) * (int)gridDim.x;
+    return P.one || units <= (int)(blockDim.x / (2 * kWarp)) * (int)gridDim.x;
 #endif
 }
 
@@ -1057,7 +1126,7 @@ __device__ void row_pass_pair(const Params& P, const Tw& tw, const float2* src, 
     constexpr int LOGN = ilog2c(NF), HALF = NF / 2, H1 = HALF + 1, PP = padded_len(NF), E = NF / kWarp, K = 2;
     const int rows = P.rows, lane = threadIdx.x % kWarp;
     const long long Hs = P.H;
-    const Pair pr = pair_of(tw, rows / 2);
+    const Pair pr = pair_of(P, tw, rows / 2);
     char* mem = smem + (size_t)(2 * pr.id) * P.warp_bytes;
     float2* X0 = (float2*)mem;
     float2* X1 = X0 + K * PP;
@@ -1130,7 +1199,7 @@ __device__ void col_pass_pair(const Params& P, const Tw& tw, const float2* src, 
     constexpr int LOGN = ilog2c(NF), PP = padded_len(NF), E = NF / kWarp, K = 2;
     const int lane = threadIdx.x % kWarp;
     const long long Hs = P.H;
-    const Pair pr = pair_of(tw, P.ncols);
+    const Pair pr = pair_of(P, tw, P.ncols);
     char* mem = smem + (size_t)(2 * pr.id) * P.warp_bytes;
     float2* B0 = (float2*)mem;
     float2* B1 = B0 + K * PP;
@@ -1378,12 +1447,10 @@ __device__ void row_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
         const int r0 = 2 * u;
         for (int i = tid; i < 4 * kMaxK; i += nthr) red[i] = 0u;
         // the first points' state, in flight during the inverse transforms
-        S st[kCoopChunk];
-#pragma unroll
-        for (int c = 0; c < kCoopChunk; c++) {
-            const int q = tid + nthr * c;
-            if (q < 2 * n) st[c] = ld((long long)(r0 + (q >> logn)) * n + (q & (n - 1)), r0 + (q >> logn), q & (n - 1));
-        }
+        auto ldq = [&](int q) {
+            return ld((long long)(r0 + (q >> logn)) * n + (q & (n - 1)), r0 + (q >> logn), q & (n - 1));
+        };
+        S cur = ldq(tid < 2 * n ? tid : 0);
         cta_sync();
         longlong2* X = B0;
         int sc[kMaxK] = {0, 0, 0};
@@ -1392,7 +1459,7 @@ __device__ void row_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
             cta_sync();
             fxc_convert_rows(B0, kin, logn, red, red + kMaxK, tid, nthr);
             cta_sync();
-            X = fx_coop<+1, NF>(B0, B1, logn, kin, red + kMaxK, tw.tfx, tw.log, tid, nthr) ? B1 : B0;
+            X = fx_coop<+1>(B0, B1, logn, kin, red + kMaxK, tw.tfx, tw.log, tid, nthr) ? B1 : B0;
 #pragma unroll
             for (int f = 0; f < kMaxK; f++)
                 if (f < kin) sc[f] = fxc_scale(red, red + kMaxK, f) + log_npts(P);
@@ -1400,34 +1467,23 @@ __device__ void row_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
         // pointwise: point q = rr n + x of the unit; the outputs replace the
         // inputs of the same point and row
         unsigned hi[kMaxK] = {0u, 0u, 0u};
-        for (int q0 = 0; q0 < 2 * n; q0 += nthr * kCoopChunk) {
-            if (q0 > 0) {
+#pragma unroll 1
+        for (int q = tid; q < 2 * n; q += nthr) {
+            const S st = cur;
+            if (q + nthr < 2 * n) cur = ldq(q + nthr);
+            const int rr = q >> logn, x = q & (n - 1);
+            long long* slot = (long long*)(X + fxs(x)) + rr;
+            double in[kMaxK], out[kMaxK];
 #pragma unroll
-                for (int c = 0; c < kCoopChunk; c++) {
-                    const int q = q0 + tid + nthr * c;
-                    if (q < 2 * n)
-                        st[c] = ld((long long)(r0 + (q >> logn)) * n + (q & (n - 1)), r0 + (q >> logn), q & (n - 1));
-                }
-            }
+            for (int f = 0; f < kMaxK; f++)
+                if (f < kin) in[f] = fx_to(slot[f * 2 * n], sc[f]);
+            ap((long long)(r0 + rr) * n + x, r0 + rr, x, st, in, out);
 #pragma unroll
-            for (int c = 0; c < kCoopChunk; c++) {
-                const int q = q0 + tid + nthr * c;
-                if (q < 2 * n) {
-                    const int rr = q >> logn, x = q & (n - 1);
-                    long long* slot = (long long*)(X + fxs(x)) + rr;
-                    double in[kMaxK], out[kMaxK];
-#pragma unroll
-                    for (int f = 0; f < kMaxK; f++)
-                        if (f < kin) in[f] = fx_to(slot[f * 2 * n], sc[f]);
-                    ap((long long)(r0 + rr) * n + x, r0 + rr, x, st[c], in, out);
-#pragma unroll
-                    for (int g = 0; g < kMaxK; g++) {
-                        if (g < kout) {
-                            *(double*)&slot[g * 2 * n] = out[g];
-                            const unsigned m = fx_hi(out[g]);
-                            hi[g] = m > hi[g] ? m : hi[g];
-                        }
-                    }
+            for (int g = 0; g < kMaxK; g++) {
+                if (g < kout) {
+                    *(double*)&slot[g * 2 * n] = out[g];
+                    const unsigned m = fx_hi(out[g]);
+                    hi[g] = m > hi[g] ? m : hi[g];
                 }
             }
         }
@@ -1439,7 +1495,7 @@ __device__ void row_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
             fxc_convert(X, kout, logn, red + 2 * kMaxK, red + 3 * kMaxK, tid, nthr);
             cta_sync();
             longlong2* Z = X == B0 ? B1 : B0;
-            const longlong2* Y = fx_coop<-1, NF>(X, Z, logn, kout, red + 3 * kMaxK, tw.tfx, tw.log, tid, nthr) ? Z : X;
+            const longlong2* Y = fx_coop<-1>(X, Z, logn, kout, red + 3 * kMaxK, tw.tfx, tw.log, tid, nthr) ? Z : X;
             fxc_store_rows(Y, dst + r0, Hs, rows, kout, logn, red + 2 * kMaxK, red + 3 * kMaxK, tid, nthr);
         }
         cta_sync();  // the next unit reuses the buffers
@@ -1460,12 +1516,7 @@ __device__ void col_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
     for (int k1 = blockIdx.x; k1 < ncols; k1 += gridDim.x) {
         const Line ln = line_of(P, tw, k1);
         for (int i = tid; i < 4 * kMaxK; i += nthr) red[i] = 0u;
-        S st[kCoopChunk];
-#pragma unroll
-        for (int c = 0; c < kCoopChunk; c++) {
-            const int k0 = tid + nthr * c;
-            if (k0 < n) st[c] = ld(ln, k0);
-        }
+        S cur = ld(ln, tid < n ? tid : 0);
         cta_sync();
         longlong2* X = B0;
         int sc[kMaxK] = {0, 0, 0};
@@ -1474,7 +1525,7 @@ __device__ void col_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
             cta_sync();
             fxc_convert(B0, kin, logn, red, red + kMaxK, tid, nthr);
             cta_sync();
-            X = fx_coop<-1, NF>(B0, B1, logn, kin, red + kMaxK, tw.tfx, tw.log, tid, nthr) ? B1 : B0;
+            X = fx_coop<-1>(B0, B1, logn, kin, red + kMaxK, tw.tfx, tw.log, tid, nthr) ? B1 : B0;
 #pragma unroll
             for (int f = 0; f < kMaxK; f++)
                 if (f < kin) sc[f] = fxc_scale(red, red + kMaxK, f);
@@ -1483,40 +1534,30 @@ __device__ void col_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
         longlong2* Z = X == B0 ? B1 : B0;
         const int pitch = n + 2;
         unsigned hi[kMaxK] = {0u, 0u, 0u};
-        for (int q0 = 0; q0 < n; q0 += nthr * kCoopChunk) {
-            if (q0 > 0) {
+#pragma unroll 1
+        for (int k0 = tid; k0 < n; k0 += nthr) {
+            const S st = cur;
+            if (k0 + nthr < n) cur = ld(ln, k0 + nthr);
+            longlong2* slot = X + fxs(k0);
+            double2 in[kMaxK];
+            CO out[kMaxK];
 #pragma unroll
-                for (int c = 0; c < kCoopChunk; c++) {
-                    const int k0 = q0 + tid + nthr * c;
-                    if (k0 < n) st[c] = ld(ln, k0);
+            for (int f = 0; f < kMaxK; f++) {
+                if (f < kin) {
+                    const longlong2 z = slot[f * n];
+                    in[f] = double2{fx_to(z.x, sc[f]), fx_to(z.y, sc[f])};
                 }
             }
+            ap(ln, k0, st, in, out);
 #pragma unroll
-            for (int c = 0; c < kCoopChunk; c++) {
-                const int k0 = q0 + tid + nthr * c;
-                if (k0 < n) {
-                    longlong2* slot = X + fxs(k0);
-                    double2 in[kMaxK];
-                    CO out[kMaxK];
-#pragma unroll
-                    for (int f = 0; f < kMaxK; f++) {
-                        if (f < kin) {
-                            const longlong2 z = slot[f * n];
-                            in[f] = double2{fx_to(z.x, sc[f]), fx_to(z.y, sc[f])};
-                        }
-                    }
-                    ap(ln, k0, st[c], in, out);
-#pragma unroll
-                    for (int g = 0; g < kMaxK; g++) {
-                        if (g < kout) {
-                            if constexpr (sizeof(TO) == 8) {
-                                *(CO*)&slot[g * n] = out[g];
-                                const unsigned a = fx_hi(out[g].x), c2 = fx_hi(out[g].y), m = a > c2 ? a : c2;
-                                hi[g] = m > hi[g] ? m : hi[g];
-                            } else {
-                                ((CO*)Z)[(size_t)g * pitch + k0] = out[g];
-                            }
-                        }
+            for (int g = 0; g < kMaxK; g++) {
+                if (g < kout) {
+                    if constexpr (sizeof(TO) == 8) {
+                        *(CO*)&slot[g * n] = out[g];
+                        const unsigned a = fx_hi(out[g].x), c2 = fx_hi(out[g].y), m = a > c2 ? a : c2;
+                        hi[g] = m > hi[g] ? m : hi[g];
+                    } else {
+                        ((CO*)Z)[(size_t)g * pitch + k0] = out[g];
                     }
                 }
             }
@@ -1530,12 +1571,12 @@ __device__ void col_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
                 fxc_convert(X, kout, logn, red + 2 * kMaxK, red + 3 * kMaxK, tid, nthr);
                 cta_sync();
                 const longlong2* Y =
-                    fx_coop<+1, NF>(X, Z, logn, kout, red + 3 * kMaxK, tw.tfx, tw.log, tid, nthr) ? Z : X;
+                    fx_coop<+1>(X, Z, logn, kout, red + 3 * kMaxK, tw.tfx, tw.log, tid, nthr) ? Z : X;
                 fxc_store(Y, dst + (size_t)k1 * n, Hs, kout, logn, red + 2 * kMaxK, red + 3 * kMaxK, tid, nthr);
             } else {
                 cta_sync();  // the inputs' buffers become the second set of the FP32 lines
                 float2 *f0 = (float2*)Z, *f1 = (float2*)X;
-                const float2* Y = fft_coop<+1, float, NF>(f0, f1, logn, pitch, kout, tw.t32, tw.log, tid, nthr) ? f1 : f0;
+                const float2* Y = fft_coop<+1, float>(f0, f1, logn, pitch, kout, tw.t32, tw.log, tid, nthr) ? f1 : f0;
                 for (int it = tid; it < kout * n; it += nthr) {
                     const int g = it >> logn, x = it & (n - 1);
                     dst[(size_t)g * Hs + (size_t)k1 * n + x] = Y[(size_t)g * pitch + x];
@@ -1574,7 +1615,7 @@ __device__ void row_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
             X0[(size_t)l * pitch + x] = (x <= half) ? CI{A.x - B.y, A.y + B.x} : CI{A.x + B.y, B.x - A.y};
         }
         const CI* Xr = X0;
-        if (kin > 0) Xr = fft_coop<+1, TI, NF>(X0, X1, logn, pitch, kin, tw.t32, tw.log, tid, nthr) ? X1 : X0;
+        if (kin > 0) Xr = fft_coop<+1, TI>(X0, X1, logn, pitch, kin, tw.t32, tw.log, tid, nthr) ? X1 : X0;
         // pointwise: point q = rr n + x of the unit (consecutive threads, consecutive x)
         for (int q0 = 0; q0 < 2 * n; q0 += nthr * kCoopChunk) {
             S st[kCoopChunk];
@@ -1613,7 +1654,7 @@ __device__ void row_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
             }
         }
         if (kout > 0) {
-            const CO* Yr = fft_coop<-1, TO, NF>(Y0, Y1, logn, pitch, kout, tw.t32, tw.log, tid, nthr) ? Y1 : Y0;
+            const CO* Yr = fft_coop<-1, TO>(Y0, Y1, logn, pitch, kout, tw.t32, tw.log, tid, nthr) ? Y1 : Y0;
             const TO hf = (TO)0.5;
             for (int it = tid; it < kout * (half + 1); it += nthr) {
                 const int g = it / (half + 1), k = it - g * (half + 1);
@@ -1650,7 +1691,7 @@ __device__ void col_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
         const C* Xr = B0;
         C* Xi = B1;
         if (kin > 0) {
-            const int r = fft_coop<-1, TI, NF>(B0, B1, logn, pitch, kin, tw.t32, tw.log, tid, nthr);
+            const int r = fft_coop<-1, TI>(B0, B1, logn, pitch, kin, tw.t32, tw.log, tid, nthr);
             Xr = r ? B1 : B0;
             Xi = r ? B0 : B1;
         }
@@ -1680,7 +1721,7 @@ __device__ void col_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
         }
         if (kout > 0) {
             CO* scratch = (CO*)Xr;
-            const int r = fft_coop<+1, TO, NF>(Xo, scratch, logn, pitch, kout, tw.t32, tw.log, tid, nthr);
+            const int r = fft_coop<+1, TO>(Xo, scratch, logn, pitch, kout, tw.t32, tw.log, tid, nthr);
             const CO* Yr = r ? scratch : Xo;
             for (int it = tid; it < kout * n; it += nthr) {
                 const int g = it >> logn, x = it & (n - 1);
@@ -1870,10 +1911,9 @@ __device__ void mid_pass_fx(const Params& P, const Tw& tw, int k, const double2*
 // iteration passes: a unit (kMidG lines of one field) is 16-byte pieces, each
 // two neighbouring lines' values at one position (row side: i1 pairs of one
 // line; transposed side: the kMidG values at one km), copied by cp.async into
-// one of two slots while the warp transforms the previous unit; transforms in
-// the padded layout.
+// the warp's slot; transforms in the padded layout.
 __host__ __device__ constexpr size_t mid_staged_smem(int n) {
-    return 2 * (size_t)kMidG * (size_t)padded_len(n) * 8 + 2 * (size_t)n * 16;
+    return 2 * (size_t)kMidG * (size_t)padded_len(n) * 8 + (size_t)n * 16;
 }
 
 template <int NF, int S>
@@ -1885,64 +1925,48 @@ __device__ void mid_pass_staged(const Params& P, const Tw& tw, int k, const floa
     const WarpCtx w = warp_ctx(P, smem);
     float2* B0 = (float2*)w.mem;
     float2* B1 = B0 + kMidG * PP;
-    float4* slots = (float4*)(B1 + kMidG * PP);  // 2 x NF pieces
+    float4* slot = (float4*)(B1 + kMidG * PP);  // NF pieces
     const URange ur = units_of(tw, P.h1 * gpp);
-    auto issue = [&](int u, int f, int s) {
+    for (int u = ur.b; u < ur.e; u += ur.s) {
         const int k1 = u / gpp, i0 = (u - k1 * gpp) * kMidG;
-        const float2* sf = src + (size_t)f * H;
-        float4* sl = slots + s * NF;
-        if (S < 0) {
-            const float2* rb = sf + (size_t)k1 * rows + (size_t)i0 * NF;  // [k1][i0][i1]
-            for (int j = w.lane; j < NF; j += kWarp) cp_async16(sl + j, rb + 2 * j);
-        } else {
-            const float2* cb = sf + (size_t)k1 * NF * n0 + i0;  // [k1][km][i0]
-            for (int km = w.lane; km < NF; km += kWarp) cp_async16(sl + km, cb + (size_t)km * n0);
-        }
-    };
-    int u = ur.b, f = 0, s = 0;
-    if (u < ur.e && k > 0) issue(u, 0, 0);
-    cp_async_commit();
-    while (u < ur.e && k > 0) {
-        int un = u, fn = f + 1;
-        if (fn == k) {
-            fn = 0;
-            un = u + ur.s;
-        }
-        if (un < ur.e) issue(un, fn, s ^ 1);
-        cp_async_commit();
-        cp_async_wait<1>();
-        warp_sync();
-        const float2* sl = (const float2*)(slots + s * NF);
+        for (int f = 0; f < k; f++) {
+            const float2* sf = src + (size_t)f * H;
+            if (S < 0) {
+                const float2* rb = sf + (size_t)k1 * rows + (size_t)i0 * NF;  // [k1][i0][i1]
+                for (int j = w.lane; j < NF; j += kWarp) cp_async16(slot + j, rb + 2 * j);
+            } else {
+                const float2* cb = sf + (size_t)k1 * NF * n0 + i0;  // [k1][km][i0]
+                for (int km = w.lane; km < NF; km += kWarp) cp_async16(slot + km, cb + (size_t)km * n0);
+            }
+            cp_async_commit();
+            cp_async_wait<0>();
+            warp_sync();
+            const float2* sl = (const float2*)slot;
 #pragma unroll 4
-        for (int j = w.lane; j < kMidG * NF; j += kWarp) {
-            if (S < 0) B0[(j / NF) * PP + pix<true>(j % NF)] = sl[j];         // line g = j / NF
-            else B0[(j % kMidG) * PP + pix<true>(j / kMidG)] = sl[j];         // km = j / kMidG
-        }
-        const int r = fft_lines_fixed<S, float, LOGN, kMidG, true>(B0, B1, PP, kMidG, tw.t32, tw.log, w.lane);
-        const float2* Br = r ? B1 : B0;
-        const int k1 = u / gpp, i0 = (u - k1 * gpp) * kMidG;
-        float2* df = dst + (size_t)f * H;
-        if (S < 0) {
-            float4* cb = (float4*)(df + (size_t)k1 * NF * n0 + i0);
-            for (int km = w.lane; km < NF; km += kWarp) {
-                const float2 a = Br[pix<true>(km)], b = Br[PP + pix<true>(km)];
-                cb[(size_t)km * (n0 / 2)] = float4{a.x, a.y, b.x, b.y};
+            for (int j = w.lane; j < kMidG * NF; j += kWarp) {
+                if (S < 0) B0[(j / NF) * PP + pix<true>(j % NF)] = sl[j];         // line g = j / NF
+                else B0[(j % kMidG) * PP + pix<true>(j / kMidG)] = sl[j];         // km = j / kMidG
             }
-        } else {
-            float4* rb = (float4*)(df + (size_t)k1 * rows + (size_t)i0 * NF);
-            for (int j = w.lane; j < NF; j += kWarp) {
-                const int g = (2 * j) / NF, q = pix<true>((2 * j) % NF);  // i1 and i1 + 1 share a group
-                const float2 a = Br[g * PP + q], b = Br[g * PP + q + 1];
-                rb[j] = float4{a.x, a.y, b.x, b.y};
+            const int r = fft_lines_fixed<S, float, LOGN, kMidG, true>(B0, B1, PP, kMidG, tw.t32, tw.log, w.lane);
+            const float2* Br = r ? B1 : B0;
+            float2* df = dst + (size_t)f * H;
+            if (S < 0) {
+                float4* cb = (float4*)(df + (size_t)k1 * NF * n0 + i0);
+                for (int km = w.lane; km < NF; km += kWarp) {
+                    const float2 a = Br[pix<true>(km)], b = Br[PP + pix<true>(km)];
+                    cb[(size_t)km * (n0 / 2)] = float4{a.x, a.y, b.x, b.y};
+                }
+            } else {
+                float4* rb = (float4*)(df + (size_t)k1 * rows + (size_t)i0 * NF);
+                for (int j = w.lane; j < NF; j += kWarp) {
+                    const int g = (2 * j) / NF, q = pix<true>((2 * j) % NF);  // i1 and i1 + 1 share a group
+                    const float2 a = Br[g * PP + q], b = Br[g * PP + q + 1];
+                    rb[j] = float4{a.x, a.y, b.x, b.y};
+                }
             }
+            warp_sync();
         }
-        warp_sync();
-        u = un;
-        f = fn;
-        s ^= 1;
     }
-    cp_async_wait<0>();
-    warp_sync();
 }
 
 // Column passes read the last row pass's output and write the next row pass's
@@ -2199,13 +2223,9 @@ __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, cons
             }
         });
     if (!reb) {
-        publish_sum(&P.sc->beta_sum[c.bsel][0], s0);
-        if (!pfc) {
-            publish_sum(&P.sc->beta_sum[c.bsel][1], s2);
-        }
-    }
-    if (acc) {
-        publish_sum(&P.mass[1], dmass);
+        double* const a[3] = {&P.sc->beta_sum[c.bsel][0], &P.sc->beta_sum[c.bsel][1], &P.mass[1]};
+        const double v[3] = {s0.warp_total(), pfc ? 0.0 : s2.warp_total(), acc ? warp_sum(dmass) : 0.0};
+        publish_group<3>(tw, true, nullptr, 0ull, a, v);
     }
 }
 
@@ -2511,16 +2531,14 @@ __device__ __noinline__ void phase_R_staged(const Params& P, const Ctl& c, const
                                      asum);
     };
     if constexpr (!PFC && NF % (2 * kWarp) == 0) {
-        if (P.coop && pairs_hold(tw, P.rows / 2)) {
+        if (P.coop && pairs_hold(P, P.rows / 2)) {
             row_pass_pair<NF, NS>(P, tw, src, (float2*)P.NB, sp, smem, pt);
-            amax.publish(&P.norms[(size_t)bank * P.nslots + c.ev]);
-            publish_sum(&P.sums[(size_t)bank * P.nslots + c.ev], asum);
+            publish_eval(P, tw, false, bank, c.ev, amax, asum);  // two warps of the CTA
             return;
         }
     }
     row_pass_staged<NF, K, NS, SL>(P, tw, src, (float2*)P.NB, sp, smem, pt);
-    amax.publish(&P.norms[(size_t)bank * P.nslots + c.ev]);
-    publish_sum(&P.sums[(size_t)bank * P.nslots + c.ev], asum);
+    publish_eval(P, tw, !P.coop, bank, c.ev, amax, asum);  // coop: one warp of the CTA
 }
 
 template <int L>
@@ -2553,9 +2571,7 @@ __device__ __noinline__ void phase_R_coop(const Params& P, const Ctl& c, const T
             if (pfc) row_point<float, float, true>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
             else row_point<float, float, false>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
         });
-    // every warp publishes its threads' norm and sum
-    amax.publish(&P.norms[(size_t)bank * P.nslots + c.ev]);
-    publish_sum(&P.sums[(size_t)bank * P.nslots + c.ev], asum);
+    publish_eval(P, tw, true, bank, c.ev, amax, asum);
 }
 
 // Iteration row pass (R1 reads the FP64 base direction, RI the T one):
@@ -2612,8 +2628,7 @@ __device__ PAGD_HOT void phase_R(const Params& P, const Ctl& c, const Tw& tw, ch
             if (pfc) row_point<T, TI, true>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
             else row_point<T, TI, false>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
         });
-    amax.publish(&P.norms[(size_t)bank * P.nslots + c.ev]);
-    publish_sum(&P.sums[(size_t)bank * P.nslots + c.ev], asum);
+    publish_eval(P, tw, true, bank, c.ev, amax, asum);
 }
 
 // Constants of the iteration column pass: the momentum factors, theta_v s, the
@@ -2679,7 +2694,7 @@ __device__ __noinline__ void phase_CI_staged(const Params& P, const Ctl& c, cons
         col_point<float, PFC>(P, q, sprev, k1, k0, sv[0], sv[1], sv[2], in, out);
     };
     if constexpr (!PFC && NF % (2 * kWarp) == 0) {
-        if (P.coop && pairs_hold(tw, P.ncols)) {
+        if (P.coop && pairs_hold(P, P.ncols)) {
             col_pass_pair<NF, 3>(P, tw, csrcT<float>(P), cdstT<float>(P), sc3, smem, pt);
             return;
         }
@@ -2787,7 +2802,11 @@ __device__ PAGD_COLD void phase_accept(const Params& P, const Ctl& c, const Tw& 
         dmass += x - a;
         if (P.out_real) P.out_real[p] = x;
     }
-    publish_sum(&P.mass[1], dmass);
+    {
+        double* const a[1] = {&P.mass[1]};
+        const double v[1] = {warp_sum(dmass)};
+        publish_group<1>(tw, true, nullptr, 0ull, a, v);
+    }
     if (c.rec_pending && leader(tw)) P.mass[2] = bits_dbl(ldcg(&P.norms[(size_t)c.rec_bank * P.nslots + c.rec_ev]));
     if (leader(tw)) {
         P.stats[c.step].iters = c.ev;
@@ -3128,6 +3147,7 @@ __host__ __device__ inline Ctl ctl_init(const Params& P) {
     c.rec_pending = 0; c.rec_ev = 0; c.rec_bank = 0;
     c.inc = inc_eval(P, c.ref_ok, P.step0, 1);
     c.bt = betas_from(P, step_coeffs(P, 0), 0.0, 0.0);
+    c.reb_nrm = 0.0;
     c.resid = 0.0; c.base_nrm = 0.0; c.best_nrm = 0.0; c.acc_resid = 0.0;
     switch (P.prog) {
         case PROG_RUN:
@@ -3228,7 +3248,10 @@ __device__ void ctl_eval(const Params& P, Ctl& c, double nrm) {
     c.resid = nrm;
     if (!nn_le(nrm, 1.0e300)) { c.fail = ST_ENAN; c.ph = PH_FAIL; return; }
     if (c.ph == PH_R1 || !nn_le(c.best_nrm, nrm)) { c.best_nrm = nrm; c.best_ev = c.ev; }
-    if (c.ph == PH_R1) c.base_nrm = nrm;
+    if (c.ph == PH_R1) {
+        c.base_nrm = nrm;
+        c.reb_nrm = kRebaseRatio * nrm;
+    }
     // the first direction of a step from the extrapolation (Sec. 3.4.2): the
     // record a caller's guess is judged against
     if (c.ph == PH_R1 && !c.ereb && (c.gmode == 0 || c.gmode == 2 || c.gmode == 4)) {
@@ -3291,7 +3314,7 @@ __device__ void ctl_eval(const Params& P, Ctl& c, double nrm) {
         c.bsel = 3;
         c.inc = t64 ? 0 : inc_eval(P, c.ref_ok, P.step0 + c.step, 1);
         c.ph = PH_B;
-    } else if ((fp32_norm && (conv || nn_le(nrm, kRebaseRatio * c.base_nrm) ||
+    } else if ((fp32_norm && (conv || nn_le(nrm, c.reb_nrm) ||
                               c.ev - c.best_ev >= kStagnation)) ||
                (inc_norm && conv)) {
         if (c.rech >= P.max_recheck) { c.fail = ST_ENOCONV; c.ph = PH_FAIL; return; }
@@ -3304,6 +3327,35 @@ __device__ void ctl_eval(const Params& P, Ctl& c, double nrm) {
     } else {
         c.ph = PH_CI;
     }
+}
+
+// The two transitions of an iteration, without the rest of the machine: CI ->
+// RI, and RI -> CI when the norm neither stops nor moves anything (ctl_eval's
+// last branch).  Thread 0 of every CTA decides between two barriers, 1700
+// cycles through the whole machine.  Returns false for ctl_advance to decide.
+template <class T> __device__ __forceinline__ bool ctl_fast(const Params& P, Ctl& c) {
+    if (P.nm > 1 || P.prog != PROG_RUN) return false;
+    if (c.ph == PH_CI) {
+        c.ph = PH_RI;
+        c.it++;
+        return true;
+    }
+    if (c.ph != PH_RI) return false;
+    const int ev = c.ev;
+    const unsigned long long b = ldcg(&P.norms[(size_t)(c.step & 1) * P.nslots + ev]);
+    const bool mixed = sizeof(T) == 4;
+    const unsigned long long thr = dbl_bits(P.tol), reb = mixed ? dbl_bits(c.reb_nrm) : 0ull, best = dbl_bits(c.best_nrm);
+    const int best_ev = b < best ? ev + 1 : c.best_ev;
+    if (b <= thr || b <= reb || b > dbl_bits(1.0e300) || ev + 1 >= P.max_iter || ev + 2 >= P.nslots ||
+        (mixed && ev + 1 - best_ev >= kStagnation))
+        return false;
+    c.lastev = ev;
+    c.ev = ev + 1;
+    c.resid = bits_dbl(b);
+    c.best_ev = best_ev;
+    if (b < best) c.best_nrm = bits_dbl(b);
+    c.ph = PH_CI;
+    return true;
 }
 
 template <class T>
@@ -3583,16 +3635,16 @@ __host__ __device__ inline int phase_weight(const Params& P, const Ctl& c) {
         }
     }
     switch (c.ph) {
-        case PH_B: return c.inc ? 6 : 9;
+        case PH_B: return 5;
         case PH_C:
         case PH_D:
-        case PH_E: return c.inc ? 5 : 8;
+        case PH_E: return c.inc ? 5 : 6;
         case PH_R1:
         case PH_RI:
         case PH_CI: return t64 ? 3 : 1;
         case PH_MF:
         case PH_MI: return (c.m64 || t64) ? 3 * (c.mk > 0 ? c.mk : 1) : 1;
-        case PH_ACCEPT: return 5;
+        case PH_ACCEPT: return 2;
         default: return t64 ? 4 : 2;
     }
 }
@@ -3631,14 +3683,14 @@ __host__ __device__ inline void batch_split(Tw& t, long long gw, long long nw, l
     const long long ra = (g * nw + total - 1) / total, rb = ((g + cost) * nw + total - 1) / total - 1;
     if (rb - ra + 1 >= 16 && (long long)units >= 32 * (rb - ra + 1)) {
         if (gw < ra || gw > rb) {
-            t.wr = kIdleRank;
-            t.wn = 1;
+            t.wr = t.ur = kIdleRank;
+            t.wn = t.un = 1;
             t.ulo = 0;
             t.uhi = 0;
             return;
         }
-        t.wr = (int)(gw - ra);
-        t.wn = (int)(rb - ra + 1);
+        t.wr = t.ur = (int)(gw - ra);
+        t.wn = t.un = (int)(rb - ra + 1);
         t.ulo = 0;
         t.uhi = -1;
         return;
