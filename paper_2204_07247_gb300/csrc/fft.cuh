@@ -255,8 +255,7 @@ __host__ __device__ constexpr int ilog2c(int v) { return v <= 1 ? 0 : 1 + ilog2c
 // CTA-cooperative transforms: all threads of the CTA share the nl lines of one
 // unit, the butterflies of a stage dealt round robin over (line, butterfly),
 // stages separated by a CTA barrier.  Used where a phase has fewer units than
-// warps: the lines of one unit then occupy every SM sub-partition instead of
-// one, which is what bounds an FP64 transform on a part with a low FP64 rate.
+// warps: the lines of one unit then occupy every SM sub-partition instead of one.
 
 __device__ __forceinline__ void cta_sync() {
 #ifndef PAGD_EMU
@@ -297,13 +296,21 @@ __device__ __forceinline__ void stage_coop(const cx<T>* src, cx<T>* dst, int log
 // -> result in b0 (returns 0) or b1 (1), visible to every thread on return.
 // Radix 4, and 8 for the first stage of an odd number of levels (radix 2, which
 // gives every thread a butterfly, needs twice the barriers and shared-memory
-// round trips and was slower); the stages share their code.
+// round trips and was slower); the stages share their code.  64 points go as
+// 8 x 8, like the warp-owned transform, whose results they give bit for bit.
 template <int S, class T>
 __device__ __noinline__ int fft_coop(cx<T>* b0, cx<T>* b1, int logn, int pitch, int nl, const cx<T>* tw, int logTw,
                                      int tid, int nthr) {
     cx<T>*s = b0, *d = b1;
     int logNs = 2, r = 1;
     cta_sync();
+    if (logn == 6) {
+        stage_coop<8, S, T, true>(s, d, logn, 0, pitch, nl, tw, logTw, tid, nthr);
+        cta_sync();
+        stage_coop<8, S, T, false>(d, s, logn, 3, pitch, nl, tw, logTw, tid, nthr);
+        cta_sync();
+        return 0;
+    }
     if (logn & 1) {
         stage_coop<8, S, T, true>(s, d, logn, 0, pitch, nl, tw, logTw, tid, nthr);
         logNs = 3;
