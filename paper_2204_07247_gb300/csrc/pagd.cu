@@ -65,7 +65,7 @@ struct pagd_solver {
 };
 
 enum {
-    O_SC, O_NORMS, O_SUMS, O_STATS, O_TW64, O_TW32, O_U0, O_U1, O_VB, O_G64, O_VBT, O_LBT, O_DD0,
+    O_SC, O_STATS, O_NORMS, O_SUMS, O_TW64, O_TW32, O_U0, O_U1, O_VB, O_G64, O_VBT, O_LBT, O_DD0,
     O_DD1, O_SS0, O_SS1, O_C0, O_NB, O_DB, O_CL64, O_NB64, O_DB64, O_MASS, O_TRACE, O_VR64, O_NR64, O_WR64, O_LB64, O_YB, O_X, O_X64, O_GH64, O_LCTL, O_TWFX, O_END
 };
 
@@ -621,19 +621,19 @@ static Params run_params(const pagd_solver* s, double* u_out, double dt, int nst
 static pagd_status run_finish(pagd_solver* s, const Params& P, double dt, int nsteps, int* iters, double* resid,
                               bool bar_error, int* used_guess = nullptr) {
     const bool imex = s->scheme == PAGD_LBDF2 || s->scheme == PAGD_LMP;
-    Scal sc;
-    pagd_status st = dcopy(s, &sc, P.sc, sizeof(Scal));
+    // the run's scalars and its per-step results, which follow them in the
+    // workspace, in one copy (each read-back costs about 10 us)
+    const size_t so = s->off[O_STATS] - s->off[O_SC];
+    std::vector<char> back(so + sizeof(StepStat) * (size_t)(nsteps > 0 ? nsteps : 1));
+    pagd_status st = dcopy(s, back.data(), P.sc, back.size());
     if (st == PAGD_OK) st = dsync(s);
     if (st != PAGD_OK) return st;
+    Scal sc;
+    std::memcpy(&sc, back.data(), sizeof(sc));
+    const StepStat* stats = (const StepStat*)(back.data() + so);
     bar_error = bar_error || sc.bar_error;
-    std::vector<StepStat> stats(nsteps > 0 ? nsteps : 1);
     const int ndone = sc.steps_done;
     const int nrec = (sc.status != ST_OK) ? ndone + 1 : ndone;
-    if (nrec > 0) {
-        st = dcopy(s, stats.data(), P.stats, sizeof(StepStat) * (size_t)(nrec < nsteps ? nrec : nsteps));
-        if (st == PAGD_OK) st = dsync(s);
-        if (st != PAGD_OK) return st;
-    }
     for (int i = 0; i < nrec && i < nsteps; i++) {
         if (iters) iters[i] = stats[i].iters;
         if (resid) resid[i] = stats[i].resid;
@@ -651,7 +651,7 @@ static pagd_status run_finish(pagd_solver* s, const Params& P, double dt, int ns
     if (sc.status != ST_OK) {
         char buf[160];
         std::snprintf(buf, sizeof(buf), "step %d (global %d) failed with status %d after %d evaluations",
-                      sc.fail_step, s->step, sc.status, nrec > 0 ? stats[nrec - 1].iters : 0);
+                      sc.fail_step, s->step, sc.status, nrec > 0 && nrec <= nsteps ? stats[nrec - 1].iters : 0);
         return fail(s, status_from(sc.status), buf);
     }
     if (ndone != nsteps) return fail(s, PAGD_ECUDA, "kernel ended early");
