@@ -49,6 +49,7 @@ constexpr int kPitch = kTile + 4;  // of a channel's points in shared memory: ro
 struct SnoDims {
     int n0, n1, np, C, L, M0, M1, M;
     int QC, J, JB, R, NT;  // NT: tiles of a sample
+    int ljb;               // log2 JB
 };
 
 // tanh form of GELU (Hendrycks and Gimpel, 2016), x (1 + tanh u) / 2 = x sigma(2 u)
@@ -66,14 +67,17 @@ __device__ __forceinline__ float gelu_grad(float x, float s) {
 
 __device__ __forceinline__ int k0_of(int m0, int M0, int n0) { return m0 < M0 / 2 ? m0 : n0 - M0 + m0; }
 
-// exp(-2 pi i j / n), j < n, from sincospif: the tables of both axes, written
-// once when the workspace is handed in
-__global__ void k_tables(float2* t, int n) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// exp(-2 pi i j / n), j < n, from sincospif, for both axes: written by every
+// call in one small launch, so that nothing in the workspace has to be kept
+__global__ void k_tables(float2* t0, int n0, float2* t1, int n1) {
+    int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool first = j < n0;
+    if (!first) j -= n0;
+    const int n = first ? n0 : n1;
     if (j >= n) return;
-    float s, c;
-    sincospif(2.f * (float)j / (float)n, &s, &c);
-    t[j] = make_float2(c, -s);
+    float sn, cs;
+    sincospif(-2.f * (float)j / (float)n, &sn, &cs);
+    (first ? t0 : t1)[j] = float2{cs, sn};
 }
 
 // cos(2 pi k / 16)
@@ -200,7 +204,7 @@ __global__ void __launch_bounds__(kThr, CT <= 16 ? 3 : 1) k_tile(SnoDims d, Tile
     float2* U = tj + d.M1 * 32;                     // [R][C][M1]
     float2* e0 = U + R * d.C * d.M1;                // [R][M0] exp(-2 pi i k0 x0 / n0)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.y;
-    const int rg = blockIdx.x / d.JB, jb = blockIdx.x - rg * d.JB, x00 = rg * R, j = jb * 32 + lane;
+    const int rg = blockIdx.x >> d.ljb, jb = blockIdx.x & (d.JB - 1), x00 = rg * R, j = jb * 32 + lane;
     const size_t bc = (size_t)b * d.C;
     for (int i = tid; i < d.M1 * 32; i += kThr) tj[i] = a.tw1[((i >> 5) * (jb * 32 + (i & 31))) & (d.n1 - 1)];
     if constexpr (MODE != T_LIFT) {
@@ -306,6 +310,15 @@ __global__ void __launch_bounds__(kThr, CT <= 16 ? 3 : 1) k_tile(SnoDims d, Tile
             for (int t = 0; t < PT; t++)
 #pragma unroll
                 for (int c = 0; c < CT; c++) vin[t][c] = (c < d.C && in[t]) ? a.vin[(bc + c) * d.np + pp[t]] : 0.f;
+            // (z_{l-1} with the other loads, not one by one in the loop below)
+            float zp[PT][MODE == T_BACK ? CT : 1];
+            if constexpr (MODE == T_BACK) {
+#pragma unroll
+                for (int t = 0; t < PT; t++)
+#pragma unroll
+                    for (int c = 0; c < CT; c++)
+                        zp[t][c] = (c < d.C && in[t]) ? a.zprev[(bc + c) * d.np + pp[t]] : 0.f;
+            }
             float out[PT];
             float sg[MODE == T_LOSS ? CT : 1], zz[MODE == T_LOSS ? CT : 1];
 #pragma unroll
@@ -342,7 +355,7 @@ __global__ void __launch_bounds__(kThr, CT <= 16 ? 3 : 1) k_tile(SnoDims d, Tile
                             zz[o] = f[t];
                             out[t] = fmaf(a.Q[o], f[t] * sg[o], out[t]);
                         } else if constexpr (MODE == T_BACK) {
-                            const float z = in[t] ? a.zprev[i] : 0.f;
+                            const float z = zp[t][o];
                             const float g = f[t] * gelu_grad(z, gelu_s(z));
                             if (in[t]) a.vout[i] = g;
                             *ys = in[t] ? g : 0.f;
@@ -485,7 +498,7 @@ __global__ void __launch_bounds__(kColThr) k_cols(SnoDims d, const float2* T, co
         if (m < d.M) {
 #pragma unroll 4
             for (int r = q; r < cr; r += nq) {
-                const float2 v = rw[r * d.M1 + m1], e = cs[(k0 * ((c0 + r) / d.JB)) & (d.n0 - 1)];
+                const float2 v = rw[r * d.M1 + m1], e = cs[(k0 * ((c0 + r) >> d.ljb)) & (d.n0 - 1)];
                 s.x += v.x * e.x - v.y * e.y;
                 s.y += v.x * e.y + v.y * e.x;
             }
@@ -810,6 +823,9 @@ static pagd_status forward(sno_net* s, TileArgs& a, int B, bool train) {
     float2* F = (float2*)(w + s->off_F);
     float2* G = (float2*)(w + s->off_G);
     const size_t vs = (size_t)B * d.C * d.np;  // one layer of activations
+    k_tables<<<(d.n0 + d.n1 + kThr - 1) / kThr, kThr, 0, st>>>((float2*)(w + s->off_tw0), d.n0,
+                                                                (float2*)(w + s->off_tw1), d.n1);
+    CK(cudaGetLastError());
     a.vout = v;
     CK(tile<T_LIFT>(d, a, B, st));
     for (int l = 0; l < d.L; l++) {
@@ -842,10 +858,11 @@ pagd_status sno_create(sno_net** out, int n0, int n1, int channels, int layers, 
     sno_net* s = new (std::nothrow) sno_net();
     if (!s) return PAGD_ENOMEM;
     SnoDims& d = s->d;
-    d = SnoDims{n0, n1, n0 * n1, channels, layers, modes0, modes1, modes0 * modes1, 0, 0, 0, 0, 0};
+    d = SnoDims{n0, n1, n0 * n1, channels, layers, modes0, modes1, modes0 * modes1, 0, 0, 0, 0, 0, 0};
     d.QC = n1 >= 512 ? 16 : n1 >= 64 ? 4 : 1;
     d.J = n1 / d.QC;
     d.JB = d.J > 32 ? d.J / 32 : 1;
+    while ((1 << d.ljb) < d.JB) d.ljb++;
     d.R = 16 / d.QC;
     d.NT = (n0 + d.R - 1) / d.R * d.JB;
     s->batch = batch;
@@ -873,12 +890,6 @@ pagd_status sno_set_workspace(sno_net* s, void* dev, size_t bytes) {
     if (((uintptr_t)dev & 255) != 0) return sno_fail(s, PAGD_EINVAL, "workspace not 256-byte aligned");
     if (bytes < s->ws_bytes) return sno_fail(s, PAGD_ENOMEM, "workspace too small");
     s->ws = (char*)dev;
-    // the twiddle tables, once per workspace, on the network's stream
-    cudaStream_t st = (cudaStream_t)s->stream;
-    const SnoDims& d = s->d;
-    k_tables<<<(d.n0 + kThr - 1) / kThr, kThr, 0, st>>>((float2*)(s->ws + s->off_tw0), d.n0);
-    k_tables<<<(d.n1 + kThr - 1) / kThr, kThr, 0, st>>>((float2*)(s->ws + s->off_tw1), d.n1);
-    CK(cudaGetLastError());
     return PAGD_OK;
 }
 
