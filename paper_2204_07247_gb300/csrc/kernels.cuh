@@ -34,27 +34,27 @@ __device__ __forceinline__ void red_release_add(unsigned long long* p, unsigned 
 // acquire loads.  The wait is bounded: after kBarrierTimeoutNs, or once another
 // CTA has flagged an error, the CTA records the error and returns false
 // instead of spinning on.
+// grid_arrive is thread 0's part, between the CTA's barriers on both sides.
+__device__ __forceinline__ bool grid_arrive(Scal* sc, unsigned gen) {
+    const unsigned long long target = (unsigned long long)(gen + 1) * gridDim.x;
+    red_release_add(&sc->bar_count, 1ull);
+    if (ld_acquire(&sc->bar_count) < target) {
+        const unsigned long long t0 = gtimer();
+        volatile int* ve = &sc->bar_error;
+        while (ld_acquire(&sc->bar_count) < target) {
+            if (*ve) return false;
+            if (gtimer() - t0 > kBarrierTimeoutNs) {
+                atomicOr(&sc->bar_error, 1);
+                return false;
+            }
+        }
+    }
+    return true;
+}
 static __device__ bool grid_barrier(Scal* sc, unsigned& gen) {
     __shared__ int s_ok;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        const unsigned long long target = (unsigned long long)(gen + 1) * gridDim.x;
-        red_release_add(&sc->bar_count, 1ull);
-        if (ld_acquire(&sc->bar_count) < target) {
-            const unsigned long long t0 = gtimer();
-            volatile int* ve = &sc->bar_error;
-            while (ld_acquire(&sc->bar_count) < target) {
-                if (*ve) { ok = 0; break; }
-                if (gtimer() - t0 > kBarrierTimeoutNs) {
-                    atomicOr(&sc->bar_error, 1);
-                    ok = 0;
-                    break;
-                }
-            }
-        }
-        s_ok = ok;
-    }
+    if (threadIdx.x == 0) s_ok = grid_arrive(sc, gen) ? 1 : 0;
     gen++;
     __syncthreads();
     return s_ok != 0;
@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxCtas) pagd_kernel(const __gri
     // and thread 0 advances it between two CTA barriers, which keeps its ~40
     // values out of the registers of the phase code.
     __shared__ Ctl c;
+    __shared__ int s_ok;
     unsigned gen = 0;
     int ntr = 0;
     if (threadIdx.x == 0) {
@@ -105,8 +106,11 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxCtas) pagd_kernel(const __gri
         const bool cl_phase = P.cl && c.ph == PH_CI;
         if (cl_phase) cluster_iterate<T, NF>(P, c, tw, wsm, &ntr);
         else exec_phase<T, NF>(P, c, tw, wsm, red);
-        if (!grid_barrier(P.sc, gen)) break;
+        // thread 0 meets the other CTAs and advances the control state between
+        // two barriers of the CTA
+        __syncthreads();
         if (threadIdx.x == 0) {
+            s_ok = grid_arrive(P.sc, gen) ? 1 : 0;
             if (P.trace && blockIdx.x == 0 && ntr < P.trace_cap && !cl_phase) {
                 // bit 16: a phase of an incremental (T-transform) base evaluation
                 const bool incb = c.inc && (c.ph == PH_B || c.ph == PH_C || c.ph == PH_D || c.ph == PH_E);
@@ -120,9 +124,11 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxCtas) pagd_kernel(const __gri
                 unsigned* dst = (unsigned*)&c;
                 for (int i = 0; i < (int)(sizeof(Ctl) / sizeof(unsigned)); i++) dst[i] = __ldcg(src + i);
             }
-            if (cl_phase || !ctl_fast<T>(P, c)) ctl_advance<T>(P, c);
+            if (s_ok && (cl_phase || !ctl_fast<T>(P, c))) ctl_advance<T>(P, c);
         }
+        gen++;
         __syncthreads();
+        if (!s_ok) break;
     }
     if (P.trace && blockIdx.x == 0 && threadIdx.x == 0) P.sc->ntrace = ntr;
 }
