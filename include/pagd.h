@@ -180,7 +180,8 @@ pagd_status pagd_get_state(pagd_solver* s, double* un_dev, double* unm1_dev, int
  * 8 MiB that the library carries; every GPU that loads the library holds that
  * array until the process exits.  The array's head keeps the twiddle tables;
  * the rest, 8,364,032 bytes, holds the step's scratch, so the solver's
- * pagd_workspace_size must not exceed that: every 2D grid up to 128 x 128
+ * pagd_workspace_size, less the 24,576 bytes of a table that the library
+ * carries apart, must not exceed that: every 2D grid up to 128 x 128
  * points and every 3D grid up to 16 x 16 x 16 fits in either precision
  * (FP32_MIXED also up to 128 x 256 and 32 x 32 x 32).  Larger grids are
  * rejected with PAGD_EINVAL and a message giving both sizes.
@@ -254,7 +255,7 @@ pagd_status pagd_pass_probe(pagd_solver* s, int pass, int count, double* us_per_
  * distributed shared memory), whether the passes with FP64 lines run
  * CTA-cooperative units, the dynamic shared memory per CTA, and whether the
  * FP32 iteration passes stage their inputs through shared memory by
- * asynchronous copies (PFC, FP32-mixed, square power-of-two grids; the same
+ * asynchronous copies (FP32-mixed, first and last axis of 64 to 512 points; the same
  * arithmetic either way).  Every output nullable. */
 pagd_status pagd_launch_info(const pagd_solver* s, int* grid, int* threads, int* cluster, int* coop,
                              size_t* smem, int* staged);

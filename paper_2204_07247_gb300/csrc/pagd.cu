@@ -359,7 +359,7 @@ static pagd_status run_program(pagd_solver* s, Params& P) {
 
 // The FP32 iteration passes stage their inputs through shared memory
 // (row_pass_staged / col_pass_staged; line lengths 64 to 512): bytes a warp's
-// slice needs for the staging slots (PFC two, FCH one), 0 where they do not
+// slice needs for a staging slot, 0 where they do not
 // stage.  PAGD_STAGED=0 keeps the register-staged passes (the same arithmetic,
 // for comparison).
 static size_t staged_bytes(const pagd_solver* s) {
@@ -367,8 +367,8 @@ static size_t staged_bytes(const pagd_solver* s) {
     if (!stage_len(n0) || !stage_len(n1) || s->tsize != 4) return 0;
     if (const char* e = std::getenv("PAGD_STAGED"))
         if (e[0] == '0' && e[1] == 0) return 0;
-    const int k = k_iter(s->model), sl = staged_slots(s->model);
-    size_t m = std::max(row_staged_smem(n1, k, staged_row_state(s->model), sl), col_staged_smem(n0, k, 3, sl));
+    const int k = k_iter(s->model);
+    size_t m = std::max(row_staged_smem(n1, k, staged_row_state(s->model)), col_staged_smem(n0, k, 3));
     // the middle passes of a cubic grid stage too (mid_pass_staged)
     if (s->dim == 3 && n0 == n1 && s->n[1] == n0) m = std::max(m, mid_staged_smem(n0));
     return (m + 15) & ~(size_t)15;
@@ -414,8 +414,9 @@ static void make_plan(pagd_solver* s) {
     if (s->grid < 1) s->grid = 1;
     s->smem = tw_smem_bytes(s->logtw) + (size_t)wpb * s->warp_bytes;
     // CTA-cooperative units for the passes with FP64 lines when a phase has
-    // fewer units than half the warps (most warps would otherwise idle and an
-    // pass's FP64 work would run on one SM sub-partition).
+    // fewer units than half the warps: most warps would otherwise idle and a
+    // unit's pointwise FP64 work and integer butterflies run on one SM
+    // sub-partition.
     // PAGD_COOP=0 / 1 overrides the choice.
     s->coop = 2 * units <= (long long)s->grid * wpb ? 1 : 0;
     if (const char* e = std::getenv("PAGD_COOP")) {
@@ -1039,12 +1040,14 @@ pagd_status pagd_step_static(pagd_solver* s, const double* un_dev, const double*
     if (step_index < 0 || !(dt > 0.0) || !std::isfinite(dt) || !(tol >= 0.0) ||
         (step_index > 0 && !(dt_prev > 0.0)))
         return fail(s, PAGD_EINVAL, "bad step index / dt / dt_prev / tol");
-    if (s->ws_bytes > kStaticWorkspaceBytes) {
+    // (the fixed-point twiddle table, the layout's last part, is apart: g_static_twfx)
+    const size_t need = s->off[O_TWFX];
+    if (need > kStaticWorkspaceBytes) {
         char buf[200];
         std::snprintf(buf, sizeof(buf),
                       "grid too large for the static scratch: needs %zu bytes, the maximum is %zu "
                       "(use pagd_set_workspace and pagd_step)",
-                      s->ws_bytes, kStaticWorkspaceBytes);
+                      need, kStaticWorkspaceBytes);
         return fail(s, PAGD_EINVAL, buf);
     }
     char* head = nullptr;

@@ -70,9 +70,8 @@ struct StepStat {
 };
 
 constexpr int kMaxK = 3;        // fields per pass
-// CTA size of the persistent kernels: up to 8 warps (255 registers each fill
-// the register file); the launch picks as many as the warps' shared memory
-// slices allow
+// CTA size of the persistent kernels: up to 8 warps; the launch picks as many
+// as the warps' shared memory slices allow
 constexpr int kMaxThreads = 256;
 // CTAs of the single-instance kernel per SM (128 registers a thread): a warp's
 // line transform is a chain of shared-memory round trips and integer products
@@ -186,24 +185,30 @@ struct Beta {
     double m2, b0, b2, b4;
 };
 
+// (flags and small numbers in bytes: a batch keeps one of these per member in
+// every CTA's shared memory, which limits the members it can take)
 struct Ctl {
-    int ph, step, it, ev, lastev, cur, rech, fail, best_ev;
-    int after, mk, m64;  // 3D middle pass: the phase after it, its fields, FP64 buffers
-    int gok;             // GH64 holds this step's g_hat (an exact evaluation made it)
-    int bsel;            // bank of the averaged-Newton sums of the current evaluation
-    int gmode;           // caller's guess: 0 none, 1 at it (kept when its first direction is no
-                         // larger than the record), 2 probing the extrapolation,
-                         // 3 iterating from it, 4 iterating from the extrapolation
-    double gnorm;        // ||d_0||_inf at the caller's guess
-    int acc_used;        // the step pending acceptance started from the caller's guess
+    int step, it, ev, lastev, best_ev;
+    int rec_ev;  // see rec_pending
+    int acc_it, acc_lastev, acc_ev;
+    signed char ph, cur, rech, fail;
+    signed char after, mk, m64;  // 3D middle pass: the phase after it, its fields, FP64 buffers
+    signed char gok;             // GH64 holds this step's g_hat (an exact evaluation made it)
+    signed char bsel;            // bank of the averaged-Newton sums of the current evaluation
+    signed char gmode;           // caller's guess: 0 none, 1 at it (kept when its first direction is no
+                                 // larger than the record), 2 probing the extrapolation,
+                                 // 3 iterating from it, 4 iterating from the extrapolation
+    signed char acc_used;        // the step pending acceptance started from the caller's guess
     // record of the extrapolation's first direction: evaluation rec_ev of bank
     // rec_bank was one; the next phase B / ACCEPT stores its norm (P.mass[2])
-    int rec_pending, rec_ev, rec_bank;
-    int acc, acc_cur, acc_it, acc_lastev, acc_ev, reb, ereb, inc, ref_ok, exact_done;
+    signed char rec_pending, rec_bank;
+    signed char acc, acc_cur, reb, ereb, inc, ref_ok, exact_done;
+    double gnorm;        // ||d_0||_inf at the caller's guess
     double resid, base_nrm, best_nrm, acc_resid;
     Beta bt;             // averaged Newton constants of the current evaluation
     double reb_nrm;      // kRebaseRatio base_nrm
 };
+static_assert(sizeof(Ctl) % 4 == 0, "the cluster loop hands it back in words");
 
 // FP32 iterations stop improving once ||d|| reaches about 1e-7 of the FP64
 // direction at the base point (the FP32 rounding of C0); the base is moved
@@ -487,10 +492,6 @@ __host__ __device__ __forceinline__ size_t row_warp_smem(int n1, int kin, int sz
 }
 __host__ __device__ __forceinline__ size_t col_warp_smem(int n0, int k, int sz) {
     return (size_t)(k + 1) * pitch_of(n0) * 2 * sz;
-}
-// inputs in szi, outputs in szo < szi (separate buffers)
-__host__ __device__ __forceinline__ size_t col_warp_smem_mixed(int n0, int kin, int szi, int kout, int szo) {
-    return (size_t)(kin + 1) * pitch_of(n0) * 2 * szi + (size_t)(kout + 1) * pitch_of(n0) * 2 * szo;
 }
 
 struct WarpCtx {
@@ -886,12 +887,14 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
 
 // ------------------------------------------- staged FP32 iteration passes
 //
-// The FP32 row and column passes of the PFC iterations with every input of a
-// unit staged in shared memory by asynchronous 16-byte copies (cp.async): a
-// warp issues all reads of its next unit (the half-spectrum pieces and the
-// pointwise state) before it transforms the current one, so that they are in
-// flight while it computes and hold no registers meanwhile.  Two staging slots
-// per warp alternate.  The transforms run on two buffers in the padded layout
+// The FP32 row and column passes of the iterations with every input of a unit
+// staged in shared memory by asynchronous 16-byte copies (cp.async): a warp
+// issues all reads of its unit (the half-spectrum pieces and the pointwise
+// state) at once, so that they are in flight together and hold no registers
+// meanwhile.  A warp has one staging slot: with a second one for its next unit
+// the slices leave an SM half the warps, which hide more of the reads than the
+// slot did (256^3, 8 warps with two slots -> 16 with one: row pass 129 -> 109,
+// column pass 140 -> 90 us).  The transforms run on two buffers in the padded layout
 // (fft.cuh: no bank conflicts in the strided stages).  Selected on the host
 // (Params::stage) where a warp's slice of shared memory, sized for the FP64
 // phases, holds them; K fields per line (PFC: 1), NS arrays of pointwise state.
@@ -903,36 +906,29 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
 // Slot = K lines of the input spectrum + NS lines of complex state, pitch N;
 // the first stage of the forward transform reads the slot's lines.
 
-__host__ __device__ constexpr size_t row_staged_smem(int n, int k, int ns, int slots) {
-    return 2 * (size_t)k * (size_t)padded_len(n) * 8 +
-           (size_t)slots * ((size_t)k * (size_t)(n / 2 + 1) * 16 + (size_t)ns * 2 * n * 4);
+__host__ __device__ constexpr size_t row_staged_smem(int n, int k, int ns) {
+    return 2 * (size_t)k * (size_t)padded_len(n) * 8 + (size_t)k * (size_t)(n / 2 + 1) * 16 + (size_t)ns * 2 * n * 4;
 }
-__host__ __device__ constexpr size_t col_staged_smem(int n, int k, int ns, int slots) {
-    return 2 * (size_t)k * (size_t)padded_len(n) * 8 + (size_t)slots * (size_t)(k + ns) * n * 8;
+__host__ __device__ constexpr size_t col_staged_smem(int n, int k, int ns) {
+    return 2 * (size_t)k * (size_t)padded_len(n) * 8 + (size_t)(k + ns) * n * 8;
 }
-// staging slots per model: PFC (one field) prefetches the next unit into a
-// second slot; FCH (two fields, four state arrays) has room for one slot,
-// which still puts all of a unit's reads in flight at once
-__host__ __device__ constexpr int staged_slots(int) { return 1; }
 __host__ __device__ constexpr int staged_row_state(int model) { return model == 0 ? 3 : 4; }
 
-template <int NF, int K, int NS, int SLOTS, class Ap>
+template <int NF, int K, int NS, class Ap>
 __device__ void row_pass_staged(const Params& P, const Tw& tw, const float2* src, float2* dst,
                                 const float* const* sp, char* smem, Ap&& ap) {
     constexpr int LOGN = ilog2c(NF), HALF = NF / 2, H1 = HALF + 1, PP = padded_len(NF), E = NF / kWarp;
-    constexpr int SLOT = K * H1 * 16 + NS * 2 * NF * 4;  // bytes
     const int rows = P.rows;
     const long long Hs = P.H;
     const WarpCtx w = warp_ctx(P, smem);
     float2* X0 = (float2*)w.mem;
     float2* X1 = X0 + K * PP;
-    char* slots = (char*)(X1 + K * PP);
+    float4* const sq = (float4*)(X1 + K * PP);
+    float* const st = (float*)(sq + K * H1);
     const float iscale = (float)P.inv_npts;
     const URange ur = units_of(tw, rows / 2);
-    auto issue = [&](int u, int s) {
+    for (int u = ur.b; u < ur.e; u += ur.s) {
         const int r0 = 2 * u;
-        float4* sq = (float4*)(slots + (size_t)s * SLOT);
-        float* st = (float*)(sq + K * H1);
 #pragma unroll
         for (int f = 0; f < K; f++)
             for (int k = w.lane; k < H1; k += kWarp)
@@ -941,25 +937,9 @@ __device__ void row_pass_staged(const Params& P, const Tw& tw, const float2* src
         for (int a = 0; a < NS; a++)
             for (int j = w.lane; j < NF / 2; j += kWarp)
                 cp_async16(st + a * 2 * NF + 4 * j, sp[a] + (size_t)r0 * NF + 4 * j);
-    };
-    if (SLOTS == 2 && ur.b < ur.e) issue(ur.b, 0);
-    if (SLOTS == 2) cp_async_commit();
-    int s = 0;
-    for (int u = ur.b; u < ur.e; u += ur.s, s ^= (SLOTS - 1)) {
-        const int r0 = 2 * u;
-        if constexpr (SLOTS == 2) {
-            // this unit's copies were issued with the previous unit
-            if (u + ur.s < ur.e) issue(u + ur.s, s ^ 1);
-            cp_async_commit();
-            cp_async_wait<1>();
-        } else {
-            issue(u, 0);
-            cp_async_commit();
-            cp_async_wait<0>();
-        }
+        cp_async_commit();
+        cp_async_wait<0>();
         warp_sync();
-        const float4* sq = (const float4*)(slots + (size_t)s * SLOT);
-        const float* st = (const float*)(sq + K * H1);
         // the two rows' half spectra -> one complex line (real part row r0)
 #pragma unroll
         for (int f = 0; f < K; f++) {
@@ -1013,24 +993,22 @@ __device__ void row_pass_staged(const Params& P, const Tw& tw, const float2* src
         }
         warp_sync();
     }
-    cp_async_wait<0>();
-    warp_sync();
 }
 
-template <int NF, int K, int NS, int SLOTS, class Ap>
+template <int NF, int K, int NS, class Ap>
 __device__ void col_pass_staged(const Params& P, const Tw& tw, const float2* src, float2* dst,
                                 const float2* const* sc, char* smem, Ap&& ap) {
     constexpr int LOGN = ilog2c(NF), PP = padded_len(NF), E = NF / kWarp;
-    constexpr int SLOT = (K + NS) * NF * 8;  // bytes
     const int ncols = P.ncols;
     const long long Hs = P.H;
     const WarpCtx w = warp_ctx(P, smem);
     float2* B0 = (float2*)w.mem;
     float2* B1 = B0 + K * PP;
-    char* slots = (char*)(B1 + K * PP);
+    float2* const sl = B1 + K * PP;
+    const float2* const st = sl + K * NF;
     const URange ur = units_of(tw, ncols);
-    auto issue = [&](int k1, int s) {
-        float2* sl = (float2*)(slots + (size_t)s * SLOT);
+    for (int k1 = ur.b; k1 < ur.e; k1 += ur.s) {
+        const Line ln = line_of(P, tw, k1);
 #pragma unroll
         for (int f = 0; f < K; f++)
             for (int j = w.lane; j < NF / 2; j += kWarp)
@@ -1039,24 +1017,9 @@ __device__ void col_pass_staged(const Params& P, const Tw& tw, const float2* src
         for (int a = 0; a < NS; a++)
             for (int j = w.lane; j < NF / 2; j += kWarp)
                 cp_async16(sl + (K + a) * NF + 2 * j, sc[a] + (size_t)k1 * NF + 2 * j);
-    };
-    if (SLOTS == 2 && ur.b < ur.e) issue(ur.b, 0);
-    if (SLOTS == 2) cp_async_commit();
-    int s = 0;
-    for (int k1 = ur.b; k1 < ur.e; k1 += ur.s, s ^= (SLOTS - 1)) {
-        const Line ln = line_of(P, tw, k1);
-        if constexpr (SLOTS == 2) {
-            if (k1 + ur.s < ur.e) issue(k1 + ur.s, s ^ 1);
-            cp_async_commit();
-            cp_async_wait<1>();
-        } else {
-            issue(k1, 0);
-            cp_async_commit();
-            cp_async_wait<0>();
-        }
+        cp_async_commit();
+        cp_async_wait<0>();
         warp_sync();
-        const float2* sl = (const float2*)(slots + (size_t)s * SLOT);
-        const float2* st = sl + K * NF;
         const int r = fft_lines_fixed_into_padded<-1, float, LOGN, K>(sl, NF, B0, B1, PP, K, tw.t32, tw.log, w.lane);
         float2* Xr = r ? B1 : B0;
         float2* Xi = r ? B0 : B1;
@@ -1085,8 +1048,6 @@ __device__ void col_pass_staged(const Params& P, const Tw& tw, const float2* src
         }
         warp_sync();
     }
-    cp_async_wait<0>();
-    warp_sync();
 }
 
 // ------------------------------------------- staged passes by pairs of warps
@@ -1732,9 +1693,9 @@ __device__ void col_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
     }
 }
 
-// Only passes with an FP64 line have the cooperative variant: an FP32 line is
-// latency-bound, not rate-bound, on one sub-partition, and the extra code
-// costs the FP32 passes registers.
+// By default only passes with an FP64 line have the variant of shared lines:
+// their integer butterflies are most of a unit's time and split well; the FP32
+// passes stage their inputs, and pairs of warps share them on small grids.
 template <class TI, class TO> constexpr bool kHasCoop = sizeof(TI) == 8 || sizeof(TO) == 8;
 // NF | kNoCoop: line length NF without the cooperative variants (batched
 // launches, whose warps own their units, never use them)
@@ -2519,7 +2480,7 @@ __device__ __forceinline__ void row_point(const RowK<T>& q, T* dcur, long long p
 template <int NF, bool PFC>
 __device__ __noinline__ void phase_R_staged(const Params& P, const Ctl& c, const Tw& tw, char* smem,
                                             const float2* src) {
-    constexpr int K = PFC ? 1 : 2, NS = staged_row_state(PFC ? 0 : 1), SL = staged_slots(PFC ? 0 : 1);
+    constexpr int K = PFC ? 1 : 2, NS = staged_row_state(PFC ? 0 : 1);
     const RowK<float> q = row_consts<float>(P, c);
     const int bank = c.step & 1;
     float* dcur = (float*)P.DD[c.it & 1];
@@ -2537,7 +2498,7 @@ __device__ __noinline__ void phase_R_staged(const Params& P, const Ctl& c, const
             return;
         }
     }
-    row_pass_staged<NF, K, NS, SL>(P, tw, src, (float2*)P.NB, sp, smem, pt);
+    row_pass_staged<NF, K, NS>(P, tw, src, (float2*)P.NB, sp, smem, pt);
     publish_eval(P, tw, !P.coop, bank, c.ev, amax, asum);  // coop: one warp of the CTA
 }
 
@@ -2686,7 +2647,7 @@ __device__ __forceinline__ void col_point(const Params& P, const ColK<T>& q, cx<
 // fields out (PFC: the direction; FCH: also the Laplacian of ybar_{it+1}).
 template <int NF, bool PFC>
 __device__ __noinline__ void phase_CI_staged(const Params& P, const Ctl& c, const Tw& tw, char* smem) {
-    constexpr int K = PFC ? 1 : 2, SL = staged_slots(PFC ? 0 : 1);
+    constexpr int K = PFC ? 1 : 2;
     const ColK<float> q = col_consts<float>(P, c);
     float2* sprev = (float2*)P.SS[(c.it - 1) & 1];
     const float2* sc3[3] = {(const float2*)P.SS[c.it & 1], sprev, (const float2*)P.C0};
@@ -2699,7 +2660,7 @@ __device__ __noinline__ void phase_CI_staged(const Params& P, const Ctl& c, cons
             return;
         }
     }
-    col_pass_staged<NF, K, 3, SL>(P, tw, csrcT<float>(P), cdstT<float>(P), sc3, smem, pt);
+    col_pass_staged<NF, K, 3>(P, tw, csrcT<float>(P), cdstT<float>(P), sc3, smem, pt);
 }
 
 template <int L> __device__ __forceinline__ void phase_CI_staged_of(const Params& P, const Ctl& c, const Tw& tw, char* smem) {
@@ -3608,11 +3569,11 @@ __host__ __device__ inline int unit_cost(const Params& P, int ph) {
 }
 // Device time per point of a member's current phase, in units of a PFC FP32
 // iteration pass, measured on GB300 with pure phases of batched launches.
-// PFC (96 members): exact base row / column passes 8.8x / 7.8x, incremental
-// ones ~2/3 of that, the last step's accept 5x.  FCH (8 members of 512^2): its
-// iteration passes carry two fields, about 2x a PFC pass per point; relative
-// to them, exact base passes 4.5-5x, incremental B / C / D / E
-// 4.0 / 2.3 / 1.7 / 3.2x, accept 1.5x.  The batched
+// PFC (96 members): exact base passes 5-6x, incremental ones 5x, the last step's
+// accept 2x (8.8x, 6x and 5x while lines were transformed in FP64).  FCH (8
+// members of 512^2): its iteration passes carry two fields, about 2x a PFC pass
+// per point; relative to them, exact base passes 4.5-5x, incremental B / C / D /
+// E 4.0 / 2.3 / 1.7 / 3.2x, accept 1.5x.  The batched
 // launch lays members out on a cost axis of points x this weight, so that a
 // global phase mixing members in FP64 base evaluations with members in FP32
 // iterations gives every warp about the same time of work.  Only the dealing
