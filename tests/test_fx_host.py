@@ -94,3 +94,23 @@ def test_ranges_and_non_finite_lines(emu, n):
         u = np.zeros(n)
         u[3, 2] = bad
         assert np.all(np.isnan(S.fft_r2c(u)))
+
+
+@pytest.mark.parametrize("n", [(64, 64), (128, 64), (64, 128)])
+def test_pair_passes_match_the_warp_passes(emu, monkeypatch, n):
+    """The FCH staged passes of two warps per unit and the lines shared by a CTA
+    (PAGD_COOP=1) against one warp per unit: two solves accepted at
+    ||d|| <= tol differ by at most about 2 tol / (1 - q), q <= 0.9: 20 tol."""
+    tol, out = 1e-8, []
+    rng = np.random.default_rng(3)
+    u0 = -0.3 + 0.05 * rng.uniform(-1, 1, n)
+    for coop in ("0", "1"):
+        monkeypatch.setenv("PAGD_COOP", coop)
+        S = pagd.Solver("fch", n, tuple(v * 4 * np.pi / 256 for v in n), 0.1, 0.1, 0.1, scheme="bdf2",
+                        precision="fp32_mixed", lib=emu)
+        assert S.launch_info()["coop"] == int(coop) and S.launch_info()["staged"]
+        S.set_state(u0)
+        o = S.empty_field()
+        S.run(1e-3, 2, tol, o)
+        out.append(o.copy())
+    assert np.abs(out[0] - out[1]).max() <= 20 * tol
