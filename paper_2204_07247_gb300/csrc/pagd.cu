@@ -417,8 +417,14 @@ static void make_plan(pagd_solver* s) {
     // fewer units than half the warps: most warps would otherwise idle and a
     // unit's pointwise FP64 work and integer butterflies run on one SM
     // sub-partition.
-    // PAGD_COOP=0 / 1 overrides the choice.
-    s->coop = 2 * units <= (long long)s->grid * wpb ? 1 : 0;
+    // PAGD_COOP=0 / 1 overrides the choice.  3D grids of other lengths than 64
+    // to 512 with more units than SMs keep a warp per unit: their short lines
+    // gain less from sharing than the rounds cost (32^3, 544 units, two steps of
+    // PFC FP64: 1479 us shared, 803 with a warp per unit).
+    s->coop = 2 * units <= (long long)s->grid * wpb &&
+                      (s->dim == 2 || units <= sms || fixed_len(s->n[0], s->n[last]) != 0)
+                  ? 1
+                  : 0;
     if (const char* e = std::getenv("PAGD_COOP")) {
         if ((e[0] == '0' || e[0] == '1') && e[1] == 0) s->coop = e[0] - '0';
     }
