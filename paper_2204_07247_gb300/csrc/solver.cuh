@@ -1355,6 +1355,8 @@ __device__ void col_pass_fx(const Params& P, const Tw& tw, int kin, int kout, co
                 }
             }
         }
+        // the FP32 lines lie in the third line's slots: every lane has read its own there
+        if constexpr (sizeof(TO) == 4) warp_sync();
 #pragma unroll 1
         for (int g = 0; g < kout; g++) {
             longlong2* b = B + g * n;

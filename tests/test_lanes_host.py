@@ -1,0 +1,75 @@
+"""The passes of csrc/solver.cuh with every thread of a CTA as a fiber of its own
+(tests/lanes): between two barriers a whole lane runs before the next one, in
+either order, and a shuffle orders no memory.  A hand-over through shared memory
+without a barrier gives wrong results here; on a GPU it may or may not.
+
+Tolerances: an FP32 line is transformed forward and back, 2 log2(n) stages of at
+most 2^-23 relative each to the largest value: 18 2^-23 < 2.2e-6 for 512 points,
+3e-6 with the conversions; an FP64 one 18 2^-52: 4e-15."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2204_07247_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def lanes(tmp_path_factory):
+    d = str(tmp_path_factory.mktemp("lanes"))
+    for src in (CSRC, os.path.join(HERE, "lanes")):  # the latter's compat.cuh replaces the former's
+        for f in os.listdir(src):
+            if f.endswith((".cuh", ".cpp")):
+                shutil.copy(os.path.join(src, f), d)
+    so = os.path.join(d, "liblanes.so")
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-w", "-fno-strict-aliasing", "-fPIC", "-shared", "-o", so,
+                           os.path.join(d, "lanes.cpp")])
+    return ctypes.CDLL(so)
+
+
+def ptr(a):
+    return ctypes.c_void_p(a.ctypes.data)
+
+
+def spectrum(k, lead, rows, seed):
+    """k fields of half spectra [field][lead][rows], real in the first and last of lead"""
+    r = np.random.default_rng(seed)
+    s = r.uniform(-1, 1, (k, lead, rows)) + 1j * r.uniform(-1, 1, (k, lead, rows))
+    s[:, [0, -1]] = s[:, [0, -1]].real
+    return s
+
+
+PASSES = [("col_sum_fx", 3), ("col_sum_coop_fx", 3), ("row_fx", 3), ("row_coop_fx", 3), ("col_fx", 3), ("col_coop_fx", 3),
+          ("row_coop", 2), ("col_coop", 2), ("mid_fx_fwd", 2), ("mid_fx_inv", 2), ("row_staged", 1), ("row_staged", 2),
+          ("col_staged", 1), ("col_staged", 2), ("row_pair", 2), ("col_pair", 2), ("mid_staged_fwd", 2), ("mid_staged_inv", 2)]
+# (points of a line, compile-time length or 0; the staged passes have compile-time lengths only)
+CASES = [(p, k, n, nf) for p, k in PASSES for n, nf in [(8, 0), (16, 0), (32, 0), (64, 0), (64, 64), (512, 512)]
+         if nf or not ("staged" in p or "pair" in p)]
+
+
+@pytest.mark.parametrize("up", [1, 0])
+@pytest.mark.parametrize("name,k,n,nf", CASES)
+def test_passes_do_not_depend_on_the_order_of_lanes(lanes, name, k, n, nf, up):
+    if name[0] == "r":      # [k][n / 2 + 1][8 rows]: inverse and forward along n, scaled by 1 / (8 n)
+        src = spectrum(k, n // 2 + 1, 8, n)
+        want = src / 8
+    elif name[0] == "c":    # [k][5 lines][n]: forward and inverse along n
+        src = spectrum(k, 5, n, n)
+        want = src * n
+        if "sum" in name:
+            want = np.concatenate([want.sum(0, keepdims=True), np.zeros((k - 1,) + want.shape[1:])])
+    else:                   # [k][5 planes][8 lines][n] <-> [k][5][n][8]
+        src = spectrum(k, 5, 8 * n, n)
+        if "fwd" in name:
+            want = np.swapaxes(np.fft.fft(src.reshape(k, 5, 8, n)), 2, 3)
+        else:
+            want = n * np.fft.ifft(np.swapaxes(src.reshape(k, 5, n, 8), 2, 3))
+    src = np.ascontiguousarray(src)
+    dst = np.zeros_like(src)
+    assert lanes.lanes_pass(name.encode(), n, nf, k, up, ptr(src), ptr(dst)) == 1
+    tol = 4e-15 if name.endswith("_fx") and "sum" not in name or "mid_fx" in name else 3e-6
+    assert np.abs(dst - want.reshape(dst.shape)).max() <= tol * np.abs(want).max()
