@@ -414,6 +414,7 @@ __device__ __forceinline__ void publish_group(const Tw& tw, bool all, unsigned l
         __threadfence_block();
     }
     if (!warp_bcast(last)) return;
+    warp_sync();  // the other lanes' reads come after lane 0's fence (a shuffle orders no memory)
     const bool in = (unsigned)lane < nw;
     unsigned long long mt = in ? cr->m[lane] : 0ull;
     double t[N];

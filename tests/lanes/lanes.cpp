@@ -118,4 +118,18 @@ int lanes_pass(const char* pass, int n, int nf, int k, int up, const double* src
     }
     return 0;
 }
+// publish_group by one CTA of nw warps: maximum and sums of the warps' values
+int lanes_publish(int nw, int up, const unsigned long long* m, const double* v, unsigned long long* mo, double* vo) {
+    gridDim.x = kFewCtas + 1;
+    *mo = 0;
+    for (int i = 0; i < 3; i++) vo[i] = 0.0;
+    return emu_cta(nw * 32, up != 0, sizeof(CtaRed), [&](int t) {
+        Tw tw{};
+        tw.cr = (CtaRed*)emu_region();
+        double* const a[3] = {vo, vo + 1, vo + 2};
+        const int w = t / 32;
+        const double x[3] = {v[3 * w], v[3 * w + 1], v[3 * w + 2]};
+        publish_group<3>(tw, true, mo, m[w], a, x);
+    });
+}
 }

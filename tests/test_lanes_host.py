@@ -73,3 +73,13 @@ def test_passes_do_not_depend_on_the_order_of_lanes(lanes, name, k, n, nf, up):
     assert lanes.lanes_pass(name.encode(), n, nf, k, up, ptr(src), ptr(dst)) == 1
     tol = 4e-15 if name.endswith("_fx") and "sum" not in name or "mid_fx" in name else 3e-6
     assert np.abs(dst - want.reshape(dst.shape)).max() <= tol * np.abs(want).max()
+
+
+@pytest.mark.parametrize("up", [1, 0])
+@pytest.mark.parametrize("warps", [1, 3, 8])
+def test_a_cta_publishes_what_its_warps_hold(lanes, warps, up):
+    m = np.arange(1, warps + 1, dtype=np.uint64)[::-1].copy()
+    v = np.arange(3.0 * warps).reshape(warps, 3) + 0.5
+    mo, vo = np.zeros(1, np.uint64), np.zeros(3)
+    assert lanes.lanes_publish(warps, up, ptr(m), ptr(v), ptr(mo), ptr(vo)) == 1
+    assert mo[0] == warps and np.array_equal(vo, v.sum(0))  # small whole and half numbers: exact
