@@ -143,21 +143,24 @@ __device__ __forceinline__ int fx_scale(int emax, int sh) { return emax == 0x7ff
 
 // FP64 <-> FP32 conversions with integer instructions: the hardware's issue
 // at the FP64 rate (64 cycles per warp and sub-partition), these are about
-// nine integer instructions each.  Rounded to nearest even; FP32 results below 2^-126
-// become zero, as do FP32 inputs below 2^-126.
+// ten integer instructions each.  The same values, rounded to nearest even;
+// subnormal FP32 numbers, which need a shift by the value, go through the
+// hardware's.
 __device__ __forceinline__ float to_f32(double x) {
     const unsigned long long b = dbl_bits(x), m = b & 0x7fffffffffffffffull;
     const unsigned hi = (unsigned)(m >> 32);
+    if (hi - 0x36900000u < 0x01800000u) return (float)x;  // 2^-150 <= |x| < 2^-126
     const unsigned long long t = m - (896ull << 52);
     unsigned r = (unsigned)((t + 0x0fffffffull + ((t >> 29) & 1ull)) >> 29);
-    if (hi < 0x38100000u) r = 0u;                                   // below 2^-126
+    if (hi < 0x38100000u) r = 0u;                                   // below 2^-150
     if (hi >= 0x47f00000u) r = m > 0x7ff0000000000000ull ? 0x7fc00000u : 0x7f800000u;  // 2^128 and above, inf, NaN
     return bits_flt(r | ((unsigned)(b >> 32) & 0x80000000u));
 }
 __device__ __forceinline__ double to_f64(float x) {
     const unsigned b = flt_bits(x), m = b & 0x7fffffffu;
+    if (m - 1u < 0x007fffffu) return (double)x;
     unsigned hi = (m >> 3) + (896u << 20), lo = m << 29;
-    if (m < 0x00800000u) { hi = 0u; lo = 0u; }
+    if (m == 0u) hi = 0u;
     if (m >= 0x7f800000u) hi += 896u << 20;  // inf, NaN
     hi |= b & 0x80000000u;
     return bits_dbl(((unsigned long long)hi << 32) | lo);
