@@ -2622,10 +2622,9 @@ __device__ __forceinline__ void col_point(const Params& P, const ColK<T>& q, cx<
     const C yh = C{sc.x + q.l * (sc.x - sp.x), sc.y + q.l * (sc.y - sp.y)};
     C d{(T)0, (T)0};
     if (kap != (T)0) {
-        // 1 / kappa and 1 / L = kappa / den from one reciprocal
-        const T den = q.m2 + kap * (q.b0 + kap * (q.b2 + kap * q.b4));
-        const T r = rcp64(kap * den);
-        const T ik = r * den, il = -(r * kap) * kap;
+        // (one reciprocal of kappa^2 L for both overflows in FP32 from kappa = 4e9)
+        const T ik = rcp64(kap);
+        const T il = -rcp64(q.m2 * ik + (q.b0 + kap * (q.b2 + kap * q.b4)));
         if (PFC) {
             const T m = q.aim * ik + (q.c0 + kap * (kap - (T)2));
             d.x = il * (g0.x + m * yh.x + in[0].x);

@@ -1,0 +1,23 @@
+"""Grids far from the usual spacing, through the CPU emulation: the FP32 iteration
+passes carry wavenumbers up to kappa = 1e13 (their squares are FP32 numbers) and
+take as many evaluations there as on an ordinary domain."""
+import numpy as np
+import pytest
+
+from paper_2204_07247_gb300 import pagd
+
+
+@pytest.mark.parametrize("n", [(16, 16), (64, 64)])
+@pytest.mark.parametrize("model,eta", [("pfc", 0.0), ("fch", 0.1)])
+def test_small_domains_iterate_like_ordinary_ones(model, eta, n):
+    evals = []
+    for L in (0.01, 1e-3, 1e-5):
+        S = pagd.Solver(model, n, (L, L), 0.1, eta, eta, scheme="bdf2", precision="fp32_mixed",
+                        lib=pagd.load_emulation())
+        S.set_state(0.1 + 0.05 * np.random.default_rng(0).uniform(-1, 1, n))
+        it, res = S.run(0.1, 2, 1e-10, S.empty_field())
+        assert np.all(res <= 1e-10)
+        evals.append(np.array(it))
+    # every mode but the mean decays at once on each of them: the same steps, up
+    # to one evaluation of rounding
+    assert max(np.abs(e - evals[0]).max() for e in evals) <= 1, evals
