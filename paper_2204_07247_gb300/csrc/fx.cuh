@@ -169,17 +169,27 @@ __device__ __forceinline__ double to_f64(float x) {
 // division takes 364 cycles, six times one): an FP32 reciprocal of the
 // significand, then one step of Newton's iteration for 1 / x with its next
 // term, x0 (1 + e + e^2) with e = 1 - m x0 (|e| <= 2^-21, so e^3 is below the
-// rounding), and the exponent by integer arithmetic.  Other x: the division.
+// rounding), and the exponent by integer arithmetic: within 0.501 ulp, the
+// division 0.5.  Other x (rcp_plain): the division.
+__device__ __forceinline__ bool rcp_plain(double x) { return (unsigned)(dbl_bits(x) >> 32) - 0x00100000u >= 0x7fa00000u; }
 __device__ __forceinline__ double rcp64(double x) {
+    if (rcp_plain(x)) return 1.0 / x;
     const unsigned long long b = dbl_bits(x);
     const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
-    if (hi - 0x00100000u >= 0x7fa00000u) return 1.0 / x;
     const float m = bits_flt(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
     const double x0 = to_f64(1.0f / m), md = bits_dbl((b & 0xfffffffffffffull) | 0x3ff0000000000000ull);
     const double e = fma(-md, x0, 1.0), y = fma(x0, fma(e, e, e), x0);
     return bits_dbl(dbl_bits(y) + ((unsigned long long)(1023u - (hi >> 20)) << 52));
 }
 __device__ __forceinline__ float rcp64(float x) { return 1.0f / x; }
+// a / x and b / x: the product with the reciprocal, corrected by its remainder
+// (Markstein 1990), within 0.501 ulp where the plain product has 1
+__device__ __forceinline__ double2 div64(double2 n, double x) {
+    if (rcp_plain(x)) return double2{n.x / x, n.y / x};
+    const double r = rcp64(x);
+    const double2 q{n.x * r, n.y * r};
+    return double2{fma(fma(-x, q.x, n.x), r, q.x), fma(fma(-x, q.y, n.y), r, q.y)};
+}
 template <class T> __device__ __forceinline__ T cvt(double x) {
     if constexpr (sizeof(T) == 8) return x;
     else return to_f32(x);

@@ -171,7 +171,6 @@ static Params params_for(const pagd_solver* s, char* w) {
     P.eta2 = s->eta2;
     P.tau = s->tau;
     P.M = s->M;
-    P.iM = 1.0 / s->M;
     P.s = s->opts.s;
     P.n_eta = s->opts.n_eta;
     P.accel = s->opts.accel;

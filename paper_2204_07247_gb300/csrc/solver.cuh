@@ -100,7 +100,7 @@ struct Params {
     double k0sq, k1sq, kmsq;  // (2 pi / L)^2 of the first, last and middle axes
     float k0sqf, k1sqf, kmsqf;
     double cellvol;           // product of the spacings
-    double eps, eta1, eta2, tau, M, iM;  // iM = 1 / M
+    double eps, eta1, eta2, tau, M;
     double s;
     int n_eta, accel, max_iter, max_recheck, theta_mode;
     // the PFC FP32 iteration passes stage their inputs by asynchronous copies
@@ -2204,25 +2204,29 @@ __device__ PAGD_COLD void phase_B_inc(const Params& P, const Ctl& c, const Tw& t
 
 // Spectral base gradient C0 = G'_N(VB) (Eqs. misc07 / obj:G'), its
 // preconditioned direction d0 and the first correction delta_1 = theta_v s d0.
-// kappa G = w / M + kappa (rest), with w = A_i v_hat + g_hat and the rest of G
-// in t; the preconditioner is L = den / kappa.  One reciprocal, of kappa den,
-// gives both 1 / kappa and 1 / L (an FP64 division costs as much as six
-// products, and every FP64 instruction 19 SM cycles per warp).
-__device__ __forceinline__ double precond_den(const Beta& B, double kap) {
-    return fma(kap, fma(kap, fma(kap, B.b4, B.b2), B.b0), B.m2);
+// G = w / (M kappa) + t with w = A_i v_hat + g_hat, d = -G / L, and the
+// preconditioner L = a / (M kappa) + beta_0 + beta_2 kappa + beta_4 kappa^2.
+// 1 / (M kappa) is rounded twice (the product and the reciprocal), as 1 / M
+// divided by kappa is, and serves both.  (rcp64 takes three FP64 instructions,
+// of 19 SM cycles per warp each, a division as much as six.)
+struct Precond {
+    double ik, L;
+};
+__device__ __forceinline__ Precond precond64(double a, double M, const Beta& B, double kap) {
+    const double ik = rcp64(M * kap);
+    return Precond{ik, fma(a, ik, fma(kap, fma(kap, B.b4, B.b2), B.b0))};
 }
 template <class T>
-__device__ __forceinline__ void base_direction(const Params& P, const StepK& k, const Beta& B, double iM, long long idx,
-                                               double kap, double2 w, double2 t, double2& d) {
+__device__ __forceinline__ void base_direction(const Params& P, const StepK& k, const Beta& B, long long idx, double kap,
+                                               double2 w, double2 t, double2& d) {
     double2 G{0.0, 0.0};
     d = double2{0.0, 0.0};
     if (dbl_bits(kap) != 0ull) {
-        const double den = precond_den(B, kap);
+        const Precond p = precond64(k.a, P.M, B, kap);
         // not positive, or a NaN
-        if (dbl_bits(den) - 1ull >= 0x7ff0000000000000ull) atomicOr(&P.sc->flags, FLAG_PRECOND);
-        const double r = rcp64(kap * den);
-        const double ik = r * den * iM, il = -(r * kap) * kap;
-        G = double2{fma(w.x, ik, t.x), fma(w.y, ik, t.y)};
+        if (dbl_bits(p.L) - 1ull >= 0x7ff0000000000000ull) atomicOr(&P.sc->flags, FLAG_PRECOND);
+        const double il = -rcp64(p.L);
+        G = double2{fma(w.x, p.ik, t.x), fma(w.y, p.ik, t.y)};
         d = double2{il * G.x, il * G.y};
     }
     ((cx<T>*)P.C0)[idx] = cx<T>{cvt<T>(G.x), cvt<T>(G.y)};
@@ -2240,7 +2244,6 @@ __device__ PAGD_COLD void phase_C(const Params& P, const Ctl& c, const Tw& tw, c
     const StepK& k = step_coeffs(P, c.step);
     const Beta B = c.bt;
     const int kb = k_base(P.model);
-    const double iM = P.iM;
     const bool gcached = c.ereb && c.gok;  // g_hat from GH64, not among the inputs
     const int kin = gcached ? kb - 1 : kb;
     auto ldg_hat = [&](const Line& k1, int k0) {
@@ -2261,7 +2264,7 @@ __device__ PAGD_COLD void phase_C(const Params& P, const Ctl& c, const Tw& tw, c
                                  P.WR64[idx] = w;
                                  const double Lh = fma(kap, kap - 2.0, c0);
                                  double2 d;
-                                 base_direction<T>(P, k, B, iM, idx, kap, w,
+                                 base_direction<T>(P, k, B, idx, kap, w,
                                                    double2{fma(Lh, v.x, nl.x), fma(Lh, v.y, nl.y)}, d);
                                  out[0] = cx<T>{cvt<T>(d.x), cvt<T>(d.y)};
                              });
@@ -2301,7 +2304,7 @@ template <class T, int NF>
 __device__ PAGD_COLD void phase_E(const Params& P, const Ctl& c, const Tw& tw, char* smem) {
     const StepK& k = step_coeffs(P, c.step);
     const Beta B = c.bt;
-    const double e2 = P.eps * P.eps, e4 = e2 * e2, iM = P.iM;
+    const double e2 = P.eps * P.eps, e4 = e2 * e2;
     const double fl = -(1.0 + lam_at(P, 1)) * k.ts;
     struct St { double2 v, w; };
     // the direction (and Lap of the first correction) are small: inverse in T
@@ -2317,7 +2320,7 @@ __device__ PAGD_COLD void phase_E(const Params& P, const Ctl& c, const Tw& tw, c
                              P.NR64[idx + P.H] = in[1];
                              const double q = e4 * kap * kap, r = e2 * kap;
                              double2 d;
-                             base_direction<T>(P, k, B, iM, idx, kap, s.w,
+                             base_direction<T>(P, k, B, idx, kap, s.w,
                                                double2{fma(q, s.v.x, fma(r, in[0].x, in[1].x)),
                                                        fma(q, s.v.y, fma(r, in[0].y, in[1].y))}, d);
                              out[0] = cx<T>{cvt<T>(d.x), cvt<T>(d.y)};
@@ -2342,7 +2345,7 @@ __device__ PAGD_COLD void phase_CN(const Params& P, const Ctl& c, const Tw& tw, 
     const int kb = k_base(P.model);
     const int kin = reb ? kb - 1 : kb;
     const int o = reb ? 0 : 1;  // in[o] = y_hat, in[o + 1] = dN_hat (PFC), in[0] = W_hat (new step)
-    const double iM = P.iM, Ai = k.Ai, c0 = 1.0 - P.eps;
+    const double Ai = k.Ai, c0 = 1.0 - P.eps;
     const bool pfc = P.model == M_PFC;
     struct St { double2 v, n, w; };
     colp<T, NF, true>(
@@ -2367,10 +2370,10 @@ __device__ PAGD_COLD void phase_CN(const Params& P, const Ctl& c, const Tw& tw, 
                 P.NR64[idx] = nl;
                 const double Lh = fma(kap, kap - 2.0, c0);
                 double2 d;
-                base_direction<T>(P, k, B, iM, idx, kap, w, double2{fma(Lh, v.x, nl.x), fma(Lh, v.y, nl.y)}, d);
+                base_direction<T>(P, k, B, idx, kap, w, double2{fma(Lh, v.x, nl.x), fma(Lh, v.y, nl.y)}, d);
                 out[0] = C{cvt<T>(d.x), cvt<T>(d.y)};
             } else {
-                const T f = -kappa_t<T>(P, k1, k0);
+                const T f = -cvt<T>(kappa_at(P, k1, k0));
                 out[0] = C{f * yt.x, f * yt.y};
             }
         });
@@ -2411,7 +2414,7 @@ __device__ PAGD_COLD void phase_EN(const Params& P, const Ctl& c, const Tw& tw, 
     using C = cx<T>;
     const StepK& k = step_coeffs(P, c.step);
     const Beta B = c.bt;
-    const double e2 = P.eps * P.eps, e4 = e2 * e2, iM = P.iM;
+    const double e2 = P.eps * P.eps, e4 = e2 * e2;
     const double fl = -(1.0 + lam_at(P, 1)) * k.ts;
     const long long H = P.H;
     struct St { double2 f1, pp, v, w; };
@@ -2430,7 +2433,7 @@ __device__ PAGD_COLD void phase_EN(const Params& P, const Ctl& c, const Tw& tw, 
             P.NR64[idx + H] = pp;
             const double q = e4 * kap * kap, r = e2 * kap;
             double2 d;
-            base_direction<T>(P, k, B, iM, idx, kap, s.w,
+            base_direction<T>(P, k, B, idx, kap, s.w,
                               double2{fma(q, s.v.x, fma(r, f1.x, pp.x)), fma(q, s.v.y, fma(r, f1.y, pp.y))}, d);
             out[0] = C{cvt<T>(d.x), cvt<T>(d.y)};
             const double f = fl * kap;
@@ -3009,8 +3012,7 @@ __device__ __forceinline__ double2 imex_solve(const Params& P, const StepK& k, d
         rx -= M * kap * 0.5 * Lh * un.x;
         ry -= M * kap * 0.5 * Lh * un.y;
     }
-    const double den = rcp64(k.a + M * kap * half * Lh);
-    return double2{rx * den, ry * den};
+    return div64(double2{rx, ry}, k.a + M * kap * half * Lh);
 }
 template <int NF>
 __device__ PAGD_COLD void phase_im_c0(const Params& P, const Ctl& c, const Tw& tw, char* smem) {

@@ -1,12 +1,22 @@
-// The number helpers of fx.cuh over arrays: as host code (g++, the emulation's
+// The number helpers of fx.cuh and solver.cuh over arrays: as host code (g++, the emulation's
 // compat.cuh) and, compiled by nvcc, as a kernel per helper.
-#include "fft.cuh"
+#include "solver.cuh"
 
 using namespace pagd;
 
 namespace {
 struct ToF32 { __device__ float operator()(double x) const { return to_f32(x); } };
 struct ToF64 { __device__ double operator()(float x) const { return to_f64(x); } };
+struct Rcp { __device__ double operator()(double x) const { return rcp64(x); } };
+struct Div { __device__ double2 operator()(double2 n) const { return div64(double2{n.x, 1.0}, n.y); } };  // n.x / n.y, 1 / n.y
+// kappa, a / M = 4 / M -> 1 / (M kappa), L
+struct Pre {
+    double M, b0, b2, b4;
+    __device__ double2 operator()(double kap) const {
+        const Precond p = precond64(4.0, M, Beta{4.0 / M, b0, b2, b4}, kap);
+        return double2{p.ik, p.L};
+    }
+};
 
 #ifdef __CUDACC__
 template <class F, class A, class B> __global__ void each(F f, const A* a, B* b, long long n) {
@@ -28,4 +38,7 @@ template <class F, class A, class B> int apply(F f, const A* a, B* b, long long 
 extern "C" {
 int arith_f32(const double* a, float* b, long long n) { return apply(ToF32{}, a, b, n); }
 int arith_f64(const float* a, double* b, long long n) { return apply(ToF64{}, a, b, n); }
+int arith_rcp(const double* a, double* b, long long n) { return apply(Rcp{}, a, b, n); }
+int arith_div(const double2* a, double2* b, long long n) { return apply(Div{}, a, b, n / 2); }
+int arith_pre(const double* a, double2* b, long long n) { return apply(Pre{1.3, 0.7, -2.0, 1.0}, a, b, n / 2); }
 }

@@ -1,6 +1,10 @@
-"""The number helpers of csrc/fx.cuh against IEEE arithmetic: on the CPU through
-the host build of the same source, and on the GPU (marked gpu).  Conversions are
-exact or rounded to nearest even, so they have to agree bit for bit."""
+"""The number helpers of csrc/fx.cuh and solver.cuh against IEEE arithmetic: on
+the CPU through the host build of the same source, and on the GPU (marked gpu).
+
+Conversions are exact or rounded to nearest even, so they have to agree bit for
+bit.  The reciprocal is one rounding of x0 (1 + e + e^2) with |e| <= 2^-21, the
+inner sum's rounding being 2^-53 of e: at most 0.5 + 2^-10 ulp, and 0.501 with the
+rounding of the check itself; the quotient's correction leaves as much."""
 import ctypes
 import os
 import subprocess
@@ -76,6 +80,54 @@ def same(a, b):
     u = np.uint32 if a.dtype == np.float32 else np.uint64
     bad = np.flatnonzero(a.view(u)[~n] != b.view(u)[~n])
     assert bad.size == 0, (a[~n][bad[:4]], b[~n][bad[:4]])
+
+
+def ulps(got, ref):
+    """|got - ref| in units of the last place of ref (extended precision)"""
+    u = np.spacing(np.abs(ref.astype(np.float64)))
+    return np.abs((got.astype(np.longdouble) - ref) / u)
+
+
+def normals(seed=1):
+    """positive normal numbers whose reciprocals are normal, and significands next to 1 and 2"""
+    r = np.random.default_rng(seed)
+    e = np.repeat(np.arange(1, 2042, dtype=np.uint64), 64)
+    m = r.integers(0, 2 ** 52, e.size, dtype=np.uint64)
+    m[::8] >>= np.uint64(40)
+    m[1::8] |= np.uint64(0xffffff0000000)
+    return ((e << np.uint64(52)) | m).view(np.float64)
+
+
+def test_reciprocal(run):
+    x = normals()
+    assert ulps(run("arith_rcp", np.float64, x), 1 / x.astype(np.longdouble)).max() <= 0.501
+    rest = doubles()
+    rest = rest[(rest <= 0) | (rest >= 2.0 ** 1020) | (np.abs(rest) < 2.0 ** -1022) | np.isnan(rest)]
+    with np.errstate(all="ignore"):  # every other number: the division
+        same(run("arith_rcp", np.float64, rest), 1 / rest)
+
+
+def test_quotient(run):
+    x = normals()
+    x = x[(x > 2.0 ** -900) & (x < 2.0 ** 900)]
+    n = np.random.default_rng(2).uniform(-3, 3, x.size) * 2.0 ** np.random.default_rng(3).integers(-60, 60, x.size)
+    got = run("arith_div", np.float64, np.stack([n, x], 1).ravel()).reshape(-1, 2)
+    lx = x.astype(np.longdouble)
+    assert ulps(got[:, 0], n / lx).max() <= 0.501 and ulps(got[:, 1], 1 / lx).max() <= 0.501
+    pairs = np.array([[1.0, np.inf], [0.0, 3.0], [2.0, 0.0], [3.0, -7.0], [1.0, 5e-324], [np.nan, 1.0], [1.0, np.nan]])
+    with np.errstate(all="ignore"):
+        same(run("arith_div", np.float64, pairs.ravel()).reshape(-1, 2)[:, 0].copy(), pairs[:, 0] / pairs[:, 1])
+
+
+def test_preconditioner_factors(run):
+    """1 / (M kappa): two roundings; L: its sum, positive terms but one, against the
+    sum of their magnitudes: six roundings of half an ulp."""
+    kap = np.concatenate([10.0 ** np.random.default_rng(4).uniform(-12, 16, 4000), 10.0 ** np.arange(17, 120, 7.0)])
+    got = run("arith_pre", np.float64, np.concatenate([kap, np.zeros(kap.size)])).reshape(-1, 2)
+    k, M = kap.astype(np.longdouble), np.longdouble(1.3)
+    assert ulps(got[:, 0], 1 / (M * k)).max() <= 1.01 * 2  # relative 2 x 2^-53, up to 2 ulp of a smaller significand
+    terms = np.stack([4 / (M * k), np.full(kap.size, np.longdouble(0.7)), -2 * k, k * k])
+    assert (np.abs(got[:, 1] - terms.sum(0)) / np.abs(terms).sum(0)).max() <= 6 * 2.0 ** -53
 
 
 def test_fp64_to_fp32(run):
