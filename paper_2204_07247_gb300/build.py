@@ -79,7 +79,7 @@ def build_emulation(force: bool = False) -> str:
         return EMU
     tmp = EMU + f".{os.getpid()}.tmp"
     cxx = shutil.which("g++") or "g++"
-    subprocess.check_call([cxx, "-O2", "-std=c++17", "-DPAGD_EMU", "-x", "c++", "-fPIC", "-shared",
+    subprocess.check_call([cxx, "-O2", "-std=c++17", "-ffp-contract=off", "-fno-strict-aliasing", "-DPAGD_EMU", "-x", "c++", "-fPIC", "-shared",
                            "-o", tmp, os.path.join(CSRC, "pagd.cu")])
     os.replace(tmp, EMU)
     return EMU

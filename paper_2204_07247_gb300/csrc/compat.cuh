@@ -48,6 +48,7 @@ inline double bits_dbl(unsigned long long u) { double d; std::memcpy(&d, &u, 8);
 inline unsigned flt_bits(float f) { unsigned u; std::memcpy(&u, &f, 4); return u; }
 inline float bits_flt(unsigned u) { float f; std::memcpy(&f, &u, 4); return f; }
 inline float warp_xor(float v, int) { return v; }
+inline float fadd(float a, float b) { return a + b; }  // (built with -ffp-contract=off)
 #define PAGD_WARP 1
 template <class T> inline T warp_max(T v) { return v; }
 template <class T> inline T warp_sum(T v) { return v; }
@@ -70,6 +71,8 @@ __device__ __forceinline__ unsigned long long dbl_bits(double d) { return (unsig
 __device__ __forceinline__ double bits_dbl(unsigned long long u) { return __longlong_as_double((long long)u); }
 __device__ __forceinline__ unsigned flt_bits(float f) { return __float_as_uint(f); }
 __device__ __forceinline__ float bits_flt(unsigned u) { return __uint_as_float(u); }
+// an addition that is never contracted with a product
+__device__ __forceinline__ float fadd(float a, float b) { return __fadd_rn(a, b); }
 template <class T> __device__ __forceinline__ T warp_xor(T v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 // lane 0's value
 __device__ __forceinline__ unsigned warp_bcast(unsigned v) { return __shfl_sync(0xffffffffu, v, 0); }

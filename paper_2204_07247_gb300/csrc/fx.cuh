@@ -197,25 +197,41 @@ template <class T> __device__ __forceinline__ T cvt(double x) {
 __device__ __forceinline__ double wide(double x) { return x; }
 __device__ __forceinline__ double wide(float x) { return to_f64(x); }
 
-// Sum of FP32 values without FP64 instructions: the rounding error of every
-// addition is kept (Knuth's two-sum) and summed beside it, 2^-48 of the sum of
-// the magnitudes.
-struct Sum2 {
-    float h = 0.f, l = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float s = h + x, v = s - h;
-        l += (h - (s - v)) + (x - v);
-        h = s;
+// Sum of FP32 values without FP64 instructions, to the last place of an FP64
+// one and better: three words, the rounding error of each word's additions
+// (Knuth's two-sum) going into the next (Ogita, Rump and Oishi 2005, SumK), so
+// that 2^-70 of the sum of the magnitudes is left.  Thirteen FP32 additions a
+// value; an FP64 addition with its conversion takes 128 cycles.  Two words (seven
+// additions) left 2^-48, more than the 2^-53 per addition of an FP64 sum.
+// A partial sum above 3.4e38 becomes an infinity, as in FP32.
+struct Sum3 {
+    float h = 0.f, m = 0.f, l = 0.f;
+    // a + b -> a, returns the rounding error
+    static __device__ __forceinline__ float two_sum(float& a, float b) {
+        const float s = fadd(a, b), v = fadd(s, -a), e = fadd(fadd(a, -fadd(s, -v)), fadd(b, -v));
+        a = s;
+        return e;
+    }
+    __device__ __forceinline__ void add(float x) { l = fadd(l, two_sum(m, two_sum(h, x))); }
+    __device__ __forceinline__ void add(const Sum3& o) {
+        add(o.h);
+        l = fadd(l, fadd(two_sum(m, o.m), o.l));
+    }
+    __device__ __forceinline__ double value() const {
+        if ((flt_bits(h) & 0x7f800000u) == 0x7f800000u) return to_f64(h);  // (the errors are NaN)
+        return to_f64(h) + (to_f64(m) + to_f64(l));
     }
     __device__ __forceinline__ double warp_total() const {
-        Sum2 t = *this;
+        Sum3 t = *this;
 #pragma unroll
         for (int o = kWarp / 2; o > 0; o >>= 1) {
-            const float h2 = warp_xor(t.h, o), l2 = warp_xor(t.l, o);
-            t.add(h2);
-            t.l += l2;
+            Sum3 u;
+            u.h = warp_xor(t.h, o);
+            u.m = warp_xor(t.m, o);
+            u.l = warp_xor(t.l, o);
+            t.add(u);
         }
-        return (double)t.h + (double)t.l;
+        return t.value();
     }
 };
 

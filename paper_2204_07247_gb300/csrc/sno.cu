@@ -656,25 +656,23 @@ __global__ void __launch_bounds__(kThr) k_wgrad(SnoDims d, const float* dz, cons
     }
 }
 
-// out[col(j)] = sum over rows of part[row][j], the rounding errors kept (Sum2); lift: the
+// out[col(j)] = sum over rows of part[row][j], without loss (Sum3); lift: the
 // partials [C][3] = (dP0, dP1, db) go to the layout P [C][2], b_P [C]
 constexpr int kSumThr = 1024;
 __global__ void __launch_bounds__(kSumThr) k_sum_rows(const float* part, int rows, int cols, float* out, int lift) {
-    __shared__ float rh[kSumThr / 32][33], rl[kSumThr / 32][33];
+    __shared__ float red[3][kSumThr / 32][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
-    pagd::Sum2 s;
+    pagd::Sum3 s;
     if (j < cols)
         for (int r = w; r < rows; r += kSumThr / 32) s.add(part[(size_t)r * cols + j]);
-    rh[w][lane] = s.h;
-    rl[w][lane] = s.l;
+    red[0][w][lane] = s.h;
+    red[1][w][lane] = s.m;
+    red[2][w][lane] = s.l;
     __syncthreads();
     if (w == 0 && j < cols) {
-        for (int q = 1; q < kSumThr / 32; q++) {
-            s.add(rh[q][lane]);
-            s.l += rl[q][lane];
-        }
+        for (int q = 1; q < kSumThr / 32; q++) s.add(pagd::Sum3{red[0][q][lane], red[1][q][lane], red[2][q][lane]});
         const int o = !lift ? j : (j % 3 < 2 ? 2 * (j / 3) + j % 3 : 2 * lift + j / 3);
-        out[o] = s.h + s.l;
+        out[o] = pagd::to_f32(s.value());
     }
 }
 

@@ -459,9 +459,9 @@ template <> struct MaxAbs<double> {
         return ((unsigned long long)h << 32) | l;
     }
 };
-// sum of T values: FP64 as they are, FP32 by Sum2
+// sum of T values: FP64 as they are, FP32 by Sum3
 template <class T> struct SumOf;
-template <> struct SumOf<float> : Sum2 {};
+template <> struct SumOf<float> : Sum3 {};
 template <> struct SumOf<double> {
     double v = 0.0;
     __device__ __forceinline__ void add(double x) { v += x; }
@@ -2094,7 +2094,7 @@ __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, cons
         P.stats[c.step - 1].used_guess = c.acc_used;
         P.sc->steps_done = c.step;
     }
-    Sum2 s0, s2;
+    Sum3 s0, s2;
     const float c1e = to_f32(1.0 - P.eps), tauf = to_f32(P.tau), eta1f = to_f32(P.eta1), eta2f = to_f32(P.eta2),
                 e2f = to_f32(P.eps * P.eps);
     const int kb = k_base(P.model);

@@ -17,6 +17,16 @@ struct Pre {
         return double2{p.ik, p.L};
     }
 };
+// the sum of m FP32 values of each of the threads of a warp
+struct Sum {
+    const float* a;
+    int m;
+    __device__ double operator()(int i) const {
+        Sum3 s;
+        for (int q = 0; q < m; q++) s.add(a[(long long)i * m + q]);
+        return s.warp_total();
+    }
+};
 
 #ifdef __CUDACC__
 template <class F, class A, class B> __global__ void each(F f, const A* a, B* b, long long n) {
@@ -40,5 +50,6 @@ int arith_f32(const double* a, float* b, long long n) { return apply(ToF32{}, a,
 int arith_f64(const float* a, double* b, long long n) { return apply(ToF64{}, a, b, n); }
 int arith_rcp(const double* a, double* b, long long n) { return apply(Rcp{}, a, b, n); }
 int arith_div(const double2* a, double2* b, long long n) { return apply(Div{}, a, b, n / 2); }
+int arith_sum(const float* a, const int* i, double* b, long long n, int m) { return apply(Sum{a, m}, i, b, n); }
 int arith_pre(const double* a, double2* b, long long n) { return apply(Pre{1.3, 0.7, -2.0, 1.0}, a, b, n / 2); }
 }

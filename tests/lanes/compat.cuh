@@ -198,6 +198,7 @@ inline unsigned long long dbl_bits(double d) { unsigned long long u; std::memcpy
 inline double bits_dbl(unsigned long long u) { double d; std::memcpy(&d, &u, 8); return d; }
 inline unsigned flt_bits(float f) { unsigned u; std::memcpy(&u, &f, 4); return u; }
 inline float bits_flt(unsigned u) { float f; std::memcpy(&f, &u, 4); return f; }
+inline float fadd(float a, float b) { return a + b; }
 inline int clz32(unsigned v) { return v ? __builtin_clz(v) : 32; }
 inline int clz64(unsigned long long v) { return v ? __builtin_clzll(v) : 64; }
 #define PAGD_WARP 32

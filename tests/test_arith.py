@@ -6,8 +6,10 @@ bit.  The reciprocal is one rounding of x0 (1 + e + e^2) with |e| <= 2^-21, the
 inner sum's rounding being 2^-53 of e: at most 0.5 + 2^-10 ulp, and 0.501 with the
 rounding of the check itself; the quotient's correction leaves as much."""
 import ctypes
+import math
 import os
 import subprocess
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -23,11 +25,13 @@ class Host:
                                "-fPIC", "-shared", "-o", so, os.path.join(HERE, "lanes", "arith.cu")])
         self.lib = ctypes.CDLL(so)
 
-    def __call__(self, fn, out_type, *arrays):
-        out = np.zeros(len(arrays[0]), out_type)
+    warp = 1
+
+    def __call__(self, fn, out_type, *arrays, n=None, extra=()):
+        out = np.zeros(n or len(arrays[0]), out_type)
         keep = [np.ascontiguousarray(a) for a in arrays]
         args = [ctypes.c_void_p(a.ctypes.data) for a in keep]
-        assert getattr(self.lib, fn)(*args, ctypes.c_void_p(out.ctypes.data), ctypes.c_longlong(len(out))) == 0
+        assert getattr(self.lib, fn)(*args, ctypes.c_void_p(out.ctypes.data), ctypes.c_longlong(len(out)), *extra) == 0
         return out
 
 
@@ -39,13 +43,15 @@ class Device:
                                "-shared", "-o", so, os.path.join(HERE, "lanes", "arith.cu")])
         self.lib = ctypes.CDLL(so)
 
-    def __call__(self, fn, out_type, *arrays):
+    warp = 32
+
+    def __call__(self, fn, out_type, *arrays, n=None, extra=()):
         import torch
         dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in arrays]
-        out = torch.from_numpy(np.zeros(len(arrays[0]), out_type)).cuda()
+        out = torch.from_numpy(np.zeros(n or len(arrays[0]), out_type)).cuda()
         torch.cuda.synchronize()
         args = [ctypes.c_void_p(t.data_ptr()) for t in dev]
-        assert getattr(self.lib, fn)(*args, ctypes.c_void_p(out.data_ptr()), ctypes.c_longlong(len(out))) == 0
+        assert getattr(self.lib, fn)(*args, ctypes.c_void_p(out.data_ptr()), ctypes.c_longlong(len(out)), *extra) == 0
         return out.cpu().numpy()
 
 
@@ -128,6 +134,42 @@ def test_preconditioner_factors(run):
     assert ulps(got[:, 0], 1 / (M * k)).max() <= 1.01 * 2  # relative 2 x 2^-53, up to 2 ulp of a smaller significand
     terms = np.stack([4 / (M * k), np.full(kap.size, np.longdouble(0.7)), -2 * k, k * k])
     assert (np.abs(got[:, 1] - terms.sum(0)) / np.abs(terms).sum(0)).max() <= 6 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("kind", ["same sign", "mixed", "cancelling", "wide"])
+def test_sum_no_less_exact_than_fp64(run, kind):
+    """64 sums of 32 x 400 (host: 400) values: within a last place of the
+    exact sum plus 2^-70 of the magnitudes, which is less than FP64 leaves"""
+    m, n = 400, 64 * run.warp
+    r = np.random.default_rng(5)
+    a = r.uniform(0.5, 1, (64, run.warp * m))
+    if kind != "same sign":
+        a *= r.choice([-1, 1], a.shape)
+    if kind == "cancelling":  # pairs of opposite values and a small rest
+        h = a.shape[1] // 2
+        a[:, h:] = -a[:, :h][:, ::-1]
+        a[:, ::7] += 1e-4 * r.uniform(-1, 1, a[:, ::7].shape)
+    if kind == "wide":
+        a *= 2.0 ** r.integers(-60, 60, a.shape)
+    a = a.astype(np.float32)
+    got = run("arith_sum", np.float64, a.ravel(), np.arange(n, dtype=np.int32), n=n, extra=(ctypes.c_int(m),))
+    err = err64 = 0.0
+    for i in range(64):
+        x = a[i].astype(np.float64)
+        ref, mag = math.fsum(x), math.fsum(np.abs(x))
+        e = [float(abs(Fraction(float(g)) - Fraction(ref))) for g in got[i * run.warp:(i + 1) * run.warp]]
+        assert max(e) <= np.spacing(abs(ref)) + 2.0 ** -70 * mag  # (fsum itself is rounded)
+        err = max(err, max(e) / mag)
+        err64 = max(err64, abs(float(np.cumsum(x)[-1]) - ref) / mag)
+    assert err <= err64
+
+
+def test_sum_of_infinities(run):
+    a = np.ones((run.warp, 4), np.float32)
+    for bad, want in ((np.inf, np.inf), (-np.inf, -np.inf), (np.nan, np.nan)):
+        a[0, 1] = bad
+        got = run("arith_sum", np.float64, a.ravel(), np.arange(run.warp, dtype=np.int32), n=run.warp, extra=(ctypes.c_int(4),))
+        same(got, np.full(run.warp, want))
 
 
 def test_fp64_to_fp32(run):
