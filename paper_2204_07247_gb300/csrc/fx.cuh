@@ -92,13 +92,21 @@ __device__ __forceinline__ unsigned fx_hi(double x) { return (unsigned)(dbl_bits
 // exponent field of a line from the largest fx_hi of its values
 __device__ __forceinline__ int fx_emax(unsigned hi) { return (int)(hi >> 20); }
 
-// x in units of 2^(emax - 1083): |result| < 2^61
+// x in units of 2^(emax - 1083): |result| < 2^61.  A subnormal x counts only in
+// a line of values below 2^-960 (emax < 64), which takes a path of its own.
+static __device__ __noinline__ long long fx_from_tiny(double x, int emax) {
+    const unsigned long long b = dbl_bits(x), f = b & 0xfffffffffffffull;
+    const int e = (int)(b >> 52) & 0x7ff;
+    const long long v = (long long)(e == 0 ? (f << 9) >> emax : ((f | 0x10000000000000ull) << 8) >> (emax - e));
+    return (long long)b < 0 ? -v : v;
+}
 __device__ __forceinline__ long long fx_from(double x, int emax) {
+    if (emax < 64) return fx_from_tiny(x, emax);
     const unsigned long long b = dbl_bits(x);
     const int e = (int)(b >> 52) & 0x7ff;
     unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
     int r = emax - e;
-    if (r > 63 || e == 0) r = 63;  // below 2^-62 of the largest: zero
+    if (r > 63) r = 63;  // below 2^-62 of the largest: zero
     const long long v = (long long)((m << 8) >> r);
     return (long long)b < 0 ? -v : v;
 }
@@ -119,8 +127,8 @@ __device__ __forceinline__ long long fx_shr(long long a, int sh, long long half)
 __device__ __forceinline__ long long fx_half(int sh) { return (1ll << sh) >> 1; }
 
 // a 2^-S as a double (round half away), |a| < 2^63.  FAST: S in [kFxLo, kFxUp], where
-// no value overflows or falls below 2^-1022 (else to infinity and zero; NaN
-// for a line marked kFxNaN).
+// no value overflows or falls below 2^-1022 (else to an infinity, to a subnormal
+// number or zero; NaN for a line marked kFxNaN).
 constexpr int kFxLo = -900, kFxUp = 1000;
 template <bool FAST> __device__ __forceinline__ double fx_to_t(long long a, int S) {
     const unsigned long long sgn = (unsigned long long)a & 0x8000000000000000ull;
@@ -129,7 +137,8 @@ template <bool FAST> __device__ __forceinline__ double fx_to_t(long long a, int 
     const unsigned long long n = u << ((lz - 1) & 63);
     const int E = 1085 - lz - S;
     unsigned long long t = ((n + 0x200ull) >> 10) + ((unsigned long long)(unsigned)E << 52);
-    if (u == 0 || (!FAST && E < 0)) t = 0;
+    if (!FAST && E < 0) t = E < -53 ? 0ull : (n + (0x200ull << -E)) >> (10 - E);
+    if (u == 0) t = 0;
     if (!FAST) {
         if (E >= 2046) t = 0x7ff0000000000000ull;
         if (S > kFxNaN / 2) t = 0x7ff8000000000000ull;

@@ -21,3 +21,20 @@ def test_small_domains_iterate_like_ordinary_ones(model, eta, n):
     # every mode but the mean decays at once on each of them: the same steps, up
     # to one evaluation of rounding
     assert max(np.abs(e - evals[0]).max() for e in evals) <= 1, evals
+
+
+@pytest.mark.parametrize("p", [-1000, -1022, -1040, -1060])
+@pytest.mark.parametrize("n", [(8, 8), (16, 128), (256, 32), (8, 512)])
+def test_subnormal_lines(n, p):
+    """Fields around 2^p: the spectrum is the one of the same numbers scaled up, to
+    the last place of a subnormal number: one rounding per point after each of the
+    two passes, the first ones summed by the second."""
+    S = pagd.Solver("pfc", n, (3.0, 5.0), 0.1, lib=pagd.load_emulation())
+    u = (0.1 + np.random.default_rng(1).uniform(-1, 1, n)) * 2.0 ** p
+    up = u * 2.0 ** 900 * 2.0 ** (-p - 900)  # exact
+    want = S.fft_r2c(up) * 2.0 ** p
+    assert np.any(want)
+    tol = (n[0] + 1) * 2.0 ** -1074 + 1e-15 * np.abs(want).max()
+    assert np.abs(S.fft_r2c(u) - want).max() <= tol
+    back = S.fft_c2r(S.fft_r2c(u))
+    assert np.abs(back - u).max() <= 3 * tol
