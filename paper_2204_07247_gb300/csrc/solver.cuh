@@ -2053,6 +2053,11 @@ __host__ __device__ __forceinline__ int k_base(int model) { return model == M_PF
 // linear residual W = A_i VB + g = a x + b u^n + c u^{n-1} (O(u_t)), the shift
 // y = VB_new - VB_old from the reference point, and (PFC) the nonlinear change
 // VB_new^3 - VB_old^3 = y (3 r^2 + 3 r y + y^2), r = VB_old.
+// Unit of the averaged-Newton sums: a value is an FP32 number, the sum of 2^24
+// of them is one in this unit.
+constexpr float kSumUnit = 0x1p-24f;
+constexpr double kSumUnits = 0x1p24;  // in one
+
 template <class T, int NF, bool INC>
 __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, const Tw& tw, char* smem, double* red) {
     using TO = typename std::conditional<INC, T, double>::type;
@@ -2150,11 +2155,11 @@ __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, cons
                 // averaged-Newton sums: preconditioner constants, FP32 is enough
                 const float vf = to_f32(vb);
                 if (pfc) {
-                    s0.add(3.0f * vf * vf + c1e);
+                    s0.add((3.0f * vf * vf + c1e) * kSumUnit);
                 } else {
                     const float f1 = dF1(vf, tauf), f2 = dF2(vf, tauf), f3 = dF3(vf, tauf);
-                    s0.add(f2 * f2 - eta2f * f2 + f3 * f1);
-                    s2.add(e2f * (f2 - eta1f));
+                    s0.add((f2 * f2 - eta2f * f2 + f3 * f1) * kSumUnit);
+                    s2.add((e2f * (f2 - eta1f)) * kSumUnit);
                 }
             }
             P.VB[p] = vb;
@@ -2188,7 +2193,8 @@ __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, cons
         });
     if (!reb) {
         double* const a[3] = {&P.sc->beta_sum[c.bsel][0], &P.sc->beta_sum[c.bsel][1], &P.mass[1]};
-        const double v[3] = {s0.warp_total(), pfc ? 0.0 : s2.warp_total(), acc ? warp_sum(dmass) : 0.0};
+        const double v[3] = {s0.warp_total() * kSumUnits, pfc ? 0.0 : s2.warp_total() * kSumUnits,
+                             acc ? warp_sum(dmass) : 0.0};
         publish_group<3>(tw, true, nullptr, 0ull, a, v);
     }
 }

@@ -38,3 +38,13 @@ def test_subnormal_lines(n, p):
     assert np.abs(S.fft_r2c(u) - want).max() <= tol
     back = S.fft_c2r(S.fft_r2c(u))
     assert np.abs(back - u).max() <= 3 * tol
+
+
+@pytest.mark.parametrize("model,eta,size,dt", [("pfc", 0.0, 1e18, 1e-50), ("pfc", 0.0, 5e18, 1e-50), ("fch", 0.1, 1e9, 1e-60)])
+def test_sums_of_large_values(model, eta, size, dt):
+    """Fields whose averaged-Newton values are FP32 numbers, but not their sum
+    over the grid (3 u^2 and about 45 u^4 against 3.4e38)."""
+    S = pagd.Solver(model, (64, 64), (20.0, 20.0), 0.1, eta, eta, scheme="bdf2", lib=pagd.load_emulation())
+    S.set_state(size * (1 + 0.05 * np.random.default_rng(0).uniform(-1, 1, (64, 64))))
+    _, res = S.run(dt, 1, 1e-13 * size, S.empty_field())
+    assert np.all(res <= 1e-13 * size)
