@@ -48,7 +48,8 @@ struct Setup {
 auto ld_row = [](long long, int, int) { return Nothing{}; };
 auto ld_col = [](const Line&, int) { return Nothing{}; };
 
-template <int NF> bool run(const char* pass, int n, int k, bool up, const double* src, double* dst) {
+// state: scale of the pointwise state that the staged passes add to every field (0: none)
+template <int NF> bool run(const char* pass, int n, int k, bool up, float state, const double* src, double* dst) {
     auto is = [&](const char* s) { return std::strcmp(pass, s) == 0; };
     const bool row = pass[0] == 'r', mid = pass[0] == 'm';
     const int other = 8, warps = (std::strstr(pass, "coop") || std::strstr(pass, "pair")) ? 4 : 2;
@@ -71,11 +72,21 @@ template <int NF> bool run(const char* pass, int n, int k, bool up, const double
         for (int f = 0; f < k; f++) t = cadd(t, in[f]);
         out[0] = float2{(float)t.x, (float)t.y};
     };
-    auto rs = [&](long long, int, int, const float*, const float* in, float* out) { for (int f = 0; f < k; f++) out[f] = in[f]; };
-    auto cs = [&](const Line&, int, const float2*, const float2* in, float2* out) { for (int f = 0; f < k; f++) out[f] = in[f]; };
-    std::vector<float> st((size_t)P.npts);
-    const float* sp[1] = {st.data()};
-    const float2* sc[1] = {s32.data()};
+    auto rs = [&](long long p, int row, int x, const float* sv, const float* in, float* out) {
+        const float bad = p == (long long)row * P.n1 + x ? 0.f : NAN;
+        for (int f = 0; f < k; f++) out[f] = in[f] + sv[f] + bad;
+    };
+    auto cs = [&](const Line& l, int k0, const float2* sv, const float2* in, float2* out) {
+        for (int f = 0; f < k; f++) out[f] = float2{in[f].x + sv[f].x, in[f].y + sv[f].y * (float)(l.l + k0 != 3)};
+    };
+    std::vector<float> st[2];
+    std::vector<float2> sl[2];
+    for (int a = 0; a < 2; a++) {
+        for (long long i = 0; i < P.npts; i++) st[a].push_back(state * (float)((i * 37 + a * 11) % 101));
+        for (size_t i = 0; i < H; i++) sl[a].push_back(float2{state * (float)(i * 41 % 103), state * (float)((i + a) * 43 % 107)});
+    }
+    const float* sp[2] = {st[0].data(), st[1].data()};
+    const float2* sc[2] = {sl[0].data(), sl[1].data()};
     const bool ok = emu_cta(warps * 32, up, 0, [&](int) {
         const Tw t = S.tw(warps);
         if (is("row_fx")) { f32 = false; row_pass_fx<NF>(P, t, k, k, s64, d64, mem, ld_row, rf); }
@@ -90,13 +101,13 @@ template <int NF> bool run(const char* pass, int n, int k, bool up, const double
         else if (is("mid_fx_inv")) { f32 = false; mid_pass_fx<+1, NF>(P, t, k, s64, d64, mem); }
         else if constexpr (NF > 0) {
             if (is("row_staged")) {
-                if (k == 1) row_pass_staged<NF, 1, 1>(P, t, s32.data(), d32.data(), sp, mem, rs);
-                else row_pass_staged<NF, 2, 1>(P, t, s32.data(), d32.data(), sp, mem, rs);
+                if (k == 1) row_pass_staged<NF, 1, 2>(P, t, s32.data(), d32.data(), sp, mem, rs);
+                else row_pass_staged<NF, 2, 2>(P, t, s32.data(), d32.data(), sp, mem, rs);
             } else if (is("col_staged")) {
-                if (k == 1) col_pass_staged<NF, 1, 1>(P, t, s32.data(), d32.data(), sc, mem, cs);
-                else col_pass_staged<NF, 2, 1>(P, t, s32.data(), d32.data(), sc, mem, cs);
-            } else if (is("row_pair")) row_pass_pair<NF, 1>(P, t, s32.data(), d32.data(), sp, mem, rs);
-            else if (is("col_pair")) col_pass_pair<NF, 1>(P, t, s32.data(), d32.data(), sc, mem, cs);
+                if (k == 1) col_pass_staged<NF, 1, 2>(P, t, s32.data(), d32.data(), sc, mem, cs);
+                else col_pass_staged<NF, 2, 2>(P, t, s32.data(), d32.data(), sc, mem, cs);
+            } else if (is("row_pair")) row_pass_pair<NF, 2>(P, t, s32.data(), d32.data(), sp, mem, rs);
+            else if (is("col_pair")) col_pass_pair<NF, 2>(P, t, s32.data(), d32.data(), sc, mem, cs);
             else if (is("mid_staged_fwd")) mid_pass_staged<NF, -1>(P, t, k, s32.data(), d32.data(), mem);
             else if (is("mid_staged_inv")) mid_pass_staged<NF, +1>(P, t, k, s32.data(), d32.data(), mem);
         }
@@ -110,11 +121,11 @@ template <int NF> bool run(const char* pass, int n, int k, bool up, const double
 extern "C" {
 // one pass over k fields of a grid whose transformed axis has n points and the
 // others 8; 1: done
-int lanes_pass(const char* pass, int n, int nf, int k, int up, const double* src, double* dst) {
+int lanes_pass(const char* pass, int n, int nf, int k, int up, double state, const double* src, double* dst) {
     switch (nf) {
-        case 0: return run<0>(pass, n, k, up != 0, src, dst);
-        case 64: return run<64>(pass, n, k, up != 0, src, dst);
-        case 512: return run<512>(pass, n, k, up != 0, src, dst);
+        case 0: return run<0>(pass, n, k, up != 0, (float)state, src, dst);
+        case 64: return run<64>(pass, n, k, up != 0, (float)state, src, dst);
+        case 512: return run<512>(pass, n, k, up != 0, (float)state, src, dst);
     }
     return 0;
 }
@@ -131,5 +142,42 @@ int lanes_publish(int nw, int up, const unsigned long long* m, const double* v, 
         const double x[3] = {v[3 * w], v[3 * w + 1], v[3 * w + 2]};
         publish_group<3>(tw, true, mo, m[w], a, x);
     });
+}
+// The short control path and the whole machine after the phase ph (0: CI, 1: RI)
+// of an iteration: 0: both leave the same state, 1: the short path leaves the
+// decision to the machine (and the state alone), 2: they differ.
+int lanes_ctl(int t64, int ph, int ev, int best_ev, double best, double base, double nrm, double tol, int max_iter, int last) {
+    Setup S(8, 1, 8, 1);
+    Params& P = S.P;
+    P.prog = PROG_RUN;
+    P.precision = t64 ? P_FP64 : P_MIXED;
+    P.tol = tol;
+    P.max_iter = max_iter;
+    P.max_recheck = 16;
+    P.nsteps = last ? 1 : 3;
+    P.nslots = 64;
+    std::vector<unsigned long long> norms(2 * P.nslots, 0);
+    std::vector<double> mass(3, 0.0);
+    P.norms = norms.data();
+    P.mass = mass.data();
+    Ctl c;
+    std::memset((void*)&c, 0, sizeof(c));
+    c.ph = ph ? PH_RI : PH_CI;
+    c.it = 3;
+    c.ev = ev;
+    c.best_ev = best_ev;
+    c.best_nrm = best;
+    c.base_nrm = base;
+    c.reb_nrm = kRebaseRatio * base;
+    c.exact_done = 1;
+    norms[ev] = dbl_bits(nrm);
+    Ctl a, b;
+    std::memcpy((void*)&a, (void*)&c, sizeof(c));
+    std::memcpy((void*)&b, (void*)&c, sizeof(c));
+    const bool fast = t64 ? ctl_fast<double>(P, a) : ctl_fast<float>(P, a);
+    if (!fast) return std::memcmp((void*)&a, (void*)&c, sizeof(c)) == 0 ? 1 : 2;
+    if (t64) ctl_advance<double>(P, b);
+    else ctl_advance<float>(P, b);
+    return std::memcmp((void*)&a, (void*)&b, sizeof(c)) == 0 ? 0 : 2;
 }
 }

@@ -114,3 +114,18 @@ def test_pair_passes_match_the_warp_passes(emu, monkeypatch, n):
         S.run(1e-3, 2, tol, o)
         out.append(o.copy())
     assert np.abs(out[0] - out[1]).max() <= 20 * tol
+
+
+@pytest.mark.parametrize("n", [(64, 64), (128, 64)])
+def test_pair_passes_take_as_many_evaluations(emu, monkeypatch, n):
+    """An exact base evaluation accepts every step, so that a wrong iteration pass
+    costs evaluations rather than accuracy: the forms differ by rounding, one
+    evaluation a step at most."""
+    u0, its = -0.3 + 0.05 * np.random.default_rng(3).uniform(-1, 1, n), []
+    for coop in ("0", "1"):
+        monkeypatch.setenv("PAGD_COOP", coop)
+        S = pagd.Solver("fch", n, tuple(v * 4 * np.pi / 256 for v in n), 0.1, 0.1, 0.1, scheme="bdf2",
+                        precision="fp32_mixed", lib=emu)
+        S.set_state(u0)
+        its.append(np.array(S.run(1e-3, 3, 1e-8, S.empty_field())[0]))
+    assert np.abs(its[0] - its[1]).max() <= 1, its

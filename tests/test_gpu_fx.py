@@ -93,3 +93,19 @@ def test_network_tiles(n, C, L, modes, B):
     rl, rg = SO.loss_and_grad(theta, t(un), t(um), t(tg), 1.0, 20.0, 0.02, C, L, *modes)
     assert abs(loss - rl) <= 1e-5 * abs(rl)
     assert torch.linalg.norm(grad.double().cpu() - rg) <= 1e-4 * torch.linalg.norm(rg)
+
+
+@pytest.mark.parametrize("model,n", [("fch", (64, 64)), ("fch", (64, 512)), ("fch", (256, 256)), ("fch", (512, 512)),
+                                     ("pfc", (512, 512)), ("pfc", (64, 256))])
+def test_small_grid_forms_take_as_many_evaluations(monkeypatch, model, n):
+    """The states agree as long as the iterations converge at all (an exact base
+    evaluation accepts); a wrong iteration pass shows in their number.  The forms
+    differ by rounding: one evaluation a step at most, two for a rebase it moves."""
+    h, its = math.pi / 4 if model == "pfc" else 4 * math.pi / 256, []
+    eta = 0.1 if model == "fch" else 0.0
+    for coop in ("0", "1"):
+        monkeypatch.setenv("PAGD_COOP", coop)
+        S = pagd.Solver(model, n, tuple(h * v for v in n), 0.1, eta, eta, scheme="bdf2", precision="fp32_mixed")
+        S.set_state(dev(I.noisy_field(n, -0.3 if model == "fch" else 0.1, 0.05, 5)))
+        its.append(np.array(S.run(1e-3 if model == "fch" else 0.1, 3, 1e-10, S.empty_field())[0]))
+    assert np.abs(its[0] - its[1]).max() <= 3, its

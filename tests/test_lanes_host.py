@@ -70,9 +70,23 @@ def test_passes_do_not_depend_on_the_order_of_lanes(lanes, name, k, n, nf, up):
             want = n * np.fft.ifft(np.swapaxes(src.reshape(k, 5, n, 8), 2, 3))
     src = np.ascontiguousarray(src)
     dst = np.zeros_like(src)
-    assert lanes.lanes_pass(name.encode(), n, nf, k, up, ptr(src), ptr(dst)) == 1
+    assert lanes.lanes_pass(name.encode(), n, nf, k, up, ctypes.c_double(0), ptr(src), ptr(dst)) == 1
     tol = 4e-15 if name.endswith("_fx") and "sum" not in name or "mid_fx" in name else 3e-6
     assert np.abs(dst - want.reshape(dst.shape)).max() <= tol * np.abs(want).max()
+
+
+@pytest.mark.parametrize("n", [64, 512])
+@pytest.mark.parametrize("axis", ["row", "col"])
+def test_pairs_of_warps_give_the_bits_of_one(lanes, axis, n):
+    """The pair passes do the arithmetic of the staged ones: the same bits, with
+    pointwise state that differs from point to point and field to field."""
+    src = spectrum(2, n // 2 + 1, 8, n) if axis == "row" else spectrum(2, 5, n, n)
+    src, out = np.ascontiguousarray(src), []
+    for form in ("staged", "pair"):
+        dst = np.zeros_like(src)
+        assert lanes.lanes_pass(f"{axis}_{form}".encode(), n, n, 2, 1, ctypes.c_double(0.01), ptr(src), ptr(dst)) == 1
+        out.append(dst)
+    assert np.any(out[0]) and np.array_equal(*out)
 
 
 @pytest.mark.parametrize("up", [1, 0])
@@ -83,3 +97,26 @@ def test_a_cta_publishes_what_its_warps_hold(lanes, warps, up):
     mo, vo = np.zeros(1, np.uint64), np.zeros(3)
     assert lanes.lanes_publish(warps, up, ptr(m), ptr(v), ptr(mo), ptr(vo)) == 1
     assert mo[0] == warps and np.array_equal(vo, v.sum(0))  # small whole and half numbers: exact
+
+
+@pytest.mark.parametrize("t64", [0, 1])
+@pytest.mark.parametrize("last", [0, 1])
+def test_short_control_path_decides_as_the_machine(lanes, t64, last):
+    """ctl_fast: the machine's state after an iteration that goes on, and hands over
+    whenever the norm accepts, moves the base, is not finite or the counts run out."""
+    f = lanes.lanes_ctl
+    f.argtypes = [ctypes.c_int] * 4 + [ctypes.c_double] * 4 + [ctypes.c_int] * 2
+    tol, base, best = 1e-10, 1e-2, 1e-5
+    assert f(t64, 0, 5, 4, best, base, 0.0, tol, 40, last) == 0           # after CI
+    up, down = np.nextafter(tol, 1), np.nextafter(tol, 0)
+    goes_on = {1e-6: 1, best: 1, 1e-3: 1, up: t64, np.nextafter(1e-6 * base, 1): 1, 1e300: 1,
+               tol: 0, down: 0, 0.0: 0, 1e-6 * base: t64, 1.1e300: 0, np.inf: 0, np.nan: 0}
+    for nrm, on in goes_on.items():
+        assert f(t64, 1, 5, 4, best, base, nrm, tol, 40, last) == (0 if on else 1), nrm
+    assert f(t64, 1, 5, 4, best, base, 0.0, 0.0, 40, last) == 1           # tol = 0
+    for ev in range(10, 20):                                              # stagnation: FP32 only
+        assert f(t64, 1, ev, 4, best, base, 1e-4, tol, 40, last) == (0 if t64 or ev + 1 - 4 < 12 else 1)
+    assert f(t64, 1, 38, 37, best, base, 1e-4, tol, 40, last) == 0        # max_iter
+    assert f(t64, 1, 39, 38, best, base, 1e-4, tol, 40, last) == 1
+    assert f(t64, 1, 61, 60, best, base, 1e-4, tol, 100, last) == 0       # slots
+    assert f(t64, 1, 62, 61, best, base, 1e-4, tol, 100, last) == 1
