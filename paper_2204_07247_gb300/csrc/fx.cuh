@@ -92,22 +92,16 @@ __device__ __forceinline__ unsigned fx_hi(double x) { return (unsigned)(dbl_bits
 // exponent field of a line from the largest fx_hi of its values
 __device__ __forceinline__ int fx_emax(unsigned hi) { return (int)(hi >> 20); }
 
-// x in units of 2^(emax - 1083): |result| < 2^61.  A subnormal x counts only in
-// a line of values below 2^-960 (emax < 64), which takes a path of its own.
-static __device__ __noinline__ long long fx_from_tiny(double x, int emax) {
+// x in units of 2^(emax - 1083): |result| < 2^61.  (Subnormal numbers count, in
+// lines of values below 2^-960; the select for them is 1% of a transform.  A
+// branch for such lines, per value or per line, cost 2 to 6%.)
+__device__ __forceinline__ long long fx_from(double x, int emax) {
     const unsigned long long b = dbl_bits(x), f = b & 0xfffffffffffffull;
     const int e = (int)(b >> 52) & 0x7ff;
-    const long long v = (long long)(e == 0 ? (f << 9) >> emax : ((f | 0x10000000000000ull) << 8) >> (emax - e));
-    return (long long)b < 0 ? -v : v;
-}
-__device__ __forceinline__ long long fx_from(double x, int emax) {
-    if (emax < 64) return fx_from_tiny(x, emax);
-    const unsigned long long b = dbl_bits(x);
-    const int e = (int)(b >> 52) & 0x7ff;
-    unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    const unsigned long long m = e == 0 ? f << 9 : (f | 0x10000000000000ull) << 8;
     int r = emax - e;
     if (r > 63) r = 63;  // below 2^-62 of the largest: zero
-    const long long v = (long long)((m << 8) >> r);
+    const long long v = (long long)(m >> r);
     return (long long)b < 0 ? -v : v;
 }
 // upper bound of a point's modulus, in units of 2^41
@@ -152,23 +146,27 @@ __device__ __forceinline__ int fx_scale(int emax, int sh) { return emax == 0x7ff
 
 // FP64 <-> FP32 conversions with integer instructions: the hardware's issue
 // at the FP64 rate (64 cycles per warp and sub-partition), these are about
-// ten integer instructions each.  The same values, rounded to nearest even;
-// subnormal FP32 numbers, which need a shift by the value, go through the
-// hardware's.
+// twelve instructions each.  The same values, rounded to nearest even; subnormal
+// FP32 numbers go through a normal one 2^64 times as large, so that a result
+// among them is rounded twice (within 0.5 + 2^-24 of its last place).  A branch to the
+// hardware's conversion for them cost the FP32-mixed runs 5 to 9%.
 __device__ __forceinline__ float to_f32(double x) {
     const unsigned long long b = dbl_bits(x), m = b & 0x7fffffffffffffffull;
     const unsigned hi = (unsigned)(m >> 32);
-    if (hi - 0x36900000u < 0x01800000u) return (float)x;  // 2^-150 <= |x| < 2^-126
-    const unsigned long long t = m - (896ull << 52);
+    const bool sub = hi < 0x38100000u;  // below 2^-126
+    const unsigned long long t = m - ((unsigned long long)(sub ? 832u << 20 : 896u << 20) << 32);
     unsigned r = (unsigned)((t + 0x0fffffffull + ((t >> 29) & 1ull)) >> 29);
-    if (hi < 0x38100000u) r = 0u;                                   // below 2^-150
+    if (hi < 0x34100000u) r = 0u;                                   // below 2^-190
     if (hi >= 0x47f00000u) r = m > 0x7ff0000000000000ull ? 0x7fc00000u : 0x7f800000u;  // 2^128 and above, inf, NaN
+    if (sub) r = flt_bits(bits_flt(r) * 0x1p-64f);
     return bits_flt(r | ((unsigned)(b >> 32) & 0x80000000u));
 }
 __device__ __forceinline__ double to_f64(float x) {
     const unsigned b = flt_bits(x), m = b & 0x7fffffffu;
-    if (m - 1u < 0x007fffffu) return (double)x;
-    unsigned hi = (m >> 3) + (896u << 20), lo = m << 29;
+    const bool sub = m < 0x00800000u;
+    const unsigned n = sub ? flt_bits(bits_flt(m) * 0x1p64f) : m;
+    unsigned hi = (n >> 3) + (sub ? 832u << 20 : 896u << 20);
+    const unsigned lo = n << 29;
     if (m == 0u) hi = 0u;
     if (m >= 0x7f800000u) hi += 896u << 20;  // inf, NaN
     hi |= b & 0x80000000u;
