@@ -179,6 +179,12 @@ static Params params_for(const pagd_solver* s, char* w) {
     P.theta_mode = s->opts.theta_mode;
     const double sq = std::sqrt(s->opts.s);
     for (int j = 0; j < s->opts.n_eta; j++) P.lam[j] = (1.0 - s->opts.eta[j] * sq) / (1.0 + s->opts.eta[j] * sq);
+    for (int j = 0; j < s->opts.n_eta; j++) P.lamf[j] = (float)P.lam[j];
+    P.e2f = (float)(P.eps * P.eps);
+    P.c0f = (float)(1.0 - P.eps);
+    P.tauf = (float)P.tau;
+    P.eta1f = (float)P.eta1;
+    P.eta2f = (float)P.eta2;
     P.nslots = s->nslots;
     P.cur0 = s->cur;
     P.step0 = s->step;

@@ -83,6 +83,7 @@ constexpr int kMaxCtas = 2;
 // scheme coefficients of one step (see compute_step_coeffs)
 struct StepK {
     double a, b, c, thv, ts, Ai, rho, gun, thpc, m2, ith, aim;  // ith = 1 / thv, aim = Ai / M
+    float tsf, m2f, aimf;                                       // rounded to FP32, for the FP32 passes
 };
 
 struct Params {
@@ -99,6 +100,8 @@ struct Params {
     long long npts;
     double k0sq, k1sq, kmsq;  // (2 pi / L)^2 of the first, last and middle axes
     float k0sqf, k1sqf, kmsqf;
+    // constants of the FP32 passes, rounded by the host: eps^2, 1 - eps, tau, ...
+    float e2f, c0f, tauf, eta1f, eta2f, lamf[16];
     double cellvol;           // product of the spacings
     double eps, eta1, eta2, tau, M;
     double s;
@@ -281,6 +284,9 @@ inline StepK compute_step_coeffs(int scheme, int n, double dt, double dtp, doubl
     k.m2 = k.a / M;
     k.ith = 1.0 / k.thv;
     k.aim = k.Ai / M;
+    k.tsf = (float)k.ts;
+    k.m2f = (float)k.m2;
+    k.aimf = (float)k.aim;
     return k;
 }
 
@@ -317,8 +323,12 @@ __device__ __forceinline__ Beta betas(const Params& P, const StepK& k, int bank)
     return betas_from(P, k, ldcg(&P.sc->beta_sum[bank][0]), ldcg(&P.sc->beta_sum[bank][1]));
 }
 
-__device__ __forceinline__ double lam_at(const Params& P, int i) {
-    return P.accel ? P.lam[i % P.n_eta] : 0.0;
+template <class T> __device__ __forceinline__ T sel(double d, float f) {
+    if constexpr (sizeof(T) == 8) return d;
+    else return f;
+}
+template <class T = double> __device__ __forceinline__ T lam_at(const Params& P, int i) {
+    return P.accel ? sel<T>(P.lam[i % P.n_eta], P.lamf[i % P.n_eta]) : (T)0;
 }
 
 // last-axis wavenumber index of column-pass line l (l = k1 nm + km)
@@ -2043,6 +2053,11 @@ struct Nil {};
 __host__ __device__ __forceinline__ int k_iter(int model) { return model == M_PFC ? 1 : 2; }
 __host__ __device__ __forceinline__ int k_base(int model) { return model == M_PFC ? 3 : 2; }
 
+// Unit of the averaged-Newton sums: a value is an FP32 number, the sum of 2^24
+// of them is one in this unit.
+constexpr float kSumUnit = 0x1p-24f;
+constexpr double kSumUnits = 0x1p24;  // in one
+
 // Phase B: (1) the pending acceptance of the previous step, (2) either the new
 // step's initial guess (Sec. 3.4.2: extrapolation of the two previous solutions),
 // base argument VB, history term g and preconditioner sums, or a move of the
@@ -2053,11 +2068,6 @@ __host__ __device__ __forceinline__ int k_base(int model) { return model == M_PF
 // linear residual W = A_i VB + g = a x + b u^n + c u^{n-1} (O(u_t)), the shift
 // y = VB_new - VB_old from the reference point, and (PFC) the nonlinear change
 // VB_new^3 - VB_old^3 = y (3 r^2 + 3 r y + y^2), r = VB_old.
-// Unit of the averaged-Newton sums: a value is an FP32 number, the sum of 2^24
-// of them is one in this unit.
-constexpr float kSumUnit = 0x1p-24f;
-constexpr double kSumUnits = 0x1p24;  // in one
-
 template <class T, int NF, bool INC>
 __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, const Tw& tw, char* smem, double* red) {
     using TO = typename std::conditional<INC, T, double>::type;
@@ -2100,8 +2110,7 @@ __device__ __forceinline__ void phase_B_impl(const Params& P, const Ctl& c, cons
         P.sc->steps_done = c.step;
     }
     Sum3 s0, s2;
-    const float c1e = to_f32(1.0 - P.eps), tauf = to_f32(P.tau), eta1f = to_f32(P.eta1), eta2f = to_f32(P.eta2),
-                e2f = to_f32(P.eps * P.eps);
+    const float c1e = P.c0f, tauf = P.tauf, eta1f = P.eta1f, eta2f = P.eta2f, e2f = P.e2f;
     const int kb = k_base(P.model);
     const bool pfc = P.model == M_PFC;
     const bool reb = c.reb != 0, acc = c.acc != 0;
@@ -2393,7 +2402,8 @@ __device__ PAGD_COLD void phase_DN(const Params& P, const Tw& tw, char* smem) {
     using C = cx<T>;
     T* lbt = (T*)P.LBt;
     const T* yb = (const T*)P.YB;
-    const T tau = (T)P.tau, e2 = (T)(P.eps * P.eps), eta1 = (T)P.eta1, eta2 = (T)P.eta2;
+    const T tau = sel<T>(P.tau, P.tauf), e2 = sel<T>(P.eps * P.eps, P.e2f), eta1 = sel<T>(P.eta1, P.eta1f),
+            eta2 = sel<T>(P.eta2, P.eta2f);
     struct St { double vb, lb; T y; };
     rowp<T, T, NF, true>(
         P, tw, 1, 2, (const C*)P.DB, (C*)P.NB, smem,
@@ -2453,8 +2463,8 @@ template <class T> struct RowK {
 };
 template <class T> __device__ __forceinline__ RowK<T> row_consts(const Params& P, const Ctl& c) {
     const StepK& k = step_coeffs(P, c.step);
-    return RowK<T>{cvt<T>(lam_at(P, c.it - 1)), cvt<T>(lam_at(P, c.it)), cvt<T>(k.ts), cvt<T>(P.tau),
-                   cvt<T>(P.eps * P.eps), cvt<T>(P.eta1), cvt<T>(P.eta2)};
+    return RowK<T>{lam_at<T>(P, c.it - 1),        lam_at<T>(P, c.it),       sel<T>(k.ts, k.tsf),     sel<T>(P.tau, P.tauf),
+                   sel<T>(P.eps * P.eps, P.e2f), sel<T>(P.eta1, P.eta1f), sel<T>(P.eta2, P.eta2f)};
 }
 
 // One point of the iteration row pass: delta_{i+1} from the direction
@@ -2613,9 +2623,9 @@ template <class T> struct ColK {
 template <class T> __device__ __forceinline__ ColK<T> col_consts(const Params& P, const Ctl& c) {
     const StepK& k = step_coeffs(P, c.step);
     const Beta B = c.bt;
-    const T e2 = cvt<T>(P.eps * P.eps);
-    return ColK<T>{cvt<T>(lam_at(P, c.it)), cvt<T>(lam_at(P, c.it + 1)), cvt<T>(k.ts), cvt<T>(B.m2), cvt<T>(B.b0),
-                   cvt<T>(B.b2), cvt<T>(B.b4), cvt<T>(k.aim), cvt<T>(1.0 - P.eps), e2, e2 * e2};
+    const T e2 = sel<T>(P.eps * P.eps, P.e2f);
+    return ColK<T>{lam_at<T>(P, c.it), lam_at<T>(P, c.it + 1), sel<T>(k.ts, k.tsf), sel<T>(B.m2, k.m2f), cvt<T>(B.b0),
+                   cvt<T>(B.b2),       cvt<T>(B.b4),           sel<T>(k.aim, k.aimf), sel<T>(1.0 - P.eps, P.c0f), e2, e2 * e2};
 }
 
 // One wavenumber of the iteration column pass: ybar_hat, the spectral residual
