@@ -422,12 +422,15 @@ static void make_plan(pagd_solver* s) {
     // fewer units than half the warps: most warps would otherwise idle and a
     // unit's pointwise FP64 work and integer butterflies run on one SM
     // sub-partition.
-    // PAGD_COOP=0 / 1 overrides the choice.  3D grids of other lengths than 64
-    // to 512 with more units than SMs keep a warp per unit: their short lines
-    // gain less from sharing than the rounds cost (32^3, 544 units, two steps of
-    // PFC FP64: 1479 us shared, 803 with a warp per unit).
+    // PAGD_COOP=0 / 1 overrides the choice.  On 3D grids the CTAs take the shared
+    // units in rounds, and the middle passes keep a warp per unit: with more
+    // units than SMs a warp per unit is faster (PFC FP64, two steps, shared
+    // against a warp per unit: 32 x 16 x 32, 272 units, 1102 / 889 us; 64 x 16 x
+    // 64, 528, 1539 / 1093; 128 x 8 x 128, 520, 2423 / 1882; 32^3, 544, 1718 / 917),
+    // except for two rounds of long lines (64 x 8 x 64, 264: 1020 / 1020,
+    // FP32-mixed 716 / 770).
     s->coop = 2 * units <= (long long)s->grid * wpb &&
-                      (s->dim == 2 || units <= sms || fixed_len(s->n[0], s->n[last]) != 0)
+                      (s->dim == 2 || units <= sms || (units <= 2ll * sms && fixed_len(s->n[0], s->n[last]) != 0))
                   ? 1
                   : 0;
     if (const char* e = std::getenv("PAGD_COOP")) {

@@ -109,3 +109,17 @@ def test_small_grid_forms_take_as_many_evaluations(monkeypatch, model, n):
         S.set_state(dev(I.noisy_field(n, -0.3 if model == "fch" else 0.1, 0.05, 5)))
         its.append(np.array(S.run(1e-3 if model == "fch" else 0.1, 3, 1e-10, S.empty_field())[0]))
     assert np.abs(its[0] - its[1]).max() <= 3, its
+
+
+@pytest.mark.parametrize("n,shared", [((64, 8, 64), 1), ((64, 16, 64), 0), ((128, 8, 128), 0), ((32, 16, 32), 0), ((32, 32, 32), 0),
+                                      ((16, 16, 16), 1), ((8, 8, 8), 1)])
+def test_3d_grids_share_units_only_in_few_rounds(n, shared):
+    """Which of the two forms a 3D grid takes on 152 SMs, and that they agree: the
+    tolerance of the transforms above."""
+    S = pagd.Solver("pfc", n, (3.0,) * 3, 0.1)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert S.launch_info()["coop"] == shared
+    u = 0.1 + 0.05 * np.random.default_rng(sum(n)).uniform(-1, 1, n)
+    sp = S.fft_r2c(dev(u)).cpu().numpy()
+    ref = np.fft.rfftn(u)
+    assert np.linalg.norm(sp[..., 0] + 1j * sp[..., 1] - ref) <= 1e-15 * np.linalg.norm(ref)
