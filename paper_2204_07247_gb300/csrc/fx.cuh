@@ -483,7 +483,7 @@ template <int S, int LOGN> __device__ __forceinline__ void fx_first(const longlo
 // b (all stages but the last done) -> v
 template <int S, int LOGN>
 __device__ __forceinline__ void fx_last(longlong2* v, const longlong2* b, const FxTw* tw, int logTw, int lane) {
-    constexpr int R = LOGN == 9 ? 8 : 4, LR = radix_log(R), NB = (1 << LOGN) / R, PER = NB / kWarp;
+    constexpr int R = LOGN == 9 ? 8 : 4, NB = (1 << LOGN) / R, PER = NB / kWarp;
     const int twshift = logTw - LOGN;
 #pragma unroll
     for (int i = 0; i < PER; i++) {
@@ -499,7 +499,6 @@ __device__ __forceinline__ void fx_last(longlong2* v, const longlong2* b, const 
         for (int r = 0; r < R; r++) v[i + r * PER] = u[r];
     }
     warp_sync();
-    (void)LR;
 }
 template <int S, int LOGN, int LOGNS, int END>
 __device__ __forceinline__ void fx_middle(longlong2* b, const FxTw* tw, int logTw, int lane) {
@@ -541,22 +540,22 @@ template <int E> __device__ __forceinline__ void fx_put(const longlong2* v, int 
         }
     }
 }
-// points s[i stride] of a line -> its transform in the slots of b; returns the exponent
+// n contiguous points -> their transform in the slots of b; returns the exponent
 template <int S, int LOGN>
-__device__ __noinline__ int fx_line_in(longlong2* b, const double2* s, int stride, const FxTw* tw, int logTw, int lane) {
+__device__ __noinline__ int fx_line_in(longlong2* b, const double2* s, const FxTw* tw, int logTw, int lane) {
     constexpr int E = (1 << LOGN) / kWarp;
     double2 z[E];
     longlong2 v[E];
 #pragma unroll
-    for (int i = 0; i < E; i++) z[i] = s[(size_t)(lane + kWarp * i) * stride];
+    for (int i = 0; i < E; i++) z[i] = s[lane + kWarp * i];
     const FxExp x = fx_regs<E>(z, v);
     fx_first<S, LOGN>(v, b, x.sh, lane);
     fx_middle<S, LOGN, radix_log(fx_radix(LOGN, 0)), LOGN>(b, tw, logTw, lane);
     return x.e - x.sh;
 }
-// doubles in the lane's slots of b -> the transform at d[i stride]
+// doubles in the lane's slots of b -> the transform at d, contiguous
 template <int S, int LOGN>
-__device__ __noinline__ void fx_line_out(longlong2* b, double2* d, int stride, const FxTw* tw, int logTw, int lane) {
+__device__ __noinline__ void fx_line_out(longlong2* b, double2* d, const FxTw* tw, int logTw, int lane) {
     constexpr int E = (1 << LOGN) / kWarp, END = LOGN - (LOGN == 9 ? 3 : 2);
     longlong2 v[E];
     double2 z[E];
@@ -566,7 +565,7 @@ __device__ __noinline__ void fx_line_out(longlong2* b, double2* d, int stride, c
     fx_first<S, LOGN>(v, b, x.sh, lane);
     fx_middle<S, LOGN, radix_log(fx_radix(LOGN, 0)), END>(b, tw, logTw, lane);
     fx_last<S, LOGN>(v, b, tw, logTw, lane);
-    fx_put<E>(v, x.e - x.sh, d, stride, lane);
+    fx_put<E>(v, x.e - x.sh, d, 1, lane);
 }
 // doubles in the lane's slots of b -> the transform in the slots; returns the exponent
 template <int S, int LOGN>
@@ -605,7 +604,7 @@ __host__ __device__ constexpr bool fx_regs_ok(int nf) { return nf == 128 || nf =
 // hi: this lane's largest fx_hi of its slots.  in and mid return the exponent.
 template <int S, int NF>
 __device__ __forceinline__ int fx_in(longlong2* b, const double2* s, int n, int logn, const FxTw* tw, int logTw, int lane) {
-    if constexpr (fx_regs_ok(NF)) return fx_line_in<S, ilog2c(NF)>(b, s, 1, tw, logTw, lane);
+    if constexpr (fx_regs_ok(NF)) return fx_line_in<S, ilog2c(NF)>(b, s, tw, logTw, lane);
     const FxExp x = fx_convert(b, n, fx_load(b, s, n, lane, kWarp), lane);
     fx_line<S, NF>(b, logn, x.sh, tw, logTw, lane);
     return x.e - x.sh;
@@ -621,7 +620,7 @@ template <int S, int NF>
 __device__ __forceinline__ void fx_out(longlong2* b, unsigned hi, double2* d, int n, int logn, const FxTw* tw, int logTw,
                                        int lane) {
     if constexpr (fx_regs_ok(NF)) {
-        fx_line_out<S, ilog2c(NF)>(b, d, 1, tw, logTw, lane);
+        fx_line_out<S, ilog2c(NF)>(b, d, tw, logTw, lane);
     } else {
         const FxExp x = fx_convert(b, n, hi, lane);
         fx_line<S, NF>(b, logn, x.sh, tw, logTw, lane);

@@ -476,7 +476,8 @@ static void make_plan(pagd_solver* s) {
 #endif
     s->stage = (!s->cl && stage_fits(s, s->warp_bytes)) ? 1 : 0;
     // FP32 iteration passes with CTA-cooperative units (unstaged FP32 passes
-    // of fixed line length): opt-in with PAGD_COOP32=1.  Measured slower on
+    // of fixed line length): opt-in with PAGD_COOP32=1 PAGD_STAGED=0 (the staged
+    // passes, which such grids otherwise take, come first).  Measured slower on
     // FCH 256^2 (128 row pairs on 152 SMs), where the FP64 passes gain from
     // them: 382.7 against 359.3 us per step, the column pass 13.4 against
     // 10.3 us.
@@ -1440,6 +1441,7 @@ static pagd_status batch_chunk(pagd_batch* b, double dt, int nsteps, double tol,
         PI[i].warp_bytes = (long long)b->warp_bytes;
         PI[i].coop = 0;  // batch warps own their units: no CTA-wide barriers
         PI[i].coop32 = 0;
+        PI[i].one = 0;
         PI[i].cl = 0;    // and every phase of a batch is device-wide
         PI[i].stage = stage_fits(s, b->warp_bytes) ? 1 : 0;
         PI[i].logtw = b->logtw;

@@ -106,8 +106,8 @@ struct Params {
     double eps, eta1, eta2, tau, M;
     double s;
     int n_eta, accel, max_iter, max_recheck, theta_mode;
-    // the PFC FP32 iteration passes stage their inputs by asynchronous copies
-    // (row_pass_staged / col_pass_staged; fixed line lengths)
+    // the FP32 iteration passes stage their inputs by asynchronous copies
+    // (row_pass_staged / col_pass_staged; first and last axis of 64 to 512 points)
     int stage;
     // PROG_PASS: the iteration pass it repeats (PH_RI, PH_CI, PH_MF, PH_MI)
     int pass;
@@ -154,7 +154,7 @@ struct Params {
     void* YB;
     int ref_valid, refresh;
     // the passes with an FP64 line run CTA-cooperative units (single-instance
-    // launches with fixed line lengths only)
+    // launches only)
     int coop;
     // cluster-resident iterations (cluster.cuh): the cluster size (0: off) and
     // the control state the loop hands back to the device-wide machine (a Ctl)
@@ -478,9 +478,9 @@ template <> struct SumOf<double> {
     __device__ __forceinline__ double warp_total() const { return warp_sum(v); }
 };
 // the norm and the sum of a row pass's evaluation
-template <class TI, class T>
+template <class T>
 __device__ __forceinline__ void publish_eval(const Params& P, const Tw& tw, bool all, int bank, int ev,
-                                             const MaxAbs<TI>& amax, const SumOf<T>& asum) {
+                                             const MaxAbs<T>& amax, const SumOf<T>& asum) {
     double* const a[1] = {&P.sums[(size_t)bank * P.nslots + ev]};
     const double v[1] = {asum.warp_total()};
     publish_group<1>(tw, all, &P.norms[(size_t)bank * P.nslots + ev], amax.warp_bits(), a, v);
@@ -520,40 +520,38 @@ __device__ __forceinline__ WarpCtx warp_ctx(const Params& P, char* smem) {
 // Row pass.  src/dst: column-major half spectra, field f, column k, row r at
 // f*H + k*rows + r.  A unit is ru = 2 rows;
 // real line l = f*ru + rr; lines 2j and 2j+1 are packed as the real and
-// imaginary parts of complex line j.  fn(p, row, x, const TI* in, TO* out).
-template <class TI, class TO, class Fn>
-__device__ void row_pass(const Params& P, const Tw& tw, int kin, int kout, const cx<TI>* src,
-                         cx<TO>* dst, char* smem, Fn&& fn) {
-    using CI = cx<TI>;
-    using CO = cx<TO>;
+// imaginary parts of complex line j.  fn(p, row, x, const float* in, float* out).
+template <class Fn>
+__device__ void row_pass(const Params& P, const Tw& tw, int kin, int kout, const float2* src,
+                         float2* dst, char* smem, Fn&& fn) {
     const int rows = P.rows, n1 = P.n1, logn1 = P.logn1, half = n1 >> 1;
     const long long H = P.H;
     const int pitch = pitch_of(n1);
     const int ru = row_unit(kin, kout);
     const WarpCtx w = warp_ctx(P, smem);
-    TI* Rin = (TI*)w.mem;
-    TO* Rout = (TO*)(w.mem + (size_t)kin * ru * n1 * sizeof(TI));
-    char* zb = w.mem + (size_t)kin * ru * n1 * sizeof(TI) + (size_t)kout * ru * n1 * sizeof(TO);
-    const TI iscale = (TI)P.inv_npts;
+    float* Rin = (float*)w.mem;
+    float* Rout = (float*)(w.mem + (size_t)kin * ru * n1 * sizeof(float));
+    char* zb = w.mem + (size_t)kin * ru * n1 * sizeof(float) + (size_t)kout * ru * n1 * sizeof(float);
+    const float iscale = (float)P.inv_npts;
     const URange ur = units_of(tw, rows / ru);
     for (int u = ur.b; u < ur.e; u += ur.s) {
         const int r0 = u * ru;
         for (int j = 0; 2 * j < kin * ru; j++) {
-            CI* Z0 = (CI*)zb;
-            CI* Z1 = Z0 + pitch;
+            float2* Z0 = (float2*)zb;
+            float2* Z1 = Z0 + pitch;
             const int la = 2 * j, lb = 2 * j + 1;
-            const CI* sa = src + (size_t)(la / ru) * H + r0 + (la % ru);
-            const CI* sb = src + (size_t)(lb / ru) * H + r0 + (lb % ru);
+            const float2* sa = src + (size_t)(la / ru) * H + r0 + (la % ru);
+            const float2* sb = src + (size_t)(lb / ru) * H + r0 + (lb % ru);
             for (int x = w.lane; x < n1; x += kWarp) {
                 const int k = (x <= half) ? x : n1 - x;
-                CI A = sa[(size_t)k * rows], B = sb[(size_t)k * rows];
+                float2 A = sa[(size_t)k * rows], B = sb[(size_t)k * rows];
                 if (x == 0 || x == half) { A.y = 0; B.y = 0; }
-                Z0[x] = (x <= half) ? CI{A.x - B.y, A.y + B.x} : CI{A.x + B.y, B.x - A.y};
+                Z0[x] = (x <= half) ? float2{A.x - B.y, A.y + B.x} : float2{A.x + B.y, B.x - A.y};
             }
-            const int res = fft_line_w<+1, TI>(Z0, Z1, logn1, tw.t32, tw.log, w.lane);
-            const CI* Zr = res ? Z1 : Z0;
+            const int res = fft_line_w<+1, float>(Z0, Z1, logn1, tw.t32, tw.log, w.lane);
+            const float2* Zr = res ? Z1 : Z0;
             for (int x = w.lane; x < n1; x += kWarp) {
-                const CI z = Zr[x];
+                const float2 z = Zr[x];
                 Rin[(size_t)la * n1 + x] = z.x * iscale;
                 Rin[(size_t)lb * n1 + x] = z.y * iscale;
             }
@@ -561,30 +559,30 @@ __device__ void row_pass(const Params& P, const Tw& tw, int kin, int kout, const
         }
         for (int x = w.lane; x < n1; x += kWarp) {
             for (int rr = 0; rr < ru; rr++) {
-                TI in[kMaxK];
-                TO out[kMaxK];
+                float in[kMaxK];
+                float out[kMaxK];
                 for (int f = 0; f < kin; f++) in[f] = Rin[(size_t)(f * ru + rr) * n1 + x];
                 fn((long long)(r0 + rr) * n1 + x, r0 + rr, x, in, out);
                 for (int g = 0; g < kout; g++) Rout[(size_t)(g * ru + rr) * n1 + x] = out[g];
             }
         }
         for (int j = 0; 2 * j < kout * ru; j++) {
-            CO* Z0 = (CO*)zb;
-            CO* Z1 = Z0 + pitch;
+            float2* Z0 = (float2*)zb;
+            float2* Z1 = Z0 + pitch;
             const int la = 2 * j, lb = 2 * j + 1;
             warp_sync();
             for (int x = w.lane; x < n1; x += kWarp)
-                Z0[x] = CO{Rout[(size_t)la * n1 + x], Rout[(size_t)lb * n1 + x]};
-            const int res = fft_line_w<-1, TO>(Z0, Z1, logn1, tw.t32, tw.log, w.lane);
-            const CO* Zr = res ? Z1 : Z0;
-            CO* da = dst + (size_t)(la / ru) * H + r0 + (la % ru);
-            CO* db = dst + (size_t)(lb / ru) * H + r0 + (lb % ru);
-            const TO hf = (TO)0.5;
+                Z0[x] = float2{Rout[(size_t)la * n1 + x], Rout[(size_t)lb * n1 + x]};
+            const int res = fft_line_w<-1, float>(Z0, Z1, logn1, tw.t32, tw.log, w.lane);
+            const float2* Zr = res ? Z1 : Z0;
+            float2* da = dst + (size_t)(la / ru) * H + r0 + (la % ru);
+            float2* db = dst + (size_t)(lb / ru) * H + r0 + (lb % ru);
+            const float hf = 0.5f;
             for (int k = w.lane; k <= half; k += kWarp) {
-                const CO zk = Zr[k];
-                const CO zn = Zr[(n1 - k) & (n1 - 1)];
-                da[(size_t)k * rows] = CO{hf * (zk.x + zn.x), hf * (zk.y - zn.y)};
-                db[(size_t)k * rows] = CO{hf * (zk.y + zn.y), hf * (zn.x - zk.x)};
+                const float2 zk = Zr[k];
+                const float2 zn = Zr[(n1 - k) & (n1 - 1)];
+                da[(size_t)k * rows] = float2{hf * (zk.x + zn.x), hf * (zk.y - zn.y)};
+                db[(size_t)k * rows] = float2{hf * (zk.y + zn.y), hf * (zn.x - zk.x)};
             }
         }
         warp_sync();
@@ -592,52 +590,41 @@ __device__ void row_pass(const Params& P, const Tw& tw, int kin, int kout, const
 }
 
 // Column pass over the ncols contiguous lines of length n0: one warp per line.
-// fn(k1, k0, in, out); outputs may overwrite inputs of the same point.  The
-// forward transforms run in TI, the inverse ones in TO (TO narrower than TI:
-// outputs whose size is a small fraction of the inputs', e.g. a direction
-// computed from FP64 spectra, go back to physical space in FP32).
-template <class TI, class TO, class Fn>
-__device__ void col_pass(const Params& P, const Tw& tw, int kin, int kout, const cx<TI>* src, cx<TO>* dst,
+// fn(k1, k0, in, out); outputs overwrite inputs of the same point.
+template <class Fn>
+__device__ void col_pass(const Params& P, const Tw& tw, int kin, int kout, const float2* src, float2* dst,
                          char* smem, Fn&& fn) {
-    using CI = cx<TI>;
-    using CO = cx<TO>;
-    constexpr bool same = sizeof(TI) == sizeof(TO);
     const int n0 = P.n0, ncols = P.ncols, logn0 = P.logn0;
     const long long H = P.H;
     const int pitch = pitch_of(n0);
-    const int nbi = same ? (kin > kout ? kin : kout) + 1 : kin + 1;
+    const int nb = (kin > kout ? kin : kout) + 1;
     const WarpCtx w = warp_ctx(P, smem);
     const URange ur = units_of(tw, ncols);
     for (int k1 = ur.b; k1 < ur.e; k1 += ur.s) {
         const Line ln = line_of(P, tw, k1);
-        CI* buf[kMaxK + 1];
-        CO* obuf[kMaxK + 1];
-        for (int i = 0; i < nbi; i++) buf[i] = (CI*)w.mem + (size_t)i * pitch;
+        float2* buf[kMaxK + 1];
+        for (int i = 0; i < nb; i++) buf[i] = (float2*)w.mem + (size_t)i * pitch;
         for (int f = 0; f < kin; f++) {
-            const CI* s = src + (size_t)f * H + (size_t)k1 * n0;
+            const float2* s = src + (size_t)f * H + (size_t)k1 * n0;
             for (int k0 = w.lane; k0 < n0; k0 += kWarp) buf[f][k0] = s[k0];
-            const int res = fft_line_w<-1, TI>(buf[f], buf[nbi - 1], logn0, tw.t32, tw.log, w.lane);
+            const int res = fft_line_w<-1, float>(buf[f], buf[nb - 1], logn0, tw.t32, tw.log, w.lane);
             if (res) {
-                CI* t = buf[f];
-                buf[f] = buf[nbi - 1];
-                buf[nbi - 1] = t;
+                float2* t = buf[f];
+                buf[f] = buf[nb - 1];
+                buf[nb - 1] = t;
             }
         }
-        // outputs: in place of the inputs (same precision) or after them
-        for (int i = 0; i <= kout; i++)
-            obuf[i] = same ? (CO*)(i < kout ? buf[i] : buf[nbi - 1])
-                           : (CO*)((CI*)w.mem + (size_t)nbi * pitch) + (size_t)i * pitch;
         for (int k0 = w.lane; k0 < n0; k0 += kWarp) {
-            CI in[kMaxK];
-            CO out[kMaxK];
+            float2 in[kMaxK];
+            float2 out[kMaxK];
             for (int f = 0; f < kin; f++) in[f] = buf[f][k0];
             fn(ln, k0, in, out);
-            for (int g = 0; g < kout; g++) obuf[g][k0] = out[g];
+            for (int g = 0; g < kout; g++) buf[g][k0] = out[g];
         }
         for (int g = 0; g < kout; g++) {
-            const int res = fft_line_w<+1, TO>(obuf[g], obuf[kout], logn0, tw.t32, tw.log, w.lane);
-            const CO* r = res ? obuf[kout] : obuf[g];
-            CO* d = dst + (size_t)g * H + (size_t)k1 * n0;
+            const int res = fft_line_w<+1, float>(buf[g], buf[nb - 1], logn0, tw.t32, tw.log, w.lane);
+            const float2* r = res ? buf[nb - 1] : buf[g];
+            float2* d = dst + (size_t)g * H + (size_t)k1 * n0;
             for (int k0 = w.lane; k0 < n0; k0 += kWarp) d[k0] = r[k0];
             warp_sync();
         }
@@ -662,18 +649,9 @@ __host__ __device__ constexpr int chunk_for(int bytes, int n) {
     return c;
 }
 
-template <int NF> __host__ __device__ __forceinline__ size_t row_fixed_smem(int kin, int szin, int kout, int szout) {
-    return 2 * (size_t)(NF + 2) * ((size_t)kin * 2 * szin + (size_t)kout * 2 * szout);
-}
-template <int NF> __host__ __device__ __forceinline__ size_t col_fixed_smem(int k, int sz) {
-    return 2 * (size_t)(NF + 2) * (size_t)k * 2 * sz;
-}
-
-template <class TI, class TO, int NF, class Ld, class Ap>
-__device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout, const cx<TI>* src,
-                               cx<TO>* dst, char* smem, Ld&& ld, Ap&& ap) {
-    using CI = cx<TI>;
-    using CO = cx<TO>;
+template <int NF, class Ld, class Ap>
+__device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout, const float2* src,
+                               float2* dst, char* smem, Ld&& ld, Ap&& ap) {
     using S = decltype(ld(0ll, 0, 0));
     constexpr int LOGN = ilog2c(NF), HALF = NF / 2, H1 = HALF + 1, PITCH = NF + 2;
     constexpr int E = NF / kWarp, EH = (H1 + kWarp - 1) / kWarp;
@@ -682,11 +660,11 @@ __device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
     const int rows = P.rows;
     const long long Hs = P.H;
     const WarpCtx w = warp_ctx(P, smem);
-    CI* X0 = (CI*)w.mem;
-    CI* X1 = X0 + (size_t)kin * PITCH;
-    CO* Y0 = (CO*)(X1 + (size_t)kin * PITCH);
-    CO* Y1 = Y0 + (size_t)kout * PITCH;
-    const TI iscale = (TI)P.inv_npts;
+    float2* X0 = (float2*)w.mem;
+    float2* X1 = X0 + (size_t)kin * PITCH;
+    float2* Y0 = (float2*)(X1 + (size_t)kin * PITCH);
+    float2* Y1 = Y0 + (size_t)kout * PITCH;
+    const float iscale = (float)P.inv_npts;
     const URange ur = units_of(tw, rows / 2);
     constexpr int NCH = E / GCH;  // load chunks per field
     for (int u = ur.b; u < ur.e; u += ur.s) {
@@ -700,12 +678,12 @@ __device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
             const int x = w.lane + kWarp * i;
             st[q] = ld((long long)(r0 + rr) * NF + x, r0 + rr, x);
         }
-        // spectra of the kin fields, chunk t = (field, GCH points); FP32 lines
-        // load chunk t + 1 before storing chunk t to shared memory (the
-        // compiler cannot move a global load above a shared store itself)
-        auto load_chunk = [&](int t, CI* a, CI* b) {
+        // spectra of the kin fields, chunk t = (field, GCH points): chunk t + 1 is
+        // loaded before chunk t is stored to shared memory (the compiler cannot
+        // move a global load above a shared store itself)
+        auto load_chunk = [&](int t, float2* a, float2* b) {
             const int l = t / NCH, c = (t % NCH) * GCH;
-            const CI* s0 = src + (size_t)l * Hs + r0;
+            const float2* s0 = src + (size_t)l * Hs + r0;
 #pragma unroll
             for (int i = 0; i < GCH; i++) {
                 const int x = w.lane + kWarp * (c + i);
@@ -714,34 +692,26 @@ __device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
                 b[i] = s0[(size_t)k * rows + 1];
             }
         };
-        auto put_chunk = [&](int t, const CI* a, const CI* b) {
+        auto put_chunk = [&](int t, const float2* a, const float2* b) {
             const int l = t / NCH, c = (t % NCH) * GCH;
 #pragma unroll
             for (int i = 0; i < GCH; i++) {
                 const int x = w.lane + kWarp * (c + i);
-                CI A = a[i], B = b[i];
+                float2 A = a[i], B = b[i];
                 if (x == 0 || x == HALF) { A.y = 0; B.y = 0; }
-                X0[(size_t)l * PITCH + x] = (x <= HALF) ? CI{A.x - B.y, A.y + B.x} : CI{A.x + B.y, B.x - A.y};
+                X0[(size_t)l * PITCH + x] = (x <= HALF) ? float2{A.x - B.y, A.y + B.x} : float2{A.x + B.y, B.x - A.y};
             }
         };
         const int nt = kin * NCH;
-        if constexpr (sizeof(TI) == 4) {
-            CI a[2][GCH], b[2][GCH];
+        float2 a[2][GCH], b[2][GCH];
 #pragma unroll
-            for (int t = 0; t <= kMaxK * NCH; t++) {
-                if (t < nt) load_chunk(t, a[t & 1], b[t & 1]);
-                if (t >= 1 && t <= nt) put_chunk(t - 1, a[(t - 1) & 1], b[(t - 1) & 1]);
-            }
-        } else {
-            for (int t = 0; t < nt; t++) {
-                CI a[GCH], b[GCH];
-                load_chunk(t, a, b);
-                put_chunk(t, a, b);
-            }
+        for (int t = 0; t <= kMaxK * NCH; t++) {
+            if (t < nt) load_chunk(t, a[t & 1], b[t & 1]);
+            if (t >= 1 && t <= nt) put_chunk(t - 1, a[(t - 1) & 1], b[(t - 1) & 1]);
         }
-        const CI* Xr = X0;
+        const float2* Xr = X0;
         if (kin > 0)
-            Xr = fft_lines_fixed<+1, TI, LOGN, kMaxK>(X0, X1, PITCH, kin, tw.t32, tw.log, w.lane) ? X1 : X0;
+            Xr = fft_lines_fixed<+1, float, LOGN, kMaxK>(X0, X1, PITCH, kin, tw.t32, tw.log, w.lane) ? X1 : X0;
 #pragma unroll 1
         for (int c0 = 0; c0 < NPT; c0 += PCH) {
             if (c0 > 0) {
@@ -756,12 +726,12 @@ __device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
             for (int q = 0; q < PCH; q++) {
                 const int i = (c0 + q) >> 1, rr = (c0 + q) & 1;
                 const int x = w.lane + kWarp * i;
-                TI in[kMaxK];
-                TO out[kMaxK];
+                float in[kMaxK];
+                float out[kMaxK];
 #pragma unroll
                 for (int f = 0; f < kMaxK; f++) {
                     if (f < kin) {
-                        const CI z = Xr[(size_t)f * PITCH + x];
+                        const float2 z = Xr[(size_t)f * PITCH + x];
                         in[f] = (rr ? z.y : z.x) * iscale;
                     }
                 }
@@ -769,7 +739,7 @@ __device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
 #pragma unroll
                 for (int g = 0; g < kMaxK; g++) {
                     if (g < kout) {
-                        CO* qq = Y0 + (size_t)g * PITCH + x;
+                        float2* qq = Y0 + (size_t)g * PITCH + x;
                         if (rr) qq->y = out[g];
                         else qq->x = out[g];
                     }
@@ -777,20 +747,20 @@ __device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
             }
         }
         if (kout > 0) {
-            const CO* Yr =
-                fft_lines_fixed<-1, TO, LOGN, kMaxK>(Y0, Y1, PITCH, kout, tw.t32, tw.log, w.lane) ? Y1 : Y0;
-            const TO hf = (TO)0.5;
+            const float2* Yr =
+                fft_lines_fixed<-1, float, LOGN, kMaxK>(Y0, Y1, PITCH, kout, tw.t32, tw.log, w.lane) ? Y1 : Y0;
+            const float hf = 0.5f;
             for (int g = 0; g < kout; g++) {
-                CO* d0 = dst + (size_t)g * Hs + r0;
-                const CO* zl = Yr + (size_t)g * PITCH;
+                float2* d0 = dst + (size_t)g * Hs + r0;
+                const float2* zl = Yr + (size_t)g * PITCH;
 #pragma unroll
                 for (int i = 0; i < EH; i++) {
                     const int k = w.lane + kWarp * i;
                     if (k <= HALF) {
-                        const CO zk = zl[k];
-                        const CO zn = zl[(NF - k) & (NF - 1)];
-                        d0[(size_t)k * rows] = CO{hf * (zk.x + zn.x), hf * (zk.y - zn.y)};
-                        d0[(size_t)k * rows + 1] = CO{hf * (zk.y + zn.y), hf * (zn.x - zk.x)};
+                        const float2 zk = zl[k];
+                        const float2 zn = zl[(NF - k) & (NF - 1)];
+                        d0[(size_t)k * rows] = float2{hf * (zk.x + zn.x), hf * (zk.y - zn.y)};
+                        d0[(size_t)k * rows + 1] = float2{hf * (zk.y + zn.y), hf * (zn.x - zk.x)};
                     }
                 }
             }
@@ -799,11 +769,9 @@ __device__ void row_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
     }
 }
 
-template <class TI, class TO, int NF, class Ld, class Ap>
-__device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout, const cx<TI>* src,
-                               cx<TO>* dst, char* smem, Ld&& ld, Ap&& ap) {
-    using C = cx<TI>;
-    using CO = cx<TO>;
+template <int NF, class Ld, class Ap>
+__device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout, const float2* src,
+                               float2* dst, char* smem, Ld&& ld, Ap&& ap) {
     using S = decltype(ld(Line{}, 0));
     constexpr int LOGN = ilog2c(NF), PITCH = NF + 2, E = NF / kWarp;
     constexpr int GCH = E < 8 ? E : 8;
@@ -812,8 +780,8 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
     const long long Hs = P.H;
     const int kl = kin > kout ? kin : kout;
     const WarpCtx w = warp_ctx(P, smem);
-    C* B0 = (C*)w.mem;
-    C* B1 = B0 + (size_t)kl * PITCH;
+    float2* B0 = (float2*)w.mem;
+    float2* B1 = B0 + (size_t)kl * PITCH;
     const URange ur = units_of(tw, ncols);
     constexpr int NCH = E / GCH;  // load chunks per field
     for (int k1 = ur.b; k1 < ur.e; k1 += ur.s) {
@@ -823,44 +791,35 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
         S st[PCH];
 #pragma unroll
         for (int q = 0; q < PCH; q++) st[q] = ld(ln, w.lane + kWarp * q);
-        // lines of the kin fields, chunk t = (field, GCH points); FP32 lines
-        // load chunk t + 1 before storing chunk t to shared memory
-        auto load_chunk = [&](int t, C* v) {
+        // lines of the kin fields, chunk t = (field, GCH points): chunk t + 1 is
+        // loaded before chunk t is stored to shared memory
+        auto load_chunk = [&](int t, float2* v) {
             const int f = t / NCH, c = (t % NCH) * GCH;
-            const C* s = src + (size_t)f * Hs + (size_t)k1 * NF;
+            const float2* s = src + (size_t)f * Hs + (size_t)k1 * NF;
 #pragma unroll
             for (int i = 0; i < GCH; i++) v[i] = s[w.lane + kWarp * (c + i)];
         };
-        auto put_chunk = [&](int t, const C* v) {
+        auto put_chunk = [&](int t, const float2* v) {
             const int f = t / NCH, c = (t % NCH) * GCH;
 #pragma unroll
             for (int i = 0; i < GCH; i++) B0[(size_t)f * PITCH + w.lane + kWarp * (c + i)] = v[i];
         };
         const int nt = kin * NCH;
-        if constexpr (sizeof(TI) == 4) {
-            C v[2][GCH];
+        float2 v[2][GCH];
 #pragma unroll
-            for (int t = 0; t <= kMaxK * NCH; t++) {
-                if (t < nt) load_chunk(t, v[t & 1]);
-                if (t >= 1 && t <= nt) put_chunk(t - 1, v[(t - 1) & 1]);
-            }
-        } else {
-            for (int t = 0; t < nt; t++) {
-                C v[GCH];
-                load_chunk(t, v);
-                put_chunk(t, v);
-            }
+        for (int t = 0; t <= kMaxK * NCH; t++) {
+            if (t < nt) load_chunk(t, v[t & 1]);
+            if (t >= 1 && t <= nt) put_chunk(t - 1, v[(t - 1) & 1]);
         }
-        const C* Xr = B0;
-        C* Xi = B1;
+        const float2* Xr = B0;
+        float2* Xi = B1;
         if (kin > 0) {
-            const int r = fft_lines_fixed<-1, TI, LOGN, kMaxK>(B0, B1, PITCH, kin, tw.t32, tw.log, w.lane);
+            const int r = fft_lines_fixed<-1, float, LOGN, kMaxK>(B0, B1, PITCH, kin, tw.t32, tw.log, w.lane);
             Xr = r ? B1 : B0;
             Xi = r ? B0 : B1;
         }
-        // outputs (TO, PITCH apart) in the buffer the inputs do not occupy;
-        // kl lines of TI hold kout lines of TO
-        CO* Xo = (CO*)Xi;
+        // outputs in the buffer the inputs do not occupy
+        float2* Xo = Xi;
 #pragma unroll 1
         for (int c0 = 0; c0 < E; c0 += PCH) {
             if (c0 > 0) {
@@ -870,8 +829,8 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
 #pragma unroll
             for (int q = 0; q < PCH; q++) {
                 const int k0 = w.lane + kWarp * (c0 + q);
-                C in[kMaxK];
-                CO out[kMaxK];
+                float2 in[kMaxK];
+                float2 out[kMaxK];
 #pragma unroll
                 for (int f = 0; f < kMaxK; f++)
                     if (f < kin) in[f] = Xr[(size_t)f * PITCH + k0];
@@ -882,12 +841,12 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
             }
         }
         if (kout > 0) {
-            CO* scratch = (CO*)Xr;
+            float2* scratch = (float2*)Xr;
             const int r =
-                fft_lines_fixed<+1, TO, LOGN, kMaxK>(Xo, scratch, PITCH, kout, tw.t32, tw.log, w.lane);
-            const CO* Yr = r ? scratch : Xo;
+                fft_lines_fixed<+1, float, LOGN, kMaxK>(Xo, scratch, PITCH, kout, tw.t32, tw.log, w.lane);
+            const float2* Yr = r ? scratch : Xo;
             for (int g = 0; g < kout; g++) {
-                CO* d = dst + (size_t)g * Hs + (size_t)k1 * NF;
+                float2* d = dst + (size_t)g * Hs + (size_t)k1 * NF;
 #pragma unroll
                 for (int i = 0; i < E; i++) d[w.lane + kWarp * i] = Yr[(size_t)g * PITCH + w.lane + kWarp * i];
             }
@@ -907,8 +866,8 @@ __device__ void col_pass_fixed(const Params& P, const Tw& tw, int kin, int kout,
 // slot did (256^3, 8 warps with two slots -> 16 with one: row pass 129 -> 109,
 // column pass 140 -> 90 us).  The transforms run on two buffers in the padded layout
 // (fft.cuh: no bank conflicts in the strided stages).  Selected on the host
-// (Params::stage) where a warp's slice of shared memory, sized for the FP64
-// phases, holds them; K fields per line (PFC: 1), NS arrays of pointwise state.
+// (Params::stage) for those lengths, a warp's slice of shared memory being sized
+// for them; K fields per line (PFC: 1), NS arrays of pointwise state.
 //
 // Row unit: rows r0, r0 + 1.  Slot = K x (N/2 + 1) 16-byte pieces (the two
 // rows' coefficients at k, adjacent in the [k][row] layout) + NS x 2 rows of
@@ -1393,7 +1352,7 @@ __device__ void col_pass_fx(const Params& P, const Tw& tw, int kin, int kout, co
 // ------------------------------------------------ CTA-cooperative variants
 //
 // One unit per CTA: the threads of the CTA load and convert the unit's lines,
-// transform them together (fx_lines_coop), share the pointwise work and store,
+// transform them together (fx_coop), share the pointwise work and store,
 // with CTA barriers in between.  For phases with fewer units than warps (a
 // 256^2 grid has 128 row units and 129 columns).  The FP64 instructions left
 // in a pass are its pointwise ones: an SM sub-partition issues one in 64
@@ -1563,33 +1522,31 @@ __device__ void col_pass_coop_fx(const Params& P, const Tw& tw, int kin, int kou
 
 // FP32 lines with one unit per CTA (the incremental base evaluations, whose
 // pointwise work is FP64, and the opt-in FP32 iteration passes)
-template <class TI, class TO, int NF, class Ld, class Ap>
-__device__ void row_pass_coop(const Params& P, const Tw& tw, int kin, int kout, const cx<TI>* src, cx<TO>* dst,
+template <int NF, class Ld, class Ap>
+__device__ void row_pass_coop(const Params& P, const Tw& tw, int kin, int kout, const float2* src, float2* dst,
                               char* smem, Ld&& ld, Ap&& ap) {
-    using CI = cx<TI>;
-    using CO = cx<TO>;
     using S = decltype(ld(0ll, 0, 0));
     const int n = NF > 0 ? NF : P.n1, logn = NF > 0 ? ilog2c(NF) : P.logn1, half = n >> 1, pitch = n + 2, rows = P.rows;
     const long long Hs = P.H;
     const int tid = threadIdx.x, nthr = blockDim.x;
-    CI* X0 = (CI*)smem;
-    CI* X1 = X0 + (size_t)kin * pitch;
-    CO* Y0 = (CO*)(X1 + (size_t)kin * pitch);
-    CO* Y1 = Y0 + (size_t)kout * pitch;
-    const TI iscale = (TI)P.inv_npts;
+    float2* X0 = (float2*)smem;
+    float2* X1 = X0 + (size_t)kin * pitch;
+    float2* Y0 = (float2*)(X1 + (size_t)kin * pitch);
+    float2* Y1 = Y0 + (size_t)kout * pitch;
+    const float iscale = (float)P.inv_npts;
     for (int u = blockIdx.x; u < rows / 2; u += gridDim.x) {
         const int r0 = 2 * u;
         // inverse x-DFT inputs: complex line x of field l packs rows r0, r0 + 1
         for (int it = tid; it < kin * n; it += nthr) {
             const int l = it >> logn, x = it & (n - 1);
             const int k = (x <= half) ? x : n - x;
-            const CI* s0 = src + (size_t)l * Hs + (size_t)k * rows + r0;
-            CI A = s0[0], B = s0[1];
+            const float2* s0 = src + (size_t)l * Hs + (size_t)k * rows + r0;
+            float2 A = s0[0], B = s0[1];
             if (x == 0 || x == half) { A.y = 0; B.y = 0; }
-            X0[(size_t)l * pitch + x] = (x <= half) ? CI{A.x - B.y, A.y + B.x} : CI{A.x + B.y, B.x - A.y};
+            X0[(size_t)l * pitch + x] = (x <= half) ? float2{A.x - B.y, A.y + B.x} : float2{A.x + B.y, B.x - A.y};
         }
-        const CI* Xr = X0;
-        if (kin > 0) Xr = fft_coop<+1, TI>(X0, X1, logn, pitch, kin, tw.t32, tw.log, tid, nthr) ? X1 : X0;
+        const float2* Xr = X0;
+        if (kin > 0) Xr = fft_coop<+1, float>(X0, X1, logn, pitch, kin, tw.t32, tw.log, tid, nthr) ? X1 : X0;
         // pointwise: point q = rr n + x of the unit (consecutive threads, consecutive x)
         for (int q0 = 0; q0 < 2 * n; q0 += nthr * kCoopChunk) {
             S st[kCoopChunk];
@@ -1606,12 +1563,12 @@ __device__ void row_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
                 const int q = q0 + tid + nthr * c;
                 if (q < 2 * n) {
                     const int rr = q >> logn, x = q & (n - 1);
-                    TI in[kMaxK];
-                    TO out[kMaxK];
+                    float in[kMaxK];
+                    float out[kMaxK];
 #pragma unroll
                     for (int f = 0; f < kMaxK; f++) {
                         if (f < kin) {
-                            const CI z = Xr[(size_t)f * pitch + x];
+                            const float2 z = Xr[(size_t)f * pitch + x];
                             in[f] = (rr ? z.y : z.x) * iscale;
                         }
                     }
@@ -1619,7 +1576,7 @@ __device__ void row_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
 #pragma unroll
                     for (int g = 0; g < kMaxK; g++) {
                         if (g < kout) {
-                            CO* qq = Y0 + (size_t)g * pitch + x;
+                            float2* qq = Y0 + (size_t)g * pitch + x;
                             if (rr) qq->y = out[g];
                             else qq->x = out[g];
                         }
@@ -1628,48 +1585,46 @@ __device__ void row_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
             }
         }
         if (kout > 0) {
-            const CO* Yr = fft_coop<-1, TO>(Y0, Y1, logn, pitch, kout, tw.t32, tw.log, tid, nthr) ? Y1 : Y0;
-            const TO hf = (TO)0.5;
+            const float2* Yr = fft_coop<-1, float>(Y0, Y1, logn, pitch, kout, tw.t32, tw.log, tid, nthr) ? Y1 : Y0;
+            const float hf = 0.5f;
             for (int it = tid; it < kout * (half + 1); it += nthr) {
                 const int g = it / (half + 1), k = it - g * (half + 1);
-                CO* d0 = dst + (size_t)g * Hs + r0;
-                const CO* zl = Yr + (size_t)g * pitch;
-                const CO zk = zl[k];
-                const CO zn = zl[(n - k) & (n - 1)];
-                d0[(size_t)k * rows] = CO{hf * (zk.x + zn.x), hf * (zk.y - zn.y)};
-                d0[(size_t)k * rows + 1] = CO{hf * (zk.y + zn.y), hf * (zn.x - zk.x)};
+                float2* d0 = dst + (size_t)g * Hs + r0;
+                const float2* zl = Yr + (size_t)g * pitch;
+                const float2 zk = zl[k];
+                const float2 zn = zl[(n - k) & (n - 1)];
+                d0[(size_t)k * rows] = float2{hf * (zk.x + zn.x), hf * (zk.y - zn.y)};
+                d0[(size_t)k * rows + 1] = float2{hf * (zk.y + zn.y), hf * (zn.x - zk.x)};
             }
         }
         cta_sync();  // the next unit reuses the buffers
     }
 }
 
-template <class TI, class TO, int NF, class Ld, class Ap>
-__device__ void col_pass_coop(const Params& P, const Tw& tw, int kin, int kout, const cx<TI>* src, cx<TO>* dst,
+template <int NF, class Ld, class Ap>
+__device__ void col_pass_coop(const Params& P, const Tw& tw, int kin, int kout, const float2* src, float2* dst,
                               char* smem, Ld&& ld, Ap&& ap) {
-    using C = cx<TI>;
-    using CO = cx<TO>;
     using S = decltype(ld(Line{}, 0));
     const int n = NF > 0 ? NF : P.n0, logn = NF > 0 ? ilog2c(NF) : P.logn0, pitch = n + 2, ncols = P.ncols;
     const long long Hs = P.H;
     const int kl = kin > kout ? kin : kout;
     const int tid = threadIdx.x, nthr = blockDim.x;
-    C* B0 = (C*)smem;
-    C* B1 = B0 + (size_t)kl * pitch;
+    float2* B0 = (float2*)smem;
+    float2* B1 = B0 + (size_t)kl * pitch;
     for (int k1 = blockIdx.x; k1 < ncols; k1 += gridDim.x) {
         const Line ln = line_of(P, tw, k1);
         for (int it = tid; it < kin * n; it += nthr) {
             const int f = it >> logn, x = it & (n - 1);
             B0[(size_t)f * pitch + x] = src[(size_t)f * Hs + (size_t)k1 * n + x];
         }
-        const C* Xr = B0;
-        C* Xi = B1;
+        const float2* Xr = B0;
+        float2* Xi = B1;
         if (kin > 0) {
-            const int r = fft_coop<-1, TI>(B0, B1, logn, pitch, kin, tw.t32, tw.log, tid, nthr);
+            const int r = fft_coop<-1, float>(B0, B1, logn, pitch, kin, tw.t32, tw.log, tid, nthr);
             Xr = r ? B1 : B0;
             Xi = r ? B0 : B1;
         }
-        CO* Xo = (CO*)Xi;
+        float2* Xo = (float2*)Xi;
         for (int q0 = 0; q0 < n; q0 += nthr * kCoopChunk) {
             S st[kCoopChunk];
 #pragma unroll
@@ -1681,8 +1636,8 @@ __device__ void col_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
             for (int c = 0; c < kCoopChunk; c++) {
                 const int k0 = q0 + tid + nthr * c;
                 if (k0 < n) {
-                    C in[kMaxK];
-                    CO out[kMaxK];
+                    float2 in[kMaxK];
+                    float2 out[kMaxK];
 #pragma unroll
                     for (int f = 0; f < kMaxK; f++)
                         if (f < kin) in[f] = Xr[(size_t)f * pitch + k0];
@@ -1694,9 +1649,9 @@ __device__ void col_pass_coop(const Params& P, const Tw& tw, int kin, int kout, 
             }
         }
         if (kout > 0) {
-            CO* scratch = (CO*)Xr;
-            const int r = fft_coop<+1, TO>(Xo, scratch, logn, pitch, kout, tw.t32, tw.log, tid, nthr);
-            const CO* Yr = r ? scratch : Xo;
+            float2* scratch = (float2*)Xr;
+            const int r = fft_coop<+1, float>(Xo, scratch, logn, pitch, kout, tw.t32, tw.log, tid, nthr);
+            const float2* Yr = r ? scratch : Xo;
             for (int it = tid; it < kout * n; it += nthr) {
                 const int g = it >> logn, x = it & (n - 1);
                 dst[(size_t)g * Hs + (size_t)k1 * n + x] = Yr[(size_t)g * pitch + x];
@@ -1729,30 +1684,29 @@ __host__ __device__ __forceinline__ size_t mid_warp_smem(int nm, int sz) {
 }
 __host__ __device__ __forceinline__ int mid_units(const Params& P) { return P.h1 * (P.n0 / kMidG); }
 
-template <class T, int S, int NF>
-__device__ void mid_pass(const Params& P, const Tw& tw, int k, const cx<T>* src, cx<T>* dst, char* smem) {
-    using C = cx<T>;
+template <int S, int NF>
+__device__ void mid_pass(const Params& P, const Tw& tw, int k, const float2* src, float2* dst, char* smem) {
     constexpr int L = NF & (kNoCoop - 1);  // fixed line length of the launch (0: runtime)
     // values per lane loaded before any of them is stored to shared memory
     // (the compiler cannot move a global load above a shared store itself)
-    constexpr int CH = sizeof(T) == 4 ? 16 : 8;
+    constexpr int CH = 16;
     const int nm = P.nm, logm = P.logm, n0 = P.n0, rows = P.rows, gpp = P.n0 / kMidG;
     const long long H = P.H;
     const int pitch = pitch_of(nm);
     const int nv = kMidG * nm;
     const WarpCtx w = warp_ctx(P, smem);
-    C* B0 = (C*)w.mem;
-    C* B1 = B0 + (size_t)kMidG * pitch;
+    float2* B0 = (float2*)w.mem;
+    float2* B1 = B0 + (size_t)kMidG * pitch;
     const URange ur = units_of(tw, P.h1 * gpp);
     for (int u = ur.b; u < ur.e; u += ur.s) {
         const int k1 = u / gpp, i0 = (u - k1 * gpp) * kMidG;
         for (int f = 0; f < k; f++) {
-            const C* sf = src + (size_t)f * H;
-            C* df = dst + (size_t)f * H;
+            const float2* sf = src + (size_t)f * H;
+            float2* df = dst + (size_t)f * H;
             const size_t rowbase = (size_t)k1 * rows + (size_t)i0 * nm;    // [k1][i0][i1]
             const size_t colbase = (size_t)k1 * nm * n0 + (size_t)i0;      // [k1][km][i0]
             for (int j0 = 0; j0 < nv; j0 += CH * kWarp) {
-                C v[CH];
+                float2 v[CH];
 #pragma unroll
                 for (int q = 0; q < CH; q++) {
                     const int j = j0 + w.lane + q * kWarp;
@@ -1778,16 +1732,16 @@ __device__ void mid_pass(const Params& P, const Tw& tw, int k, const cx<T>* src,
             if constexpr (L > 0) {
                 if (nm == L) {
                     // cubic grid: both lines in lockstep through the fixed-length stages
-                    r = fft_lines_fixed<S, T, ilog2c(L), kMidG>(B0, B1, pitch, kMidG, tw.t32, tw.log, w.lane);
+                    r = fft_lines_fixed<S, float, ilog2c(L), kMidG>(B0, B1, pitch, kMidG, tw.t32, tw.log, w.lane);
                 } else {
                     for (int g = 0; g < kMidG; g++)
-                        r = fft_line_w<S, T>(B0 + g * pitch, B1 + g * pitch, logm, tw.t32, tw.log, w.lane);
+                        r = fft_line_w<S, float>(B0 + g * pitch, B1 + g * pitch, logm, tw.t32, tw.log, w.lane);
                 }
             } else {
                 for (int g = 0; g < kMidG; g++)
-                    r = fft_line_w<S, T>(B0 + g * pitch, B1 + g * pitch, logm, tw.t32, tw.log, w.lane);
+                    r = fft_line_w<S, float>(B0 + g * pitch, B1 + g * pitch, logm, tw.t32, tw.log, w.lane);
             }
-            const C* Br = r ? B1 : B0;
+            const float2* Br = r ? B1 : B0;
             for (int j = w.lane; j < nv; j += kWarp) {
                 if (S < 0) {
                     const int km = j / kMidG, g = j - km * kMidG;
@@ -1982,18 +1936,18 @@ __device__ __forceinline__ void rowp(const Params& P, const Tw& tw, int kin, int
     } else {
         if constexpr (COOP && !(NF & kNoCoop)) {
             if (P.coop) {
-                row_pass_coop<TI, TO, L>(P, tw, kin, kout, src, dst, smem, ld, ap);
+                row_pass_coop<L>(P, tw, kin, kout, src, dst, smem, ld, ap);
                 return;
             }
         }
         if constexpr (L == 0)
-            row_pass<TI, TO>(P, tw, kin, kout, src, dst, smem,
+            row_pass(P, tw, kin, kout, src, dst, smem,
                              [&](long long p, int row, int x, const TI* in, TO* out) {
                                  const auto s = ld(p, row, x);
                                  ap(p, row, x, s, in, out);
                              });
         else
-            row_pass_fixed<TI, TO, L>(P, tw, kin, kout, src, dst, smem, ld, ap);
+            row_pass_fixed<L>(P, tw, kin, kout, src, dst, smem, ld, ap);
     }
 }
 
@@ -2012,17 +1966,17 @@ __device__ __forceinline__ void colp2(const Params& P, const Tw& tw, int kin, in
     } else {
         if constexpr (COOP && !(NF & kNoCoop)) {
             if (P.coop) {
-                col_pass_coop<TI, TO, L>(P, tw, kin, kout, src, dst, smem, ld, ap);
+                col_pass_coop<L>(P, tw, kin, kout, src, dst, smem, ld, ap);
                 return;
             }
         }
         if constexpr (L == 0)
-            col_pass<TI, TO>(P, tw, kin, kout, src, dst, smem, [&](const Line& k1, int k0, const cx<TI>* in, cx<TO>* out) {
+            col_pass(P, tw, kin, kout, src, dst, smem, [&](const Line& k1, int k0, const cx<TI>* in, cx<TO>* out) {
                 const auto s = ld(k1, k0);
                 ap(k1, k0, s, in, out);
             });
         else
-            col_pass_fixed<TI, TO, L>(P, tw, kin, kout, src, dst, smem, ld, ap);
+            col_pass_fixed<L>(P, tw, kin, kout, src, dst, smem, ld, ap);
     }
 }
 template <class T, int NF, bool COOP = kHasCoop<T, T>, class Ld, class Ap>
@@ -2472,11 +2426,11 @@ template <class T> __device__ __forceinline__ RowK<T> row_consts(const Params& P
 // max-norm and sum accumulators, the extrapolated iterate y and the nonlinear
 // term(s) at it (PFC: (b + y)^3 - b^3; FCH: the differences of F' and of the
 // second variation's nonlinear part).
-template <class T, class TI, bool PFC>
+template <class T, bool PFC>
 __device__ __forceinline__ void row_point(const RowK<T>& q, T* dcur, long long p, T dp, T dpp, T b, T lb,
-                                          const TI* in, T* out, MaxAbs<TI>& amax, SumOf<T>& asum) {
-    const TI dd = in[0];
-    const T de = dp + q.lp * (dp - dpp) + q.ts * (T)dd;
+                                          const T* in, T* out, MaxAbs<T>& amax, SumOf<T>& asum) {
+    const T dd = in[0];
+    const T de = dp + q.lp * (dp - dpp) + q.ts * dd;
     dcur[p] = de;
     amax.add(dd);
     asum.add(de);
@@ -2485,7 +2439,7 @@ __device__ __forceinline__ void row_point(const RowK<T>& q, T* dcur, long long p
         out[0] = y * ((T)3 * b * (b + y) + y * y);
     } else {
         const T tau = q.tau;
-        const T ly = (T)in[1];
+        const T ly = in[1];
         const T f1b = dF1(b, tau), f2b = dF2(b, tau);
         const T df1 = y * ((T)3 * b * (b + y) + y * y + tau * ((T)2 * b + y) - (T)1);
         const T df2 = y * ((T)6 * b + (T)3 * y + (T)2 * tau);
@@ -2510,7 +2464,7 @@ __device__ __noinline__ void phase_R_staged(const Params& P, const Ctl& c, const
     MaxAbs<float> amax;
     SumOf<float> asum;
     auto pt = [&](long long p, int, int, const float* sv, const float* in, float* out) {
-        row_point<float, float, PFC>(q, dcur, p, sv[0], sv[1], sv[2], NS > 3 ? sv[NS > 3 ? 3 : 0] : 0.f, in, out, amax,
+        row_point<float, PFC>(q, dcur, p, sv[0], sv[1], sv[2], NS > 3 ? sv[NS > 3 ? 3 : 0] : 0.f, in, out, amax,
                                      asum);
     };
     if constexpr (!PFC && NF % (2 * kWarp) == 0) {
@@ -2547,23 +2501,23 @@ __device__ __noinline__ void phase_R_coop(const Params& P, const Ctl& c, const T
     MaxAbs<float> amax;
     SumOf<float> asum;
     struct St { float dp, dpp, b, lb; };
-    row_pass_coop<float, float, NF>(
+    row_pass_coop<NF>(
         P, tw, K, K, src, (float2*)P.NB, smem,
         [&](long long p, int, int) { return St{dprev[p], dcur[p], vbt[p], pfc ? 0.f : lbt[p]}; },
         [&](long long p, int, int, const St& s, const float* in, float* out) {
-            if (pfc) row_point<float, float, true>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
-            else row_point<float, float, false>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
+            if (pfc) row_point<float, true>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
+            else row_point<float, false>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
         });
     publish_eval(P, tw, true, bank, c.ev, amax, asum);
 }
 
-// Iteration row pass (R1 reads the FP64 base direction, RI the T one):
+// Iteration row pass (R1 reads the base's direction, RI the column pass's, both in T):
 // delta_it = ybar_{it-1} + theta_v s d_{it-1}; ||d_{it-1}||_inf; then the
 // nonlinear differences at ybar_it and their forward x-DFT.
-template <class TI, class T, int NF>
+template <class T, int NF>
 __device__ PAGD_HOT void phase_R(const Params& P, const Ctl& c, const Tw& tw, char* smem, double* red,
-                        const cx<TI>* src) {
-    if constexpr (sizeof(TI) == 4 && sizeof(T) == 4) {
+                        const cx<T>* src) {
+    if constexpr (sizeof(T) == 4) {
         if (P.stage) {
             constexpr int L = NF & (kNoCoop - 1);
             if constexpr (L != 0) {
@@ -2593,11 +2547,11 @@ __device__ PAGD_HOT void phase_R(const Params& P, const Ctl& c, const Tw& tw, ch
     const T* vbt = (const T*)P.VBt;
     const T* lbt = (const T*)P.LBt;
     const int K = k_iter(P.model);
-    MaxAbs<TI> amax;
+    MaxAbs<T> amax;
     SumOf<T> asum;
     const bool pfc = P.model == M_PFC;
     struct St { T dp, dpp, b, lb; };
-    rowp<TI, T, NF>(
+    rowp<T, T, NF>(
         P, tw, K, K, src, (cx<T>*)P.NB, smem,
         [&](long long p, int, int) {
             St s;
@@ -2607,9 +2561,9 @@ __device__ PAGD_HOT void phase_R(const Params& P, const Ctl& c, const Tw& tw, ch
             s.lb = pfc ? (T)0 : lbt[p];
             return s;
         },
-        [&](long long p, int, int, const St& s, const TI* in, T* out) {
-            if (pfc) row_point<T, TI, true>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
-            else row_point<T, TI, false>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
+        [&](long long p, int, int, const St& s, const T* in, T* out) {
+            if (pfc) row_point<T, true>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
+            else row_point<T, false>(q, dcur, p, s.dp, s.dpp, s.b, s.lb, in, out, amax, asum);
         });
     publish_eval(P, tw, true, bank, c.ev, amax, asum);
 }
@@ -2699,7 +2653,7 @@ __device__ __noinline__ void phase_CI_coop(const Params& P, const Ctl& c, const 
     const int K = k_iter(P.model);
     const bool pfc = P.model == M_PFC;
     struct St { float2 sc, sp, g0; };
-    col_pass_coop<float, float, NF>(
+    col_pass_coop<NF>(
         P, tw, K, K, csrcT<float>(P), cdstT<float>(P), smem,
         [&](const Line& k1, int k0) {
             const long long idx = (long long)k1 * P.n0 + k0;
@@ -3488,7 +3442,7 @@ __device__ __forceinline__ void mid_iter(const Params& P, const Tw& tw, int k, c
                 return;
             }
         }
-        mid_pass<float, S, NF>(P, tw, k, (const float2*)src, (float2*)dst, smem);
+        mid_pass<S, NF>(P, tw, k, (const float2*)src, (float2*)dst, smem);
     }
 }
 
@@ -3496,7 +3450,7 @@ template <class T, int NF>
 __device__ __forceinline__ void exec_phase(const Params& P, const Ctl& c, const Tw& tw, char* smem, double* red) {
     switch (c.ph) {
         case PH_R1:
-        case PH_RI: phase_R<T, T, NF>(P, c, tw, smem, red, (const cx<T>*)P.DB); break;
+        case PH_RI: phase_R<T, NF>(P, c, tw, smem, red, (const cx<T>*)P.DB); break;
         case PH_CI: phase_CI<T, NF>(P, c, tw, smem); break;
         case PH_MF:
             if (c.m64) mid_pass_fx<-1, NF>(P, tw, c.mk, P.NB64, P.X64, smem);
@@ -3593,7 +3547,8 @@ __host__ __device__ inline int unit_cost(const Params& P, int ph) {
 // accept 2x (8.8x, 6x and 5x while lines were transformed in FP64).  FCH (8
 // members of 512^2): its iteration passes carry two fields, about 2x a PFC pass
 // per point; relative to them, exact base passes 4.5-5x, incremental B / C / D /
-// E 4.0 / 2.3 / 1.7 / 3.2x, accept 1.5x.  The batched
+// E 4.0 / 2.3 / 1.7 / 3.2x, accept 1.5x.  (The FCH figures were taken while lines
+// were transformed in FP64 and are due to be taken again.)  The batched
 // launch lays members out on a cost axis of points x this weight, so that a
 // global phase mixing members in FP64 base evaluations with members in FP32
 // iterations gives every warp about the same time of work.  Only the dealing

@@ -95,8 +95,8 @@ template <int NF> bool run(const char* pass, int n, int k, bool up, float state,
         else if (is("col_coop_fx")) { f32 = false; col_pass_coop_fx<double, NF>(P, t, k, k, s64, d64, mem, ld_col, cf); }
         else if (is("col_sum_fx")) col_pass_fx<float, NF>(P, t, k, 1, s64, d32.data(), mem, ld_col, csum);
         else if (is("col_sum_coop_fx")) col_pass_coop_fx<float, NF>(P, t, k, 1, s64, d32.data(), mem, ld_col, csum);
-        else if (is("row_coop")) row_pass_coop<float, float, NF>(P, t, k, k, s32.data(), d32.data(), mem, ld_row, rf);
-        else if (is("col_coop")) col_pass_coop<float, float, NF>(P, t, k, k, s32.data(), d32.data(), mem, ld_col, cf);
+        else if (is("row_coop")) row_pass_coop<NF>(P, t, k, k, s32.data(), d32.data(), mem, ld_row, rf);
+        else if (is("col_coop")) col_pass_coop<NF>(P, t, k, k, s32.data(), d32.data(), mem, ld_col, cf);
         else if (is("mid_fx_fwd")) { f32 = false; mid_pass_fx<-1, NF>(P, t, k, s64, d64, mem); }
         else if (is("mid_fx_inv")) { f32 = false; mid_pass_fx<+1, NF>(P, t, k, s64, d64, mem); }
         else if constexpr (NF > 0) {
