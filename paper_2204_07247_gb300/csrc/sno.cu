@@ -857,6 +857,12 @@ pagd_status sno_create(sno_net** out, int n0, int n1, int channels, int layers, 
     if (!s) return PAGD_ENOMEM;
     SnoDims& d = s->d;
     d = SnoDims{n0, n1, n0 * n1, channels, layers, modes0, modes1, modes0 * modes1, 0, 0, 0, 0, 0, 0};
+    // QC points of a row per lane: more points share the twiddle sums of their
+    // residue, but fewer than 32 residues leave lanes idle.  Inference / gradient in
+    // us, 16 channels, 4 layers, 16 x 16 modes, QC = 1, 4, 16: 64 samples of 32^2
+    // 263 / 706, 300 / 807, 451 / 1191; 64 of 64^2 554 / 1395, 417 / 1147, 757 /
+    // 1971; 8 of 256^2 904 / 2050, 400 / 1007, 431 / 1121; 4 of 512^2 2164 / 4678,
+    // 814 / 1972, 476 / 1322.
     d.QC = n1 >= 512 ? 16 : n1 >= 64 ? 4 : 1;
     d.J = n1 / d.QC;
     d.JB = d.J > 32 ? d.J / 32 : 1;
