@@ -134,12 +134,22 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxCtas) pagd_kernel(const __gri
 }
 
 
+// The dynamic shared memory a kernel may take, whatever this launch needs: the
+// attribute is the process's, and a launch that lowered it to its own size would
+// fail another thread's.  (2 KB of the SM's 227 are left to the kernels' static
+// shared memory; a launch that needs them asks for its own size.)
+template <class K> cudaError_t allow_smem(K* kern, size_t smem) {
+    const size_t most = (227 - 2) * 1024;
+    return cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(smem > most ? smem : most));
+}
+
 // Launch pagd_kernel<T, NF> cooperatively: the grid is capped at the number of
 // co-resident CTAs so that the device-wide barrier is safe.
 template <class T, int NF>
 cudaError_t pagd_launch(const Params& P, int grid, int threads, size_t smem, void* stream, int* grid_used) {
     void (*kern)(const Params) = pagd_kernel<T, NF>;
-    cudaError_t e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)kern, threads, smem);

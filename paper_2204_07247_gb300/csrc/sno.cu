@@ -753,12 +753,19 @@ static void plan(sno_net* s) {
         if (e_ != cudaSuccess) return sno_fail(s, PAGD_ECUDA, cudaGetErrorString(e_)); \
     } while (0)
 
+// A kernel may take all of an SM's shared memory, whatever this call needs: the
+// attribute is the process's, and a call that lowered it to its own size would
+// fail another thread's launch.
+constexpr int kMaxSmem = 227 * 1024;
+template <class K> static cudaError_t allow_smem(K* kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+}
+
 template <int MODE, int QC, int CT, int MM>
 static cudaError_t launch_tile(const SnoDims& d, const TileArgs& a, int B, cudaStream_t st) {
     const size_t smem = tile_smem(d, CT);
     if (smem > 48 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_tile<MODE, QC, CT, MM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(k_tile<MODE, QC, CT, MM>);
         if (e != cudaSuccess) return e;
     }
     k_tile<MODE, QC, CT, MM><<<dim3(d.NT, B), kThr, smem, st>>>(d, a);
@@ -776,7 +783,7 @@ template <int MODE> static cudaError_t tile(const SnoDims& d, const TileArgs& a,
 template <int CT> static cudaError_t launch_wgrad(const SnoDims& d, const float* dz, const float* v, float* part, int B,
                                                   cudaStream_t st) {
     const size_t smem = std::max<size_t>((size_t)2 * CT * kPitch, (size_t)8 * CT * (CT + 1)) * sizeof(float);
-    const cudaError_t e = cudaFuncSetAttribute(k_wgrad<CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k_wgrad<CT>);
     if (e != cudaSuccess) return e;
     k_wgrad<CT><<<dim3((d.np + kTile - 1) / kTile, B), kThr, smem, st>>>(d, dz, v, part);
     return cudaGetLastError();
@@ -804,7 +811,7 @@ static void set_layer(TileArgs& a, const SnoDims& d, int l) {
 static cudaError_t launch_cols(const sno_net* s, int G, const float2* T, float2* F) {
     const SnoDims& d = s->d;
     const size_t smem = sizeof(float2) * (d.n0 + (size_t)kColRows * d.M1 + kColThr);
-    const cudaError_t e = cudaFuncSetAttribute(k_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k_cols);
     if (e != cudaSuccess) return e;
     k_cols<<<G, kColThr, smem, (cudaStream_t)s->stream>>>(d, T, (const float2*)(s->ws + s->off_tw0), F);
     return cudaGetLastError();
