@@ -1686,7 +1686,9 @@ __host__ __device__ __forceinline__ int mid_units(const Params& P) { return P.h1
 
 // (A function of its own, and eight values a lane: inlined into the kernel of 128
 // registers with sixteen it spilled.  FCH FP32-mixed, inverse pass: 8 x 128 x 16
-// 12.8 -> 8.8 us, 16 x 64 x 16 10.1 -> 7.9, 32^3 9.1 -> 7.1.)
+// 12.8 -> 8.8 us, 16 x 64 x 16 10.1 -> 7.9, 32^3 9.1 -> 7.1.  The FP64 one below stays
+// inlined: apart, FCH 256^2 LBDF2 took 5627 us instead of 5393, 256^3 transforms
+// 1289 instead of 1270.)
 template <int S, int NF>
 __device__ __noinline__ void mid_pass(const Params& P, const Tw& tw, int k, const float2* src, float2* dst, char* smem) {
     constexpr int L = NF & (kNoCoop - 1);  // fixed line length of the launch (0: runtime)
@@ -1762,7 +1764,7 @@ __device__ __noinline__ void mid_pass(const Params& P, const Tw& tw, int k, cons
 // The same pass on FP64 lines in fixed point: the unit's kMidG lines one
 // after the other through a warp's line buffers.
 template <int S, int NF>
-__device__ __noinline__ void mid_pass_fx(const Params& P, const Tw& tw, int k, const double2* src, double2* dst, char* smem) {
+__device__ void mid_pass_fx(const Params& P, const Tw& tw, int k, const double2* src, double2* dst, char* smem) {
     constexpr int L = NF & (kNoCoop - 1);
     constexpr int CH = 8;
     const int nm = P.nm, logm = P.logm, n0 = P.n0, rows = P.rows, gpp = P.n0 / kMidG;
