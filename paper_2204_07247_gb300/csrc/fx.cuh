@@ -244,12 +244,14 @@ struct Sum3 {
 
 // ---------------------------------------------------------- warp-owned line
 
-// radix of the stage that starts at LOGNS: as stage_radix, but 4, 8, 4 for 128
-// points, whose first and last butterflies then cover all lanes, and 4 (2 at the
-// end) up to 64 points, where a warp has eight butterflies of radix 8 or fewer:
-// PFC FP64 64^3 1701 -> 1452 us for two steps, 32 x 16 x 64 1094 -> 1002.
+// radix of the stage that starts at LOGNS: as stage_radix, but 4 (and one 2) up
+// to 128 points, where a warp has fewer butterflies of radix 8 than lanes.  128
+// points go 2, 4, 4, 4: their first and last butterflies then cover all lanes.
+// PFC FP64, two steps, radix 8 / 4: 64^3 1701 / 1452 us, 32 x 16 x 64 1094 / 1002,
+// a batch of 32 members of 128^2 1964 / 1616, of 4 987 / 904.
 __host__ __device__ constexpr int fx_radix(int logn, int logns) {
-    return logn == 7 ? (logns == 2 ? 8 : 4) : logn < 7 ? (logn - logns >= 2 ? 4 : 2) : stage_radix(logn, logns);
+    if (logn == 7) return logns == 0 ? 2 : 4;
+    return logn < 7 ? (logn - logns >= 2 ? 4 : 2) : stage_radix(logn, logns);
 }
 
 template <int R, int S, int LOGN, int LOGNS, bool FIRST>

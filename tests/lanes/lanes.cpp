@@ -125,6 +125,7 @@ int lanes_pass(const char* pass, int n, int nf, int k, int up, double state, con
     switch (nf) {
         case 0: return run<0>(pass, n, k, up != 0, (float)state, src, dst);
         case 64: return run<64>(pass, n, k, up != 0, (float)state, src, dst);
+        case 128: return run<128>(pass, n, k, up != 0, (float)state, src, dst);
         case 512: return run<512>(pass, n, k, up != 0, (float)state, src, dst);
     }
     return 0;

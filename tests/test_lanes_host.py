@@ -47,7 +47,7 @@ PASSES = [("col_sum_fx", 3), ("col_sum_coop_fx", 3), ("row_fx", 3), ("row_coop_f
           ("row_coop", 2), ("col_coop", 2), ("mid_fx_fwd", 2), ("mid_fx_inv", 2), ("row_staged", 1), ("row_staged", 2),
           ("col_staged", 1), ("col_staged", 2), ("row_pair", 2), ("col_pair", 2), ("mid_staged_fwd", 2), ("mid_staged_inv", 2)]
 # (points of a line, compile-time length or 0; the staged passes have compile-time lengths only)
-CASES = [(p, k, n, nf) for p, k in PASSES for n, nf in [(8, 0), (16, 0), (32, 0), (64, 0), (64, 64), (512, 512)]
+CASES = [(p, k, n, nf) for p, k in PASSES for n, nf in [(8, 0), (16, 0), (32, 0), (64, 0), (128, 0), (64, 64), (128, 128), (512, 512)]
          if nf or not ("staged" in p or "pair" in p)]
 
 
