@@ -163,6 +163,28 @@ template <int V> __device__ __forceinline__ void reduce_deal(float* v, int lane)
     }
 }
 
+// The same with the rounding errors beside the sums (two-sum): on return v holds
+// the sums and e the errors.
+template <int V> __device__ __forceinline__ void reduce_deal2(float* v, float* e, int lane) {
+    int cnt = V;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const bool up = (lane & s) != 0;
+        const int hf = cnt / 2;
+#pragma unroll
+        for (int i = 0; i < V / 2; i++) {
+            if (i < hf) {
+                const float got = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + hf], s);
+                const float gotE = s < 16 ? __shfl_xor_sync(0xffffffffu, up ? e[i] : e[i + hf], s) : 0.f;
+                const float keepE = s < 16 ? (up ? e[i + hf] : e[i]) : 0.f;
+                v[i] = up ? v[i + hf] : v[i];
+                e[i] = pagd::Sum3::two_sum(v[i], got) + (keepE + gotE);
+            }
+        }
+        cnt = hf;
+    }
+}
+
 // What a tile kernel does at its points (k_tile)
 enum { T_LIFT, T_LAYER, T_GUESS, T_LOSS, T_BACK, T_BACK0 };
 
@@ -183,7 +205,7 @@ struct TileArgs {
     const float2 *tw0, *tw1;
     double* guess;
     double* loss;
-    float* part;          // per-block sums: T_LOSS [C + 1], T_BACK0 [C][3]
+    float* part;          // per-block sums: T_LOSS [C + 1][2], T_BACK0 [C][3]
 };
 
 // One tile of every channel, in one block:
@@ -411,28 +433,56 @@ __global__ void __launch_bounds__(kThr, CT <= 16 ? 3 : 1) k_tile(SnoDims d, Tile
             }
         }
     }
-    if constexpr (MODE == T_LOSS || MODE == T_BACK0) {
-        // block sums of the per-thread accumulators -> one row of part
-        constexpr int NV = MODE == T_LOSS ? CT + 1 : 3 * CT;
-        float* red = (float*)U;  // [kThr / 32][NV]: the spectral part's buffers are free
-        const int nv = MODE == T_LOSS ? d.C + 1 : 3 * d.C;
+    float* red = (float*)U;  // the spectral part's buffers are free
+    if constexpr (MODE == T_LOSS) {
+        // block sums of the per-thread accumulators -> one row of part, two words
+        // each: they nearly cancel over the grid (half the rounding errors of
+        // dQ, db_Q came from here)
+        constexpr int NV = CT + 1, V = CT <= 16 ? 32 : 64, PL = V / 32;
+        float v[V], e[V];
+#pragma unroll
+        for (int c = 0; c < V; c++) {
+            v[c] = c < NV ? qacc[c] : 0.f;
+            e[c] = 0.f;
+        }
+        reduce_deal2<V>(v, e, lane);
+#pragma unroll
+        for (int q = 0; q < PL; q++) {
+            const int c = lane * PL + q;
+            if (c < NV) {
+                red[(warp * NV + c) * 2] = v[q];
+                red[(warp * NV + c) * 2 + 1] = e[q];
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, o);
+        if (lane == 0) atomicAdd(a.loss, lacc * (0.5 * a.dscale));
+        __syncthreads();
+        const int nv = d.C + 1;
+        for (int i = tid; i < nv; i += kThr) {
+            const int c = i == d.C ? CT : i;
+            pagd::Sum3 t;
+            for (int w = 0; w < kThr / 32; w++) {
+                t.add(red[(w * NV + c) * 2]);
+                t.add(red[(w * NV + c) * 2 + 1]);
+            }
+            float* row = a.part + (((size_t)b * gridDim.x + blockIdx.x) * nv + i) * 2;
+            row[0] = t.h;
+            row[1] = t.m;
+        }
+    }
+    if constexpr (MODE == T_BACK0) {
+        constexpr int NV = 3 * CT;
+        const int nv = 3 * d.C;
 #pragma unroll
         for (int c = 0; c < NV; c++) {
-            float v;
-            if constexpr (MODE == T_LOSS) v = qacc[c];
-            else v = pacc[c % 3][c / 3];
+            float v = pacc[c % 3][c / 3];
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (lane == 0) red[warp * NV + c] = v;
         }
-        if constexpr (MODE == T_LOSS) {
-            for (int o = 16; o > 0; o >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, o);
-            if (lane == 0) atomicAdd(a.loss, lacc * (0.5 * a.dscale));
-        }
         __syncthreads();
         for (int i = tid; i < nv; i += kThr) {
-            const int c = (MODE == T_LOSS && i == d.C) ? CT : i;
             float v = 0.f;
-            for (int w = 0; w < kThr / 32; w++) v += red[w * NV + c];
+            for (int w = 0; w < kThr / 32; w++) v += red[w * NV + i];
             a.part[((size_t)b * gridDim.x + blockIdx.x) * nv + i] = v;
         }
     }
@@ -658,15 +708,19 @@ __global__ void __launch_bounds__(kThr) k_wgrad(SnoDims d, const float* dz, cons
     }
 }
 
-// out[col(j)] = sum over rows of part[row][j], without loss (Sum3); lift: the
-// partials [C][3] = (dP0, dP1, db) go to the layout P [C][2], b_P [C]
+// out[col(j)] = sum over rows of part[row][j], without loss (Sum3), of `words`
+// words each; lift: the partials [C][3] = (dP0, dP1, db) go to the layout P [C][2], b_P [C]
 constexpr int kSumThr = 1024;
-__global__ void __launch_bounds__(kSumThr) k_sum_rows(const float* part, int rows, int cols, float* out, int lift) {
+__global__ void __launch_bounds__(kSumThr) k_sum_rows(const float* part, int rows, int cols, int words, float* out, int lift) {
     __shared__ float red[3][kSumThr / 32][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
     pagd::Sum3 s;
     if (j < cols)
-        for (int r = w; r < rows; r += kSumThr / 32) s.add(part[(size_t)r * cols + j]);
+        for (int r = w; r < rows; r += kSumThr / 32) {
+            const float* p = part + ((size_t)r * cols + j) * words;
+            s.add(p[0]);
+            if (words > 1) s.add(p[1]);
+        }
     red[0][w][lane] = s.h;
     red[1][w][lane] = s.m;
     red[2][w][lane] = s.l;
@@ -741,7 +795,7 @@ static void plan(sno_net* s) {
     s->off_dz = take(sizeof(float) * B * d.C * np);
     s->off_dz2 = take(sizeof(float) * B * d.C * np);
     const size_t rows = B * std::max<size_t>((size_t)d.NT, (np + kTile - 1) / kTile);
-    s->off_part = take(sizeof(float) * rows * std::max<size_t>((size_t)d.C * d.C + d.C, (size_t)3 * d.C));
+    s->off_part = take(sizeof(float) * rows * std::max<size_t>({(size_t)d.C * d.C + d.C, (size_t)3 * d.C, (size_t)2 * (d.C + 1)}));
     s->off_dF = take(sizeof(float2) * B * d.C * d.M);
     s->off_loss = take(sizeof(double));
     s->off_tw0 = take(sizeof(float2) * d.n0);
@@ -956,10 +1010,10 @@ pagd_status sno_loss_grad(sno_net* s, const float* params, const double* un, con
     // last layer, projection, loss, and the way back to dz of the last layer
     a.vout = dz;
     CK(tile<T_LOSS>(d, a, B, st));
-    auto sum_rows = [&](int rows, int cols, float* out, int lift) {
-        k_sum_rows<<<(cols + 31) / 32, kSumThr, 0, st>>>(part, rows, cols, out, lift);
+    auto sum_rows = [&](int rows, int cols, int words, float* out, int lift) {
+        k_sum_rows<<<(cols + 31) / 32, kSumThr, 0, st>>>(part, rows, cols, words, out, lift);
     };
-    sum_rows(tiles, d.C + 1, grad + off_Q(d), 0);
+    sum_rows(tiles, d.C + 1, 2, grad + off_Q(d), 0);
     a.G = dF;
     for (int l = d.L - 1; l >= 0; l--) {
         float* gL = grad + off_layer(d, l);
@@ -969,7 +1023,7 @@ pagd_status sno_loss_grad(sno_net* s, const float* params, const double* un, con
                                                               gL + nrow, dF, B);
         if (d.C <= 16) CK(launch_wgrad<16>(d, dz, v + (size_t)l * vs, part, B, st));
         else CK(launch_wgrad<32>(d, dz, v + (size_t)l * vs, part, B, st));
-        sum_rows(wrows, nrow, gL, 0);
+        sum_rows(wrows, nrow, 1, gL, 0);
         a.vin = dz;
         a.vout = dz2;
         if (l > 0) {
@@ -980,7 +1034,7 @@ pagd_status sno_loss_grad(sno_net* s, const float* params, const double* un, con
         }
         std::swap(dz, dz2);
     }
-    sum_rows(tiles, 3 * d.C, grad, d.C);
+    sum_rows(tiles, 3 * d.C, 1, grad, d.C);
     CK(cudaGetLastError());
     if (loss) CK(cudaMemcpyAsync(loss, dloss, sizeof(double), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
