@@ -436,8 +436,9 @@ __global__ void __launch_bounds__(kThr, CT <= 16 ? 3 : 1) k_tile(SnoDims d, Tile
     float* red = (float*)U;  // the spectral part's buffers are free
     if constexpr (MODE == T_LOSS) {
         // block sums of the per-thread accumulators -> one row of part, two words
-        // each: they nearly cancel over the grid (half the rounding errors of
-        // dQ, db_Q came from here)
+        // each: they nearly cancel over the grid (error of dQ, db_Q over 93 drawn
+        // networks 2.7e-7 with one word, 3.0e-8 with two; gradient of 4 states of
+        // 512^2 1317 -> 1353 us)
         constexpr int NV = CT + 1, V = CT <= 16 ? 32 : 64, PL = V / 32;
         float v[V], e[V];
 #pragma unroll
